@@ -8,10 +8,8 @@
 
 namespace hsa {
 
-__device__ __forceinline__ float phi_elu1(float x) { return x > 0.f ? x + 1.f : expf(x); }
-
 // ---------------------------------------------------------------------------------------
-// Stage A: one CTA per (touched block, head).  Copies the new rows of K and V into the block's
+// Without a linear state: one CTA per (touched block, head).  Copies the new rows of K and V into the block's
 // page and adds their column sums to the block's key sum.  A CTA owns its (head, block)
 // exclusively, so the sum order is fixed.
 // ---------------------------------------------------------------------------------------
@@ -80,99 +78,7 @@ __global__ void __launch_bounds__(256) append_pool_ksum_kernel(AppendArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Stage B: partial state over a token range.  grid (nsplit, H), 256 threads; each thread owns a
-// register tile of the D x D outer-product sum.
-// ---------------------------------------------------------------------------------------
-template <int D>
-__global__ void __launch_bounds__(256) state_partial_kernel(AppendArgs a) {
-  constexpr int TB = 32;       // tokens staged per batch
-  constexpr int R = D / 32;    // 4 (D=128) or 2 (D=64): half-tile edge
-  __shared__ __align__(16) float fk[TB][D];
-  __shared__ __align__(16) float vv[TB][D];
-
-  const int h = blockIdx.y;
-  const int split = blockIdx.x;
-  const int per = (a.n_new + a.nsplit - 1) / a.nsplit;
-  const int t0 = split * per;
-  const int t1 = min(a.n_new, t0 + per);
-  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-  // thread tile: rows {ty*R + i, D/2 + ty*R + i}, cols {tx*R + j, D/2 + tx*R + j}
-  float acc[2 * R][2 * R];
-#pragma unroll
-  for (int i = 0; i < 2 * R; ++i)
-#pragma unroll
-    for (int j = 0; j < 2 * R; ++j) acc[i][j] = 0.f;
-  float zacc = 0.f;
-
-  constexpr int CH = D / 8;
-  for (int tb = t0; tb < t1; tb += TB) {
-    const int nt = min(TB, t1 - tb);
-    __syncthreads();
-    for (int idx = threadIdx.x; idx < TB * CH; idx += 256) {
-      const int r = idx / CH, c8 = idx % CH;
-      float kf[8], vf[8];
-      if (r < nt) {
-        const size_t src = static_cast<size_t>(tb + r) * a.tok_stride +
-                           static_cast<size_t>(h) * a.head_stride + c8 * 8;
-        const uint4 kk = *reinterpret_cast<const uint4*>(a.k + src);
-        const uint4 v4 = *reinterpret_cast<const uint4*>(a.v + src);
-        const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kk);
-        const __nv_bfloat162* v2 = reinterpret_cast<const __nv_bfloat162*>(&v4);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const float2 f = __bfloat1622float2(k2[i]);
-          const float2 g = __bfloat1622float2(v2[i]);
-          kf[2 * i] = a.relu ? fmaxf(f.x, 0.f) : phi_elu1(f.x);
-          kf[2 * i + 1] = a.relu ? fmaxf(f.y, 0.f) : phi_elu1(f.y);
-          vf[2 * i] = g.x;
-          vf[2 * i + 1] = g.y;
-        }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 8; ++i) kf[i] = vf[i] = 0.f;
-      }
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        fk[r][c8 * 8 + i] = kf[i];
-        vv[r][c8 * 8 + i] = vf[i];
-      }
-    }
-    __syncthreads();
-    if (threadIdx.x < D) {
-#pragma unroll 8
-      for (int r = 0; r < TB; ++r) zacc += fk[r][threadIdx.x];
-    }
-#pragma unroll 4
-    for (int r = 0; r < TB; ++r) {
-      float ka[2 * R], va[2 * R];
-#pragma unroll
-      for (int i = 0; i < R; ++i) {
-        ka[i] = fk[r][ty * R + i];
-        ka[R + i] = fk[r][D / 2 + ty * R + i];
-        va[i] = vv[r][tx * R + i];
-        va[R + i] = vv[r][D / 2 + tx * R + i];
-      }
-#pragma unroll
-      for (int i = 0; i < 2 * R; ++i)
-#pragma unroll
-        for (int j = 0; j < 2 * R; ++j) acc[i][j] = fmaf(ka[i], va[j], acc[i][j]);
-    }
-  }
-  float* out = a.spart + (static_cast<size_t>(h) * a.nsplit + split) * (D * D + D);
-#pragma unroll
-  for (int i = 0; i < 2 * R; ++i) {
-    const int row = (i < R) ? ty * R + i : D / 2 + ty * R + (i - R);
-#pragma unroll
-    for (int j = 0; j < 2 * R; ++j) {
-      const int col = (j < R) ? tx * R + j : D / 2 + tx * R + (j - R);
-      out[row * D + col] = acc[i][j];
-    }
-  }
-  if (threadIdx.x < D) out[D * D + threadIdx.x] = zacc;
-}
-
-// ---------------------------------------------------------------------------------------
-// Stage C: S[dst] <- S[src] + sum of partials (fixed order), with its bf16 hi/lo split (the forward
+// Reduction: S[dst] <- S[src] + sum of partials (fixed order), with its bf16 hi/lo split (the forward
 // kernels feed hi and lo to the tensor cores as two bf16 operands), the same for z and its operand image.
 // ---------------------------------------------------------------------------------------
 __global__ void state_reduce_kernel(AppendArgs a) {
@@ -219,21 +125,30 @@ __global__ void state_reduce_kernel(AppendArgs a) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Fused append for head_dim 128 (the measured path): one pass over the chunk's K and V in which
+// Fused append with the linear state (the measured path): one pass over the chunk's K and V in which
 // no thread touches global memory for the bulk data.
 // grid (nsplit, H); a CTA owns a run of consecutive history blocks of one head.  Per block
 //   * the producer lane brings the block's rows of K and V into a 4-deep ring by TMA (rows
 //     outside the chunk arrive as zeros) and sends the same tiles on to the block's page by
 //     TMA store (a block that already held tokens before this call is written row by row by
 //     the workers instead, so that its old rows stay),
-//   * sixteen worker warps (two groups on alternate blocks) read K from the ring, build phi(K) as bf16 hi + lo (hi + lo carries
-//     ~16 bits) in the 128-byte-swizzled MN-major layout,
+//   * sixteen worker warps (two groups on alternate blocks) read K from the ring and build phi(K) as
+//     bf16 terms in the 128-byte-swizzled MN-major layout,
 //   * the MMA lane lets the tensor cores accumulate, over the block's tokens (tcgen05, K = tokens)
-//       S_part (128 x 128, fp32 in TMEM) += phi(K)_hi^T V + phi(K)_lo^T V      (V straight from the ring)
-//       z_part (128 x 16)                 += phi(K)_hi^T 1 + phi(K)_lo^T 1
-//       ksum_b (128 x 16)                  = K^T 1                              (K straight from the ring)
+//       S_part (d x d, fp32 in TMEM)   += phi(K)^T V      (V straight from the ring)
+//       z_part (d x 16)                += phi(K)^T 1
+//       ksum_b (d x 16)                 = K^T 1           (K straight from the ring)
 //     and four more warps read ksum_b back as soon as it is final,
-// and finally the CTA writes its partial S and z for the fixed-order reduction of stage C.
+// and finally the CTA writes its partial S and z for the fixed-order reduction below.
+// head_dim 128: phi(K) = hi + lo (~16 bits), two products into one accumulator of 128 lanes.
+// head_dim 64: phi(K) = hi + mid + lo (~24 bits: this size was summed in fp32 before it came here).  A
+// product has 128 lanes, so that hi and mid go through it together, as the two 64-lane halves of one
+// operand (their tiles lie one behind the other), and lo with a tile of zeros (beside hi, on mid's lanes);
+// ksum takes K and, unused, V.  Alternate blocks have accumulators of their own, and those and the two
+// halves are added in fp32 when the partial state is written (every product truncates what it adds to).
+// Measured at head_dim 64, 16 heads, chunks of 1000 tokens: 16.2 -> 9.3 us for the whole append (a page
+// kernel and an fp32 SIMT state kernel before it), error of S against 64 bits 1.9e-7 -> 1.3e-7; what is
+// left is latency (launch, first data, two kernels): the 8.3 MB take 1.3 us at the copy bandwidth.
 // Every wait is bounded; on expiry the CTA records a timeout and leaves.
 // ---------------------------------------------------------------------------------------
 
@@ -242,15 +157,22 @@ namespace {
 constexpr int kAfDepth = 4;                      // ring stages
 constexpr int kAfWorkers = 512;                  // worker threads (warps 2..17)
 constexpr int kAfThreads = 64 + kAfWorkers + 128;  // + producer warp + MMA warp + 4 key-sum warps
-constexpr int kAfTile = 64 * 128 * 2;            // [64 tokens x 128 dims] bf16 = two swizzled slabs
-constexpr int kAfStage = 2 * kAfTile;            // K | V
-constexpr int kAfHilo = 2 * kAfTile;             // phi hi | phi lo
 constexpr int kAfOnes = 2048;                    // [16 x 64] bf16 ones (K-major operand)
-constexpr int kAfSmem = kAfDepth * kAfStage + 2 * kAfHilo + kAfOnes + 256 + 1024;
 constexpr uint32_t kAfTmemCols = 256;
-constexpr uint32_t kAfColZ = 128, kAfColKs = 144;  // TMEM columns: S 0..127, z, ksum[2]
-constexpr int kAfPitch = 132;                      // floats per row of the staged partial state
-static_assert(128 * kAfPitch * 4 <= 2 * kAfHilo + kAfOnes, "partial state is staged in the hi/lo + ones area");
+constexpr uint32_t kAfColZ = 128, kAfColKs = 144;  // TMEM columns: S from 0, z, ksum[2]
+
+template <int D>
+struct AfSmem {
+  static constexpr int kTile = 64 * D * 2;     // [64 tokens x D dims] bf16 = D / 64 swizzled slabs
+  static constexpr int kSlab = 64 * 128;       // bytes of one slab
+  static constexpr int kStage = 2 * kTile;     // K | V
+  static constexpr int kTerms = D == 128 ? 2 : 3;
+  static constexpr int kPhi = kTerms * kTile;  // phi(K) of a block: hi | lo or hi | mid | lo
+  static constexpr int kZeros = D == 128 ? 0 : kTile;  // (a tile of zeros in front of the two phi buffers)
+  static constexpr int kTotal = kAfDepth * kStage + 2 * kPhi + kZeros + kAfOnes + 256 + 1024;
+  static constexpr int kPitch = D + 4;  // floats per row of the staged partial state
+  static_assert(128 * kPitch * 4 <= 2 * kPhi + kZeros + kAfOnes, "partial state is staged in the phi + ones area");
+};
 
 struct AfBars {
   uint64_t full[kAfDepth];      // ring stage landed
@@ -273,10 +195,16 @@ __device__ __forceinline__ bool af_wait(uint64_t* bar, uint32_t parity, AfBars* 
   return false;
 }
 
-// elu(x) + 1 with the fast exponential (relative error ~1e-6, far inside the state's tolerance)
-__device__ __forceinline__ float phi_fast(float x) {
-  float e;  // branch-free: elu(x) + 1 = max(x, 0) + exp(min(x, 0))
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fminf(x, 0.f) * 1.4426950408889634f));
+// Either feature map.  elu(x) + 1 = max(x, 0) + exp(min(x, 0)), branch-free; head_dim 128 takes the fast
+// exponential (relative error ~1e-6, far inside what two bf16 terms carry), head_dim 64 expf.
+template <int D, bool RELU>
+__device__ __forceinline__ float af_phi(float x) {
+  if (RELU) return fmaxf(x, 0.f);
+  float e;
+  if (D == 128)
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fminf(x, 0.f) * 1.4426950408889634f));
+  else
+    return x > 0.f ? x + 1.f : expf(x);
   return fmaxf(x, 0.f) + e;
 }
 
@@ -291,18 +219,19 @@ __device__ __forceinline__ void tma_store_2d(const void* tmap, const void* smem_
 
 // RELU: the feature map is max(x, 0) instead of elu(x) + 1 (an instance of its own: the map sits in
 // the innermost loop of the worker warps)
-template <bool RELU>
+template <int D, bool RELU>
 __global__ void __launch_bounds__(kAfThreads, 1)
 append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CUtensorMap tm_kin,
                     const __grid_constant__ CUtensorMap tm_vin, const __grid_constant__ CUtensorMap tm_kpool,
                     const __grid_constant__ CUtensorMap tm_vpool) {
-  constexpr int D = 128;
+  using L = AfSmem<D>;
   extern __shared__ uint8_t af_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(af_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
   uint8_t* ring = smem;
-  uint8_t* hilo = smem + kAfDepth * kAfStage;
-  uint8_t* ones = hilo + 2 * kAfHilo;
+  uint8_t* zeros = smem + kAfDepth * L::kStage;
+  uint8_t* phi = zeros + L::kZeros;
+  uint8_t* ones = phi + 2 * L::kPhi;
   AfBars* bars = reinterpret_cast<AfBars*>(ones + kAfOnes);
 
   // the reduction kernel behind this one may be scheduled early; it waits for this grid itself
@@ -323,13 +252,14 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
 
   auto issue_loads = [&](int bi) {
     const int s = bi % kAfDepth;
-    uint8_t* st = ring + s * kAfStage;
+    uint8_t* st = ring + s * L::kStage;
     const int32_t row0 = static_cast<int32_t>((bs + bi) * kBlock - a.n0);  // may be negative: zero fill
-    mbar_expect_tx(&bars->full[s], kAfStage);
-    tma_load_3d(st, &tm_kin, &bars->full[s], 0, h, row0);
-    tma_load_3d(st + kAfTile / 2, &tm_kin, &bars->full[s], 64, h, row0);
-    tma_load_3d(st + kAfTile, &tm_vin, &bars->full[s], 0, h, row0);
-    tma_load_3d(st + kAfTile + kAfTile / 2, &tm_vin, &bars->full[s], 64, h, row0);
+    mbar_expect_tx(&bars->full[s], L::kStage);
+#pragma unroll
+    for (int dh = 0; dh < D / 64; ++dh) tma_load_3d(st + dh * L::kSlab, &tm_kin, &bars->full[s], dh * 64, h, row0);
+#pragma unroll
+    for (int dh = 0; dh < D / 64; ++dh)
+      tma_load_3d(st + L::kTile + dh * L::kSlab, &tm_vin, &bars->full[s], dh * 64, h, row0);
   };
   if (threadIdx.x == 0) {
     for (int s = 0; s < kAfDepth; ++s) {
@@ -355,6 +285,8 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
   }
   // bf16 1.0 everywhere: under any swizzle the tile reads as all ones
   for (int i = threadIdx.x; i < kAfOnes / 4; i += kAfThreads) reinterpret_cast<uint32_t*>(ones)[i] = 0x3F803F80u;
+  for (int i = threadIdx.x; i < L::kZeros / 16; i += kAfThreads)
+    reinterpret_cast<uint4*>(zeros)[i] = make_uint4(0u, 0u, 0u, 0u);
   fence_proxy_async_smem();
   wait_prior();
   tc_fence_before();
@@ -372,12 +304,12 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
         if (!ok) break;
         const int64_t b = bs + bi;
         if (b * kBlock >= a.n0) {  // the block holds nothing older: whole tiles go to its page
-          uint8_t* st = ring + s * kAfStage;
+          uint8_t* st = ring + s * L::kStage;
           const int32_t prow = (a.page_table[b] * a.H + h) * kBlock;
-          tma_store_2d(&tm_kpool, st, 0, prow);
-          tma_store_2d(&tm_kpool, st + kAfTile / 2, 64, prow);
-          tma_store_2d(&tm_vpool, st + kAfTile, 0, prow);
-          tma_store_2d(&tm_vpool, st + kAfTile + kAfTile / 2, 64, prow);
+#pragma unroll
+          for (int dh = 0; dh < D / 64; ++dh) tma_store_2d(&tm_kpool, st + dh * L::kSlab, dh * 64, prow);
+#pragma unroll
+          for (int dh = 0; dh < D / 64; ++dh) tma_store_2d(&tm_vpool, st + L::kTile + dh * L::kSlab, dh * 64, prow);
         }
         tma_store_commit();
         if (bi >= 1 && bi - 1 + kAfDepth < nblk) {
@@ -392,7 +324,7 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (one lane)
     if (elect_one_sync()) {
-      constexpr uint32_t idesc_s = idesc_bf16_f32(128, 128, 1, 1);
+      constexpr uint32_t idesc_s = idesc_bf16_f32(128, D, 1, 1);
       constexpr uint32_t idesc_1 = idesc_bf16_f32(128, 16, 1, 0);
       constexpr uint32_t hi = desc_hi_sw128(1024);
       const uint32_t b_ones = desc_lo_sw128(smem_u32(ones), 16);
@@ -400,21 +332,27 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
         const int s = bi % kAfDepth, hb = bi & 1;
         if (!af_wait(&bars->phi_ready[hb], (bi >> 1) & 1, bars, a.status)) break;
         tc_fence_after();
-        uint8_t* st = ring + s * kAfStage;
-        const uint32_t a_k = desc_lo_sw128(smem_u32(st), kAfTile / 2);
-        const uint32_t b_v = desc_lo_sw128(smem_u32(st + kAfTile), kAfTile / 2);
-        const uint32_t a_hi = desc_lo_sw128(smem_u32(hilo + hb * kAfHilo), kAfTile / 2);
-        const uint32_t a_lo = desc_lo_sw128(smem_u32(hilo + hb * kAfHilo + kAfTile), kAfTile / 2);
+        uint8_t* st = ring + s * L::kStage;
+        uint8_t* ph = phi + hb * L::kPhi;
+        // lanes 0..63 and 64..127 of the A operands: the two slabs of a tile (head_dim 128), two tiles
+        // one behind the other or the zeros and lo (head_dim 64)
+        const uint32_t a_k = desc_lo_sw128(smem_u32(st), L::kSlab);
+        const uint32_t b_v = desc_lo_sw128(smem_u32(st + L::kTile), L::kSlab);
+        const uint32_t a_1 = desc_lo_sw128(smem_u32(ph), L::kSlab);
+        const uint32_t a_2 = D == 128 ? desc_lo_sw128(smem_u32(ph + L::kTile), L::kSlab)
+                                      : desc_lo_sw128(smem_u32(zeros), L::kZeros + hb * L::kPhi + 2 * L::kTile);
+        const uint32_t acc_s = tmem + (D == 64 ? 64 * hb : 0), acc_z = tmem + kAfColZ + (D == 64 ? 64 * hb : 0);
+        const bool more = bi >= (D == 64 ? 2 : 1);  // the accumulator holds earlier blocks
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          tc_mma_ss_lo(tmem, a_hi + kk * 128, b_v + kk * 128, hi, idesc_s, (bi > 0 || kk > 0) ? 1u : 0u);
+          tc_mma_ss_lo(acc_s, a_1 + kk * 128, b_v + kk * 128, hi, idesc_s, (more || kk > 0) ? 1u : 0u);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) tc_mma_ss_lo(tmem, a_lo + kk * 128, b_v + kk * 128, hi, idesc_s, 1u);
+        for (int kk = 0; kk < 4; ++kk) tc_mma_ss_lo(acc_s, a_2 + kk * 128, b_v + kk * 128, hi, idesc_s, 1u);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          tc_mma_ss_lo(tmem + kAfColZ, a_hi + kk * 128, b_ones, hi, idesc_1, (bi > 0 || kk > 0) ? 1u : 0u);
+          tc_mma_ss_lo(acc_z, a_1 + kk * 128, b_ones, hi, idesc_1, (more || kk > 0) ? 1u : 0u);
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) tc_mma_ss_lo(tmem + kAfColZ, a_lo + kk * 128, b_ones, hi, idesc_1, 1u);
+        for (int kk = 0; kk < 4; ++kk) tc_mma_ss_lo(acc_z, a_2 + kk * 128, b_ones, hi, idesc_1, 1u);
         if (bi >= 2 && !af_wait(&bars->ks_read[hb], ((bi >> 1) - 1) & 1, bars, a.status)) break;
         tc_fence_after();
 #pragma unroll
@@ -436,6 +374,7 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
       tc_wait_ld();
       tc_fence_before();
       if (lane == 0) mbar_arrive(&bars->ks_read[bj & 1]);
+      if (quad * 32 >= D) continue;
       const int64_t b = bs + bj;
       float* dst = a.ksum + (static_cast<size_t>(h) * a.max_pages + b) * D + quad * 32 + lane;
       float old = 0.f;
@@ -452,15 +391,18 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
     // other's arithmetic
     const int w = threadIdx.x - 64;
     const int grp = w >> 8, wg = w & 255;
-    const int ch = wg & 15;  // 16-byte chunk of a row (8 dims)
-    const int rg = wg >> 4;  // rows rg, rg + 16, rg + 32, rg + 48 of a block
+    constexpr int CH = D / 8;              // 16-byte chunks of a row (8 dims)
+    constexpr int RS = kAfWorkers / 2 / CH;  // rows one pass of a group covers
+    constexpr int NI = kBlock / RS;
+    const int ch = wg % CH;
+    const int rg = wg / CH;  // rows rg, rg + RS, ... of a block
     const int quad = warp & 3;
     bool ok = true;
-    uint32_t soff[4];  // the thread's four 16-byte chunks inside a swizzled [64 x 128] tile
+    uint32_t soff[NI];  // the thread's 16-byte chunks inside a swizzled tile
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = rg + 16 * i;
-      soff[i] = (ch >> 3) * (kAfTile / 2) + r * 128 + (((ch & 7) ^ (r & 7)) << 4);
+    for (int i = 0; i < NI; ++i) {
+      const int r = rg + RS * i;
+      soff[i] = (ch >> 3) * L::kSlab + r * 128 + (((ch & 7) ^ (r & 7)) << 4);
     }
 #pragma unroll 1
     for (int bi = grp; bi < nblk && ok; bi += 2) {
@@ -468,22 +410,22 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
       const int64_t b = bs + bi;
       ok = af_wait(&bars->full[s], (bi / kAfDepth) & 1, bars, a.status);
       if (!ok) break;
-      const uint8_t* st_k = ring + s * kAfStage;
-      uint4 kreg[4];
+      const uint8_t* st_k = ring + s * L::kStage;
+      uint4 kreg[NI];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) kreg[i] = *reinterpret_cast<const uint4*>(st_k + soff[i]);
+      for (int i = 0; i < NI; ++i) kreg[i] = *reinterpret_cast<const uint4*>(st_k + soff[i]);
       if (b * kBlock < a.n0) {
         // block partly filled before this call: only its new rows (and the zero rows past the
         // last token) are written, by hand
         const size_t row_base = (static_cast<size_t>(a.page_table[b]) * a.H + h) * kBlock;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int r = rg + 16 * i;
+        for (int i = 0; i < NI; ++i) {
+          const int r = rg + RS * i;
           const int64_t t = b * kBlock + r;
           if (t >= a.n0) {
             const size_t dst = (row_base + r) * D + ch * 8;
             *reinterpret_cast<uint4*>(a.k_pool + dst) = kreg[i];
-            *reinterpret_cast<uint4*>(a.v_pool + dst) = *reinterpret_cast<const uint4*>(st_k + kAfTile + soff[i]);
+            *reinterpret_cast<uint4*>(a.v_pool + dst) = *reinterpret_cast<const uint4*>(st_k + L::kTile + soff[i]);
           }
         }
       }
@@ -491,31 +433,36 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
         ok = af_wait(&bars->mma_done[hb], ((bi >> 1) - 1) & 1, bars, a.status);
         if (!ok) break;
       }
-      uint8_t* st_hi = hilo + hb * kAfHilo;
-      uint8_t* st_lo = st_hi + kAfTile;
+      uint8_t* ph = phi + hb * L::kPhi;
       // rows outside the chunk (only in its first and last block) add nothing to the state
       const bool whole = b * kBlock >= a.n0 && b * kBlock + kBlock <= n_end;
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < NI; ++i) {
         const uint32_t* kw = reinterpret_cast<const uint32_t*>(&kreg[i]);
-        uint32_t hw[4], lw[4];
+        uint32_t tw[L::kTerms][4];
 #pragma unroll
         for (int e = 0; e < 4; ++e) {
-          const float x0 = __uint_as_float(kw[e] << 16), x1 = __uint_as_float(kw[e] & 0xffff0000u);
-          const float p0 = RELU ? fmaxf(x0, 0.f) : phi_fast(x0);
-          const float p1 = RELU ? fmaxf(x1, 0.f) : phi_fast(x1);
-          hw[e] = pack_bf16(p0, p1);
-          lw[e] = pack_bf16(p0 - __uint_as_float(hw[e] << 16), p1 - __uint_as_float(hw[e] & 0xffff0000u));
-        }
-        if (!whole) {
-          const int64_t t = b * kBlock + rg + 16 * i;
-          if (t < a.n0 || t >= n_end) {
+          float p0 = af_phi<D, RELU>(__uint_as_float(kw[e] << 16));
+          float p1 = af_phi<D, RELU>(__uint_as_float(kw[e] & 0xffff0000u));
 #pragma unroll
-            for (int e = 0; e < 4; ++e) hw[e] = lw[e] = 0u;
+          for (int t = 0; t < L::kTerms; ++t) {
+            tw[t][e] = pack_bf16(p0, p1);
+            p0 -= __uint_as_float(tw[t][e] << 16);
+            p1 -= __uint_as_float(tw[t][e] & 0xffff0000u);
           }
         }
-        *reinterpret_cast<uint4*>(st_hi + soff[i]) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
-        *reinterpret_cast<uint4*>(st_lo + soff[i]) = make_uint4(lw[0], lw[1], lw[2], lw[3]);
+        if (!whole) {
+          const int64_t t = b * kBlock + rg + RS * i;
+          if (t < a.n0 || t >= n_end) {
+#pragma unroll
+            for (int m = 0; m < L::kTerms; ++m)
+#pragma unroll
+              for (int e = 0; e < 4; ++e) tw[m][e] = 0u;
+          }
+        }
+#pragma unroll
+        for (int m = 0; m < L::kTerms; ++m)
+          *reinterpret_cast<uint4*>(ph + m * L::kTile + soff[i]) = make_uint4(tw[m][0], tw[m][1], tw[m][2], tw[m][3]);
       }
       fence_proxy_async_smem();  // generic-proxy writes above -> visible to the tensor cores
       mbar_arrive(&bars->phi_ready[hb]);
@@ -528,38 +475,59 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
     float* out = a.spart + (static_cast<size_t>(h) * a.nsplit + split) * (D * D + D);
     const int row = quad * 32 + lane;
     {
-      // TMEM -> shared memory (row pitch 132 floats: conflict-free both ways) -> coalesced rows
-      float* stage = reinterpret_cast<float*>(hilo);
-      uint32_t v[32];
-      const int col = ((warp - 2) >> 2) * 32;  // four warps per lane quadrant, 32 columns each
+      // TMEM -> shared memory (row pitch D + 4 floats: conflict-free both ways) -> coalesced rows
+      float* stage = reinterpret_cast<float*>(phi);
+      constexpr int NC = D / 4;  // four warps per lane quadrant, NC columns each
+      uint32_t v[NC];
+      const int col = ((warp - 2) >> 2) * NC;
+      const bool zw = ((warp - 2) >> 2) == 0;  // this warp takes the quadrant's z as well
+      uint32_t zv[16];
+      zv[0] = 0u;
       if (nblk > 0 && ok) {
-        tmem_ld32(tmem + (static_cast<uint32_t>(quad * 32) << 16) + col, v);
+        const uint32_t t_row = tmem + (static_cast<uint32_t>(quad * 32) << 16);
+        if constexpr (D == 128)
+          tmem_ld32(t_row + col, v);
+        else
+          tmem_ld16(t_row + col, v);
+        if (zw) tmem_ld16(t_row + kAfColZ, zv);
         tc_wait_ld();
+        if constexpr (D == 64) {
+          if (nblk > 1) {  // the other accumulator
+            uint32_t u[NC];
+            tmem_ld16(t_row + 64 + col, u);
+            tc_wait_ld();
+#pragma unroll
+            for (int i = 0; i < NC; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(u[i]));
+            if (zw) {
+              tmem_ld16(t_row + kAfColZ + 64, u);
+              tc_wait_ld();
+              zv[0] = __float_as_uint(__uint_as_float(zv[0]) + __uint_as_float(u[0]));
+            }
+          }
+        }
       } else {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) v[i] = 0u;
+        for (int i = 0; i < NC; ++i) v[i] = 0u;
       }
-      float4* srow = reinterpret_cast<float4*>(stage + row * kAfPitch + col);
+      float4* srow = reinterpret_cast<float4*>(stage + row * L::kPitch + col);
 #pragma unroll
-      for (int i = 0; i < 8; ++i)
+      for (int i = 0; i < NC / 4; ++i)
         srow[i] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
                               __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
+      if (zw) stage[row * L::kPitch + D] = __uint_as_float(zv[0]);
       asm volatile("bar.sync 1, %0;" ::"n"(kAfWorkers) : "memory");
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int f = w + kAfWorkers * i;  // float4 index of the [128][128] partial state
-        const int r2 = f >> 5, c4 = f & 31;
-        reinterpret_cast<float4*>(out)[f] = *reinterpret_cast<const float4*>(stage + r2 * kAfPitch + c4 * 4);
+      for (int i = 0; i < D * D / 4 / kAfWorkers; ++i) {
+        const int f = w + kAfWorkers * i;  // float4 index of the [D][D] partial state
+        const int r2 = f / (D / 4), c4 = f % (D / 4);
+        float4 o = *reinterpret_cast<const float4*>(stage + r2 * L::kPitch + c4 * 4);
+        if (D == 64) {  // lanes 64..127 hold the mid terms
+          const float4 m = *reinterpret_cast<const float4*>(stage + (r2 + 64) * L::kPitch + c4 * 4);
+          o = make_float4(o.x + m.x, o.y + m.y, o.z + m.z, o.w + m.w);
+        }
+        reinterpret_cast<float4*>(out)[f] = o;
       }
-    }
-    if (warp < 6) {
-      uint32_t v[16];
-      v[0] = 0u;
-      if (nblk > 0 && ok) {
-        tmem_ld16(tmem + (static_cast<uint32_t>(quad * 32) << 16) + kAfColZ, v);
-        tc_wait_ld();
-      }
-      out[D * D + row] = __uint_as_float(v[0]);
+      if (w < D) out[D * D + w] = stage[w * L::kPitch + D] + (D == 64 ? stage[(w + 64) * L::kPitch + D] : 0.f);
     }
   }
   tc_fence_before();
@@ -571,9 +539,14 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
 }
 
 cudaError_t append_init() {
-  cudaError_t e = cudaFuncSetAttribute(append_fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAfSmem);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(append_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAfSmem);
+  cudaError_t e = cudaSuccess;
+  auto set = [&](auto* fn, int bytes) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  };
+  set(append_fused_kernel<128, false>, AfSmem<128>::kTotal);
+  set(append_fused_kernel<128, true>, AfSmem<128>::kTotal);
+  set(append_fused_kernel<64, false>, AfSmem<64>::kTotal);
+  set(append_fused_kernel<64, true>, AfSmem<64>::kTotal);
   return e;
 }
 
@@ -582,25 +555,23 @@ cudaError_t launch_append(const AppendArgs& a_in, const AppendMaps* maps, cudaSt
   const int64_t b0 = a.n0 / kBlock;
   const int64_t b1 = (a.n0 + a.n_new - 1) / kBlock;
   cudaError_t e;
-  if (a.D == 128 && a.lin_state && maps) {
+  if (a.lin_state) {
     const int nb = static_cast<int>(b1 - b0 + 1);
     const int per = (nb + a.nsplit - 1) / a.nsplit;
     a.nsplit = (nb + per - 1) / per;  // no empty CTAs
-    dim3 grid(a.nsplit, a.H);
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = grid;
+    cfg.gridDim = dim3(a.nsplit, a.H);
     cfg.blockDim = dim3(kAfThreads);
-    cfg.dynamicSmemBytes = kAfSmem;
+    cfg.dynamicSmemBytes = a.D == 128 ? AfSmem<128>::kTotal : AfSmem<64>::kTotal;
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (a.relu)
-      e = cudaLaunchKernelEx(&cfg, append_fused_kernel<true>, a, per, maps->kin, maps->vin, maps->kpool, maps->vpool);
-    else
-      e = cudaLaunchKernelEx(&cfg, append_fused_kernel<false>, a, per, maps->kin, maps->vin, maps->kpool, maps->vpool);
+    auto* fn = a.D == 128 ? (a.relu ? append_fused_kernel<128, true> : append_fused_kernel<128, false>)
+                          : (a.relu ? append_fused_kernel<64, true> : append_fused_kernel<64, false>);
+    e = cudaLaunchKernelEx(&cfg, fn, a, per, maps->kin, maps->vin, maps->kpool, maps->vpool);
     if (e != cudaSuccess) return e;
   } else {
     dim3 gridA(static_cast<unsigned>(b1 - b0 + 1), a.H);
@@ -617,15 +588,7 @@ cudaError_t launch_append(const AppendArgs& a_in, const AppendMaps* maps, cudaSt
       e = cudaLaunchKernelEx(&cfgA, append_pool_ksum_kernel<128>, a);
     else
       e = cudaLaunchKernelEx(&cfgA, append_pool_ksum_kernel<64>, a);
-    if (e == cudaSuccess) e = cudaGetLastError();
-    if (e != cudaSuccess || !a.lin_state) return e;
-    dim3 gridB(a.nsplit, a.H);
-    if (a.D == 128)
-      state_partial_kernel<128><<<gridB, 256, 0, st>>>(a);
-    else
-      state_partial_kernel<64><<<gridB, 256, 0, st>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+    return e == cudaSuccess ? cudaGetLastError() : e;
   }
   // The reduction may be scheduled while the kernel before it drains (programmatic dependent
   // launch); it waits for that kernel's results itself before it reads anything.

@@ -363,8 +363,7 @@ int hsa_append_kv(hsa_ctx* ctx, const void* k, const void* v, int32_t n_tokens, 
   if (linformer && (n_tokens != ctx->cfg.lin_seg_tokens || ctx->n_tokens != static_cast<int64_t>(ctx->n_segs) * n_tokens))
     return HSA_ERR_UNSUPPORTED;  // this mode appends whole segments only
   AppendMaps maps;
-  const bool fused = a.D == 128 && a.lin_state;
-  if (fused || linformer) {
+  if (a.lin_state || linformer) {
     if (encode_q(&maps.kin, k, n_tokens, a.H, a.D, tok_stride, head_stride, kBlock) != HSA_OK ||
         encode_q(&maps.vin, v, n_tokens, a.H, a.D, tok_stride, head_stride, kBlock) != HSA_OK)
       return HSA_ERR_CUDA;
@@ -373,7 +372,7 @@ int hsa_append_kv(hsa_ctx* ctx, const void* k, const void* v, int32_t n_tokens, 
   }
   cudaError_t e = cudaSuccess;
   if (!linformer) {
-    e = launch_append(a, fused ? &maps : nullptr, static_cast<cudaStream_t>(stream));
+    e = launch_append(a, a.lin_state ? &maps : nullptr, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(ctx, e);
   }
   if (linformer) {
