@@ -463,6 +463,13 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
 #pragma unroll
         for (int m = 0; m < L::kTerms; ++m)
           *reinterpret_cast<uint4*>(ph + m * L::kTile + soff[i]) = make_uint4(tw[m][0], tw[m][1], tw[m][2], tw[m][3]);
+        if (a.phik) {  // causal contexts: the first two terms of phi(K) stay for the chunk's own forward
+          const size_t row = (static_cast<size_t>(h) * 2 * a.phik_blocks + (b - b_first)) * kBlock + rg + RS * i;
+#pragma unroll
+          for (int m = 0; m < 2; ++m)
+            *reinterpret_cast<uint4*>(a.phik + (row + static_cast<size_t>(m) * a.phik_blocks * kBlock) * D + ch * 8) =
+                make_uint4(tw[m][0], tw[m][1], tw[m][2], tw[m][3]);
+        }
       }
       fence_proxy_async_smem();  // generic-proxy writes above -> visible to the tensor cores
       mbar_arrive(&bars->phi_ready[hb]);

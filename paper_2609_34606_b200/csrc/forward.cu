@@ -197,7 +197,10 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   // read before the wait; the plain kernel does its set-up first, under that kernel's tail (a split
   // CTA may still leave without any set-up, so it sets up after it has seen its list).
   if (!SPLIT) setup();
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // wait_late: the kernel before this one supplies the causal partials only, which the epilogue reads;
+  // it let this grid start after it had itself waited for everything before it (lists, pages, state),
+  // so that the tiles' loops run on the SMs it has left already while its longest tiles finish
+  if (SPLIT || !p.wait_late) asm volatile("griddepcontrol.wait;" ::: "memory");
   int tile = blockIdx.x, h = blockIdx.y, part = blockIdx.z;
   // Parts of a list of `st` two-page steps.  balance > 0: the steps one SM would run if the whole
   // launch were spread evenly; a list is cut into the fewest parts none of which is longer than that
@@ -849,6 +852,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       // branch has not looked at Q at all: its TMA load may still be in flight and must land first.
       if (ok && epi && nsteps == 0 && (!p.do_linear || LINF))
         ok = __all_sync(0xffffffffu, wait_bar(&bars->q_full, 0, bars, p.status));
+      if (!SPLIT && p.wait_late) asm volatile("griddepcontrol.wait;" ::: "memory");  // the causal partials
       if (ok && epi && do_output) {  // warp-uniform: the TMEM loads below are warp-collective
         const bool wr = row < p.n_q;  // rows past the end of the chunk compute but never store
         float lin_den = den;

@@ -38,9 +38,10 @@ struct Layout {
   // state
   size_t S, z, slot_S, slot_z, hilo, zop, ksum_saved, ksum, state_total;  // S, z: slot 0; slot_*: bytes per slot
   // workspace
-  size_t status, page_table, qpart, keys, spart, lin_num, lin_den, ctable, csel, ccnt, olin, ad_w, ad_idx, ad_gini, ad_wsum,
+  size_t status, page_table, qpart, keys, spart, lin_num, lin_den, phik, ctable, csel, ccnt, olin, ad_w, ad_idx, ad_gini, ad_wsum,
       part_o, part_l, part_ref, part_ticket, ws_total;
   int fwd_splits, split_blocks;
+  int phik_blocks;  // pages a chunk can touch (causal contexts with a linear state, else 0)
   // Linformer
   size_t n_cpages, cpool;
 };
@@ -90,6 +91,10 @@ Layout make_layout(const hsa_config* c) {
   if (c->flags & HSA_CFG_CAUSAL) {
     L.lin_num = o;  o = align_up(o + static_cast<size_t>(c->max_q_tokens) * H * D * 4, 256);
     L.lin_den = o;  o = align_up(o + static_cast<size_t>(c->max_q_tokens) * H * 4, 256);
+    if (c->lin_mode == HSA_LIN_STATE) {
+      L.phik_blocks = (c->max_q_tokens + kBlock - 1) / kBlock + 1;
+      L.phik = o;   o = align_up(o + H * 2 * static_cast<size_t>(L.phik_blocks) * kBlock * D * 2, 256);
+    }
   }
   if (c->flags & HSA_CFG_ADAPTIVE) {
     L.ad_w = o;    o = align_up(o + H * tiles * P * 8, 256);
@@ -137,7 +142,7 @@ struct hsa_ctx {
   int cur_slot;         // state slot that holds the running state of the current history
   int64_t tail_saved_for;  // history length whose tail-block key sum sits in the saved-tail buffer (-1: none)
   int nsm;
-  CUtensorMap tm_k, tm_v, tm_state, tm_kc, tm_vc, tm_olin, tm_ek, tm_ev;
+  CUtensorMap tm_k, tm_v, tm_state, tm_kc, tm_vc, tm_olin, tm_ek, tm_ev, tm_phik;
   int32_t n_segs;  // Linformer: complete segments compressed so far
   std::vector<int32_t> page_table_host;  // history block -> physical page
   std::vector<uint8_t> resident;         // per history block: tiles present in the pool (tier migration)
@@ -282,6 +287,7 @@ int hsa_create(hsa_ctx** out, const hsa_config* cfg, const hsa_buffers* bufs,
   if (e == cudaSuccess) e = forward_init();
   if (e == cudaSuccess) e = append_init();
   if (e == cudaSuccess) e = linear_only_init();
+  if (e == cudaSuccess) e = causal_linear_init();
   if (e == cudaSuccess && linformer) {
     e = linformer_init();
     // identity page table and "every page" selection of the compressed pool
@@ -303,6 +309,8 @@ int hsa_create(hsa_ctx** out, const hsa_config* cfg, const hsa_buffers* bufs,
   if (r == HSA_OK)
     r = encode_2d_rows(&ctx->tm_state, static_cast<uint8_t*>(bufs->state) + ctx->lay.hilo,
                        static_cast<uint64_t>(cfg->num_heads) * 4 * D, D);
+  if (r == HSA_OK && ctx->lay.phik_blocks > 0)
+    r = encode_2d_rows(&ctx->tm_phik, ws + ctx->lay.phik, static_cast<uint64_t>(cfg->num_heads) * 2 * ctx->lay.phik_blocks * kBlock, D);
   if (r == HSA_OK && linformer) {
     const uint64_t crows = static_cast<uint64_t>(ctx->lay.n_cpages) * cfg->num_heads * kBlock;
     r = encode_2d_rows(&ctx->tm_kc, bufs->kc_pool, crows, D);
@@ -358,6 +366,8 @@ int hsa_append_kv(hsa_ctx* ctx, const void* k, const void* v, int32_t n_tokens, 
   a.nsplit = nsplit;
   a.lin_state = ctx->cfg.lin_mode == HSA_LIN_STATE;
   a.relu = ctx->cfg.feature_map == HSA_PHI_RELU;
+  a.phik_blocks = ctx->lay.phik_blocks;
+  a.phik = a.phik_blocks > 0 ? reinterpret_cast<__nv_bfloat16*>(ws + ctx->lay.phik) : nullptr;
   a.status = reinterpret_cast<int32_t*>(ws + ctx->lay.status);
   const bool linformer = ctx->cfg.lin_mode == HSA_LIN_LINFORMER;
   if (linformer && (n_tokens != ctx->cfg.lin_seg_tokens || ctx->n_tokens != static_cast<int64_t>(ctx->n_segs) * n_tokens))
@@ -603,12 +613,8 @@ int hsa_forward(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride, in
   }
   if (causal_lin) {
     CausalLinArgs c{};
-    c.q = static_cast<const __nv_bfloat16*>(q);
     c.n_q = n_q;
-    c.q_ts = tok_stride;
-    c.q_hs = head_stride;
-    c.k_pool = static_cast<const __nv_bfloat16*>(ctx->buf.k_pool);
-    c.v_pool = static_cast<const __nv_bfloat16*>(ctx->buf.v_pool);
+    c.phik_blocks = ctx->lay.phik_blocks;
     c.page_table = p.page_table;
     c.q_pos0 = q_pos0;
     c.n_tokens = ctx->n_tokens;
@@ -617,10 +623,12 @@ int hsa_forward(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride, in
     c.relu = p.relu;
     c.lin_num = reinterpret_cast<float*>(ws + ctx->lay.lin_num);
     c.lin_den = reinterpret_cast<float*>(ws + ctx->lay.lin_den);
-    cudaError_t e = launch_causal_linear(c, st);
+    c.status = p.status;
+    cudaError_t e = launch_causal_linear(c, tm_q, ctx->tm_phik, ctx->tm_v, st);
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     p.lin_num = c.lin_num;
     p.lin_den = c.lin_den;
+    p.wait_late = 1;
   }
   if (do_linformer && p.max_splits == 1 && D == 128) {
     // one launch: the kernel's loop runs over the compressed pool first (its own accumulator,

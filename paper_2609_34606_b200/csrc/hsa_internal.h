@@ -52,6 +52,10 @@ struct AppendArgs {
   int lin_state;  // update the linear state?
   int beside_prior;  // SIMT page write: may run beside the kernel launched just before it (see launch_append)
   int relu;       // feature map of the state: 0 elu(x) + 1, 1 max(x, 0)
+  // causal contexts: phi(K) of the chunk as bf16 hi and lo, [H][hi/lo][phik_blocks][64][D], block 0 being
+  // the chunk's first page (rows of that page before the chunk: zeros); null otherwise
+  __nv_bfloat16* phik;
+  int phik_blocks;
   int32_t* status;  // device status word
 };
 
@@ -124,6 +128,7 @@ struct FwdParams {
   int do_linear, do_sparse;
   const float* lin_num;  // causal intra-chunk partials [n_q][H][D] (or null)
   const float* lin_den;  // [n_q][H]
+  int wait_late;         // 1: the kernel before this one wrote lin_num and lin_den and nothing else this one reads
   const __nv_bfloat16* ext_lin;  // linear-branch output computed elsewhere, [n_q][H][D] (or null)
   // Linformer form inside the kernel: the loop first runs over the lf_pages pages of the compressed
   // pool (page ids through lf_table), with an accumulator and row sums of their own (null: none)
@@ -147,18 +152,16 @@ struct FwdParams {
 };
 
 struct CausalLinArgs {
-  const __nv_bfloat16* q;
   int n_q;
-  int64_t q_ts, q_hs;
-  const __nv_bfloat16* k_pool;
-  const __nv_bfloat16* v_pool;
   const int32_t* page_table;
+  int phik_blocks;  // blocks per (head, hi/lo) of the phi(K) tiles the chunk's append left (AppendArgs::phik)
   int64_t q_pos0;   // first query position == first token of the intra-chunk part
   int64_t n_tokens;
   int H, D;
   int relu;  // feature map: 0 elu(x) + 1, 1 max(x, 0)
   float* lin_num;
   float* lin_den;
+  int32_t* status;  // device status word
 };
 
 struct LinformerArgs {
@@ -201,7 +204,10 @@ cudaError_t launch_forward(const FwdParams& p, int D, const CUtensorMap& tm_q,
                            const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                            const CUtensorMap& tm_state, const CUtensorMap& tm_out, cudaStream_t st,
                            const CUtensorMap* tm_kc = nullptr, const CUtensorMap* tm_vc = nullptr);
-cudaError_t launch_causal_linear(const CausalLinArgs& a, cudaStream_t st);
+// tm_q: box of 128 tokens of one head; tm_phik, tm_v: rows of phi(K) and of the V pool, box 64 x 64
+cudaError_t launch_causal_linear(const CausalLinArgs& a, const CUtensorMap& tm_q, const CUtensorMap& tm_phik,
+                                 const CUtensorMap& tm_v, cudaStream_t st);
+cudaError_t causal_linear_init();
 // linear branch alone (head_dim 128): lean HBM-bound kernel, nsm = SMs of the device
 cudaError_t launch_linear_only(const FwdParams& p, int nsm, const CUtensorMap& tm_q, const CUtensorMap& tm_state,
                                const CUtensorMap& tm_out, cudaStream_t st);

@@ -1,12 +1,57 @@
 """Kernels at the sizes where they can go wrong: edges of tiles, remainders, the smallest and the largest
-of a range, against plain fp64 arithmetic on the identical bf16 inputs."""
+of a range, against the oracle or plain fp64 arithmetic on the identical bf16 inputs."""
+import numpy as np
 import pytest
 import torch
 
+import hsa_harness as Hn
+from oracle import hsa_oracle as O
+
 pytestmark = pytest.mark.gpu
+
+# largest error of a row that is computed in 32 bits and rounded to bf16 once: half a unit in the last of
+# 8 bits (2^-9 of the value) and, where a bf16 phi(q) is applied to the state, as much again
+BF16_REL = 2.0 ** -8
+
 
 def _randn(g, *shape):
     return torch.randn(*shape, generator=g).to(torch.bfloat16)
+
+
+@pytest.mark.parametrize("n0,n_q,d,relu", [
+    (0, 1, 128, 0), (0, 64, 128, 0), (0, 128, 128, 0), (0, 129, 128, 1), (64, 127, 128, 0), (63, 65, 128, 0),
+    (1, 257, 128, 0), (190, 385, 128, 1), (33, 640, 128, 0), (0, 1, 64, 0), (63, 130, 64, 0), (17, 300, 64, 1)])
+def test_causal_intra_chunk_products(n0, n_q, d, relu, cuda_device):
+    """Intra-chunk part of the causal linear branch (one tile, several tiles, a ragged last one; a chunk
+    that starts at, just before and just behind a page boundary) through both kernels that add it."""
+    from paper_2609_34606_b200 import hsa
+    H = 3
+    g = torch.Generator().manual_seed(1000 * n0 + n_q)
+    n = n0 + n_q
+    K, V, q = _randn(g, n, H, d), _randn(g, n, H, d), _randn(g, n_q, H, d)
+    n_blocks = (n + 63) // 64
+    ctx = hsa.HSAContext(H, d, max_pages=n_blocks + 1, max_q_tokens=max(n_q, n0, 1), max_topk=n_blocks, causal=True,
+                         device=cuda_device, feature_map=relu,
+                         page_order=torch.arange(n_blocks, -1, -1, dtype=torch.int32))
+    ctx.k_pool.fill_(0xFF)
+    ctx.v_pool.fill_(0xFF)
+    if n0:
+        ctx.append_kv(K[:n0].to(cuda_device), V[:n0].to(cuda_device))
+    ctx.append_kv(K[n0:].to(cuda_device), V[n0:].to(cuda_device))
+    qd = q.to(cuda_device)
+    budgets = torch.full((H,), -1, dtype=torch.int32, device=cuda_device)
+    idx, cnt = ctx.select_blocks(qd, budgets, q_pos0=n0, causal=True)
+    alone = ctx.forward(qd, idx, cnt, q_pos0=n0, causal=True, flags=hsa.HSA_FWD_NO_SPARSE)
+    both = ctx.forward(qd, idx, cnt, q_pos0=n0, causal=True)
+    assert ctx.device_status() == 0
+    fmap = "relu" if relu else "elu1"
+    lin = O.linear_parallel(Hn.f32(q), Hn.f32(K), Hn.f32(V), n0, True, fmap=fmap)
+    sp = O.dense_attention(Hn.f32(q), Hn.f32(K), Hn.f32(V), n0, True)
+    assert np.linalg.norm(Hn.f64(alone) - lin) <= BF16_REL * np.linalg.norm(lin)
+    ref = lin + sp
+    # (the sparse branch's weights are bf16 as well: one more rounding)
+    assert np.linalg.norm(Hn.f64(both) - ref) <= 1.5 * BF16_REL * np.linalg.norm(ref)
+    ctx.destroy()
 
 
 @pytest.mark.parametrize("n0,n,H,relu", [
