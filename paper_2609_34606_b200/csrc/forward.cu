@@ -158,13 +158,16 @@ __device__ __forceinline__ void init_barriers(Bars* bars) {
 
 // SPLIT: compiled with the split-tile path (grid z > 1); the plain kernel carries none of it
 // LINF: compiled with the compressed-pool segment in front of the selected pages (tm_kc, tm_vc)
-template <int D, bool SPLIT, bool LINF>
+// GT: per-dim gate logits arrive as tiles by TMA (tm_gl, tm_gs); an instance of its own, so that the others
+// keep their registers
+template <int D, bool SPLIT, bool LINF, bool GT>
 __global__ void __launch_bounds__(kThreads, 1)
 hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v,
                    const __grid_constant__ CUtensorMap tm_state,
                    const __grid_constant__ CUtensorMap tm_out, const __grid_constant__ CUtensorMap tm_kc,
-                   const __grid_constant__ CUtensorMap tm_vc, const FwdParams p) {
+                   const __grid_constant__ CUtensorMap tm_vc, const __grid_constant__ CUtensorMap tm_gl,
+                   const __grid_constant__ CUtensorMap tm_gs, const FwdParams p) {
   static_assert(!(SPLIT && LINF), "split lists and the compressed segment are not combined");
   constexpr int NSB = LINF ? 2 : kSBufs;                 // score buffers in use
   constexpr uint32_t kColSb = LINF ? 256 : kColS;        // first score buffer
@@ -279,6 +282,9 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   auto in_a = [&](int j) -> bool { return LINF && j < nA; };
   auto pages_of = [&](int j) -> int { return in_a(j) ? min(2, lf_pages - 2 * j) : min(2, cnt - 2 * (j - nA)); };
 
+  // K steps that pass through ring stage s: a gate tile is the next one of its stage
+  auto gate_uses = [&](int s) -> int { return nsteps > s ? (nsteps - 1 - s) / kStages + 1 : 0; };
+
   if (SPLIT) setup();
   const uint32_t tmem = bars->tmem_base;
 
@@ -319,6 +325,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           tma_load_3d(smem + L::kQ + dh * L::kHalf, &tm_q, &bars->q_full, dh * 64, h, row0);
         bool ok = true;
         int armed_k = 0, armed_v = 0;  // loads issued per ring, for the drain on abort
+        int gates_armed = 0;
         auto page_row = [&](int idx) -> int32_t {
           int blk = sel[idx];
           if (blk < 0 || blk >= p.n_blocks) {  // never follow a bad index into the pool
@@ -375,8 +382,24 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             ++armed_v;
           }
         }
+        if (GT && ok) {
+          // per-dim gates: the tile's logits follow the last K pages into stages 1 and 2 of the K ring
+          // (stage 0 holds the row statistics by then), ahead of the epilogue that applies them
+          for (int i = 0; i < 2 && ok; ++i) {
+            if ((p.gate_tiles & (1 << i)) == 0) continue;
+            const int s = 1 + i;
+            ok = wait_bar(&bars->k_empty[s], (gate_uses(s) & 1) ^ 1, bars, p.status);
+            if (!ok) break;
+            mbar_expect_tx(&bars->k_full[s], L::kTile);
+            for (int dh = 0; dh < DH; ++dh)
+              tma_load_3d(smem + L::kK + s * L::kTile + dh * L::kHalf, i == 0 ? &tm_gl : &tm_gs, &bars->k_full[s], dh * 64, h, row0);
+            gates_armed |= 1 << i;
+          }
+        }
         if (!ok) {
           // drain: let every copy already issued land before the CTA's shared memory goes away
+          for (int i = 0; i < 2; ++i)
+            if (gates_armed & (1 << i)) mbar_wait(&bars->k_full[1 + i], gate_uses(1 + i) & 1, 1u << 16);
           for (int s = 0; s < kStages; ++s) {
             for (int i = 0; i < 2; ++i) {
               const int arms = i == 0 ? armed_k : armed_v;
@@ -754,6 +777,28 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 
       // ---------------------------------------------------------------- epilogue
       // (this group's columns of the output row: group 0 -> [0, D/2), group 1 -> [D/2, D))
+      const bool sig = p.gate_act == 1;
+      auto gate_w = [&](float w0) -> float { return sig ? __fdividef(1.f, 1.f + __expf(-w0)) : w0; };
+      // 16 gate weights of this thread's row: two 16-byte chunks of a tile in the K ring
+      auto tile_gates16 = [&](int s, int c0, float (&w)[16]) {
+        const int cc = c0 >> 3;
+        const uint8_t* grow = smem + L::kK + s * L::kTile + (cc >> 3) * L::kHalf + r * 128;
+        const uint4 q0 = *reinterpret_cast<const uint4*>(grow + (((cc & 7) ^ (r & 7)) << 4));
+        const uint4 q1 = *reinterpret_cast<const uint4*>(grow + ((((cc + 1) & 7) ^ (r & 7)) << 4));
+        const uint32_t gw[8] = {q0.x, q0.y, q0.z, q0.w, q1.x, q1.y, q1.z, q1.w};
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          w[2 * i] = gate_w(__uint_as_float(gw[i] << 16));
+          w[2 * i + 1] = gate_w(__uint_as_float(gw[i] & 0xffff0000u));
+        }
+      };
+      // (every attempt and every part of a split list waits for the tiles: they must have landed before the
+      // barriers start over or the CTA leaves)
+      if (GT && ok) {
+        for (int i = 0; i < 2; ++i)
+          if (p.gate_tiles & (1 << i)) ok = ok && wait_bar(&bars->k_full[1 + i], gate_uses(1 + i) & 1, bars, p.status);
+        ok = __all_sync(0xffffffffu, ok);
+      }
       if (ok && nsteps > 0) {
         ok = __all_sync(0xffffffffu, wait_bar(&bars->o_done, 0, bars, p.status));
         tc_fence_after();
@@ -864,14 +909,21 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         // (relu: a row may have no weight at all, hence 1e-6 in its denominator; 0 / 1e-6 = 0)
         const float den_eps = lin_den + ((!LINF && p.relu) ? 1e-6f : 0.f);
         const float inv_den = (p.do_linear && den_eps > 0.f) ? 1.f / den_eps : 0.f;
+        // one gate per token and head: its weight is worked out once; per-dim gates: from the tiles in
+        // shared memory, or with any other strides value by value
+        float wl0 = 1.f, ws0 = 1.f;
+        if (wr && p.g_lin && p.g_ds == 0)
+          wl0 = gate_w(__bfloat162float(p.g_lin[static_cast<size_t>(row) * p.g_ts + static_cast<size_t>(h) * p.g_hs]));
+        if (wr && p.g_sp && p.g_ds == 0)
+          ws0 = gate_w(__bfloat162float(p.g_sp[static_cast<size_t>(row) * p.g_ts + static_cast<size_t>(h) * p.g_hs]));
+        const bool gather = wr && p.g_ds != 0;
         const __nv_bfloat16* gl =
-            (wr && p.g_lin) ? p.g_lin + static_cast<size_t>(row) * p.g_ts + static_cast<size_t>(h) * p.g_hs : nullptr;
+            (gather && p.g_lin && !(p.gate_tiles & 1)) ? p.g_lin + static_cast<size_t>(row) * p.g_ts + static_cast<size_t>(h) * p.g_hs : nullptr;
         const __nv_bfloat16* gs =
-            (wr && p.g_sp) ? p.g_sp + static_cast<size_t>(row) * p.g_ts + static_cast<size_t>(h) * p.g_hs : nullptr;
+            (gather && p.g_sp && !(p.gate_tiles & 2)) ? p.g_sp + static_cast<size_t>(row) * p.g_ts + static_cast<size_t>(h) * p.g_hs : nullptr;
         const __nv_bfloat16* ext =
             (wr && p.ext_lin) ? p.ext_lin + (static_cast<size_t>(row) * p.H + h) * D : nullptr;
-        const int g_ds = static_cast<int>(p.g_ds);
-        const bool sig = p.gate_act == 1;
+        const int64_t g_ds = p.g_ds;
         // (decided from the launch parameters, not from this thread's pointers: the branch holds
         // warp-collective TMEM loads and must not diverge inside a warp)
         const bool plain = !p.g_lin && !p.g_sp && !(p.do_linear && p.lin_num != nullptr) && !p.ext_lin &&
@@ -900,9 +952,44 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             }
           }
         }
+        // gate tiles without causal partials, external linear output or merge.  (Working the
+        // weights out ahead of the accumulators, in registers, needs the trips unrolled, and code that a
+        // CTA runs once is fetched cold: 176 us a pass against 164 with this loop, 12 heads of 128, 4680
+        // tokens; value by value from global memory, which this replaces: 207.)
+        const bool gated = GT && !(p.do_linear && p.lin_num != nullptr) && !p.ext_lin && !(SPLIT && nsplit > 1);
+        if (gated) {
+          const float il = has_o ? inv_l : 0.f, id = has_lin ? inv_den : 0.f;
+#pragma unroll 1
+          for (int c0 = cbase; c0 < cbase + HC; c0 += 16) {
+            uint32_t oa[16], ln[16], packed[8];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) oa[i] = ln[i] = 0u;
+            if (has_o) tmem_ld16(o_tmem + c0, oa);
+            if (has_lin) tmem_ld16(tmem + lane_off + kColLn + c0, ln);
+            float wl[16], ws[16];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) wl[i] = ws[i] = 1.f;
+            if (p.gate_tiles & 1) tile_gates16(1, c0, wl);
+            if (p.gate_tiles & 2) tile_gates16(2, c0, ws);
+            tc_wait_ld();
+#pragma unroll
+            for (int i = 0; i < 16; i += 2) {
+              float res[2];
+#pragma unroll
+              for (int e = 0; e < 2; ++e)
+                res[e] = fmaf(wl[i + e], __uint_as_float(ln[i + e]) * id, ws[i + e] * (__uint_as_float(oa[i + e]) * il));
+              packed[i >> 1] = pack_bf16(res[0], res[1]);
+            }
+            uint8_t* srow = smem + L::kQ + (c0 >> 6) * L::kHalf + r * 128;
+#pragma unroll
+            for (int q2 = 0; q2 < 2; ++q2)
+              *reinterpret_cast<uint4*>(srow + (((((c0 >> 3) + q2) & 7) ^ (r & 7)) << 4)) =
+                  make_uint4(packed[4 * q2], packed[4 * q2 + 1], packed[4 * q2 + 2], packed[4 * q2 + 3]);
+          }
+        }
         // rolled on purpose: 16 columns per trip keeps this once-per-tile code small
 #pragma unroll 1
-        for (int c0 = cbase; c0 < (plain ? cbase : cbase + HC); c0 += 16) {
+        for (int c0 = cbase; c0 < (plain || gated ? cbase : cbase + HC); c0 += 16) {
           uint32_t oa[16], ln[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) oa[i] = ln[i] = 0u;
@@ -939,27 +1026,29 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           float wl[16], ws[16], ladd[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) {
-            wl[i] = 1.f;
-            ws[i] = 1.f;
+            wl[i] = wl0;
+            ws[i] = ws0;
             ladd[i] = 0.f;
           }
+          if (GT && (p.gate_tiles & 1)) tile_gates16(1, c0, wl);
+          if (GT && (p.gate_tiles & 2)) tile_gates16(2, c0, ws);
           if (gl) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float w0 = __bfloat162float(gl[(c0 + i) * g_ds]);
-              wl[i] = sig ? __fdividef(1.f, 1.f + __expf(-w0)) : w0;
-            }
+            for (int i = 0; i < 16; ++i) wl[i] = gate_w(__bfloat162float(gl[(c0 + i) * g_ds]));
           }
           if (gs) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              const float w0 = __bfloat162float(gs[(c0 + i) * g_ds]);
-              ws[i] = sig ? __fdividef(1.f, 1.f + __expf(-w0)) : w0;
-            }
+            for (int i = 0; i < 16; ++i) ws[i] = gate_w(__bfloat162float(gs[(c0 + i) * g_ds]));
           }
           if (lnum) {
 #pragma unroll
-            for (int i = 0; i < 16; ++i) ladd[i] = lnum[c0 + i];
+            for (int i = 0; i < 4; ++i) {
+              const float4 v = *reinterpret_cast<const float4*>(lnum + c0 + 4 * i);
+              ladd[4 * i] = v.x;
+              ladd[4 * i + 1] = v.y;
+              ladd[4 * i + 2] = v.z;
+              ladd[4 * i + 3] = v.w;
+            }
           }
           if (ext) {  // linear branch computed by an earlier pass (Linformer form): already normalised
             const uint4 e0 = *reinterpret_cast<const uint4*>(ext + c0);
@@ -1023,27 +1112,34 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 }
 
 
+namespace {
+using FwdKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap,
+                           CUtensorMap, FwdParams);
+template <int D>
+FwdKernel fwd_kernel(bool split, bool linf, bool gt) {
+  if constexpr (D == 128) {
+    if (linf) return gt ? hsa_forward_kernel<128, false, true, true> : hsa_forward_kernel<128, false, true, false>;
+  }
+  if (split) return gt ? hsa_forward_kernel<D, true, false, true> : hsa_forward_kernel<D, true, false, false>;
+  return gt ? hsa_forward_kernel<D, false, false, true> : hsa_forward_kernel<D, false, false, false>;
+}
+}  // namespace
+
 cudaError_t forward_init() {
-  cudaError_t e = cudaFuncSetAttribute(hsa_forward_kernel<128, false, false>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<128>::kTotal);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(hsa_forward_kernel<128, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             Smem<128>::kTotal);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(hsa_forward_kernel<128, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             Smem<128>::kTotal);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(hsa_forward_kernel<64, false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             Smem<64>::kTotal);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(hsa_forward_kernel<64, true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             Smem<64>::kTotal);
+  cudaError_t e = cudaSuccess;
+  for (int i = 0; i < 8 && e == cudaSuccess; ++i) {
+    const bool split = i & 1, linf = (i & 2) && !split, gt = i & 4;
+    e = cudaFuncSetAttribute(fwd_kernel<128>(split, linf, gt), cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<128>::kTotal);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(fwd_kernel<64>(split, false, gt), cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<64>::kTotal);
+  }
   return e;
 }
 
 cudaError_t launch_forward(const FwdParams& p_in, int D, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                            const CUtensorMap& tm_v, const CUtensorMap& tm_state, const CUtensorMap& tm_out,
-                           cudaStream_t st, const CUtensorMap* tm_kc, const CUtensorMap* tm_vc) {
+                           cudaStream_t st, const CUtensorMap* tm_kc, const CUtensorMap* tm_vc, const CUtensorMap* tm_gl,
+                           const CUtensorMap* tm_gs) {
   const int n_tiles = (p_in.n_q + kTileM - 1) / kTileM;
   FwdParams p = p_in;
   p.n_tiles = n_tiles;
@@ -1068,13 +1164,13 @@ cudaError_t launch_forward(const FwdParams& p_in, int D, const CUtensorMap& tm_q
   // (kernels without the compressed segment never look at the last two maps)
   const CUtensorMap& kc = linf ? *tm_kc : tm_k;
   const CUtensorMap& vc = linf ? *tm_vc : tm_v;
-  if (D == 128) {
-    if (linf) return cudaLaunchKernelEx(&cfg, hsa_forward_kernel<128, false, true>, tm_q, tm_k, tm_v, tm_state, tm_out, kc, vc, p);
-    if (split) return cudaLaunchKernelEx(&cfg, hsa_forward_kernel<128, true, false>, tm_q, tm_k, tm_v, tm_state, tm_out, kc, vc, p);
-    return cudaLaunchKernelEx(&cfg, hsa_forward_kernel<128, false, false>, tm_q, tm_k, tm_v, tm_state, tm_out, kc, vc, p);
-  }
-  if (split) return cudaLaunchKernelEx(&cfg, hsa_forward_kernel<64, true, false>, tm_q, tm_k, tm_v, tm_state, tm_out, kc, vc, p);
-  return cudaLaunchKernelEx(&cfg, hsa_forward_kernel<64, false, false>, tm_q, tm_k, tm_v, tm_state, tm_out, kc, vc, p);
+  // (nor, without gate tiles, at these)
+  p.gate_tiles = (tm_gl ? 1 : 0) | (tm_gs ? 2 : 0);
+  const CUtensorMap& gl = tm_gl ? *tm_gl : tm_q;
+  const CUtensorMap& gs = tm_gs ? *tm_gs : tm_q;
+  const bool gt = p.gate_tiles != 0;
+  return cudaLaunchKernelEx(&cfg, D == 128 ? fwd_kernel<128>(split, linf, gt) : fwd_kernel<64>(split, false, gt), tm_q, tm_k, tm_v,
+                            tm_state, tm_out, kc, vc, gl, gs, p);
 }
 
 }  // namespace hsa

@@ -630,13 +630,23 @@ int hsa_forward(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride, in
     p.lin_den = c.lin_den;
     p.wait_late = 1;
   }
+  // Per-dim gates with unit dim stride travel as tiles; strides or a base that a tensor map cannot
+  // describe (and gates per token and head) are read by the kernel's threads.
+  CUtensorMap gate_map[2];
+  const CUtensorMap* tm_gate[2] = {nullptr, nullptr};
+  const void* gate_ptr[2] = {g_lin, g_sp};
+  for (int i = 0; i < 2; ++i)
+    if (gate_ptr[i] && gate_dim_stride == 1 && tensor_args_ok(ctx, gate_ptr[i], gate_tok_stride, gate_head_stride) &&
+        encode_q(&gate_map[i], gate_ptr[i], n_q, H, D, gate_tok_stride, gate_head_stride) == HSA_OK)
+      tm_gate[i] = &gate_map[i];
   if (do_linformer && p.max_splits == 1 && D == 128) {
     // one launch: the kernel's loop runs over the compressed pool first (its own accumulator,
     // exponent reference and row sums), then over the selected pages, and merges in its epilogue
     p.lf_table = reinterpret_cast<const int32_t*>(ws + ctx->lay.ctable);
     p.lf_pages = static_cast<int>(static_cast<int64_t>(ctx->n_segs) * ctx->cfg.lin_rank / kBlock);
     p.do_linear = 1;  // the compressed segment is this launch's linear branch
-    cudaError_t ef = launch_forward(p, D, tm_q, ctx->tm_k, ctx->tm_v, ctx->tm_state, tm_out, st, &ctx->tm_kc, &ctx->tm_vc);
+    cudaError_t ef = launch_forward(p, D, tm_q, ctx->tm_k, ctx->tm_v, ctx->tm_state, tm_out, st, &ctx->tm_kc, &ctx->tm_vc,
+                                   tm_gate[0], tm_gate[1]);
     if (ef != cudaSuccess) return cuda_fail(ctx, ef);
     return HSA_OK;
   }
@@ -677,7 +687,7 @@ int hsa_forward(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride, in
   if (D == 128 && do_linear && !do_sparse && !p.ext_lin)
     e = launch_linear_only(p, ctx->nsm, tm_q, ctx->tm_state, tm_out, st);  // nothing but Q in, out out
   else
-    e = launch_forward(p, D, tm_q, ctx->tm_k, ctx->tm_v, ctx->tm_state, tm_out, st);
+    e = launch_forward(p, D, tm_q, ctx->tm_k, ctx->tm_v, ctx->tm_state, tm_out, st, nullptr, nullptr, tm_gate[0], tm_gate[1]);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   return HSA_OK;
 }

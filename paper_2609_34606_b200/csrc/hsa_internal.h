@@ -121,6 +121,7 @@ struct FwdParams {
   const __nv_bfloat16* g_sp;
   int64_t g_ts, g_hs, g_ds;
   int gate_act;
+  int gate_tiles;  // set by the launcher: bit 0 / 1 = the logits of g_lin / g_sp arrive as tiles by TMA
   __nv_bfloat16* out;
   int64_t o_ts, o_hs;
   float scale_log2;  // softmax scale * log2(e)
@@ -199,11 +200,13 @@ cudaError_t launch_select(const SelectArgs& a, cudaStream_t st);
 cudaError_t launch_qsum(const SelectArgs& a, cudaStream_t st);  // stage 1 alone: query tile sums
 cudaError_t launch_retrieve(const RetrieveArgs& a, int n_pages, cudaStream_t st);
 cudaError_t launch_select_adaptive(const SelectArgs& a, const AdaptiveArgs& ad, cudaStream_t st);
-// tm_kc / tm_vc: maps of the compressed pools, used when p.lf_table is set (else null)
+// tm_kc / tm_vc: maps of the compressed pools, used when p.lf_table is set (else null); tm_gl / tm_gs: maps
+// of per-dim gate logits with the geometry of tm_q (null: no such gate, or its strides do not allow one)
 cudaError_t launch_forward(const FwdParams& p, int D, const CUtensorMap& tm_q,
                            const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                            const CUtensorMap& tm_state, const CUtensorMap& tm_out, cudaStream_t st,
-                           const CUtensorMap* tm_kc = nullptr, const CUtensorMap* tm_vc = nullptr);
+                           const CUtensorMap* tm_kc = nullptr, const CUtensorMap* tm_vc = nullptr,
+                           const CUtensorMap* tm_gl = nullptr, const CUtensorMap* tm_gs = nullptr);
 // tm_q: box of 128 tokens of one head; tm_phik, tm_v: rows of phi(K) and of the V pool, box 64 x 64
 cudaError_t launch_causal_linear(const CausalLinArgs& a, const CUtensorMap& tm_q, const CUtensorMap& tm_phik,
                                  const CUtensorMap& tm_v, cudaStream_t st);
