@@ -38,7 +38,7 @@ struct Layout {
   // state
   size_t S, z, slot_S, slot_z, hilo, zop, ksum_saved, ksum, state_total;  // S, z: slot 0; slot_*: bytes per slot
   // workspace
-  size_t status, page_table, qpart, keys, spart, lin_num, lin_den, phik, ctable, csel, ccnt, olin, ad_w, ad_idx, ad_gini, ad_wsum,
+  size_t status, page_table, qpart, keys, spart, lin_num, lin_den, phik, rpart, ctable, csel, ccnt, olin, ad_w, ad_idx, ad_gini, ad_wsum,
       part_o, part_l, part_ref, part_ticket, ws_total;
   int fwd_splits, split_blocks;
   int phik_blocks;  // pages a chunk can touch (causal contexts with a linear state, else 0)
@@ -87,6 +87,9 @@ Layout make_layout(const hsa_config* c) {
   L.page_table = o; o = align_up(o + P * 4, 256);
   L.qpart = o;      o = align_up(o + tiles * H * D * 4, 256);
   L.keys = o;       o = align_up(o + H * tiles * P * 4, 256);
+  // partial dots of the KV page retrieval: one per head for up to 2048 pages, or per run of 256 blocks of
+  // a longer page (at most two runs per 257 blocks and one page more)
+  L.rpart = o;      o = align_up(o + H * ((P < 2048 ? P : 2048) + P / 64 + 2) * 8, 256);
   L.spart = o;      o = align_up(o + H * kStateSplitMax * (D * D + D) * 4, 256);
   if (c->flags & HSA_CFG_CAUSAL) {
     L.lin_num = o;  o = align_up(o + static_cast<size_t>(c->max_q_tokens) * H * D * 4, 256);
@@ -728,7 +731,7 @@ int hsa_retrieve_kv_pages(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_
   ra.kv_page_blocks = kv_page_blocks;
   ra.top_kp = top_kp;
   ra.scale = ctx->scale;
-  ra.keys = reinterpret_cast<uint32_t*>(ws + ctx->lay.keys);
+  ra.part = reinterpret_cast<double*>(ws + ctx->lay.rpart);
   ra.scores_out = scores_dev;
   ra.page_ids = page_ids_dev;
   e = launch_retrieve(ra, static_cast<int>(n_pages), st);

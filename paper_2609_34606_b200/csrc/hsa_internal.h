@@ -99,7 +99,7 @@ struct RetrieveArgs {
   const float* ksum;   // [H][max_pages][D]
   int kv_page_blocks, top_kp;
   float scale;
-  uint32_t* keys;      // [pages] scratch
+  double* part;        // [pages][H][runs] scratch: partial dots of a page
   float* scores_out;   // [pages] or null
   int32_t* page_ids;   // [min(top_kp, pages)] ascending (output)
 };

@@ -971,16 +971,6 @@ bool coop_info(int* nsm) {
 }  // namespace
 
 
-cudaError_t launch_qsum(const SelectArgs& a, cudaStream_t st) {
-  const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
-  dim3 g1(n_tiles, a.H);
-  if (a.D == 128)
-    qsum_partial_kernel<128><<<g1, 256, 0, st>>>(a);
-  else
-    qsum_partial_kernel<64><<<g1, 256, 0, st>>>(a);
-  return cudaGetLastError();
-}
-
 namespace {
 // Cluster size (8 CTAs, the portable maximum) if the cluster form can be launched on this device for
 // the given instance and shared-memory size, else 0.
@@ -1030,6 +1020,14 @@ cudaError_t launch_pdl(const void* fn, dim3 grid, dim3 block, size_t smem, void*
   return cudaLaunchKernelExC(&cfg, fn, params);
 }
 }  // namespace
+
+cudaError_t launch_qsum(const SelectArgs& a, cudaStream_t st) {
+  SelectArgs aa = a;
+  void* p_args[1] = {&aa};
+  const void* fn = a.D == 128 ? reinterpret_cast<const void*>(qsum_partial_kernel<128>)
+                              : reinterpret_cast<const void*>(qsum_partial_kernel<64>);
+  return launch_pdl(fn, dim3((a.n_q + kTileM - 1) / kTileM, a.H), dim3(256), 0, p_args, st);
+}
 
 // Three forms, all programmatic dependents of the kernel before them:
 //   cluster form        query tile sums as a kernel of their own (they read the whole chunk and want

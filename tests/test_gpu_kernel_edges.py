@@ -129,3 +129,29 @@ def test_gate_layouts(d, n_q, topk, layout, act, split, cuda_device):
     size = (weight(gl) * lin).abs() + (weight(gs) * sp).abs()
     assert float(((out.double() - ref).abs() - 2 * BF16_REL * size - 1e-6).max()) <= 0.0
     ctx.destroy()
+
+
+@pytest.mark.parametrize("d,H,n,kvb", [(128, 3, 65, 1), (128, 2, 5000, 7), (64, 5, 5000, 195), (128, 12, 70000, 195),
+                                       (64, 2, 70000, 256), (128, 2, 70000, 257), (128, 1, 70000, 700), (128, 2, 70000, 5000)])
+def test_kv_page_scores(d, H, n, kvb, cuda_device):
+    """Scores of KV pages of one block, of less, as many and more blocks than one CTA takes, and of one page
+    that is longer than the history, against fp64; the ids are the best pages in ascending order."""
+    from paper_2609_34606_b200 import hsa
+    g = torch.Generator().manual_seed(n + kvb)
+    nb, n_q = (n + 63) // 64, 150
+    K, q = _randn(g, n, H, d), _randn(g, n_q, H, d)
+    ctx = hsa.HSAContext(H, d, max_pages=nb + 3, max_q_tokens=max(n, n_q), max_topk=4, lin_mode=hsa.HSA_LIN_NONE, device=cuda_device)
+    kd = K.to(cuda_device)
+    ctx.append_kv(kd, kd)
+    ids, scores = ctx.retrieve_kv_pages(q.to(cuda_device), kvb, top_kp=3, with_scores=True)
+    assert ctx.device_status() == 0
+    n_pages = (nb + kvb - 1) // kvb
+    qbar = q.double().mean(0)
+    ref = torch.stack([(qbar * K[j * kvb * 64:(j + 1) * kvb * 64].double().mean(0)).sum() / H * d ** -0.5
+                       for j in range(n_pages)])
+    # key and query sums are fp32 sums of up to 128 values (2^-24 of partial sums each), the rest is fp64;
+    # the scores are sums of H d products of random sign
+    assert float((scores.double().cpu() - ref).abs().max()) <= 2.0 ** -20 * float(ref.abs().max())
+    best = torch.sort(scores.cpu(), descending=True, stable=True).indices[:min(3, n_pages)]
+    assert ids.cpu().tolist() == sorted(best.tolist())
+    ctx.destroy()
