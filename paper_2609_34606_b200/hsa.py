@@ -139,7 +139,8 @@ def _ptr(t: Optional[torch.Tensor]) -> Optional[int]:
 
 
 def _stream() -> int:
-    return torch.cuda.current_stream().cuda_stream
+    # the current stream of the current device, without building a torch.cuda.Stream (3.1 -> 0.2 us a call)
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def _thd(t: torch.Tensor, name: str) -> Tuple[int, int]:
@@ -342,27 +343,38 @@ class HSAContext:
                                self.workspace.data_ptr(), _ptr(self.kc_pool), _ptr(self.vc_pool),
                                _ptr(e_k), _ptr(e_v))
             self.ctx = hsa_create(self.cfg, bufs, page_order)
-        self._off_ksum = hsa_state_layout(self.ctx)[2]
+        # -- state views (fp32): S and z of either slot, the key sums
+        self._ksum = self._view(hsa_state_layout(self.ctx)[2], (H, max_pages, d))
+        self._slots = {}  # byte offset in the state buffer -> view of it
 
-    # -- state views (fp32) for tests and snapshots
     def _view(self, off: int, shape) -> torch.Tensor:
         n = 1
         for s in shape:
             n *= s
         return self.state[off:off + 4 * n].view(torch.float32).view(*shape)
 
+    def _slot(self, off: int, *shape) -> torch.Tensor:
+        v = self._slots.get(off)
+        if v is None:
+            v = self._slots[off] = self._view(off, shape)
+        return v
+
     @property
     def S(self) -> torch.Tensor:
         # (the state lives in two slots that take turns: ask where the current one is)
-        return self._view(hsa_state_layout(self.ctx)[0], (self.H, self.d, self.d))
+        off = C.c_size_t()
+        _check(_lib.hsa_state_layout(self.ctx, C.byref(off), None, None), "hsa_state_layout")
+        return self._slot(off.value, self.H, self.d, self.d)
 
     @property
     def z(self) -> torch.Tensor:
-        return self._view(hsa_state_layout(self.ctx)[1], (self.H, self.d))
+        off = C.c_size_t()
+        _check(_lib.hsa_state_layout(self.ctx, None, C.byref(off), None), "hsa_state_layout")
+        return self._slot(off.value, self.H, self.d)
 
     @property
     def ksum(self) -> torch.Tensor:
-        return self._view(self._off_ksum, (self.H, self.max_pages, self.d))
+        return self._ksum
 
     @property
     def n_tokens(self) -> int:
@@ -406,7 +418,7 @@ class HSAContext:
     def retrieve_kv_pages(self, q: torch.Tensor, kv_page_blocks: int, top_kp: int = 4, with_scores: bool = False):
         """Stage-2 page retrieval: (int32 ids of the kept KV pages, ascending[, fp32 score of every page])."""
         n_pages = (self.n_blocks + kv_page_blocks - 1) // kv_page_blocks
-        ids = torch.zeros(max(1, min(top_kp, n_pages)), dtype=torch.int32, device=self.device)
+        ids = torch.empty(max(1, min(top_kp, n_pages)), dtype=torch.int32, device=self.device)  # all of [:n] is written
         scores = torch.zeros(max(1, n_pages), dtype=torch.float32, device=self.device) if with_scores else None
         n = hsa_retrieve_kv_pages(self.ctx, q, kv_page_blocks, top_kp, ids, scores)
         return (ids[:n], scores[:n_pages]) if with_scores else ids[:n]
@@ -430,8 +442,12 @@ class HSAContext:
         """Cumulative-mass selection with the Gini threshold map; returns (sel_idx, sel_cnt, gini_tau)
         with gini_tau fp32 [2, H] = (Gini, threshold) per head."""
         q_pos0 = self.n_tokens if q_pos0 is None else q_pos0
-        sel_idx, sel_cnt = self.alloc_selection(q.shape[0], group_tokens)
-        gt = torch.zeros(2, self.H, dtype=torch.float32, device=self.device)
+        g, H = self.n_groups(q.shape[0], group_tokens), self.H
+        # lists, counts and (as fp32) Gini and threshold in one zeroed buffer: one fill instead of three
+        n_idx, n_cnt = H * g * self.max_topk, H * g
+        buf = torch.zeros(n_idx + n_cnt + 2 * H, dtype=torch.int32, device=self.device)
+        idx, cnt, gt = buf.split((n_idx, n_cnt, 2 * H))
+        sel_idx, sel_cnt, gt = idx.view(H, g, self.max_topk), cnt.view(H, g), gt.view(torch.float32).view(2, H)
         hsa_select_blocks_adaptive(self.ctx, q, q_pos0, causal, tau_min, tau_max, group_tokens, sel_idx, sel_cnt, gt)
         return sel_idx, sel_cnt, gt
 
