@@ -690,85 +690,6 @@ __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-template <int D>
-struct ClusterSmem {
-  static constexpr int kScratch = (D + 256) * 8;  // per sub-block; together: mean query [D] + partial sums [768 / D][D], fp64
-  static constexpr int kFixed = (kSubBlocks * kScratch + static_cast<int>(sizeof(TopkShared)) + 15) / 16 * 16;
-};
-
-template <int D, bool MIXED>
-__global__ void __launch_bounds__(256 * kSubBlocks, 1) select_cluster_kernel(SelectArgs a, int cluster_ctas) {
-  // dynamic shared memory: per sub-block scratch (mean query and its partial sums) | top-k
-  // bookkeeping | the head's keys
-  extern __shared__ __align__(16) unsigned char cl_smem[];
-  constexpr int kScratch = ClusterSmem<D>::kScratch;
-  const int sub = static_cast<int>(threadIdx.x) / 256;
-  const Blk blk{static_cast<int>(threadIdx.x) % 256, 1 + sub};
-  TopkShared* sh_all = reinterpret_cast<TopkShared*>(cl_smem + kSubBlocks * kScratch);
-  uint32_t* cl_keys = reinterpret_cast<uint32_t*>(cl_smem + ClusterSmem<D>::kFixed);
-  const int h = static_cast<int>(blockIdx.x) / cluster_ctas;
-  const int slot = (static_cast<int>(blockIdx.x) % cluster_ctas) * kSubBlocks + sub;
-  const int n_slots = cluster_ctas * kSubBlocks;
-  const int n_chunks = (cand_geom<MIXED>(a).nc + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta;
-  // (one list per head: the launcher sends per-tile selections to the grid-barrier form)
-  // The key sums of this block's first score item are requested first, ahead of the wait for the
-  // kernel before this one: that kernel (the query tile sums) writes none of them, and it has itself
-  // waited for everything before it, so they are final when any CTA of this grid runs.
-  ScoreOperands<D, MIXED> op;
-  if (slot < n_chunks) scores_load<D, MIXED>(blk, a, slot, h, op);
-  // A CTA's shared memory may be written by its peers only once it runs: every CTA says so here and
-  // checks, before its first such write, that all of the cluster have (the two halves of one
-  // cluster barrier; by then nobody waits).
-  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-  // launched as a programmatic dependent: the kernel before this one is complete from here on
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  // The head's mean query, once per CTA: all 768 threads add up the tile sums (a column's partials
-  // split over 768 / D ways, every load of a thread in flight at once, fp64, fixed order), then one
-  // thread per column adds the ways.  The three sub-blocks share the result.
-  double* qmean = reinterpret_cast<double*>(cl_smem);  // [D], then the per-way partial sums [WAYS][D]
-  {
-    constexpr int WAYS = 256 * kSubBlocks / D;
-    constexpr int kInFlight = 8;
-    const int tid = static_cast<int>(threadIdx.x), col = tid % D, way = tid / D;
-    const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
-    double sum = 0.0;
-    for (int t0 = way; t0 < n_tiles; t0 += kInFlight * WAYS) {
-      float v[kInFlight];
-#pragma unroll
-      for (int i = 0; i < kInFlight; ++i)
-        v[i] = (t0 + i * WAYS < n_tiles) ? __ldcg(&a.qpart[(static_cast<size_t>(t0 + i * WAYS) * a.H + h) * D + col]) : 0.f;
-#pragma unroll
-      for (int i = 0; i < kInFlight; ++i) sum += static_cast<double>(v[i]);
-    }
-    qmean[D + way * D + col] = sum;
-    __syncthreads();
-    if (tid < D) {
-      double t = 0.0;
-#pragma unroll
-      for (int w = 0; w < WAYS; ++w) t += qmean[D + w * D + tid];
-      qmean[tid] = t / static_cast<double>(a.n_q) * static_cast<double>(a.scale);
-    }
-    __syncthreads();
-  }
-  // the budgets are asked for now by the block that will need them, far ahead of their use
-  int budget = 0, intra_budget = -1;
-  if (slot == 0) {
-    budget = a.budgets[h];
-    if (MIXED && a.intra_budgets) intra_budget = a.intra_budgets[h];
-  }
-  // the score keys go straight into the key array of the cluster's first CTA (distributed shared
-  // memory), where the lists are extracted: no trip through global memory between the two stages
-  uint32_t keys_addr;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(keys_addr) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(cl_keys))), "r"(0u));
-  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every CTA of the cluster is running
-  for (int chunk = slot; chunk < n_chunks; chunk += n_slots)
-    scores_item<D, MIXED>(blk, a, chunk, 0, h, qmean, op, false, chunk == slot, keys_addr);
-  cluster_sync_all();  // the score keys of the head are complete and visible to its first CTA
-  // the kernel behind this one may take the places of the CTAs that leave now
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  if (slot == 0) topk_item<MIXED>(blk, a, 0, h, cl_keys, sh_all, budget, intra_budget, true);
-}
-
 // ---------------------------------------------------------------------------------------
 // Head-adaptive selection (Appendix "Sparse Branch"): block weights p = softmax of the pooled
 // scores over the candidates, sorted in descending order; Gini coefficient of the sorted weights
@@ -921,37 +842,253 @@ __global__ void __launch_bounds__(256) adaptive_pick_kernel(SelectArgs a, Adapti
   }
 }
 
-cudaError_t launch_select_adaptive(const SelectArgs& a, const AdaptiveArgs& ad, cudaStream_t st) {
-  const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
-  dim3 g1(n_tiles, a.H);
-  if (a.D == 128)
-    qsum_partial_kernel<128><<<g1, 256, 0, st>>>(a);
-  else
-    qsum_partial_kernel<64><<<g1, 256, 0, st>>>(a);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  const int64_t nblk = (a.n_tokens + kBlock - 1) / kBlock;
-  if (nblk > 0) {
-    dim3 g2(static_cast<unsigned>((nblk + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta), a.n_groups, a.H);
-    if (a.D == 128)
-      block_scores_kernel<128, false><<<g2, 256, 0, st>>>(a);
-    else
-      block_scores_kernel<64, false><<<g2, 256, 0, st>>>(a);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
+// ---------------------------------------------------------------------------------------
+// The same rule for one list per head, by the 768 threads of a cluster's first CTA behind the score stage:
+// sort, weights, Gini, threshold, prefix and list without leaving the CTA.  Sums run in fp64.  The
+// sort is bitonic over (score, block) pairs in shared memory; strides below 32 run in registers between
+// the lanes of a warp.  It is latency that bounds it: scores and lists of
+// 732 blocks, 12 heads, take 15 us in one kernel, where scores, sort and pick took 39 us in three.
+// ---------------------------------------------------------------------------------------
+struct AdaptiveShared {
+  double e_sum[24], g_sum[24];
+  int cnt[24];
+  int k;
+};
+
+// bytes of the head's keys in shared memory, up to where the 8-byte pairs may start
+__device__ __host__ __forceinline__ size_t adaptive_key_bytes(const SelectArgs& a) {
+  return (static_cast<size_t>((a.n_tokens + kBlock - 1) / kBlock) * sizeof(uint32_t) + 15) / 16 * 16;
+}
+
+constexpr int kAdThreads = 256 * 3, kAdSorters = 512;
+constexpr int kAdPer = 8;  // sorted positions per thread at most: 6144 blocks, the cluster form's limit
+
+__device__ __forceinline__ void adaptive_list(const SelectArgs& a, const AdaptiveArgs& ad, int h, uint32_t* keys,
+                                              unsigned long long* pairs, AdaptiveShared* sh) {
+  const int tid = static_cast<int>(threadIdx.x), lane = tid & 31, warp = tid >> 5;
+  const int nblk = static_cast<int>((a.n_tokens + kBlock - 1) / kBlock);
+  const int64_t p_last = a.q_pos0 + a.n_q - 1;
+  int ncand = nblk;
+  if (a.causal) ncand = p_last < 0 ? 0 : static_cast<int>(min64(nblk, p_last / kBlock + 1));
+  int np2 = 32;
+  while (np2 < ncand) np2 <<= 1;
+  for (int i = tid; i < np2; i += kAdThreads)
+    pairs[i] = i < ncand ? ((static_cast<unsigned long long>(keys[i]) << 32) | (0xffffffffu - static_cast<uint32_t>(i)))
+                         : 0ull;  // padding sorts last
+  if (tid == 0) sh->k = ncand;  // mass never reached (rounding at tau ~ 1): keep everything
+  __syncthreads();
+  for (int i = tid; i < ncand; i += kAdThreads) keys[i] = 0u;  // from here on: 1 = chosen
+  if (tid < kAdSorters) {
+    auto sync = [] { asm volatile("bar.sync 4, %0;" ::"n"(kAdSorters) : "memory"); };
+    // strides 16 .. 1 of the merges of size k_lo .. k_hi, 32 pairs per warp in registers
+    auto in_warp = [&](int k_lo, int k_hi) {
+      for (int seg = warp; seg < np2 / 32; seg += kAdSorters / 32) {
+        const int i = seg * 32 + lane;
+        unsigned long long x = pairs[i];
+        for (int k = k_lo; k <= k_hi; k <<= 1)
+          for (int j = min(16, k >> 1); j > 0; j >>= 1) {
+            const unsigned long long y = __shfl_xor_sync(0xffffffffu, x, j);
+            const bool want_max = ((i & k) == 0) == ((i & j) == 0);  // descending runs first
+            x = want_max == (x > y) ? x : y;
+          }
+        pairs[i] = x;
+      }
+    };
+    in_warp(2, 32);
+    sync();
+    for (int k = 64; k <= np2; k <<= 1) {
+      for (int j = k >> 1; j >= 32; j >>= 1) {
+        for (int t = tid; t < np2 / 2; t += kAdSorters) {
+          const int i = ((t & ~(j - 1)) << 1) | (t & (j - 1));  // the pair (i, i + j)
+          const unsigned long long x = pairs[i], y = pairs[i + j];
+          if (((i & k) == 0) ? (x < y) : (x > y)) {
+            pairs[i] = y;
+            pairs[i + j] = x;
+          }
+        }
+        sync();
+      }
+      in_warp(k, k);
+      sync();
+    }
   }
-  int np2 = 1;
-  while (np2 < nblk) np2 <<= 1;
-  const size_t smem_sort = static_cast<size_t>(np2) * 8;
-  if (smem_sort > 40 * 1024)
-    cudaFuncSetAttribute(adaptive_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         static_cast<int>(smem_sort));
-  dim3 g3(a.n_groups, a.H);
-  adaptive_sort_kernel<<<g3, 256, smem_sort, st>>>(a, ad);
-  e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  adaptive_pick_kernel<<<g3, 256, static_cast<size_t>(nblk > 0 ? nblk : 1), st>>>(a, ad);
-  return cudaGetLastError();
+  __syncthreads();
+  // weights in sorted order: thread t owns positions [t * per, t * per + per)
+  const int per = (ncand + kAdThreads - 1) / kAdThreads;
+  const int lo = min(ncand, tid * per), hi = min(ncand, lo + per);
+  const double smax = static_cast<double>(key_to_float(static_cast<uint32_t>(pairs[0] >> 32)));
+  double e[kAdPer];
+  double es = 0.0, gs = 0.0;
+#pragma unroll
+  for (int i = 0; i < kAdPer; ++i) {
+    e[i] = 0.0;
+    if (lo + i < hi) {
+      e[i] = exp(static_cast<double>(key_to_float(static_cast<uint32_t>(pairs[lo + i] >> 32))) - smax);
+      es += e[i];
+      gs += static_cast<double>(ncand - 2 * (lo + i + 1) + 1) * e[i];
+    }
+  }
+  // inclusive prefix of the threads' sums, total of the Gini terms
+  double incl = es;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const double n = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += n;
+    gs += __shfl_xor_sync(0xffffffffu, gs, o);
+  }
+  if (lane == 31) {
+    sh->e_sum[warp] = incl;
+    sh->g_sum[warp] = gs;
+  }
+  __syncthreads();
+  double before = 0.0, esum = 0.0, gsum = 0.0;
+  for (int w = 0; w < kAdThreads / 32; ++w) {
+    if (w == warp) before = esum;
+    esum += sh->e_sum[w];
+    gsum += sh->g_sum[w];
+  }
+  const double gini = (ncand > 0 && esum > 0.0) ? gsum / (esum * static_cast<double>(ncand)) : 0.0;
+  const double tau = static_cast<double>(ad.tau_min) + gini * (static_cast<double>(ad.tau_max) - static_cast<double>(ad.tau_min));
+  if (tid == 0 && ad.gini_out) {
+    ad.gini_out[h] = static_cast<float>(gini);
+    ad.gini_out[a.H + h] = static_cast<float>(tau);
+  }
+  const double target = tau * esum;  // mass to reach
+  double cum = before + (incl - es);
+#pragma unroll
+  for (int i = 0; i < kAdPer; ++i) {
+    cum += e[i];
+    if (lo + i < hi && cum >= target) {
+      atomicMin(&sh->k, lo + i + 1);
+      break;
+    }
+  }
+  __syncthreads();
+  const int kk = sh->k;
+  for (int m = tid; m < kk; m += kAdThreads) keys[0xffffffffu - static_cast<uint32_t>(pairs[m] & 0xffffffffu)] = 1u;
+  __syncthreads();
+  // ascending list of the chosen blocks: thread t owns blocks [lo, hi)
+  int mine = 0;
+  for (int b = lo; b < hi; ++b) mine += static_cast<int>(keys[b]);
+  int pos = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int n = __shfl_up_sync(0xffffffffu, pos, o);
+    if (lane >= o) pos += n;
+  }
+  if (lane == 31) sh->cnt[warp] = pos;
+  __syncthreads();
+  pos -= mine;
+  for (int w = 0; w < warp; ++w) pos += sh->cnt[w];
+  int32_t* out = a.sel_idx + static_cast<size_t>(h) * a.kcap;
+  for (int b = lo; b < hi; ++b)
+    if (keys[b]) {
+      if (pos < a.kcap) out[pos] = b;
+      ++pos;
+    }
+  if (tid == 0) {
+    a.sel_cnt[h] = min(kk, a.kcap);
+    if (kk > a.kcap) atomicCAS(a.status, 0, kDevBounds);
+  }
+}
+
+template <int D>
+struct ClusterSmem {
+  // per sub-block: partial column sums of a query tile (fp32 [256 / (D / 8)][D]); together: mean query [D]
+  // and partial sums [768 / D][D], fp64
+  static constexpr int kScratch = 8192;
+  static constexpr int kFixed = (kSubBlocks * kScratch + static_cast<int>(sizeof(TopkShared)) + 15) / 16 * 16;
+};
+
+// OWN_Q: the query tile sums are taken here as well, a tile per sub-block, instead of by the kernel in front
+// ADAPT: the lists are the head-adaptive ones (adaptive_list) instead of the budgets' top-k
+template <int D, bool MIXED, bool OWN_Q, bool ADAPT>
+__global__ void __launch_bounds__(256 * kSubBlocks, 1) select_cluster_kernel(SelectArgs a, AdaptiveArgs ad, int cluster_ctas) {
+  // dynamic shared memory: per sub-block scratch (mean query and its partial sums) | top-k
+  // bookkeeping | the head's keys
+  extern __shared__ __align__(16) unsigned char cl_smem[];
+  constexpr int kScratch = ClusterSmem<D>::kScratch;
+  const int sub = static_cast<int>(threadIdx.x) / 256;
+  const Blk blk{static_cast<int>(threadIdx.x) % 256, 1 + sub};
+  TopkShared* sh_all = reinterpret_cast<TopkShared*>(cl_smem + kSubBlocks * kScratch);
+  uint32_t* cl_keys = reinterpret_cast<uint32_t*>(cl_smem + ClusterSmem<D>::kFixed);
+  const int h = static_cast<int>(blockIdx.x) / cluster_ctas;
+  const int slot = (static_cast<int>(blockIdx.x) % cluster_ctas) * kSubBlocks + sub;
+  const int n_slots = cluster_ctas * kSubBlocks;
+  const int n_chunks = (cand_geom<MIXED>(a).nc + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta;
+  // (one list per head: the launcher sends per-tile selections to the grid-barrier form)
+  // The key sums of this block's first score item are requested first, ahead of the wait for the
+  // kernel before this one: that kernel (the query tile sums) writes none of them, and it has itself
+  // waited for everything before it, so they are final when any CTA of this grid runs.
+  ScoreOperands<D, MIXED> op;
+  if (!OWN_Q && slot < n_chunks) scores_load<D, MIXED>(blk, a, slot, h, op);
+  // A CTA's shared memory may be written by its peers only once it runs: every CTA says so here and
+  // checks, before its first such write, that all of the cluster have (the two halves of one
+  // cluster barrier; by then nobody waits).
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+  // launched as a programmatic dependent: the kernel before this one is complete from here on
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (OWN_Q) {
+    if (slot < n_chunks) scores_load<D, MIXED>(blk, a, slot, h, op);
+    const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
+    for (int tile = slot; tile < n_tiles; tile += n_slots) {
+      qsum_item<D>(blk, a, tile, h, reinterpret_cast<float(*)[D]>(cl_smem + sub * kScratch));
+      blk_sync(blk);
+    }
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every CTA of the cluster is running
+    cluster_sync_all();  // and the head's tile sums are written
+  }
+  // The head's mean query, once per CTA: all 768 threads add up the tile sums (a column's partials
+  // split over 768 / D ways, every load of a thread in flight at once, fp64, fixed order), then one
+  // thread per column adds the ways.  The three sub-blocks share the result.
+  double* qmean = reinterpret_cast<double*>(cl_smem);  // [D], then the per-way partial sums [WAYS][D]
+  {
+    constexpr int WAYS = 256 * kSubBlocks / D;
+    constexpr int kInFlight = 8;
+    const int tid = static_cast<int>(threadIdx.x), col = tid % D, way = tid / D;
+    const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
+    double sum = 0.0;
+    for (int t0 = way; t0 < n_tiles; t0 += kInFlight * WAYS) {
+      float v[kInFlight];
+#pragma unroll
+      for (int i = 0; i < kInFlight; ++i)
+        v[i] = (t0 + i * WAYS < n_tiles) ? __ldcg(&a.qpart[(static_cast<size_t>(t0 + i * WAYS) * a.H + h) * D + col]) : 0.f;
+#pragma unroll
+      for (int i = 0; i < kInFlight; ++i) sum += static_cast<double>(v[i]);
+    }
+    qmean[D + way * D + col] = sum;
+    __syncthreads();
+    if (tid < D) {
+      double t = 0.0;
+#pragma unroll
+      for (int w = 0; w < WAYS; ++w) t += qmean[D + w * D + tid];
+      qmean[tid] = t / static_cast<double>(a.n_q) * static_cast<double>(a.scale);
+    }
+    __syncthreads();
+  }
+  // the budgets are asked for now by the block that will need them, far ahead of their use
+  int budget = 0, intra_budget = -1;
+  if (!ADAPT && slot == 0) {
+    budget = a.budgets[h];
+    if (MIXED && a.intra_budgets) intra_budget = a.intra_budgets[h];
+  }
+  // the score keys go straight into the key array of the cluster's first CTA (distributed shared
+  // memory), where the lists are extracted: no trip through global memory between the two stages
+  uint32_t keys_addr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(keys_addr) : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(cl_keys))), "r"(0u));
+  if (!OWN_Q) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every CTA of the cluster is running
+  for (int chunk = slot; chunk < n_chunks; chunk += n_slots)
+    scores_item<D, MIXED>(blk, a, chunk, 0, h, qmean, op, false, chunk == slot, keys_addr);
+  cluster_sync_all();  // the score keys of the head are complete and visible to its first CTA
+  // the kernel behind this one may take the places of the CTAs that leave now
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if constexpr (ADAPT) {
+    if (slot < kSubBlocks)  // the cluster's first CTA
+      adaptive_list(a, ad, h, cl_keys, reinterpret_cast<unsigned long long*>(cl_smem + ClusterSmem<D>::kFixed + adaptive_key_bytes(a)),
+                    reinterpret_cast<AdaptiveShared*>(cl_smem));
+  } else {
+    if (slot == 0) topk_item<MIXED>(blk, a, 0, h, cl_keys, sh_all, budget, intra_budget, true);
+  }
 }
 
 namespace {
@@ -1029,9 +1166,72 @@ cudaError_t launch_qsum(const SelectArgs& a, cudaStream_t st) {
   return launch_pdl(fn, dim3((a.n_q + kTileM - 1) / kTileM, a.H), dim3(256), 0, p_args, st);
 }
 
+namespace {
+// Cluster form of the selection, if this call and this device allow it (-1 in *done_as: not launched).
+constexpr int kClusterMaxChunks = 192;
+// The query tile sums are taken inside the clusters while every sub-block gets at most one tile (24 of
+// 128 tokens): one launch instead of two.  Longer chunks want every SM for them, 96 of 148 are in a
+// cluster at 12 heads.  Measured: 12.6 against 12.7 us of kernels for 8 tiles x 16 heads of 64, 10.4 against
+// 10.0 for 13 tiles x 12 heads of 128, and 3.6 against 6.0 us of the caller's time to issue the call.
+constexpr int kOwnQueryTiles = 8 * kSubBlocks;
+
+template <int D>
+const void* cluster_kernel(bool mixed, bool own, bool adapt) {
+  if (adapt)
+    return own ? reinterpret_cast<const void*>(select_cluster_kernel<D, false, true, true>)
+               : reinterpret_cast<const void*>(select_cluster_kernel<D, false, false, true>);
+  if (mixed)
+    return own ? reinterpret_cast<const void*>(select_cluster_kernel<D, true, true, false>)
+               : reinterpret_cast<const void*>(select_cluster_kernel<D, true, false, false>);
+  return own ? reinterpret_cast<const void*>(select_cluster_kernel<D, false, true, false>)
+             : reinterpret_cast<const void*>(select_cluster_kernel<D, false, false, false>);
+}
+
+// true: launched (or failed with *err); false: not a case for this form
+bool launch_cluster(const SelectArgs& a, const AdaptiveArgs* ad, bool mixed, cudaStream_t st, cudaError_t* err) {
+  const int64_t nblk = (a.n_tokens + kBlock - 1) / kBlock;
+  const int64_t n_chunks = (nblk + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta;
+  if (a.n_groups != 1 || n_chunks > kClusterMaxChunks) return false;
+  size_t smem = a.D == 128 ? ClusterSmem<128>::kFixed : ClusterSmem<64>::kFixed;
+  if (ad) {
+    size_t np2 = 32;
+    while (static_cast<int64_t>(np2) < nblk) np2 <<= 1;
+    smem += adaptive_key_bytes(a) + np2 * 8;
+  } else {
+    smem += static_cast<size_t>(nblk > 0 ? nblk : 1) * sizeof(uint32_t);
+  }
+  const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
+  const bool own = n_tiles <= kOwnQueryTiles;
+  const void* fn = a.D == 128 ? cluster_kernel<128>(mixed, own, ad != nullptr) : cluster_kernel<64>(mixed, own, ad != nullptr);
+  // the cluster size is looked up once per instance, for the largest shared-memory size the form
+  // is used with (a cluster that fits with that fits with less)
+  constexpr size_t kMaxSmem = 120 * 1024;
+  if (smem > kMaxSmem) return false;
+  static int cached_cs[2][2][2][2] = {{{{-1, -1}, {-1, -1}}, {{-1, -1}, {-1, -1}}}, {{{-1, -1}, {-1, -1}}, {{-1, -1}, {-1, -1}}}};
+  int& cs = cached_cs[a.D == 128][mixed][own][ad != nullptr];
+  if (cs < 0) {
+    const bool ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMaxSmem)) == cudaSuccess;
+    cs = ok ? cluster_size_for(fn, kMaxSmem, 256 * kSubBlocks) : 0;
+    if (cs == 0) cudaGetLastError();  // no cluster of that shape on this device: the other forms
+  }
+  if (cs == 0) return false;
+  SelectArgs aa = a;
+  AdaptiveArgs none{};
+  AdaptiveArgs aad = ad ? *ad : none;
+  if (!own) {
+    *err = launch_qsum(a, st);
+    if (*err != cudaSuccess) return true;
+  }
+  int cs_arg = cs;
+  void* params[3] = {&aa, &aad, &cs_arg};
+  *err = launch_pdl(fn, dim3(static_cast<unsigned>(cs * a.H)), dim3(256 * kSubBlocks), smem, params, st, cs);
+  return true;
+}
+}  // namespace
+
 // Three forms, all programmatic dependents of the kernel before them:
 //   cluster form        query tile sums as a kernel of their own (they read the whole chunk and want
-//                       every SM), then one cluster of 8 CTAs per head for scores and lists, with one
+//                       every SM; short chunks: inside the clusters), then one cluster of 8 CTAs per head for scores and lists, with one
 //                       hardware cluster barrier between them -- the default for one list per head while
 //                       a head has at most kClusterMaxChunks score items (6144 blocks; measured against
 //                       the grid-barrier form: 17.1 against 20.0 us at 2194 blocks, 24.8 against 25.1 us
@@ -1040,8 +1240,6 @@ cudaError_t launch_qsum(const SelectArgs& a, cudaStream_t st) {
 //                       beyond that, one list per query tile (37 x H lists want more than 24 blocks
 //                       of threads per head), and on request
 //   three launches      for devices without cooperative launch and for callers without a barrier word
-constexpr int kClusterMaxChunks = 192;
-
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t st) {
   int nsm = 0;
   const bool mixed = a.inter_pages > 1 || a.intra_first_page1 > 0 || a.kv_pages != nullptr;
@@ -1053,33 +1251,8 @@ cudaError_t launch_select(const SelectArgs& a, cudaStream_t st) {
                                   : reinterpret_cast<const void*>(qsum_partial_kernel<64>);
   // candidates per head (coarse candidates make fewer; an upper bound is enough to choose the form)
   const int64_t n_chunks_max = (nblk_all + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta;
-  if (a.use_clusters && a.n_groups == 1 && n_chunks_max <= kClusterMaxChunks) {
-    const size_t key_bytes = static_cast<size_t>(nblk_all > 0 ? nblk_all : 1) * sizeof(uint32_t);
-    const size_t fixed = a.D == 128 ? ClusterSmem<128>::kFixed : ClusterSmem<64>::kFixed;
-    const size_t smem = fixed + key_bytes;
-    const void* fn = a.D == 128 ? (mixed ? reinterpret_cast<const void*>(select_cluster_kernel<128, true>)
-                                         : reinterpret_cast<const void*>(select_cluster_kernel<128, false>))
-                                : (mixed ? reinterpret_cast<const void*>(select_cluster_kernel<64, true>)
-                                         : reinterpret_cast<const void*>(select_cluster_kernel<64, false>));
-    // the cluster size is looked up once per instance, for the largest shared-memory size the form
-    // is used with (a cluster that fits with that fits with less)
-    constexpr size_t kMaxSmem = 96 * 1024;
-    static int cached_cs[2][2] = {{-1, -1}, {-1, -1}};  // [D == 128][mixed]
-    int& cs = cached_cs[a.D == 128][mixed];
-    bool ok = smem <= kMaxSmem;
-    if (ok && cs < 0) {
-      ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMaxSmem)) == cudaSuccess;
-      cs = ok ? cluster_size_for(fn, kMaxSmem, 256 * kSubBlocks) : 0;
-    }
-    if (ok && cs > 0) {
-      cudaError_t e1 = launch_pdl(f_qsum, dim3(n_tiles, a.H), dim3(256), 0, p_args, st);
-      if (e1 != cudaSuccess) return e1;
-      int cs_arg = cs;
-      void* params[2] = {&aa, &cs_arg};
-      return launch_pdl(fn, dim3(static_cast<unsigned>(cs * a.H)), dim3(256 * kSubBlocks), smem, params, st, cs);
-    }
-    cudaGetLastError();  // no cluster of that shape on this device: the forms below
-  }
+  cudaError_t ec = cudaSuccess;
+  if (a.use_clusters && launch_cluster(a, nullptr, mixed, st, &ec)) return ec;
   if (a.barrier && coop_info(&nsm)) {
     // one cooperative launch for all three stages
     const size_t smem_keys = static_cast<size_t>(nblk_all > 0 ? nblk_all : 1) * sizeof(uint32_t);
@@ -1116,6 +1289,37 @@ cudaError_t launch_select(const SelectArgs& a, cudaStream_t st) {
   const void* f3 = mixed ? reinterpret_cast<const void*>(topk_kernel<true>) : reinterpret_cast<const void*>(topk_kernel<false>);
   if (smem > 40 * 1024) cudaFuncSetAttribute(f3, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
   return launch_pdl(f3, dim3(a.n_groups, a.H), dim3(256), smem, p_args, st);
+}
+
+cudaError_t launch_select_adaptive(const SelectArgs& a, const AdaptiveArgs& ad, cudaStream_t st) {
+  cudaError_t e = cudaSuccess;
+  // one list per head: scores and lists in one cluster per head; several groups share their head's
+  // threshold (mean of the groups' Gini coefficients), which takes a kernel of its own
+  if (launch_cluster(a, &ad, false, st, &e)) return e;
+  e = launch_qsum(a, st);
+  if (e != cudaSuccess) return e;
+  const int64_t nblk = (a.n_tokens + kBlock - 1) / kBlock;
+  if (nblk > 0) {
+    dim3 g2(static_cast<unsigned>((nblk + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta), a.n_groups, a.H);
+    if (a.D == 128)
+      block_scores_kernel<128, false><<<g2, 256, 0, st>>>(a);
+    else
+      block_scores_kernel<64, false><<<g2, 256, 0, st>>>(a);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  int np2 = 1;
+  while (np2 < nblk) np2 <<= 1;
+  const size_t smem_sort = static_cast<size_t>(np2) * 8;
+  if (smem_sort > 40 * 1024)
+    cudaFuncSetAttribute(adaptive_sort_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         static_cast<int>(smem_sort));
+  dim3 g3(a.n_groups, a.H);
+  adaptive_sort_kernel<<<g3, 256, smem_sort, st>>>(a, ad);
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  adaptive_pick_kernel<<<g3, 256, static_cast<size_t>(nblk > 0 ? nblk : 1), st>>>(a, ad);
+  return cudaGetLastError();
 }
 
 }  // namespace hsa

@@ -155,3 +155,53 @@ def test_kv_page_scores(d, H, n, kvb, cuda_device):
     best = torch.sort(scores.cpu(), descending=True, stable=True).indices[:min(3, n_pages)]
     assert ids.cpu().tolist() == sorted(best.tolist())
     ctx.destroy()
+
+
+@pytest.mark.parametrize("d,H,n,n_q,causal", [
+    (128, 2, 1, 1, False), (128, 2, 64, 130, False), (64, 3, 65, 64, True), (128, 3, 31 * 64, 200, False),
+    (128, 2, 32 * 64, 128, True), (64, 2, 33 * 64 - 5, 3200, False), (128, 2, 767 * 64, 300, False),
+    (128, 1, 769 * 64 + 1, 3100, True), (64, 1, 6144 * 64, 100, False), (64, 1, 6145 * 64, 100, False)])
+def test_adaptive_lists(d, H, n, n_q, causal, cuda_device):
+    """Cumulative-mass lists at one block, at the edges of the sort's warp segments and of the threads' shares,
+    at the largest history of the one-kernel form and behind it, with the query sums taken inside the
+    clusters (up to 24 tiles) and in front of them."""
+    from paper_2609_34606_b200 import hsa
+    g = torch.Generator().manual_seed(n + n_q)
+    K, q = _randn(g, n, H, d), _randn(g, n_q, H, d)
+    nb = (n + 63) // 64
+    ctx = hsa.HSAContext(H, d, max_pages=nb, max_q_tokens=max(n, n_q), max_topk=nb, lin_mode=hsa.HSA_LIN_NONE, adaptive=True,
+                         device=cuda_device)
+    kd = K.to(cuda_device)
+    ctx.append_kv(kd, kd)
+    pos = max(0, n // 2 - n_q) if causal else n
+    idx, cnt, gt = ctx.select_blocks_adaptive(q.to(cuda_device), 0.35, 1.0, q_pos0=pos, causal=causal)
+    assert ctx.device_status() == 0
+    got = Hn.selection_lists(idx, cnt)
+    ref, gini, tau = O.adaptive_selection(Hn.f32(q), Hn.f32(K), pos, causal, 0.35, 1.0)
+    assert np.allclose(gt.cpu().numpy(), np.stack([gini, tau]), atol=1e-5)
+    for h in range(H):
+        a, b = list(got[h][0]), list(ref[h][0])
+        assert a == sorted(set(a)) and abs(len(a) - len(b)) <= 1
+        # (the GPU ranks scores rounded to fp32: neighbours in the order may change places at the boundary)
+        assert len(set(a) ^ set(b)) <= 2
+    ctx.destroy()
+
+
+@pytest.mark.parametrize("n_q", [3072, 3073])
+def test_query_sums_inside_the_clusters(n_q, cuda_device):
+    """24 query tiles are the most whose sums the clusters take themselves: lists as in the grid-barrier form."""
+    from paper_2609_34606_b200 import hsa
+    g = torch.Generator().manual_seed(n_q)
+    H, d, n = 5, 128, 20000
+    K, q = _randn(g, n, H, d).to(cuda_device), _randn(g, n_q, H, d).to(cuda_device)
+    budgets = torch.tensor([1, 0, 17, 64, -1], dtype=torch.int32, device=cuda_device)
+    lists = []
+    for grid_form in (False, True):
+        ctx = hsa.HSAContext(H, d, max_pages=313, max_q_tokens=n, max_topk=313, lin_mode=hsa.HSA_LIN_NONE, device=cuda_device,
+                             grid_barrier_select=grid_form)
+        ctx.append_kv(K, K)
+        idx, cnt = ctx.select_blocks(q, budgets)
+        assert ctx.device_status() == 0
+        lists.append([r[0].tolist() for r in Hn.selection_lists(idx, cnt)])
+        ctx.destroy()
+    assert lists[0] == lists[1] and [len(r) for r in lists[0]] == [1, 0, 17, 64, 313]
