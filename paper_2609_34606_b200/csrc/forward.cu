@@ -207,9 +207,9 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   int tile = blockIdx.x, h = blockIdx.y, part = blockIdx.z;
   // Parts of a list of `st` two-page steps.  balance > 0: the steps one SM would run if the whole
   // launch were spread evenly; a list is cut into the fewest parts none of which is longer than that
-  // (no part shorter than 16 steps).  balance == 0: parts of split_blocks blocks.
+  // (no part shorter than min_part_steps).  balance == 0: parts of split_blocks blocks.
   auto parts_of = [&](int st, int balance) -> int {
-    const int want = balance > 0 ? min((st + balance - 1) / balance, max(1, st / 16))
+    const int want = balance > 0 ? min((st + balance - 1) / balance, max(1, st / p.min_part_steps))
                                  : (st + p.split_blocks / 2 - 1) / (p.split_blocks / 2);
     int ns = min(p.max_splits, max(1, want));
     const int per = (st + ns - 1) / ns;
@@ -217,6 +217,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     return ns;
   };
   int balance = 0;
+  int slot_step = 1;  // from one part's partial-result slot to the next part's
   if (SPLIT && p.remap) {
     // Longest lists first.  With one list per head every (tile, part) of a head costs the same, so the
     // heads are ranked by the steps one part of theirs takes and the grid walks through them in that
@@ -230,7 +231,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     int total = st;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-    balance = max(1, static_cast<int>((static_cast<int64_t>(total) * n_tiles + p.nsm - 1) / p.nsm));
+    balance = max(1, static_cast<int>((static_cast<int64_t>(total) * n_tiles + p.balance_sms - 1) / p.balance_sms));
     const int ns = parts_of(st, balance);
     const int per = (st + ns - 1) / ns;
     const int n_items = lane < p.H ? ns * n_tiles : 0;
@@ -252,6 +253,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     const int local = lin - __shfl_sync(0xffffffffu, start, h);
     part = local / n_tiles;
     tile = local % n_tiles;
+    slot_step = n_tiles;
   }
   const int row0 = tile * kTileM;
   const int g = p.group_tokens > 0 ? row0 / p.group_tokens : 0;
@@ -273,7 +275,8 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       cnt = b_hi - b_lo;
     }
   }
-  const int slot = (tile * p.H + h) * p.max_splits + part;  // this CTA's partial-result slot
+  // this CTA's partial-result slot: the CTA's own number where the grid is one-dimensional
+  const int slot = (SPLIT && p.remap) ? static_cast<int>(blockIdx.x) : (tile * p.H + h) * p.max_splits + part;
   // steps of the compressed segment (LINF), then of the selected pages
   const int lf_pages = LINF ? p.lf_pages : 0;
   const int nA = (lf_pages + 1) / 2;
@@ -839,7 +842,9 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       float pf[SPLIT ? kFwdSplitMax : 1];  // merge factors 2^(ref_p - max ref) of the parts (split tiles only)
       if (SPLIT && nsplit > 1 && final_attempt) {
         if (ok) {
-          float* po = p.part_o + (static_cast<size_t>(slot) * kTileM + r) * D + cbase;
+          // (column groups of four outermost, then rows: the lanes of a warp write and, at the merge, read
+          // whole lines; row by row, every access of a warp touched 32 lines)
+          float* po = p.part_o + (static_cast<size_t>(slot) * (D / 4) + cbase / 4) * (kTileM * 4) + r * 4;
 #pragma unroll 1
           for (int c0 = 0; c0 < HC; c0 += 16) {
             uint32_t oa[16];
@@ -847,7 +852,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             tc_wait_ld();
 #pragma unroll
             for (int i = 0; i < 16; i += 4)
-              *reinterpret_cast<float4*>(po + c0 + i) =
+              *reinterpret_cast<float4*>(po + (c0 + i) * kTileM) =
                   make_float4(__uint_as_float(oa[i]), __uint_as_float(oa[i + 1]), __uint_as_float(oa[i + 2]),
                               __uint_as_float(oa[i + 3]));
           }
@@ -869,22 +874,23 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         if (do_output) {
           __threadfence();
           // common reference R = largest reference among the parts that saw a key for this row
-          const size_t s0 = static_cast<size_t>(slot - part) * kTileM + r;
+          const size_t s0 = static_cast<size_t>(slot - part * slot_step) * kTileM + r;
+          const size_t sq = static_cast<size_t>(slot_step) * kTileM;
+          // (all of them asked for at once: one round trip, where a loop took two or three per part)
+          float lq[SPLIT ? kFwdSplitMax : 1];
+#pragma unroll
+          for (int q = 0; q < (SPLIT ? kFwdSplitMax : 1); ++q) {
+            lq[q] = q < nsplit ? __ldcg(&p.part_l[s0 + q * sq]) : 0.f;
+            pf[q] = q < nsplit ? __ldcg(&p.part_ref[s0 + q * sq]) : 0.f;
+          }
           float rmax = -INFINITY;
-          for (int q = 0; q < nsplit; ++q)
-            if (__ldcg(&p.part_l[s0 + static_cast<size_t>(q) * kTileM]) > 0.f)
-              rmax = fmaxf(rmax, __ldcg(&p.part_ref[s0 + static_cast<size_t>(q) * kTileM]));
+#pragma unroll
+          for (int q = 0; q < (SPLIT ? kFwdSplitMax : 1); ++q) rmax = lq[q] > 0.f ? fmaxf(rmax, pf[q]) : rmax;
           float ltot = 0.f;
 #pragma unroll
           for (int q = 0; q < (SPLIT ? kFwdSplitMax : 1); ++q) {
-            pf[q] = 0.f;
-            if (q < nsplit) {
-              const float lq = __ldcg(&p.part_l[s0 + static_cast<size_t>(q) * kTileM]);
-              if (lq > 0.f) {
-                pf[q] = ex2(__ldcg(&p.part_ref[s0 + static_cast<size_t>(q) * kTileM]) - rmax);
-                ltot = fmaf(lq, pf[q], ltot);
-              }
-            }
+            pf[q] = lq[q] > 0.f ? ex2(pf[q] - rmax) : 0.f;
+            ltot = fmaf(lq[q], pf[q], ltot);
           }
           inv_l = ltot > 0.f ? 1.f / ltot : 0.f;
         }
@@ -998,13 +1004,13 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             float acc[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) acc[i] = 0.f;
-            const float* po = p.part_o + (static_cast<size_t>(slot - part) * kTileM + r) * D + c0;
+            const float* po = p.part_o + (static_cast<size_t>(slot - part * slot_step) * (D / 4) + c0 / 4) * (kTileM * 4) + r * 4;
 #pragma unroll
             for (int q = 0; q < (SPLIT ? kFwdSplitMax : 1); ++q) {
               if (q < nsplit && pf[q] != 0.f) {
 #pragma unroll
                 for (int i = 0; i < 16; i += 4) {
-                  const float4 v = __ldcg(reinterpret_cast<const float4*>(po + static_cast<size_t>(q) * kTileM * D + i));
+                  const float4 v = __ldcg(reinterpret_cast<const float4*>(po + static_cast<size_t>(q) * slot_step * kTileM * D + i * kTileM));
                   acc[i] = fmaf(pf[q], v.x, acc[i]);
                   acc[i + 1] = fmaf(pf[q], v.y, acc[i + 1]);
                   acc[i + 2] = fmaf(pf[q], v.z, acc[i + 2]);

@@ -15,6 +15,11 @@ constexpr int kStateSplitMax = 16;       // token-axis splits of the state updat
 // the bf16 rounding of z, row 1 the bf16 rounding of the remainder, rows 2..15 are zero, so that
 // phi(Q) times it gives the denominator phi(q).z as the sum of two accumulator columns
 constexpr int kZopBytes = 4096;
+// partial-result slots of a context whose lists are too short to be split for their length: enough for a
+// launch that has at most half as many (query tile, head) items as the GPU has SMs (see hsa_forward)
+constexpr int kFewItemsSlots = 240;
+constexpr int kFewItemsMinBlocks = 48;   // shorter lists are not split for that
+constexpr int kFewItemsPart = 8;         // shortest part of such a launch, in two-page steps
 constexpr int kFwdSplitMax = 16;         // CTAs a long (query tile, head) of the forward kernel is split over
 
 __host__ __device__ inline int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
@@ -140,11 +145,13 @@ struct FwdParams {
   // (grid z = max_splits); each dumps its unnormalised O, row sums and exponent references, the last
   // one to take a ticket merges them and writes the output
   int max_splits, split_blocks;
+  int min_part_steps;    // shortest part of the balance rule, in two-page steps
+  int balance_sms;       // SMs the balance rule spreads the steps over
   int n_tiles, remap;    // set by the launcher: query tiles; 1 = one-dimensional grid, longest lists first
   int nsm;               // SMs of the device (the split rule balances the launch over them)
-  float* part_o;         // [tiles][H][max_splits][128][D]
-  float* part_l;         // [tiles][H][max_splits][128]
-  float* part_ref;       // [tiles][H][max_splits][128]
+  float* part_o;         // [slots][D / 4][128][4]: slot (tile H + h) max_splits + part, or the CTA's number (remap)
+  float* part_l;         // [slots][128]
+  float* part_ref;       // [slots][128]
   int32_t* part_ticket;  // [tiles][H], zero between launches
   int32_t* status;
   // L2 look-ahead of the page gather: the pools themselves (null: none)

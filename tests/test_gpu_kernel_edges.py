@@ -205,3 +205,38 @@ def test_query_sums_inside_the_clusters(n_q, cuda_device):
         lists.append([r[0].tolist() for r in Hn.selection_lists(idx, cnt)])
         ctx.destroy()
     assert lists[0] == lists[1] and [len(r) for r in lists[0]] == [1, 0, 17, 64, 313]
+
+
+@pytest.mark.parametrize("d,H,n_q,budgets,gates,causal", [
+    (128, 2, 256, (128, 128), "", False), (128, 4, 600, (100, 0, 17, 100), "dim", False), (64, 4, 600, (100, 3, 100, 99), "head", False),
+    (128, 2, 100, (128, 1), "", False), (128, 3, 300, (110, 110, 110), "", True), (64, 1, 1, (128,), "", False)])
+def test_lists_of_few_items_split_over_ctas(d, H, n_q, budgets, gates, causal, cuda_device):
+    """A launch with few (query tile, head) items cuts their lists into parts: against the same lists given
+    per query tile, which one CTA walks from end to end (with one tile both calls take the rule, and the
+    oracle tests of the split kernel cover it)."""
+    from paper_2609_34606_b200 import hsa
+    n = 130 * 64 - 11
+    g = torch.Generator().manual_seed(n_q + H)
+    K, V, q = _randn(g, n, H, d), _randn(g, n, H, d), _randn(g, n_q, H, d).to(cuda_device)
+    kd, vd = K.to(cuda_device), V.to(cuda_device)
+    ctx = hsa.HSAContext(H, d, max_pages=130, max_q_tokens=n, max_topk=128, device=cuda_device, causal=causal)
+    n0 = n - n_q
+    ctx.append_kv(kd[:n0], vd[:n0])
+    ctx.append_kv(kd[n0:], vd[n0:])
+    pos = n0 if causal else n
+    idx, cnt = ctx.select_blocks(q, torch.tensor(budgets, dtype=torch.int32, device=cuda_device), q_pos0=pos, causal=causal)
+    gl = gs = None
+    if gates:
+        shape = (n_q, H, d) if gates == "dim" else (n_q, H)
+        gl, gs = _randn(g, *shape).to(cuda_device), _randn(g, *shape).to(cuda_device)
+    for _ in range(2):  # (the tickets are back at zero for the second launch)
+        out = ctx.forward(q, idx, cnt, q_pos0=pos, causal=causal, g_lin=gl, g_sp=gs)
+    # several groups never take the rule: the same list for every tile
+    tiles = (n_q + 127) // 128
+    many = ctx.forward(q, idx.expand(H, tiles, 128).contiguous(), cnt.expand(H, tiles).contiguous(), q_pos0=pos, causal=causal,
+                       group_tokens=128, g_lin=gl, g_sp=gs)
+    assert ctx.device_status() == 0
+    a, b = out.double(), many.double()
+    # the parts take their exponent references from other keys: weights round to bf16 differently
+    assert float((a - b).norm() / b.norm()) <= BF16_REL
+    ctx.destroy()
