@@ -169,6 +169,13 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                    const __grid_constant__ CUtensorMap tm_vc, const __grid_constant__ CUtensorMap tm_gl,
                    const __grid_constant__ CUtensorMap tm_gs, const FwdParams p) {
   static_assert(!(SPLIT && LINF), "split lists and the compressed segment are not combined");
+  // AHEAD: a step's bookkeeping before the wait for its scores (350 cycles that came after it), and the
+  // issuing lane's barriers looked at while P V runs (a barrier costs some 100 cycles to ask even if it is
+  // complete: shared memory is the busiest unit of this loop, 160 KB per step at 128 B per clock).  With
+  // two score buffers this shortens the chain that bounds the loop: Linformer pass 245.4 -> 236.5 us; long
+  // split lists 418.8 -> 415.4.  With three buffers and short lists it does not pay: 64 blocks 152.5 against
+  // 153.2, 128 blocks 272.6 against 270.2.
+  constexpr bool AHEAD = SPLIT || LINF;
   constexpr int NSB = LINF ? 2 : kSBufs;                 // score buffers in use
   constexpr uint32_t kColSb = LINF ? 256 : kColS;        // first score buffer
   constexpr uint32_t kColLn = LINF ? 128 : kColLin;      // linear-branch accumulator
@@ -436,9 +443,10 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         const uint32_t q_lo = desc_lo_sw128(smem_u32(smem + L::kQ), 16);
         bool ok = wait_bar(&bars->q_full, 0, bars, p.status);
         tc_fence_after();
-        auto issue_qk = [&](int j) -> bool {
+        // landed: the step's K tile has been seen complete already
+        auto issue_qk = [&](int j, bool landed) -> bool {
           const int s = j % kStages;
-          if (!wait_bar(&bars->k_full[s], (j / kStages) & 1, bars, p.status)) return false;
+          if (!landed && !wait_bar(&bars->k_full[s], (j / kStages) & 1, bars, p.status)) return false;
           tc_fence_after();
           const uint32_t k_lo = desc_lo_sw128(smem_u32(smem + L::kK + s * L::kTile), 16);
           const uint32_t d_tmem = tmem + kColSb + 128 * (j % NSB);
@@ -461,14 +469,15 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           tc_commit(&bars->s_full[j % NSB]);
           return true;
         };
-        for (int j = 0; j < min(NSB, nsteps) && ok; ++j) ok = issue_qk(j);
+        for (int j = 0; j < min(NSB, nsteps) && ok; ++j) ok = issue_qk(j, false);
+        bool p_ready = false, v_landed = false;
 #pragma unroll 1
         for (int j = 0; j < nsteps && ok; ++j) {
           const int s = j % kStages;
           const int b = j % NSB;
-          ok = wait_bar(&bars->p_full[b], (j / NSB) & 1, bars, p.status);
+          if (!p_ready) ok = wait_bar(&bars->p_full[b], (j / NSB) & 1, bars, p.status);
           if (!ok) break;
-          ok = wait_bar(&bars->v_full[s], (j / kStages) & 1, bars, p.status);
+          if (!v_landed) ok = wait_bar(&bars->v_full[s], (j / kStages) & 1, bars, p.status);
           if (!ok) break;
           tc_fence_after();
           constexpr uint32_t idesc = idesc_bf16_f32(128, D, 0, 1);
@@ -485,10 +494,17 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
               tc_mma_ts_lo(o_acc, p_op + kk * 8, v_lo + kk * 128, kHiSw, idesc, 1u);
           }
           tc_commit(&bars->v_empty[s]);
-          tc_commit(&bars->pv_done);
+          if (!AHEAD || safe) tc_commit(&bars->pv_done);  // (the fast pass never rescales)
+          bool k_landed = false;
+          if (AHEAD) {  // the next step's weights and V tile, and the K tile behind them, while P V runs
+            const int jv = j + 1, jk = j + NSB;
+            p_ready = jv < nsteps && mbar_test_wait(&bars->p_full[jv % NSB], (jv / NSB) & 1);
+            v_landed = jv < nsteps && mbar_test_wait(&bars->v_full[jv % kStages], (jv / kStages) & 1);
+            k_landed = jk < nsteps && mbar_test_wait(&bars->k_full[jk % kStages], (jk / kStages) & 1);
+          }
           // the scores of step j+3 overwrite the P just consumed: issued after the P V above,
           // the tensor pipe runs them in order
-          if (j + NSB < nsteps) ok = issue_qk(j + NSB);
+          if (j + NSB < nsteps) ok = issue_qk(j + NSB, k_landed);
         }
         if (ok) tc_commit(&bars->o_done);
         if (ok && p.do_linear && !LINF) {
@@ -612,27 +628,31 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         const uint32_t o_seg = seg_a ? tmem + lane_off + kColLn : o_tmem;
         const int b = j % NSB;
         const uint32_t s_tmem = tmem + lane_off + kColSb + 128 * b;
+        // bookkeeping of the step: page count, visible keys per page (columns [0, lim) of the page's 64)
+        const int npg = pages_of(j);
+        const int n = npg * kBlock;
+        const int nchunks = n / 32;
+        bool need_mask = false;
+        int lim0 = kBlock, lim1 = kBlock;
+        auto bookkeeping = [&]() {
+          if (blk0 < 0 || blk0 >= seg_blocks) blk0 = 0;
+          if (blk1 < 0 || blk1 >= seg_blocks) blk1 = 0;
+          const int64_t last_blk = blk0 > blk1 ? blk0 : blk1;
+          need_mask = (n != 128) || (last_blk * kBlock + kBlock > seg_tile_vis);
+          if (need_mask) {
+            lim0 = static_cast<int>(max64(0, min64(kBlock, seg_vis - static_cast<int64_t>(blk0) * kBlock)));
+            lim1 = npg > 1 ? static_cast<int>(max64(0, min64(kBlock, seg_vis - static_cast<int64_t>(blk1) * kBlock))) : 0;
+          }
+        };
+        if (AHEAD) bookkeeping();
         ok = __all_sync(0xffffffffu, wait_bar(&bars->s_full[b], (j / NSB) & 1, bars, p.status));
         if (!ok) break;
         tc_fence_after();
         uint32_t cbuf[2][32];  // two 32-column chunks of the score row in flight
-        // the first chunk is requested at once: its latency runs under the bookkeeping below
-        // (the steps that look for the row maximum first issue their own loads)
+        // the first chunk is requested at once (the steps that look for the row maximum first issue their own loads)
         const bool early_ld = !(safe || seg_first);
         if (early_ld) tmem_ld32(s_tmem, cbuf[0]);
-        const int npg = pages_of(j);
-        const int n = npg * kBlock;
-        if (blk0 < 0 || blk0 >= seg_blocks) blk0 = 0;
-        if (blk1 < 0 || blk1 >= seg_blocks) blk1 = 0;
-        const int64_t last_blk = blk0 > blk1 ? blk0 : blk1;
-        const bool need_mask = (n != 128) || (last_blk * kBlock + kBlock > seg_tile_vis);
-        // visible keys per page: columns [0, lim) of the page's 64
-        int lim0 = kBlock, lim1 = kBlock;
-        if (need_mask) {
-          lim0 = static_cast<int>(max64(0, min64(kBlock, seg_vis - static_cast<int64_t>(blk0) * kBlock)));
-          lim1 = npg > 1 ? static_cast<int>(max64(0, min64(kBlock, seg_vis - static_cast<int64_t>(blk1) * kBlock))) : 0;
-        }
-        const int nchunks = n / 32;
+        if (!AHEAD) bookkeeping();
         if (safe || seg_first) {
           // the reference needs the row maximum first: a pass over the score row in chunks
           float mxa = -INFINITY, mxb = -INFINITY;
