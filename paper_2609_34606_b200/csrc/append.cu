@@ -219,7 +219,8 @@ __device__ __forceinline__ void tma_store_2d(const void* tmap, const void* smem_
 
 // RELU: the feature map is max(x, 0) instead of elu(x) + 1 (an instance of its own: the map sits in
 // the innermost loop of the worker warps)
-template <int D, bool RELU>
+// KEEP (causal contexts): the workers leave phi(K) in the workspace as well (AppendArgs::phik)
+template <int D, bool RELU, bool KEEP>
 __global__ void __launch_bounds__(kAfThreads, 1)
 append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CUtensorMap tm_kin,
                     const __grid_constant__ CUtensorMap tm_vin, const __grid_constant__ CUtensorMap tm_kpool,
@@ -463,7 +464,7 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
 #pragma unroll
         for (int m = 0; m < L::kTerms; ++m)
           *reinterpret_cast<uint4*>(ph + m * L::kTile + soff[i]) = make_uint4(tw[m][0], tw[m][1], tw[m][2], tw[m][3]);
-        if (a.phik) {  // causal contexts: the first two terms of phi(K) stay for the chunk's own forward
+        if (KEEP) {  // the first two terms of phi(K) stay for the chunk's own forward
           const size_t row = (static_cast<size_t>(h) * 2 * a.phik_blocks + (b - b_first)) * kBlock + rg + RS * i;
 #pragma unroll
           for (int m = 0; m < 2; ++m)
@@ -521,7 +522,12 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
       for (int i = 0; i < NC / 4; ++i)
         srow[i] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]),
                               __uint_as_float(v[4 * i + 2]), __uint_as_float(v[4 * i + 3]));
-      if (zw) stage[row * L::kPitch + D] = __uint_as_float(zv[0]);
+      if (zw) {
+        if (D == 128)
+          out[D * D + row] = __uint_as_float(zv[0]);
+        else
+          stage[row * L::kPitch + D] = __uint_as_float(zv[0]);
+      }
       asm volatile("bar.sync 1, %0;" ::"n"(kAfWorkers) : "memory");
 #pragma unroll
       for (int i = 0; i < D * D / 4 / kAfWorkers; ++i) {
@@ -534,7 +540,7 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
         }
         reinterpret_cast<float4*>(out)[f] = o;
       }
-      if (w < D) out[D * D + w] = stage[w * L::kPitch + D] + (D == 64 ? stage[(w + 64) * L::kPitch + D] : 0.f);
+      if (D == 64 && w < D) out[D * D + w] = stage[w * L::kPitch + D] + stage[(w + 64) * L::kPitch + D];
     }
   }
   tc_fence_before();
@@ -545,15 +551,23 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
   }
 }
 
+namespace {
+using AppendKernel = void (*)(AppendArgs, int, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap);
+template <int D>
+AppendKernel fused_kernel(bool relu, bool keep) {
+  if (keep) return relu ? append_fused_kernel<D, true, true> : append_fused_kernel<D, false, true>;
+  return relu ? append_fused_kernel<D, true, false> : append_fused_kernel<D, false, false>;
+}
+}  // namespace
+
 cudaError_t append_init() {
   cudaError_t e = cudaSuccess;
-  auto set = [&](auto* fn, int bytes) {
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  };
-  set(append_fused_kernel<128, false>, AfSmem<128>::kTotal);
-  set(append_fused_kernel<128, true>, AfSmem<128>::kTotal);
-  set(append_fused_kernel<64, false>, AfSmem<64>::kTotal);
-  set(append_fused_kernel<64, true>, AfSmem<64>::kTotal);
+  for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
+    const bool relu = i & 1, keep = i & 2;
+    e = cudaFuncSetAttribute(fused_kernel<128>(relu, keep), cudaFuncAttributeMaxDynamicSharedMemorySize, AfSmem<128>::kTotal);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(fused_kernel<64>(relu, keep), cudaFuncAttributeMaxDynamicSharedMemorySize, AfSmem<64>::kTotal);
+  }
   return e;
 }
 
@@ -576,8 +590,8 @@ cudaError_t launch_append(const AppendArgs& a_in, const AppendMaps* maps, cudaSt
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    auto* fn = a.D == 128 ? (a.relu ? append_fused_kernel<128, true> : append_fused_kernel<128, false>)
-                          : (a.relu ? append_fused_kernel<64, true> : append_fused_kernel<64, false>);
+    const bool keep = a.phik != nullptr;
+    AppendKernel fn = a.D == 128 ? fused_kernel<128>(a.relu, keep) : fused_kernel<64>(a.relu, keep);
     e = cudaLaunchKernelEx(&cfg, fn, a, per, maps->kin, maps->vin, maps->kpool, maps->vpool);
     if (e != cudaSuccess) return e;
   } else {
