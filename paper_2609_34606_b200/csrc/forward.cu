@@ -978,11 +978,13 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             }
           }
         }
-        // gate tiles without causal partials, external linear output or merge.  (Working the
+        // every gate given is a tile (a base off the 16-byte boundary is read by the loop behind this one), no
+        // causal partials, external linear output or merge.  (Working the
         // weights out ahead of the accumulators, in registers, needs the trips unrolled, and code that a
         // CTA runs once is fetched cold: 176 us a pass against 164 with this loop, 12 heads of 128, 4680
         // tokens; value by value from global memory, which this replaces: 207.)
-        const bool gated = GT && !(p.do_linear && p.lin_num != nullptr) && !p.ext_lin && !(SPLIT && nsplit > 1);
+        const bool gated = GT && (!p.g_lin || (p.gate_tiles & 1)) && (!p.g_sp || (p.gate_tiles & 2)) &&
+                           !(p.do_linear && p.lin_num != nullptr) && !p.ext_lin && !(SPLIT && nsplit > 1);
         if (gated) {
           const float il = has_o ? inv_l : 0.f, id = has_lin ? inv_den : 0.f;
 #pragma unroll 1

@@ -131,6 +131,37 @@ def test_gate_layouts(d, n_q, topk, layout, act, split, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("d,split,form", [(128, 0, "state"), (64, 0, "state"), (128, 2, "state"), (64, 2, "state"), (128, 0, "linformer")])
+@pytest.mark.parametrize("which", ["g_lin", "g_sp"])
+def test_one_gate_off_the_tile_alignment(d, split, form, which, cuda_device):
+    """Per-dim gates of which only one starts on a 16-byte boundary (the other is a view one element into its
+    buffer): both are applied."""
+    from paper_2609_34606_b200 import hsa
+    H, n, n_q = 3, 640, 200
+    g = torch.Generator().manual_seed(d + split)
+    rand = lambda *s: _randn(g, *s).to(cuda_device)
+    opt = {}
+    if form == "linformer":
+        opt = dict(lin_mode=hsa.HSA_LIN_LINFORMER, lin_rank=64, lin_seg_tokens=n, e_k=rand(H, n, 64) * 0.04, e_v=rand(H, n, 64) * 0.04)
+    ctx = hsa.HSAContext(H, d, max_pages=10, max_q_tokens=n, max_topk=10, device=cuda_device, gate_act=1, split_blocks=split, **opt)
+    ctx.append_kv(rand(n, H, d), rand(n, H, d))
+    q = rand(n_q, H, d)
+    idx, cnt = ctx.select_blocks(q, torch.full((H,), 6, dtype=torch.int32, device=cuda_device))
+    gates = {"g_lin": rand(n_q, H, d), "g_sp": rand(n_q, H, d)}
+    both = ctx.forward(q, idx, cnt, **gates)
+    moved = torch.empty(n_q * H * d + 1, dtype=torch.bfloat16, device=cuda_device)[1:].view(n_q, H, d)
+    gates[which] = moved.copy_(gates[which])
+    out = ctx.forward(q, idx, cnt, **gates)
+    lin = ctx.forward(q, idx, cnt, flags=hsa.HSA_FWD_NO_SPARSE).double()
+    sp = ctx.forward(q, idx, cnt, flags=hsa.HSA_FWD_NO_LINEAR).double()
+    assert ctx.device_status() == 0
+    a, b = torch.sigmoid(gates["g_lin"].double()) * lin, torch.sigmoid(gates["g_sp"].double()) * sp
+    # the branches are rounded to bf16 before they are merged here, the result is once
+    assert float(((out.double() - a - b).abs() - 2 * BF16_REL * (a.abs() + b.abs()) - 1e-6).max()) <= 0.0
+    # and as with both on the boundary: the same arithmetic up to the order of two products
+    assert float((out.double() - both.double()).abs().max()) <= 2 * BF16_REL * float(both.double().abs().max())
+    ctx.destroy()
+
 @pytest.mark.parametrize("d,H,n,kvb", [(128, 3, 65, 1), (128, 2, 5000, 7), (64, 5, 5000, 195), (128, 12, 70000, 195),
                                        (64, 2, 70000, 256), (128, 2, 70000, 257), (128, 1, 70000, 700), (128, 2, 70000, 5000)])
 def test_kv_page_scores(d, H, n, kvb, cuda_device):
