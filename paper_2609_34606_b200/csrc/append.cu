@@ -3,6 +3,8 @@
 // as a deterministic two-stage reduction (no floating-point atomics).
 #include <cuda_bf16.h>
 
+#include <cfloat>
+
 #include "hsa_internal.h"
 #include "ptx.cuh"
 
@@ -77,6 +79,20 @@ __global__ void __launch_bounds__(256) append_pool_ksum_kernel(AppendArgs a) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+// One entry of the chunk's sum (idx < D * D: S[idx / D][idx % D], else z[idx - D * D]), token by token in fp32.
+__device__ __noinline__ float chunk_sum(const AppendArgs& a, int h, int idx) {
+  const bool is_s = idx < a.D * a.D;
+  const __nv_bfloat16* k = a.k + static_cast<size_t>(h) * a.head_stride + (is_s ? idx / a.D : idx - a.D * a.D);
+  const __nv_bfloat16* v = a.v + static_cast<size_t>(h) * a.head_stride + (is_s ? idx % a.D : 0);
+  float sum = 0.f;
+  for (int t = 0; t < a.n_new; ++t) {
+    const float x = __bfloat162float(k[static_cast<size_t>(t) * a.tok_stride]);
+    const float f = a.relu ? fmaxf(x, 0.f) : (x > 0.f ? x + 1.f : expf(x));
+    sum = is_s ? fmaf(f, __bfloat162float(v[static_cast<size_t>(t) * a.tok_stride]), sum) : sum + f;
+  }
+  return sum;
+}
+
 // ---------------------------------------------------------------------------------------
 // Reduction: S[dst] <- S[src] + sum of partials (fixed order), with its bf16 hi/lo split (the forward
 // kernels feed hi and lo to the tensor cores as two bf16 operands), the same for z and its operand image.
@@ -98,6 +114,9 @@ __global__ void state_reduce_kernel(AppendArgs a) {
   float add = 0.f;
 #pragma unroll
   for (int i = 0; i < kStateSplitMax; ++i) add += v[i];
+  // head_dim 64: an Inf that meets the zeros of the split products (zero terms, Inf - Inf in the split itself)
+  // gives NaN where the sum of phi(k) v is Inf, so a sum that is not finite is taken again term by term
+  if (D == 64 && !(fabsf(add) <= FLT_MAX)) add = chunk_sum(a, h, idx);
   const int dst = a.src_slot ^ 1;
   if (idx < DD) {
     const size_t o = static_cast<size_t>(h) * DD + idx;

@@ -91,6 +91,32 @@ def test_append_head_dim_64(n0, n, H, relu, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("n,relu", [(1, 0), (70, 0), (1000, 0), (1000, 1)])
+def test_append_head_dim_64_not_finite(n, relu, cuda_device):
+    """Inf and NaN in K and V reach the entries of S, z and the key sums that they reach in a plain sum, as the
+    same Inf or NaN, and no other."""
+    from paper_2609_34606_b200 import hsa
+    H, d, inf, nan = 4, 64, float("inf"), float("nan")
+    g = torch.Generator().manual_seed(n + relu)
+    K, V = _randn(g, n, H, d), _randn(g, n, H, d)
+    t = n // 2
+    V[t, 0, 5], V[t, 1, 63] = inf, -inf       # head 0, 1: a value
+    K[t, 1, 9], K[0, 2, 40], K[n - 1, 2, 41] = inf, -inf, inf  # head 1, 2: keys
+    K[t, 3, 0], V[t, 3, 1] = nan, nan
+    ctx = hsa.HSAContext(H, d, max_pages=(n + 63) // 64, max_q_tokens=n, max_topk=1, device=cuda_device, feature_map=relu)
+    ctx.append_kv(K.to(cuda_device), V.to(cuda_device))
+    assert ctx.device_status() == 0
+    Kd, Vd = K.double(), V.double()
+    # (max(NaN, 0) is 0 on the GPU, as it always was with this map)
+    phi = torch.nan_to_num(Kd, nan=0.0, posinf=inf, neginf=-inf).clamp(min=0) if relu else torch.where(Kd > 0, Kd + 1, Kd.exp())
+    S = torch.stack([(phi[:, h, :, None] * Vd[:, h, None, :]).sum(0) for h in range(H)])
+    bound = 2.0 ** -24 * (4 + n ** 0.5)
+    for got, ref in ((ctx.S, S), (ctx.z, phi.sum(0)), (ctx.ksum[:, 0], Kd[:64].sum(0))):
+        got, odd = got.double().cpu(), ~ref.isfinite()
+        assert torch.equal(torch.nan_to_num(got[odd], nan=1.0), torch.nan_to_num(ref[odd], nan=1.0))
+        assert float((got[~odd] - ref[~odd]).norm()) <= bound * float(ref[~odd].norm())
+    ctx.destroy()
+
 @pytest.mark.parametrize("d,n_q,topk,layout,act,split", [
     (128, 300, 6, "dim", 1, 0), (128, 129, 1, "dim", 0, 0), (128, 128, 2, "dim", 1, 0), (128, 260, 5, "dim", 1, 2),
     (64, 300, 6, "dim", 1, 0), (64, 257, 7, "dim", 1, 2), (128, 200, 0, "dim", 1, 0), (128, 300, 6, "head", 1, 0),
