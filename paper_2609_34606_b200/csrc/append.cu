@@ -79,16 +79,14 @@ __global__ void __launch_bounds__(256) append_pool_ksum_kernel(AppendArgs a) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-// One entry of the chunk's sum (idx < D * D: S[idx / D][idx % D], else z[idx - D * D]), token by token in fp32.
-__device__ __noinline__ float chunk_sum(const AppendArgs& a, int h, int idx) {
-  const bool is_s = idx < a.D * a.D;
-  const __nv_bfloat16* k = a.k + static_cast<size_t>(h) * a.head_stride + (is_s ? idx / a.D : idx - a.D * a.D);
-  const __nv_bfloat16* v = a.v + static_cast<size_t>(h) * a.head_stride + (is_s ? idx % a.D : 0);
+// sum of phi(k) v (v null: of phi(k)) over n tokens, one after another in fp32.  (Plain arguments: the whole
+// AppendArgs by reference would be copied to the stack by every thread of the caller.)
+__device__ __noinline__ float chunk_sum(const __nv_bfloat16* k, const __nv_bfloat16* v, int64_t tok_stride, int n, int relu) {
   float sum = 0.f;
-  for (int t = 0; t < a.n_new; ++t) {
-    const float x = __bfloat162float(k[static_cast<size_t>(t) * a.tok_stride]);
-    const float f = a.relu ? fmaxf(x, 0.f) : (x > 0.f ? x + 1.f : expf(x));
-    sum = is_s ? fmaf(f, __bfloat162float(v[static_cast<size_t>(t) * a.tok_stride]), sum) : sum + f;
+  for (int t = 0; t < n; ++t) {
+    const float x = __bfloat162float(k[t * tok_stride]);
+    const float f = relu ? fmaxf(x, 0.f) : (x > 0.f ? x + 1.f : expf(x));
+    sum = v ? fmaf(f, __bfloat162float(v[t * tok_stride]), sum) : sum + f;
   }
   return sum;
 }
@@ -97,9 +95,9 @@ __device__ __noinline__ float chunk_sum(const AppendArgs& a, int h, int idx) {
 // Reduction: S[dst] <- S[src] + sum of partials (fixed order), with its bf16 hi/lo split (the forward
 // kernels feed hi and lo to the tensor cores as two bf16 operands), the same for z and its operand image.
 // ---------------------------------------------------------------------------------------
+template <int D>
 __global__ void state_reduce_kernel(AppendArgs a) {
-  const int D = a.D;
-  const int DD = D * D;
+  constexpr int DD = D * D;
   const int idx = blockIdx.x * blockDim.x + threadIdx.x;
   const int h = blockIdx.y;
   if (idx >= DD + D) return;
@@ -116,7 +114,12 @@ __global__ void state_reduce_kernel(AppendArgs a) {
   for (int i = 0; i < kStateSplitMax; ++i) add += v[i];
   // head_dim 64: an Inf that meets the zeros of the split products (zero terms, Inf - Inf in the split itself)
   // gives NaN where the sum of phi(k) v is Inf, so a sum that is not finite is taken again term by term
-  if (D == 64 && !(fabsf(add) <= FLT_MAX)) add = chunk_sum(a, h, idx);
+  if (D == 64 && !(fabsf(add) <= FLT_MAX)) {
+    const __nv_bfloat16* kh = a.k + static_cast<size_t>(h) * a.head_stride;
+    const __nv_bfloat16* vh = a.v + static_cast<size_t>(h) * a.head_stride;
+    add = idx < DD ? chunk_sum(kh + idx / D, vh + idx % D, a.tok_stride, a.n_new, a.relu)
+                   : chunk_sum(kh + idx - DD, nullptr, a.tok_stride, a.n_new, a.relu);
+  }
   const int dst = a.src_slot ^ 1;
   if (idx < DD) {
     const size_t o = static_cast<size_t>(h) * DD + idx;
@@ -643,7 +646,7 @@ cudaError_t launch_append(const AppendArgs& a_in, const AppendMaps* maps, cudaSt
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, state_reduce_kernel, a);
+  return cudaLaunchKernelEx(&cfg, a.D == 128 ? state_reduce_kernel<128> : state_reduce_kernel<64>, a);
 }
 
 }  // namespace hsa
