@@ -165,12 +165,14 @@ __global__ void state_reduce_kernel(AppendArgs a) {
 // head_dim 128: phi(K) = hi + lo (~16 bits), two products into one accumulator of 128 lanes.
 // head_dim 64: phi(K) = hi + mid + lo (~24 bits: this size was summed in fp32 before it came here).  A
 // product has 128 lanes, so that hi and mid go through it together, as the two 64-lane halves of one
-// operand (their tiles lie one behind the other), and lo with a tile of zeros (beside hi, on mid's lanes);
-// ksum takes K and, unused, V.  Alternate blocks have accumulators of their own, and those and the two
-// halves are added in fp32 when the partial state is written (every product truncates what it adds to).
-// Measured at head_dim 64, 16 heads, chunks of 1000 tokens: 16.2 -> 9.3 us for the whole append (a page
-// kernel and an fp32 SIMT state kernel before it), error of S against 64 bits 1.9e-7 -> 1.3e-7; what is
-// left is latency (launch, first data, two kernels): the 8.3 MB take 1.3 us at the copy bandwidth.
+// operand (their tiles lie one behind the other), and lo with a tile of zeros (beside hi, on mid's lanes).
+// Every product truncates what it adds to, so the products take turns at four accumulators, and those and
+// the two halves are added in rounded fp32 when the partial state is written.  The key sums are taken by the
+// workers and the key-sum warps, in rounded fp32 and, for a block that is new as a whole, in the order of the
+// page kernel above.
+// Error against 64 bits, the fp32 SIMT kernels this replaced -> now (2-norm, N(0, 1) inputs): 16 heads, 1000
+// tokens, S 1.6e-7 -> 7.8e-8, z 7.4e-8 -> 5.1e-8; 40 heads, 4680 tokens, S 5.8e-7 -> 2.9e-7, z 4.9e-7 ->
+// 3.4e-8; with one accumulator per two blocks S was 8.4e-8 and 6.3e-7.
 // Every wait is bounded; on expiry the CTA records a timeout and leaves.
 // ---------------------------------------------------------------------------------------
 
@@ -180,8 +182,8 @@ constexpr int kAfDepth = 4;                      // ring stages
 constexpr int kAfWorkers = 512;                  // worker threads (warps 2..17)
 constexpr int kAfThreads = 64 + kAfWorkers + 128;  // + producer warp + MMA warp + 4 key-sum warps
 constexpr int kAfOnes = 2048;                    // [16 x 64] bf16 ones (K-major operand)
-constexpr uint32_t kAfTmemCols = 256;
 constexpr uint32_t kAfColZ = 128, kAfColKs = 144;  // TMEM columns: S from 0, z, ksum[2]
+constexpr uint32_t kAfColZ64 = 256;                 // head_dim 64: S[4] from 0, z[4]
 
 template <int D>
 struct AfSmem {
@@ -191,8 +193,10 @@ struct AfSmem {
   static constexpr int kTerms = D == 128 ? 2 : 3;
   static constexpr int kPhi = kTerms * kTile;  // phi(K) of a block: hi | lo or hi | mid | lo
   static constexpr int kZeros = D == 128 ? 0 : kTile;  // (a tile of zeros in front of the two phi buffers)
-  static constexpr int kTotal = kAfDepth * kStage + 2 * kPhi + kZeros + kAfOnes + 256 + 1024;
+  static constexpr int kKsum = D == 128 ? 0 : 2 * 32 * D * 4;  // column sums of every 32nd row, two buffers
+  static constexpr int kTotal = kAfDepth * kStage + 2 * kPhi + kZeros + kAfOnes + 256 + kKsum + 1024;
   static constexpr int kPitch = D + 4;  // floats per row of the staged partial state
+  static constexpr uint32_t kTmemCols = D == 128 ? 256 : 512;
   static_assert(128 * kPitch * 4 <= 2 * kPhi + kZeros + kAfOnes, "partial state is staged in the phi + ones area");
 };
 
@@ -303,7 +307,7 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
     tma_prefetch_desc(&tm_vpool);
   }
   if (warp == 1) {
-    tmem_alloc(&bars->tmem_base, kAfTmemCols);
+    tmem_alloc(&bars->tmem_base, L::kTmemCols);
     tmem_relinquish();
   }
   // bf16 1.0 everywhere: under any swizzle the tile reads as all ones
@@ -364,38 +368,52 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
         const uint32_t a_1 = desc_lo_sw128(smem_u32(ph), L::kSlab);
         const uint32_t a_2 = D == 128 ? desc_lo_sw128(smem_u32(ph + L::kTile), L::kSlab)
                                       : desc_lo_sw128(smem_u32(zeros), L::kZeros + hb * L::kPhi + 2 * L::kTile);
-        const uint32_t acc_s = tmem + (D == 64 ? 64 * hb : 0), acc_z = tmem + kAfColZ + (D == 64 ? 64 * hb : 0);
-        const bool more = bi >= (D == 64 ? 2 : 1);  // the accumulator holds earlier blocks
+        // accumulators of product kk and whether they hold earlier ones
+        auto acc_s = [&](int kk) { return tmem + (D == 64 ? 64 * (2 * hb + (kk & 1)) : 0); };
+        auto acc_z = [&](int kk) { return tmem + (D == 64 ? kAfColZ64 + 16 * (2 * hb + (kk & 1)) : kAfColZ); };
+        auto more = [&](int kk) { return (D == 64 ? bi >= 2 || kk >= 2 : bi > 0 || kk > 0) ? 1u : 0u; };
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          tc_mma_ss_lo(acc_s, a_1 + kk * 128, b_v + kk * 128, hi, idesc_s, (more || kk > 0) ? 1u : 0u);
+          tc_mma_ss_lo(acc_s(kk), a_1 + kk * 128, b_v + kk * 128, hi, idesc_s, more(kk));
 #pragma unroll
-        for (int kk = 0; kk < 4; ++kk) tc_mma_ss_lo(acc_s, a_2 + kk * 128, b_v + kk * 128, hi, idesc_s, 1u);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk)
-          tc_mma_ss_lo(acc_z, a_1 + kk * 128, b_ones, hi, idesc_1, (more || kk > 0) ? 1u : 0u);
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) tc_mma_ss_lo(acc_z, a_2 + kk * 128, b_ones, hi, idesc_1, 1u);
-        if (bi >= 2 && !af_wait(&bars->ks_read[hb], ((bi >> 1) - 1) & 1, bars, a.status)) break;
-        tc_fence_after();
+        for (int kk = 0; kk < 4; ++kk) tc_mma_ss_lo(acc_s(kk), a_2 + kk * 128, b_v + kk * 128, hi, idesc_s, 1u);
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk)
-          tc_mma_ss_lo(tmem + kAfColKs + hb * 16, a_k + kk * 128, b_ones, hi, idesc_1, kk > 0 ? 1u : 0u);
+          tc_mma_ss_lo(acc_z(kk), a_1 + kk * 128, b_ones, hi, idesc_1, more(kk));
+#pragma unroll
+        for (int kk = 0; kk < 4; ++kk) tc_mma_ss_lo(acc_z(kk), a_2 + kk * 128, b_ones, hi, idesc_1, 1u);
+        if constexpr (D == 128) {
+          if (bi >= 2 && !af_wait(&bars->ks_read[hb], ((bi >> 1) - 1) & 1, bars, a.status)) break;
+          tc_fence_after();
+#pragma unroll
+          for (int kk = 0; kk < 4; ++kk)
+            tc_mma_ss_lo(tmem + kAfColKs + hb * 16, a_k + kk * 128, b_ones, hi, idesc_1, kk > 0 ? 1u : 0u);
+        }
         tc_commit(&bars->consumed[s]);
         tc_commit(&bars->mma_done[hb]);
       }
     }
   } else if (warp >= 2 + kAfWorkers / 32) {
     // ------------------------------------------------------------------ key-sum warps
-    // one warp per TMEM lane quadrant: key sum of each block, as soon as its MMAs are done
+    // key sum of each block: one warp per TMEM lane quadrant, as soon as the block's MMAs are done
+    // (head_dim 64: two warps that add up the workers' sums)
     const int quad = warp & 3;
     for (int bj = 0; bj < nblk; ++bj) {
-      if (!af_wait(&bars->mma_done[bj & 1], (bj >> 1) & 1, bars, a.status)) break;
-      tc_fence_after();
-      uint32_t v[16];
-      tmem_ld16(tmem + (static_cast<uint32_t>(quad * 32) << 16) + kAfColKs + (bj & 1) * 16, v);
-      tc_wait_ld();
-      tc_fence_before();
+      if (!af_wait(D == 128 ? &bars->mma_done[bj & 1] : &bars->phi_ready[bj & 1], (bj >> 1) & 1, bars, a.status)) break;
+      float sum = 0.f;
+      if constexpr (D == 128) {
+        tc_fence_after();
+        uint32_t v[16];
+        tmem_ld16(tmem + (static_cast<uint32_t>(quad * 32) << 16) + kAfColKs + (bj & 1) * 16, v);
+        tc_wait_ld();
+        sum = __uint_as_float(v[0]);
+        tc_fence_before();
+      } else if (quad * 32 < D) {
+        const float* col = reinterpret_cast<const float*>(ones + kAfOnes + 256) + (bj & 1) * (L::kKsum / 8) + quad * 32 + lane;
+#pragma unroll
+        for (int r = 0; r < L::kKsum / (2 * D * 4); ++r) sum += col[r * D];
+        __syncwarp();
+      }
       if (lane == 0) mbar_arrive(&bars->ks_read[bj & 1]);
       if (quad * 32 >= D) continue;
       const int64_t b = bs + bj;
@@ -406,7 +424,7 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
         old = a.tail_from_saved ? *saved : *dst;
         if (!a.tail_from_saved) *saved = old;
       }
-      *dst = old + __uint_as_float(v[0]);
+      *dst = old + sum;
     }
   } else {
     // ------------------------------------------------------------------ workers
@@ -455,6 +473,23 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
       if (bi >= 2) {
         ok = af_wait(&bars->mma_done[hb], ((bi >> 1) - 1) & 1, bars, a.status);
         if (!ok) break;
+      }
+      if constexpr (D == 64) {
+        // the thread's column sums (rows outside the chunk are zeros) for the key-sum warps
+        if (bi >= 2) {
+          ok = af_wait(&bars->ks_read[hb], ((bi >> 1) - 1) & 1, bars, a.status);
+          if (!ok) break;
+        }
+        static_assert(NI == 2 && RS * D * 4 * 2 == L::kKsum, "a thread holds two rows of a block");
+        const uint32_t* w0 = reinterpret_cast<const uint32_t*>(&kreg[0]);
+        const uint32_t* w1 = reinterpret_cast<const uint32_t*>(&kreg[1]);
+        float4* dst = reinterpret_cast<float4*>(ones + kAfOnes + 256) + hb * (L::kKsum / 32) + (rg * D + ch * 8) / 4;
+#pragma unroll
+        for (int e = 0; e < 4; e += 2)
+          dst[e / 2] = make_float4(__uint_as_float(w0[e] << 16) + __uint_as_float(w1[e] << 16),
+                                   __uint_as_float(w0[e] & 0xffff0000u) + __uint_as_float(w1[e] & 0xffff0000u),
+                                   __uint_as_float(w0[e + 1] << 16) + __uint_as_float(w1[e + 1] << 16),
+                                   __uint_as_float(w0[e + 1] & 0xffff0000u) + __uint_as_float(w1[e + 1] & 0xffff0000u));
       }
       uint8_t* ph = phi + hb * L::kPhi;
       // rows outside the chunk (only in its first and last block) add nothing to the state
@@ -519,20 +554,26 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
           tmem_ld32(t_row + col, v);
         else
           tmem_ld16(t_row + col, v);
-        if (zw) tmem_ld16(t_row + kAfColZ, zv);
+        if (zw) tmem_ld16(t_row + (D == 64 ? kAfColZ64 : kAfColZ), zv);
         tc_wait_ld();
         if constexpr (D == 64) {
-          if (nblk > 1) {  // the other accumulator
-            uint32_t u[NC];
-            tmem_ld16(t_row + 64 + col, u);
-            tc_wait_ld();
+          // the other accumulators: (0 + 1) + (2 + 3), the last two only of a second block
+          auto add = [](uint32_t x, uint32_t y) { return __float_as_uint(__uint_as_float(x) + __uint_as_float(y)); };
+          uint32_t u[3][NC];
 #pragma unroll
-            for (int i = 0; i < NC; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(u[i]));
-            if (zw) {
-              tmem_ld16(t_row + kAfColZ + 64, u);
-              tc_wait_ld();
-              zv[0] = __float_as_uint(__uint_as_float(zv[0]) + __uint_as_float(u[0]));
-            }
+          for (int m = 0; m < 3; ++m) tmem_ld16(t_row + 64 * (m + 1) + col, u[m]);
+          tc_wait_ld();
+#pragma unroll
+          for (int i = 0; i < NC; ++i) {
+            v[i] = add(v[i], u[0][i]);
+            if (nblk > 1) v[i] = add(v[i], add(u[1][i], u[2][i]));
+          }
+          if (zw) {
+#pragma unroll
+            for (int m = 0; m < 3; ++m) tmem_ld16(t_row + kAfColZ64 + 16 * (m + 1), u[m]);
+            tc_wait_ld();
+            zv[0] = add(zv[0], u[0][0]);
+            if (nblk > 1) zv[0] = add(zv[0], add(u[1][0], u[2][0]));
           }
         }
       } else {
@@ -569,7 +610,7 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
   __syncthreads();
   if (warp == 1) {
     tc_fence_after();
-    tmem_dealloc(tmem, kAfTmemCols);
+    tmem_dealloc(tmem, L::kTmemCols);
   }
 }
 

@@ -91,6 +91,24 @@ def test_append_head_dim_64(n0, n, H, relu, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("n,H", [(1, 1), (63, 2), (64, 2), (1000, 16), (4680, 3)])
+def test_key_sums_head_dim_64_are_rounded_sums(n, H, cuda_device):
+    """Key sums of blocks that are new as a whole: bit for bit those of the page kernel of a context without a
+    linear state (rounded fp32 in a fixed order), also for keys spread over 16 octaves."""
+    from paper_2609_34606_b200 import hsa
+    d = 64
+    g = torch.Generator().manual_seed(n)
+    K = (torch.randn(n, H, d, generator=g) * torch.exp2(torch.randint(-12, 4, (n, H, d), generator=g).float()))
+    K, V = K.to(torch.bfloat16).to(cuda_device), _randn(g, n, H, d).to(cuda_device)
+    sums = []
+    for mode in (hsa.HSA_LIN_STATE, hsa.HSA_LIN_NONE):
+        ctx = hsa.HSAContext(H, d, max_pages=(n + 63) // 64, max_q_tokens=n, max_topk=1, device=cuda_device, lin_mode=mode)
+        ctx.append_kv(K, V)
+        assert ctx.device_status() == 0
+        sums.append(ctx.ksum.clone())
+        ctx.destroy()
+    assert torch.equal(*sums)
+
 @pytest.mark.parametrize("n,relu", [(1, 0), (70, 0), (1000, 0), (1000, 1)])
 def test_append_head_dim_64_not_finite(n, relu, cuda_device):
     """Inf and NaN in K and V reach the entries of S, z and the key sums that they reach in a plain sum, as the
