@@ -245,8 +245,7 @@ __device__ __forceinline__ void tma_store_2d(const void* tmap, const void* smem_
 
 // RELU: the feature map is max(x, 0) instead of elu(x) + 1 (an instance of its own: the map sits in
 // the innermost loop of the worker warps)
-// KEEP (causal contexts): the workers leave phi(K) in the workspace as well (AppendArgs::phik)
-template <int D, bool RELU, bool KEEP>
+template <int D, bool RELU>
 __global__ void __launch_bounds__(kAfThreads, 1)
 append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CUtensorMap tm_kin,
                     const __grid_constant__ CUtensorMap tm_vin, const __grid_constant__ CUtensorMap tm_kpool,
@@ -521,13 +520,6 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
 #pragma unroll
         for (int m = 0; m < L::kTerms; ++m)
           *reinterpret_cast<uint4*>(ph + m * L::kTile + soff[i]) = make_uint4(tw[m][0], tw[m][1], tw[m][2], tw[m][3]);
-        if (KEEP) {  // the first two terms of phi(K) stay for the chunk's own forward
-          const size_t row = (static_cast<size_t>(h) * 2 * a.phik_blocks + (b - b_first)) * kBlock + rg + RS * i;
-#pragma unroll
-          for (int m = 0; m < 2; ++m)
-            *reinterpret_cast<uint4*>(a.phik + (row + static_cast<size_t>(m) * a.phik_blocks * kBlock) * D + ch * 8) =
-                make_uint4(tw[m][0], tw[m][1], tw[m][2], tw[m][3]);
-        }
       }
       fence_proxy_async_smem();  // generic-proxy writes above -> visible to the tensor cores
       mbar_arrive(&bars->phi_ready[hb]);
@@ -617,19 +609,17 @@ append_fused_kernel(AppendArgs a, int blocks_per_cta, const __grid_constant__ CU
 namespace {
 using AppendKernel = void (*)(AppendArgs, int, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap);
 template <int D>
-AppendKernel fused_kernel(bool relu, bool keep) {
-  if (keep) return relu ? append_fused_kernel<D, true, true> : append_fused_kernel<D, false, true>;
-  return relu ? append_fused_kernel<D, true, false> : append_fused_kernel<D, false, false>;
+AppendKernel fused_kernel(bool relu) {
+  return relu ? append_fused_kernel<D, true> : append_fused_kernel<D, false>;
 }
 }  // namespace
 
 cudaError_t append_init() {
   cudaError_t e = cudaSuccess;
-  for (int i = 0; i < 4 && e == cudaSuccess; ++i) {
-    const bool relu = i & 1, keep = i & 2;
-    e = cudaFuncSetAttribute(fused_kernel<128>(relu, keep), cudaFuncAttributeMaxDynamicSharedMemorySize, AfSmem<128>::kTotal);
+  for (int relu = 0; relu < 2 && e == cudaSuccess; ++relu) {
+    e = cudaFuncSetAttribute(fused_kernel<128>(relu), cudaFuncAttributeMaxDynamicSharedMemorySize, AfSmem<128>::kTotal);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(fused_kernel<64>(relu, keep), cudaFuncAttributeMaxDynamicSharedMemorySize, AfSmem<64>::kTotal);
+      e = cudaFuncSetAttribute(fused_kernel<64>(relu), cudaFuncAttributeMaxDynamicSharedMemorySize, AfSmem<64>::kTotal);
   }
   return e;
 }
@@ -653,8 +643,7 @@ cudaError_t launch_append(const AppendArgs& a_in, const AppendMaps* maps, cudaSt
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const bool keep = a.phik != nullptr;
-    AppendKernel fn = a.D == 128 ? fused_kernel<128>(a.relu, keep) : fused_kernel<64>(a.relu, keep);
+    AppendKernel fn = a.D == 128 ? fused_kernel<128>(a.relu) : fused_kernel<64>(a.relu);
     e = cudaLaunchKernelEx(&cfg, fn, a, per, maps->kin, maps->vin, maps->kpool, maps->vpool);
     if (e != cudaSuccess) return e;
   } else {

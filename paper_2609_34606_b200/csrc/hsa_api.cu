@@ -372,8 +372,6 @@ int hsa_append_kv(hsa_ctx* ctx, const void* k, const void* v, int32_t n_tokens, 
   a.nsplit = nsplit;
   a.lin_state = ctx->cfg.lin_mode == HSA_LIN_STATE;
   a.relu = ctx->cfg.feature_map == HSA_PHI_RELU;
-  a.phik_blocks = ctx->lay.phik_blocks;
-  a.phik = a.phik_blocks > 0 ? reinterpret_cast<__nv_bfloat16*>(ws + ctx->lay.phik) : nullptr;
   a.status = reinterpret_cast<int32_t*>(ws + ctx->lay.status);
   const bool linformer = ctx->cfg.lin_mode == HSA_LIN_LINFORMER;
   if (linformer && (n_tokens != ctx->cfg.lin_seg_tokens || ctx->n_tokens != static_cast<int64_t>(ctx->n_segs) * n_tokens))
@@ -638,10 +636,11 @@ int hsa_forward(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride, in
   if (causal_lin) {
     CausalLinArgs c{};
     c.n_q = n_q;
+    c.k_pool = static_cast<const __nv_bfloat16*>(ctx->buf.k_pool);
+    c.phik = reinterpret_cast<__nv_bfloat16*>(ws + ctx->lay.phik);
     c.phik_blocks = ctx->lay.phik_blocks;
     c.page_table = p.page_table;
     c.q_pos0 = q_pos0;
-    c.n_tokens = ctx->n_tokens;
     c.H = H;
     c.D = D;
     c.relu = p.relu;

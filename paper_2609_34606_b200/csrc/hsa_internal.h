@@ -57,10 +57,6 @@ struct AppendArgs {
   int lin_state;  // update the linear state?
   int beside_prior;  // SIMT page write: may run beside the kernel launched just before it (see launch_append)
   int relu;       // feature map of the state: 0 elu(x) + 1, 1 max(x, 0)
-  // causal contexts: phi(K) of the chunk as bf16 hi and lo, [H][hi/lo][phik_blocks][64][D], block 0 being
-  // the chunk's first page (rows of that page before the chunk: zeros); null otherwise
-  __nv_bfloat16* phik;
-  int phik_blocks;
   int32_t* status;  // device status word
 };
 
@@ -162,9 +158,12 @@ struct FwdParams {
 struct CausalLinArgs {
   int n_q;
   const int32_t* page_table;
-  int phik_blocks;  // blocks per (head, hi/lo) of the phi(K) tiles the chunk's append left (AppendArgs::phik)
+  const __nv_bfloat16* k_pool;
+  // workspace: phi(K) of the pages that hold the chunk as bf16 hi and lo, [H][hi/lo][phik_blocks][64][D], block 0
+  // being the chunk's first page (its rows before the chunk included)
+  __nv_bfloat16* phik;
+  int phik_blocks;
   int64_t q_pos0;   // first query position == first token of the intra-chunk part
-  int64_t n_tokens;
   int H, D;
   int relu;  // feature map: 0 elu(x) + 1, 1 max(x, 0)
   float* lin_num;
@@ -214,7 +213,7 @@ cudaError_t launch_forward(const FwdParams& p, int D, const CUtensorMap& tm_q,
                            const CUtensorMap& tm_state, const CUtensorMap& tm_out, cudaStream_t st,
                            const CUtensorMap* tm_kc = nullptr, const CUtensorMap* tm_vc = nullptr,
                            const CUtensorMap* tm_gl = nullptr, const CUtensorMap* tm_gs = nullptr);
-// tm_q: box of 128 tokens of one head; tm_phik, tm_v: rows of phi(K) and of the V pool, box 64 x 64
+// tm_q: box of 128 tokens of one head; tm_phik, tm_v: rows of phik and of the V pool, box 64 x 64
 cudaError_t launch_causal_linear(const CausalLinArgs& a, const CUtensorMap& tm_q, const CUtensorMap& tm_phik,
                                  const CUtensorMap& tm_v, cudaStream_t st);
 cudaError_t causal_linear_init();

@@ -2,11 +2,11 @@
 // appended chunk, query i may only see the chunk's own keys up to its position; the state of
 // everything before the chunk is applied by the forward kernel, and this kernel supplies
 //   num[i,h,:] = sum_{q_pos0 <= j <= q_pos0+i} (phi(q_i).phi(k_j)) v_j,   den[i,h] = sum of weights
-// read from the pool pages.
+// K and V from the pool pages.
 //
-// phi(K) of the chunk, as bf16 hi and lo tiles, was left in the workspace by the chunk's append, which
-// forms it anyway (made here it would be made again for every query tile behind a key: that form was
-// bound by it, 42 us where this one takes 31 us).
+// phi(K) of the chunk is made first, by a kernel of its own, as bf16 tiles in the workspace (made in the kernel
+// of the products it would be made again for every query tile behind a key: that form was bound by it, 42 us
+// where this one takes 31 us; and left there by the append, every append would pay for it).
 //
 // One CTA per (128-row query tile, head), 576 threads:
 //   warp 0       TMA producer: Q tile, then, up to the tile's diagonal, phi(K) hi and lo and V (two 64-token
@@ -78,12 +78,7 @@ __device__ __forceinline__ bool cl_wait(uint64_t* bar, uint32_t parity, ClBars* 
   return false;
 }
 
-// max(x, 0) + w * exp(min(x, 0)): elu(x) + 1 (w = 1) or relu (w = 0)
-__device__ __forceinline__ float cl_phi(float x, float w) {
-  float e;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(fminf(x, 0.f) * 1.4426950408889634f));
-  return fmaf(w, e, fmaxf(x, 0.f));
-}
+__device__ __forceinline__ float cl_phi(float x, int relu) { return relu ? fmaxf(x, 0.f) : (x > 0.f ? x + 1.f : expf(x)); }
 // two fp32 values as packed bf16 hi and lo (hi + lo = value to about 16 bits)
 __device__ __forceinline__ void cl_split(float a, float b, uint32_t& hi, uint32_t& lo) {
   hi = pack_bf16(a, b);
@@ -92,10 +87,34 @@ __device__ __forceinline__ void cl_split(float a, float b, uint32_t& hi, uint32_
 
 }  // namespace
 
+// phi(K) of one page of one head: what bounds it is the bytes, 16 KB in and 32 KB out per page at head_dim 128.
+template <int D>
+__global__ void __launch_bounds__(256) phi_terms_kernel(CausalLinArgs a) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int h = blockIdx.y;
+  const int64_t b = a.q_pos0 / kBlock + blockIdx.x;
+  const uint4* src = reinterpret_cast<const uint4*>(a.k_pool + (static_cast<size_t>(a.page_table[b]) * a.H + h) * kBlock * D);
+  uint4* dst = reinterpret_cast<uint4*>(a.phik + (static_cast<size_t>(h) * 2 * a.phik_blocks + blockIdx.x) * kBlock * D);
+  const size_t term = static_cast<size_t>(a.phik_blocks) * kBlock * D / 8;  // from one term's tile to the next
+#pragma unroll
+  for (int i = 0; i < kBlock * D / 8 / 256; ++i) {
+    const int c = threadIdx.x + 256 * i;
+    const uint4 raw = src[c];
+    const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
+    uint32_t hi[4], lo[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      cl_split(cl_phi(__uint_as_float(w[e] << 16), a.relu), cl_phi(__uint_as_float(w[e] & 0xffff0000u), a.relu), hi[e], lo[e]);
+    dst[c] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+    dst[c + term] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+  }
+}
+
 template <int D>
 __global__ void __launch_bounds__(kClThreads, 1)
 causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                     const __grid_constant__ CUtensorMap tm_v) {  // tm_k: the phi(K) tiles of the chunk's append
+                     const __grid_constant__ CUtensorMap tm_v) {  // tm_k: the phi(K) tiles
   using L = ClSmem<D>;
   constexpr int DH = D / 64;
   extern __shared__ uint8_t cl_raw[];
@@ -238,7 +257,6 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
     const int quad = warp & 3;        // TMEM lane quadrant this warp may access
     const int r = quad * 32 + lane;   // row inside the tile
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
-    const float exp_part = a.relu ? 0.f : 1.f;
     bool ok = __all_sync(0xffffffffu, cl_wait(&bars->q_full, 0, bars, a.status));
     if (ok) {
       if (set * 32 < D) {
@@ -252,7 +270,7 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
           const uint32_t* qw = reinterpret_cast<const uint32_t*>(&raw);
 #pragma unroll
           for (int i = 0; i < 4; ++i)
-            cl_split(cl_phi(__uint_as_float(qw[i] << 16), exp_part), cl_phi(__uint_as_float(qw[i] & 0xffff0000u), exp_part),
+            cl_split(cl_phi(__uint_as_float(qw[i] << 16), a.relu), cl_phi(__uint_as_float(qw[i] & 0xffff0000u), a.relu),
                      hi[c * 4 + i], lo[c * 4 + i]);
         }
         tmem_st16(tmem + lane_off + kClColQh + set * 16, hi);
@@ -343,16 +361,21 @@ cudaError_t causal_linear_init() {
 cudaError_t launch_causal_linear(const CausalLinArgs& a, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                                  const CUtensorMap& tm_v, cudaStream_t st) {
   const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
+  const int64_t pages = (a.q_pos0 + a.n_q - 1) / kBlock - a.q_pos0 / kBlock + 1;
   cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3(static_cast<unsigned>(n_tiles) * a.H);
-  cfg.blockDim = dim3(kClThreads);
-  cfg.dynamicSmemBytes = a.D == 128 ? ClSmem<128>::kTotal : ClSmem<64>::kTotal;
+  cfg.gridDim = dim3(static_cast<unsigned>(pages), a.H);
+  cfg.blockDim = dim3(256);
   cfg.stream = st;
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, a.D == 128 ? phi_terms_kernel<128> : phi_terms_kernel<64>, a);
+  if (e != cudaSuccess) return e;
+  cfg.gridDim = dim3(static_cast<unsigned>(n_tiles) * a.H);
+  cfg.blockDim = dim3(kClThreads);
+  cfg.dynamicSmemBytes = a.D == 128 ? ClSmem<128>::kTotal : ClSmem<64>::kTotal;
   if (a.D == 128) return cudaLaunchKernelEx(&cfg, causal_linear_kernel<128>, a, tm_q, tm_k, tm_v);
   return cudaLaunchKernelEx(&cfg, causal_linear_kernel<64>, a, tm_q, tm_k, tm_v);
 }

@@ -53,6 +53,25 @@ def test_causal_intra_chunk_products(n0, n_q, d, relu, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("d", [64, 128])
+def test_causal_nan_key_reaches_the_queries_behind_it(d, cuda_device):
+    """A NaN in a key of the chunk makes the linear branch NaN for the queries at and behind it (elu), and a NaN in
+    a query makes its own row NaN."""
+    from paper_2609_34606_b200 import hsa
+    H, n0, n = 2, 100, 300
+    g = torch.Generator().manual_seed(d)
+    K, V, q = _randn(g, n, H, d), _randn(g, n, H, d), _randn(g, n, H, d)
+    K[150, 1, 3] = q[20, 0, 7] = float("nan")
+    ctx = hsa.HSAContext(H, d, max_pages=7, max_q_tokens=n, max_topk=1, causal=True, device=cuda_device)
+    ctx.append_kv(_randn(g, n0, H, d).to(cuda_device), _randn(g, n0, H, d).to(cuda_device))
+    ctx.append_kv(K.to(cuda_device), V.to(cuda_device))
+    out = ctx.forward(q.to(cuda_device), None, None, q_pos0=n0, causal=True, flags=hsa.HSA_FWD_NO_SPARSE).cpu()
+    assert ctx.device_status() == 0
+    bad = out.isnan().any(2)
+    assert bad[:, 1].tolist() == [t >= 150 for t in range(n)]
+    assert bad[:, 0].tolist() == [t == 20 for t in range(n)]
+    ctx.destroy()
+
 @pytest.mark.parametrize("n0,n,H,relu", [
     (0, 1, 2, 0), (0, 63, 2, 0), (0, 64, 3, 0), (0, 65, 2, 1), (1, 62, 2, 0), (1, 63, 2, 0), (63, 2, 2, 0), (64, 640, 2, 1),
     (100, 1000, 16, 0), (0, 1500, 40, 0)])
