@@ -97,7 +97,7 @@ Layout make_layout(const hsa_config* c) {
     L.lin_den = o;  o = align_up(o + static_cast<size_t>(c->max_q_tokens) * H * 4, 256);
     if (c->lin_mode == HSA_LIN_STATE) {
       L.phik_blocks = (c->max_q_tokens + kBlock - 1) / kBlock + 1;
-      L.phik = o;   o = align_up(o + H * 2 * static_cast<size_t>(L.phik_blocks) * kBlock * D * 2, 256);
+      L.phik = o;   o = align_up(o + H * kPhiTerms * static_cast<size_t>(L.phik_blocks) * kBlock * D * 2, 256);
     }
   }
   if (c->flags & HSA_CFG_ADAPTIVE) {
@@ -316,7 +316,7 @@ int hsa_create(hsa_ctx** out, const hsa_config* cfg, const hsa_buffers* bufs,
     r = encode_2d_rows(&ctx->tm_state, static_cast<uint8_t*>(bufs->state) + ctx->lay.hilo,
                        static_cast<uint64_t>(cfg->num_heads) * 4 * D, D);
   if (r == HSA_OK && ctx->lay.phik_blocks > 0)
-    r = encode_2d_rows(&ctx->tm_phik, ws + ctx->lay.phik, static_cast<uint64_t>(cfg->num_heads) * 2 * ctx->lay.phik_blocks * kBlock, D);
+    r = encode_2d_rows(&ctx->tm_phik, ws + ctx->lay.phik, static_cast<uint64_t>(cfg->num_heads) * kPhiTerms * ctx->lay.phik_blocks * kBlock, D);
   if (r == HSA_OK && linformer) {
     const uint64_t crows = static_cast<uint64_t>(ctx->lay.n_cpages) * cfg->num_heads * kBlock;
     r = encode_2d_rows(&ctx->tm_kc, bufs->kc_pool, crows, D);

@@ -20,6 +20,7 @@ constexpr int kZopBytes = 4096;
 constexpr int kFewItemsSlots = 240;
 constexpr int kFewItemsMinBlocks = 48;   // shorter lists are not split for that
 constexpr int kFewItemsPart = 8;         // shortest part of such a launch, in two-page steps
+constexpr int kPhiTerms = 3;             // bf16 terms of phi(K) for the causal products: 24 bits
 constexpr int kFwdSplitMax = 16;         // CTAs a long (query tile, head) of the forward kernel is split over
 
 __host__ __device__ inline int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
@@ -159,7 +160,7 @@ struct CausalLinArgs {
   int n_q;
   const int32_t* page_table;
   const __nv_bfloat16* k_pool;
-  // workspace: phi(K) of the pages that hold the chunk as bf16 hi and lo, [H][hi/lo][phik_blocks][64][D], block 0
+  // workspace: phi(K) of the pages that hold the chunk as bf16 terms, [H][hi/mid/lo][phik_blocks][64][D], block 0
   // being the chunk's first page (its rows before the chunk included)
   __nv_bfloat16* phik;
   int phik_blocks;

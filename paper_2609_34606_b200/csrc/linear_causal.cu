@@ -5,31 +5,40 @@
 // K and V from the pool pages.
 //
 // phi(K) of the chunk is made first, by a kernel of its own, as bf16 tiles in the workspace (made in the kernel
-// of the products it would be made again for every query tile behind a key: that form was bound by it, 42 us
-// where this one takes 31 us; and left there by the append, every append would pay for it).
+// of the products it would be made again for every query tile behind a key; left there by the append, every
+// append would pay for it): 5 us for a chunk of 1560 tokens, 12 heads of 128.
 //
 // One CTA per (128-row query tile, head), 576 threads:
-//   warp 0       TMA producer: Q tile, then, up to the tile's diagonal, phi(K) hi and lo and V (two 64-token
-//                pages = 128 keys per step) into rings of four and two 128-key tiles
+//   warp 0       TMA producer: Q tile, then, page by page up to the tile's diagonal, phi(K) and V (64 keys per
+//                step) into rings of two
 //   warp 1       tcgen05.mma issuer
-//   warps 2..17  phi(Q) once; weights of a step: mask, row sum, hi / lo split
-// The map and the weights are fp32 quantities, so each is carried as bf16 hi + lo (about 16 bits):
-//   A    = phi(Q)_hi phi(K)_hi^T + phi(Q)_lo phi(K)_hi^T + phi(Q)_hi phi(K)_lo^T      (fp32, TMEM)
-//   num += A_hi V + A_lo V   with A masked and split, den from the fp32 A
-// Against 64 bits the outputs of a causal forward are off by as much as with fp32 arithmetic
-// throughout: the rounding of the result to bf16 is two orders of magnitude larger.
+//   warps 2..17  phi(Q) once; weights of a step: mask, row sum, split; running sum of num
+// The map, the weights and the sums are fp32 quantities, so each operand is carried as three bf16 terms,
+// hi + mid + lo (24 bits), with the products of down to 2^-16 of the largest:
+//   A     = phi(Q) phi(K)^T  as  hi hi  +  (lo hi + hi lo + mid mid + mid hi + hi mid)    (fp32, TMEM)
+//   num_j = A_lo V + A_mid V + A_hi V  of one step's 64 keys, with A masked and split     (fp32, TMEM)
+// The tensor cores truncate what they add to.  The hi of phi(Q) and phi(K) are therefore multiples of 2^-6 of the
+// largest value's power of two (per row and 32 dims): the sum of hi hi over 128 dims needs 22 bits and
+// is exact, the other products have an accumulator of their own, and A is rounded once, when the two are added.
+// In num small terms go first and the accumulator lives for one step: num and den are running sums in
+// registers, rounded.
+// Error of num and den against 64 bits (2-norm; 12 heads of 128, chunks of 256 / 1560 / 3120 tokens), the fp32
+// SIMT kernel this replaced -> now: num 1.1e-7 / 2.2e-7 / 3.0e-7 -> 0.7e-7 / 1.0e-7 / 1.2e-7, den 0.6e-7 /
+// 0.8e-7 / 1.0e-7 -> 0.4e-7 / 0.5e-7 / 0.6e-7.  (Two terms each and sums over the whole chunk in TMEM: num
+// 2.7e-6 / 3.5e-6 / 5.2e-6, den 6.0e-7.)
 // (A non-finite V reaches every row of its 128-row tile, also those before it: 0 x inf in the product.)
 //
-// What bounds it: the tensor pipe, 40 products of 128 x 128 x 16 per step = 2560 cycles, with the
-// workers' 16384 weights per step beside it.
-// Measured, 12 heads of 128, a chunk of 1560 tokens (91 tile pairs per head): 31 us, with the forward
-// kernel running on the SMs that are through from 15 us on; one CTA per query and head in fp32 on the
-// CUDA cores, which this replaces, took 1678 us.  The longest tile alone is 13 steps of 2 us.
-// The steps of a tile grow with its position (chunk of 1560 tokens: 1 to 13), so the longest tiles are
-// launched first and the forward kernel behind this one may start on the SMs that are through (see
-// hsa_forward_kernel).
-// TMEM: num (128 columns) | phi(Q) hi (64) | phi(Q) lo (64) | A, two buffers of 128; the split weights
-// overwrite their A buffer, 32 columns of weights as 16 of packed hi and 16 of packed lo.
+// What bounds it: the tensor pipe along the longest tile, 25 steps at a chunk of 1560 tokens.  The terms of
+// phi(K) lie side by side, so that one product of phi(Q) hi with all three, one of mid with the first two and
+// one of lo with the first form all sums: 8 x (96 + 64 + 32) cycles per step at head_dim 128, and 768 for num.
+// Measured there (time stamps): 7400 cycles up to the first product (phi(Q)), then 2950 per step, 44 us for
+// the tile; all tiles of 12 heads together are 2184 steps, 18 us of the pipe on 148 SMs, and the forward
+// kernel runs on the SMs that are through.  One CTA per query and head in fp32 on the CUDA cores took 1678 us.
+// The steps of a tile grow with its position, so the longest tiles are launched first and the forward kernel
+// behind this one may start on the SMs that are through (see hsa_forward_kernel).
+// TMEM: num (128 columns) | two step buffers of 192: hi hi | hi mid + mid hi | hi lo + mid mid + lo hi, 64 columns
+// each.  The split weights overwrite them: 16 columns of hi hi become 8 of packed hi and 8 of packed mid, 16 of
+// the next sum 8 of packed lo.
 #include <cuda_bf16.h>
 
 #include "hsa_internal.h"
@@ -41,30 +50,34 @@ namespace {
 
 constexpr int kClWorkers = 512;
 constexpr int kClThreads = 64 + kClWorkers;
-constexpr int kClKSlots = 4;  // phi(K) tiles in flight: hi and lo of two steps
-constexpr int kClStages = 2;  // V
-constexpr uint32_t kClColNum = 0, kClColQh = 128, kClColQl = 192, kClColA = 256;  // A: + 128 * buffer
+constexpr int kClTerms = kPhiTerms;
+constexpr int kClStages = 2;
+constexpr uint32_t kClColNum = 0, kClColBuf = 128, kClBuf = kClTerms * kBlock;
 
 template <int D>
 struct ClSmem {
-  static constexpr int kHalf = 128 * 128;    // bytes of one [128 rows x 128 B] slab
-  static constexpr int kTile = 128 * D * 2;  // 128 keys (or queries)
-  static constexpr int kK = 0;               // phi(K) tiles: slot (2 step + hi / lo) % kClKSlots
-  static constexpr int kV = kK + kClKSlots * kTile;
-  static constexpr int kQ = kV + kClStages * kTile;
-  static constexpr int kBars = kQ + kTile;
+  static constexpr int kSlab = kBlock * 128;       // bytes of one [64 rows x 128 B] slab
+  static constexpr int kPage = kBlock * D * 2;     // 64 keys
+  static constexpr int kQHalf = kTileM * 128;      // bytes of one [128 rows x 128 B] slab of Q
+  static constexpr int kQTile = kTileM * D * 2;
+  static constexpr int kK = 0;                     // phi(K): stage, then slab, then term
+  static constexpr int kV = kK + kClStages * kClTerms * kPage;
+  static constexpr int kQ = kV + kClStages * kPage;  // terms of phi(Q); Q arrives in the last one's place
+  static constexpr int kBars = kQ + kClTerms * kQTile;
   static constexpr int kTotal = kBars + 256 + 1024;
 };
 
+// (ring stage and step buffer of step j are both j % 2)
 struct ClBars {
   uint64_t q_full, q_read;
-  uint64_t k_full[kClKSlots], k_empty[kClKSlots];
-  uint64_t v_full[kClStages], v_empty[kClStages];
-  uint64_t a_full[2], p_full[2];
-  uint64_t done;
+  uint64_t k_full[2], v_full[2];
+  uint64_t a_full[2];    // A of the step is formed, its phi(K) stage free
+  uint64_t num_full[2];  // num of the step is formed, its V stage free
+  uint64_t p_ready;      // weights of step j written, num of step j - 1 added up
   uint32_t tmem_base;
   volatile int abort_flag;
 };
+static_assert(kClStages == 2, "one barrier stands for a step buffer and a ring stage");
 static_assert(sizeof(ClBars) <= 256, "barrier block must fit its shared-memory slot");
 
 __device__ __forceinline__ bool cl_wait(uint64_t* bar, uint32_t parity, ClBars* bars, int32_t* status) {
@@ -79,15 +92,23 @@ __device__ __forceinline__ bool cl_wait(uint64_t* bar, uint32_t parity, ClBars* 
 }
 
 __device__ __forceinline__ float cl_phi(float x, int relu) { return relu ? fmaxf(x, 0.f) : (x > 0.f ? x + 1.f : expf(x)); }
-// two fp32 values as packed bf16 hi and lo (hi + lo = value to about 16 bits)
-__device__ __forceinline__ void cl_split(float a, float b, uint32_t& hi, uint32_t& lo) {
-  hi = pack_bf16(a, b);
-  lo = pack_bf16(a - __uint_as_float(hi << 16), b - __uint_as_float(hi & 0xffff0000u));
+// Adding and subtracting this rounds to multiples of 2^-6 of the power of two at or below `largest`.
+__device__ __forceinline__ float cl_grid(float largest) {
+  const uint32_t e = min(max(__float_as_uint(largest) >> 23, 27u), 227u);
+  return __uint_as_float(((e + 17u) << 23) | 0x400000u);
+}
+// two fp32 values as packed bf16 terms, hi + mid + lo = value to 24 bits; grid: see cl_grid (0: hi is the rounded value)
+__device__ __forceinline__ void cl_split(float a, float b, float grid, uint32_t& hi, uint32_t& mid, uint32_t& lo) {
+  hi = pack_bf16(__fsub_rn(__fadd_rn(a, grid), grid), __fsub_rn(__fadd_rn(b, grid), grid));
+  a -= __uint_as_float(hi << 16);
+  b -= __uint_as_float(hi & 0xffff0000u);
+  mid = pack_bf16(a, b);
+  lo = pack_bf16(a - __uint_as_float(mid << 16), b - __uint_as_float(mid & 0xffff0000u));
 }
 
 }  // namespace
 
-// phi(K) of one page of one head: what bounds it is the bytes, 16 KB in and 32 KB out per page at head_dim 128.
+// phi(K) of one page of one head: what bounds it is the bytes, 16 KB in and 48 KB out per page at head_dim 128.
 template <int D>
 __global__ void __launch_bounds__(256) phi_terms_kernel(CausalLinArgs a) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -95,19 +116,27 @@ __global__ void __launch_bounds__(256) phi_terms_kernel(CausalLinArgs a) {
   const int h = blockIdx.y;
   const int64_t b = a.q_pos0 / kBlock + blockIdx.x;
   const uint4* src = reinterpret_cast<const uint4*>(a.k_pool + (static_cast<size_t>(a.page_table[b]) * a.H + h) * kBlock * D);
-  uint4* dst = reinterpret_cast<uint4*>(a.phik + (static_cast<size_t>(h) * 2 * a.phik_blocks + blockIdx.x) * kBlock * D);
+  uint4* dst = reinterpret_cast<uint4*>(a.phik + (static_cast<size_t>(h) * kClTerms * a.phik_blocks + blockIdx.x) * kBlock * D);
   const size_t term = static_cast<size_t>(a.phik_blocks) * kBlock * D / 8;  // from one term's tile to the next
 #pragma unroll
   for (int i = 0; i < kBlock * D / 8 / 256; ++i) {
     const int c = threadIdx.x + 256 * i;
     const uint4 raw = src[c];
     const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
-    uint32_t hi[4], lo[4];
+    float f[8], largest = 0.f;
 #pragma unroll
-    for (int e = 0; e < 4; ++e)
-      cl_split(cl_phi(__uint_as_float(w[e] << 16), a.relu), cl_phi(__uint_as_float(w[e] & 0xffff0000u), a.relu), hi[e], lo[e]);
-    dst[c] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-    dst[c + term] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+    for (int e = 0; e < 8; ++e) {
+      f[e] = cl_phi(__uint_as_float(e & 1 ? w[e >> 1] & 0xffff0000u : w[e >> 1] << 16), a.relu);
+      largest = fmaxf(largest, f[e]);
+    }
+#pragma unroll
+    for (int o = 1; o < 4; o <<= 1) largest = fmaxf(largest, __shfl_xor_sync(0xffffffffu, largest, o));  // of 32 dims
+    const float grid = cl_grid(largest);
+    uint32_t t[kClTerms][4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) cl_split(f[2 * e], f[2 * e + 1], grid, t[0][e], t[1][e], t[2][e]);
+#pragma unroll
+    for (int m = 0; m < kClTerms; ++m) dst[c + m * term] = make_uint4(t[m][0], t[m][1], t[m][2], t[m][3]);
   }
 }
 
@@ -128,17 +157,13 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
   if (threadIdx.x == 0) {
     mbar_init(&bars->q_full, 1);
     mbar_init(&bars->q_read, kClWorkers / 32);
-    for (int s = 0; s < kClKSlots; ++s) {
+    for (int s = 0; s < 2; ++s) {
       mbar_init(&bars->k_full[s], 1);
-      mbar_init(&bars->k_empty[s], 1);
-    }
-    for (int s = 0; s < kClStages; ++s) {
       mbar_init(&bars->v_full[s], 1);
-      mbar_init(&bars->v_empty[s], 1);
       mbar_init(&bars->a_full[s], 1);
-      mbar_init(&bars->p_full[s], kClWorkers / 32);
+      mbar_init(&bars->num_full[s], 1);
     }
-    mbar_init(&bars->done, 1);
+    mbar_init(&bars->p_ready, kClWorkers / 32);
     bars->abort_flag = 0;
     fence_mbar_init();
   }
@@ -155,191 +180,205 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
   asm volatile("griddepcontrol.wait;" ::: "memory");
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
-  // pages of the chunk up to the last token this tile sees
+  // pages of the chunk up to the last token this tile sees, one per step
   const int b_first = static_cast<int>(a.q_pos0 / kBlock);
   const int64_t last = a.q_pos0 + min(row0 + kTileM, a.n_q) - 1;
-  const int n_pages = static_cast<int>(last / kBlock) - b_first + 1;
-  const int nsteps = (n_pages + 1) / 2;
-  auto pages_of = [&](int j) { return min(2, n_pages - 2 * j); };
+  const int nsteps = static_cast<int>(last / kBlock) - b_first + 1;
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer (one lane)
     if (elect_one_sync()) {
-      mbar_expect_tx(&bars->q_full, L::kTile);
-      for (int dh = 0; dh < DH; ++dh) tma_load_3d(smem + L::kQ + dh * L::kHalf, &tm_q, &bars->q_full, dh * 64, h, row0);
+      mbar_expect_tx(&bars->q_full, L::kQTile);
+      for (int dh = 0; dh < DH; ++dh) tma_load_3d(smem + L::kQ + 2 * L::kQTile + dh * L::kQHalf, &tm_q, &bars->q_full, dh * 64, h, row0);
       int armed_k = 0, armed_v = 0;  // loads issued per ring, for the drain on abort
-      auto load_k = [&](int j, int hl) -> bool {
-        const int i = 2 * j + hl, s = i % kClKSlots, npg = pages_of(j);
-        if (i >= kClKSlots && !cl_wait(&bars->k_empty[s], ((i / kClKSlots) - 1) & 1, bars, a.status)) return false;
-        mbar_expect_tx(&bars->k_full[s], npg * kBlock * D * 2);
-        for (int pg = 0; pg < npg; ++pg)
+      auto load_k = [&](int j) -> bool {
+        const int s = j % kClStages;
+        if (j >= kClStages && !cl_wait(&bars->a_full[s], ((j / kClStages) - 1) & 1, bars, a.status)) return false;
+        mbar_expect_tx(&bars->k_full[s], kClTerms * L::kPage);
+        for (int t = 0; t < kClTerms; ++t)
           for (int dh = 0; dh < DH; ++dh)
-            tma_load_2d(smem + L::kK + s * L::kTile + dh * L::kHalf + pg * (kBlock * 128), &tm_k, &bars->k_full[s], dh * 64,
-                        ((h * 2 + hl) * a.phik_blocks + 2 * j + pg) * kBlock);
+            tma_load_2d(smem + L::kK + s * kClTerms * L::kPage + (dh * kClTerms + t) * L::kSlab, &tm_k, &bars->k_full[s], dh * 64,
+                        ((h * kClTerms + t) * a.phik_blocks + j) * kBlock);
         ++armed_k;
         return true;
       };
       auto load_v = [&](int j) -> bool {
-        const int s = j % kClStages, npg = pages_of(j);
-        int32_t y[2] = {0, 0};  // (looked up ahead of the wait)
-        for (int pg = 0; pg < npg; ++pg) y[pg] = (a.page_table[b_first + 2 * j + pg] * a.H + h) * kBlock;
-        if (j >= kClStages && !cl_wait(&bars->v_empty[s], ((j / kClStages) - 1) & 1, bars, a.status)) return false;
-        mbar_expect_tx(&bars->v_full[s], npg * kBlock * D * 2);
-        for (int pg = 0; pg < npg; ++pg)
-          for (int dh = 0; dh < DH; ++dh)
-            tma_load_2d(smem + L::kV + s * L::kTile + dh * L::kHalf + pg * (kBlock * 128), &tm_v, &bars->v_full[s], dh * 64, y[pg]);
+        const int s = j % kClStages;
+        const int32_t y = (a.page_table[b_first + j] * a.H + h) * kBlock;  // (looked up ahead of the wait)
+        if (j >= kClStages && !cl_wait(&bars->num_full[s], ((j / kClStages) - 1) & 1, bars, a.status)) return false;
+        mbar_expect_tx(&bars->v_full[s], L::kPage);
+        for (int dh = 0; dh < DH; ++dh)
+          tma_load_2d(smem + L::kV + s * L::kPage + dh * L::kSlab, &tm_v, &bars->v_full[s], dh * 64, y);
         ++armed_v;
         return true;
       };
-      bool ok = true;
-      for (int j = 0; j < nsteps && ok; ++j) ok = load_k(j, 0) && load_k(j, 1) && load_v(j);
+      // phi(K) one step further than V: its stage is free as soon as the sums of step j - 2 are formed, before
+      // the weights of that step have met the V whose stage the next V takes (in one order 3500 cycles per step)
+      bool ok = load_k(0);
+      for (int j = 0; j < nsteps && ok; ++j) ok = (j + 1 >= nsteps || load_k(j + 1)) && load_v(j);
       if (!ok) {  // let every copy already issued land before the CTA's shared memory goes away
         mbar_wait(&bars->q_full, 0, 1u << 16);
-        for (int s = 0; s < kClKSlots; ++s)
-          if (armed_k > s) mbar_wait(&bars->k_full[s], ((armed_k - 1 - s) / kClKSlots) & 1, 1u << 16);
-        for (int s = 0; s < kClStages; ++s)
+        for (int s = 0; s < kClStages; ++s) {
+          if (armed_k > s) mbar_wait(&bars->k_full[s], ((armed_k - 1 - s) / kClStages) & 1, 1u << 16);
           if (armed_v > s) mbar_wait(&bars->v_full[s], ((armed_v - 1 - s) / kClStages) & 1, 1u << 16);
+        }
       }
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (one lane)
     if (elect_one_sync()) {
       constexpr uint32_t kHiSw = desc_hi_sw128(1024);
+      const uint32_t q_lo = desc_lo_sw128(smem_u32(smem + L::kQ), 16);
       auto issue_qk = [&](int j) -> bool {
-        const uint32_t d = tmem + kClColA + 128 * (j & 1);
-        // (one page in the last step: only its 64 columns are computed)
-        const uint32_t idesc = pages_of(j) >= 2 ? idesc_bf16_f32(128, 128, 0, 0) : idesc_bf16_f32(128, 64, 0, 0);
+        const uint32_t d = tmem + kClColBuf + kClBuf * (j & 1);
+        const int s = j % kClStages;
+        if (!cl_wait(&bars->k_full[s], (j / kClStages) & 1, bars, a.status)) return false;
+        tc_fence_after();
+        const uint32_t k_lo = desc_lo_sw128(smem_u32(smem + L::kK + s * kClTerms * L::kPage), 16);
+        // term t of phi(Q) with the first 3 - t of phi(K), onto the sums from the t-th on
 #pragma unroll
-        for (int hl = 0; hl < 2; ++hl) {
-          const int i = 2 * j + hl, s = i % kClKSlots;
-          if (!cl_wait(&bars->k_full[s], (i / kClKSlots) & 1, bars, a.status)) return false;
-          tc_fence_after();
-          const uint32_t k_lo = desc_lo_sw128(smem_u32(smem + L::kK + s * L::kTile), 16);
+        for (int t = 0; t < kClTerms; ++t)
 #pragma unroll
-          for (int qp = 0; qp < 2 - hl; ++qp)  // phi(K) hi meets phi(Q) hi and lo, phi(K) lo meets phi(Q) hi
-#pragma unroll
-            for (int kk = 0; kk < D / 16; ++kk) {
-              const uint32_t off = ((kk / 4) * L::kHalf + (kk % 4) * 32) >> 4;
-              tc_mma_ts_lo(d, tmem + (qp ? kClColQl : kClColQh) + kk * 8, k_lo + off, kHiSw, idesc, (hl > 0 || qp > 0 || kk > 0) ? 1u : 0u);
-            }
-          tc_commit(&bars->k_empty[s]);
-        }
+          for (int kk = 0; kk < D / 16; ++kk)
+            tc_mma_ss_lo(d + kBlock * t, q_lo + ((t * L::kQTile + (kk / 4) * L::kQHalf + (kk % 4) * 32) >> 4),
+                         k_lo + (((kk / 4) * kClTerms * L::kSlab + (kk % 4) * 32) >> 4), kHiSw,
+                         idesc_bf16_f32(128, kBlock * (kClTerms - t), 0, 0), (t > 0 || kk > 0) ? 1u : 0u);
         tc_commit(&bars->a_full[j & 1]);
         return true;
       };
-      bool ok = cl_wait(&bars->q_read, 0, bars, a.status);  // phi(Q) is in TMEM
+      bool ok = cl_wait(&bars->q_read, 0, bars, a.status);  // phi(Q) is in shared memory
       for (int j = 0; j < min(2, nsteps) && ok; ++j) ok = issue_qk(j);
 #pragma unroll 1
       for (int j = 0; j < nsteps && ok; ++j) {
         const int s = j % kClStages;
-        ok = cl_wait(&bars->p_full[j & 1], (j >> 1) & 1, bars, a.status) &&
-             cl_wait(&bars->v_full[s], (j / kClStages) & 1, bars, a.status);
+        // (V first, which has long landed: it is asked for while the tensor pipe still works)
+        ok = cl_wait(&bars->v_full[s], (j / kClStages) & 1, bars, a.status) && cl_wait(&bars->p_ready, j & 1, bars, a.status);
         if (!ok) break;
         tc_fence_after();
         constexpr uint32_t idesc = idesc_bf16_f32(128, D, 0, 1);
-        const uint32_t v_lo = desc_lo_sw128(smem_u32(smem + L::kV + s * L::kTile), L::kHalf);
-        const uint32_t p_op = tmem + kClColA + 128 * (j & 1);
-        const int nk = 4 * pages_of(j);  // 16 keys each; a page that was not loaded is not touched
-        for (int kk = 0; kk < nk; ++kk) {
-          const uint32_t p_hi = p_op + 32 * (kk >> 1) + 8 * (kk & 1);
-          tc_mma_ts_lo(tmem + kClColNum, p_hi, v_lo + kk * 128, kHiSw, idesc, (j > 0 || kk > 0) ? 1u : 0u);
-          tc_mma_ts_lo(tmem + kClColNum, p_hi + 16, v_lo + kk * 128, kHiSw, idesc, 1u);
-        }
-        tc_commit(&bars->v_empty[s]);
+        const uint32_t v_lo = desc_lo_sw128(smem_u32(smem + L::kV + s * L::kPage), L::kSlab);
+        const uint32_t p_op = tmem + kClColBuf + kClBuf * (j & 1);
+#pragma unroll
+        for (int t = kClTerms - 1; t >= 0; --t)
+#pragma unroll
+          for (int kk = 0; kk < kBlock / 16; ++kk)
+            tc_mma_ts_lo(tmem + kClColNum, p_op + (t == 2 ? kBlock + 16 * kk : 16 * kk + 8 * t), v_lo + kk * 128, kHiSw, idesc,
+                         (t < kClTerms - 1 || kk > 0) ? 1u : 0u);
+        tc_commit(&bars->num_full[s]);
         // the weights of step j + 2 overwrite the ones just consumed: the tensor pipe runs in order
         if (j + 2 < nsteps) ok = issue_qk(j + 2);
       }
-      if (ok) tc_commit(&bars->done);
     }
   } else {
-    // ------------------------------------------------------------------ weights, result
-    const int set = (warp - 2) >> 2;  // 32 of the 128 columns
+    // ------------------------------------------------------------------ weights, sums
+    const int set = (warp - 2) >> 2;  // 16 of the 64 columns of a step, D / 4 of the dims
     const int quad = warp & 3;        // TMEM lane quadrant this warp may access
     const int r = quad * 32 + lane;   // row inside the tile
     const uint32_t lane_off = static_cast<uint32_t>(quad * 32) << 16;
+    constexpr int NC = D / 4;
     bool ok = __all_sync(0xffffffffu, cl_wait(&bars->q_full, 0, bars, a.status));
     if (ok) {
       if (set * 32 < D) {
-        // phi(q) of this thread's row, 32 dims, as the bf16 hi and lo A operands
-        const uint8_t* qrow = smem + L::kQ + r * 128;
-        uint32_t hi[16], lo[16];
+        // phi(q) of this thread's row, 32 dims, as the three bf16 A operands
+        uint8_t* cell[4];  // 16-byte chunks of the row
+        float f[32], largest = 0.f;
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-          const int cc = set * 4 + c;  // 16-byte chunk of the row
-          const uint4 raw = *reinterpret_cast<const uint4*>(qrow + (cc >> 3) * L::kHalf + (((cc & 7) ^ (r & 7)) << 4));
-          const uint32_t* qw = reinterpret_cast<const uint32_t*>(&raw);
+          const int cc = set * 4 + c;
+          cell[c] = smem + L::kQ + r * 128 + (cc >> 3) * L::kQHalf + (((cc & 7) ^ (r & 7)) << 4);
+          const uint4 raw = *reinterpret_cast<const uint4*>(cell[c] + 2 * L::kQTile);
+          const uint32_t w[4] = {raw.x, raw.y, raw.z, raw.w};
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            cl_split(cl_phi(__uint_as_float(qw[i] << 16), a.relu), cl_phi(__uint_as_float(qw[i] & 0xffff0000u), a.relu),
-                     hi[c * 4 + i], lo[c * 4 + i]);
+          for (int e = 0; e < 8; ++e) {
+            f[c * 8 + e] = cl_phi(__uint_as_float(e & 1 ? w[e >> 1] & 0xffff0000u : w[e >> 1] << 16), a.relu);
+            largest = fmaxf(largest, f[c * 8 + e]);
+          }
         }
-        tmem_st16(tmem + lane_off + kClColQh + set * 16, hi);
-        tmem_st16(tmem + lane_off + kClColQl + set * 16, lo);
-        tc_wait_st();
+        const float grid = cl_grid(largest);
+        uint32_t t[kClTerms][16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) cl_split(f[2 * i], f[2 * i + 1], grid, t[0][i], t[1][i], t[2][i]);
+#pragma unroll
+        for (int m = 0; m < kClTerms; ++m)
+#pragma unroll
+          for (int c = 0; c < 4; ++c)
+            *reinterpret_cast<uint4*>(cell[c] + m * L::kQTile) = make_uint4(t[m][4 * c], t[m][4 * c + 1], t[m][4 * c + 2], t[m][4 * c + 3]);
+        fence_proxy_async_smem();
       }
-      tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->q_read);
     }
-    float den = 0.f;
+    float den = 0.f, num[NC];
+#pragma unroll
+    for (int i = 0; i < NC; ++i) num[i] = 0.f;
+    // adds the products of step j to the running sums
+    auto add_step = [&](int j) -> bool {
+      if (!__all_sync(0xffffffffu, cl_wait(&bars->num_full[j & 1], (j >> 1) & 1, bars, a.status))) return false;
+      tc_fence_after();
+#pragma unroll
+      for (int c = 0; c < NC; c += 16) {
+        uint32_t v[16];
+        tmem_ld16(tmem + lane_off + kClColNum + NC * set + c, v);
+        tc_wait_ld();
+#pragma unroll
+        for (int i = 0; i < 16; ++i) num[c + i] += __uint_as_float(v[i]);
+      }
+      return true;
+    };
 #pragma unroll 1
     for (int j = 0; j < nsteps && ok; ++j) {
       ok = __all_sync(0xffffffffu, cl_wait(&bars->a_full[j & 1], (j >> 1) & 1, bars, a.status));
       if (!ok) break;
       tc_fence_after();
-      const uint32_t buf = tmem + lane_off + kClColA + 128 * (j & 1) + 32 * set;
-      uint32_t v[32];
-      tmem_ld32(buf, v);
-      const int64_t base = static_cast<int64_t>(b_first + 2 * j) * kBlock;  // token of column 0
-      const int lo_col = static_cast<int>(a.q_pos0 - base);                 // first visible column (<= 0: all)
-      const int hi_col = static_cast<int>(a.q_pos0 + row0 - base);          // last visible column of row 0
+      const uint32_t buf = tmem + lane_off + kClColBuf + kClBuf * (j & 1);
+      uint32_t v[16], u1[16], u2[16];
+      tmem_ld16(buf + 16 * set, v);
+      tmem_ld16(buf + kBlock + 16 * set, u1);
+      tmem_ld16(buf + 2 * kBlock + 16 * set, u2);
+      const int64_t base = static_cast<int64_t>(b_first + j) * kBlock;  // token of column 0
+      const int lo_col = static_cast<int>(a.q_pos0 - base);             // first visible column (<= 0: all)
+      const int hi_col = static_cast<int>(a.q_pos0 + row0 - base);      // last visible column of row 0
       tc_wait_ld();
-      if (lo_col > 0 || hi_col < 127) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          const int c = 32 * set + i;
+      for (int i = 0; i < 16; ++i) v[i] = __float_as_uint(__uint_as_float(v[i]) + (__uint_as_float(u1[i]) + __uint_as_float(u2[i])));
+      if (lo_col > 0 || hi_col < kBlock - 1) {
+#pragma unroll
+        for (int i = 0; i < 16; ++i) {
+          const int c = 16 * set + i;
           if (c < lo_col || c > hi_col + r) v[i] = 0u;
         }
       }
       float s4[4] = {0.f, 0.f, 0.f, 0.f};
-      uint32_t hi[16], lo[16];
+      uint32_t t[kClTerms][8];
 #pragma unroll
-      for (int i = 0; i < 16; ++i) {
+      for (int i = 0; i < 8; ++i) {
         const float x0 = __uint_as_float(v[2 * i]), x1 = __uint_as_float(v[2 * i + 1]);
         s4[(2 * i) & 3] += x0;
         s4[(2 * i + 1) & 3] += x1;
-        cl_split(x0, x1, hi[i], lo[i]);
+        cl_split(x0, x1, 0.f, t[0][i], t[1][i], t[2][i]);
       }
       // (over the thread's own columns, which it has read)
-      tmem_st16(buf, hi);
-      tmem_st16(buf + 16, lo);
+      tmem_st8(buf + 16 * set, t[0]);
+      tmem_st8(buf + 16 * set + 8, t[1]);
+      tmem_st8(buf + kBlock + 16 * set, t[2]);
       den += (s4[0] + s4[1]) + (s4[2] + s4[3]);
       tc_wait_st();
+      if (j > 0) ok = add_step(j - 1);
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&bars->p_full[j & 1]);
+      if (ok && lane == 0) mbar_arrive(&bars->p_ready);
     }
-    if (ok) ok = __all_sync(0xffffffffu, cl_wait(&bars->done, 0, bars, a.status));
-    tc_fence_after();
+    if (ok) ok = add_step(nsteps - 1);
     float* dsum = reinterpret_cast<float*>(smem + L::kK);  // [4][128], dead by now
     if (ok) dsum[set * 128 + r] = den;
     // (an aborted wait leaves the loop as well: the barrier takes every worker)
     asm volatile("bar.sync 1, %0;" ::"n"(kClWorkers) : "memory");
-    if (ok) {
-      const int row = row0 + r;
-      if (set * 32 < D) {  // warp-uniform: the load is warp-collective
-        uint32_t v[32];
-        tmem_ld32(tmem + lane_off + kClColNum + 32 * set, v);
-        tc_wait_ld();
-        if (row < a.n_q) {
-          float4* dst = reinterpret_cast<float4*>(a.lin_num + (static_cast<size_t>(row) * a.H + h) * D + 32 * set);
+    const int row = row0 + r;
+    if (ok && row < a.n_q) {
+      float4* dst = reinterpret_cast<float4*>(a.lin_num + (static_cast<size_t>(row) * a.H + h) * D + NC * set);
 #pragma unroll
-          for (int i = 0; i < 8; ++i)
-            dst[i] = make_float4(__uint_as_float(v[4 * i]), __uint_as_float(v[4 * i + 1]), __uint_as_float(v[4 * i + 2]),
-                                 __uint_as_float(v[4 * i + 3]));
-        }
-      }
-      if (set == 0 && row < a.n_q) 
+      for (int i = 0; i < NC / 4; ++i) dst[i] = make_float4(num[4 * i], num[4 * i + 1], num[4 * i + 2], num[4 * i + 3]);
+      if (set == 0)
         a.lin_den[static_cast<size_t>(row) * a.H + h] = (dsum[r] + dsum[128 + r]) + (dsum[256 + r] + dsum[384 + r]);
     }
   }

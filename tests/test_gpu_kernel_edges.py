@@ -53,6 +53,37 @@ def test_causal_intra_chunk_products(n0, n_q, d, relu, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("n0,n,d,relu", [(0, 1, 128, 0), (100, 65, 128, 0), (64, 640, 128, 0), (1, 1000, 64, 0), (70, 300, 128, 1),
+                                         (0, 129, 64, 1)])
+def test_causal_partials_carry_24_bits(n0, n, d, relu, cuda_device):
+    """Numerator and denominator of the intra-chunk part against 64 bits.  Map, weights and sums are 32-bit
+    quantities: relative errors of 2^-24 per rounding, a few in a row, so 2^-21 is allowed; carried in 16 bits
+    anywhere they are off by 2^-17 and more."""
+    from paper_2609_34606_b200 import hsa
+    H = 3
+    g = torch.Generator().manual_seed(n)
+    k, v, q = _randn(g, n, H, d), _randn(g, n, H, d), _randn(g, n, H, d)
+    size = max(n, n0, 1)
+    ctx = hsa.HSAContext(H, d, max_pages=(n0 + n + 63) // 64, max_q_tokens=size, max_topk=1, causal=True, device=cuda_device,
+                         feature_map=relu)
+    if n0:
+        ctx.append_kv(_randn(g, n0, H, d).to(cuda_device), _randn(g, n0, H, d).to(cuda_device))
+    ctx.append_kv(k.to(cuda_device), v.to(cuda_device))
+    ctx.forward(q.to(cuda_device), None, None, q_pos0=n0, causal=True, flags=hsa.HSA_FWD_NO_SPARSE)
+    assert ctx.device_status() == 0
+    # the partials come first in what the causal flag adds to the workspace
+    plain = hsa.hsa_config.from_buffer_copy(ctx.cfg)
+    plain.flags = 0
+    lo = hsa.hsa_query_sizes(plain).workspace
+    num = ctx.workspace[lo:lo + 4 * n * H * d].view(torch.float32).view(n, H, d).double().cpu()
+    lo += (4 * size * H * d + 255) // 256 * 256
+    den = ctx.workspace[lo:lo + 4 * n * H].view(torch.float32).view(n, H).double().cpu()
+    phi = lambda x: x.clamp(min=0) if relu else torch.where(x > 0, x + 1, x.exp())
+    A = torch.einsum("ihd,jhd->hij", phi(q.double()), phi(k.double())).tril()
+    for got, ref in ((num, torch.einsum("hij,jhd->ihd", A, v.double())), (den, A.sum(2).T)):
+        assert float((got - ref).norm()) <= 2.0 ** -21 * float(ref.norm())
+    ctx.destroy()
+
 @pytest.mark.parametrize("d", [64, 128])
 def test_causal_nan_key_reaches_the_queries_behind_it(d, cuda_device):
     """A NaN in a key of the chunk makes the linear branch NaN for the queries at and behind it (elu), and a NaN in
