@@ -637,6 +637,7 @@ int hsa_forward(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride, in
     CausalLinArgs c{};
     c.n_q = n_q;
     c.k_pool = static_cast<const __nv_bfloat16*>(ctx->buf.k_pool);
+    c.v_pool = static_cast<const __nv_bfloat16*>(ctx->buf.v_pool);
     c.phik = reinterpret_cast<__nv_bfloat16*>(ws + ctx->lay.phik);
     c.phik_blocks = ctx->lay.phik_blocks;
     c.page_table = p.page_table;

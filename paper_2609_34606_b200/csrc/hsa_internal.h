@@ -160,6 +160,7 @@ struct CausalLinArgs {
   int n_q;
   const int32_t* page_table;
   const __nv_bfloat16* k_pool;
+  const __nv_bfloat16* v_pool;
   // workspace: phi(K) of the pages that hold the chunk as bf16 terms, [H][hi/mid/lo][phik_blocks][64][D], block 0
   // being the chunk's first page (its rows before the chunk included)
   __nv_bfloat16* phik;

@@ -26,7 +26,8 @@
 // SIMT kernel this replaced -> now: num 1.1e-7 / 2.2e-7 / 3.0e-7 -> 0.7e-7 / 1.0e-7 / 1.2e-7, den 0.6e-7 /
 // 0.8e-7 / 1.0e-7 -> 0.4e-7 / 0.5e-7 / 0.6e-7.  (Two terms each and sums over the whole chunk in TMEM: num
 // 2.7e-6 / 3.5e-6 / 5.2e-6, den 6.0e-7.)
-// (A non-finite V reaches every row of its 128-row tile, also those before it: 0 x inf in the product.)
+// An Inf or NaN meets zeros in the products (masked weights, terms of the split), also in rows before it: a row
+// whose result is not finite is taken again key by key (cl_plain_row).
 //
 // What bounds it: the tensor pipe along the longest tile, 25 steps at a chunk of 1560 tokens.  The terms of
 // phi(K) lie side by side, so that one product of phi(Q) hi with all three, one of mid with the first two and
@@ -40,6 +41,8 @@
 // each.  The split weights overwrite them: 16 columns of hi hi become 8 of packed hi and 8 of packed mid, 16 of
 // the next sum 8 of packed lo.
 #include <cuda_bf16.h>
+
+#include <cfloat>
 
 #include "hsa_internal.h"
 #include "ptx.cuh"
@@ -104,6 +107,53 @@ __device__ __forceinline__ void cl_split(float a, float b, float grid, uint32_t&
   b -= __uint_as_float(hi & 0xffff0000u);
   mid = pack_bf16(a, b);
   lo = pack_bf16(a - __uint_as_float(mid << 16), b - __uint_as_float(mid & 0xffff0000u));
+}
+
+// element e of 8 that three bf16 terms make up
+__device__ __forceinline__ float cl_join(const uint4 (&t)[kClTerms], int e) {
+  float f[kClTerms];
+#pragma unroll
+  for (int m = 0; m < kClTerms; ++m) {
+    const uint32_t w = (e >> 1) == 0 ? t[m].x : (e >> 1) == 1 ? t[m].y : (e >> 1) == 2 ? t[m].z : t[m].w;
+    f[m] = __uint_as_float(e & 1 ? w & 0xffff0000u : w << 16);
+  }
+  return fabsf(f[0]) <= FLT_MAX ? f[0] + f[1] + f[2] : f[0];  // (the remainders of Inf are NaN)
+}
+
+// num of one row (D / 4 columns) and den, key by key in fp32.  q: terms of phi(Q) in shared memory, row r; phik: the
+// head's hi tiles, mid and lo `term` elements further on each; keys `first` and the n_keys - 1 behind it, counted
+// from the first of `pages`.
+template <int D>
+__device__ __noinline__ void cl_plain_row(const uint8_t* q, int r, const __nv_bfloat16* phik, size_t term,
+                                          const __nv_bfloat16* v_pool, const int32_t* pages, int H, int h, int first, int n_keys,
+                                          int col, float* num, float* den) {
+  using L = ClSmem<D>;
+  constexpr int NC = D / 4;
+  float acc[NC], sum = 0.f;
+#pragma unroll
+  for (int i = 0; i < NC; ++i) acc[i] = 0.f;
+#pragma unroll 1
+  for (int t = first; t < first + n_keys; ++t) {
+    float w = 0.f;
+#pragma unroll 1
+    for (int c = 0; c < D / 8; ++c) {
+      uint4 qt[kClTerms], kt[kClTerms];
+#pragma unroll
+      for (int m = 0; m < kClTerms; ++m) {
+        qt[m] = *reinterpret_cast<const uint4*>(q + m * L::kQTile + r * 128 + (c >> 3) * L::kQHalf + (((c & 7) ^ (r & 7)) << 4));
+        kt[m] = *reinterpret_cast<const uint4*>(phik + m * term + static_cast<size_t>(t) * D + c * 8);
+      }
+#pragma unroll
+      for (int e = 0; e < 8; ++e) w = fmaf(cl_join(qt, e), cl_join(kt, e), w);
+    }
+    sum += w;
+    const __nv_bfloat16* v = v_pool + ((static_cast<size_t>(pages[t / kBlock]) * H + h) * kBlock + t % kBlock) * D + col;
+#pragma unroll
+    for (int i = 0; i < NC; ++i) acc[i] = fmaf(w, __bfloat162float(v[i]), acc[i]);
+  }
+#pragma unroll
+  for (int i = 0; i < NC; ++i) num[i] = acc[i];
+  if (den) *den = sum;
 }
 
 }  // namespace
@@ -375,11 +425,22 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
     asm volatile("bar.sync 1, %0;" ::"n"(kClWorkers) : "memory");
     const int row = row0 + r;
     if (ok && row < a.n_q) {
-      float4* dst = reinterpret_cast<float4*>(a.lin_num + (static_cast<size_t>(row) * a.H + h) * D + NC * set);
+      float* dst = a.lin_num + (static_cast<size_t>(row) * a.H + h) * D + NC * set;
+      float* dst_den = set == 0 ? a.lin_den + static_cast<size_t>(row) * a.H + h : nullptr;
+      den = (dsum[r] + dsum[128 + r]) + (dsum[256 + r] + dsum[384 + r]);
+      bool finite = fabsf(den) <= FLT_MAX;
 #pragma unroll
-      for (int i = 0; i < NC / 4; ++i) dst[i] = make_float4(num[4 * i], num[4 * i + 1], num[4 * i + 2], num[4 * i + 3]);
-      if (set == 0)
-        a.lin_den[static_cast<size_t>(row) * a.H + h] = (dsum[r] + dsum[128 + r]) + (dsum[256 + r] + dsum[384 + r]);
+      for (int i = 0; i < NC; ++i) finite = finite && fabsf(num[i]) <= FLT_MAX;
+      if (finite) {
+#pragma unroll
+        for (int i = 0; i < NC / 4; ++i)
+          reinterpret_cast<float4*>(dst)[i] = make_float4(num[4 * i], num[4 * i + 1], num[4 * i + 2], num[4 * i + 3]);
+        if (dst_den) *dst_den = den;
+      } else {
+        const size_t term = static_cast<size_t>(a.phik_blocks) * kBlock * D;
+        cl_plain_row<D>(smem + L::kQ, r, a.phik + h * kClTerms * term, term, a.v_pool, a.page_table + b_first, a.H, h,
+                        static_cast<int>(a.q_pos0 - static_cast<int64_t>(b_first) * kBlock), row + 1, NC * set, dst, dst_den);
+      }
     }
   }
   tc_fence_before();

@@ -53,6 +53,18 @@ def test_causal_intra_chunk_products(n0, n_q, d, relu, cuda_device):
     ctx.destroy()
 
 
+def _causal_partials(ctx, n, size):
+    """Numerator [n, H, d] and denominator [n, H] in the workspace of a context for chunks of `size` tokens: they
+    come first in what the causal flag adds to it (short lists, no adaptive selection)."""
+    from paper_2609_34606_b200 import hsa
+    plain = hsa.hsa_config.from_buffer_copy(ctx.cfg)
+    plain.flags = 0
+    lo, H, d = hsa.hsa_query_sizes(plain).workspace, ctx.H, ctx.d
+    num = ctx.workspace[lo:lo + 4 * n * H * d].view(torch.float32).view(n, H, d).double().cpu()
+    lo += (4 * size * H * d + 255) // 256 * 256
+    return num, ctx.workspace[lo:lo + 4 * n * H].view(torch.float32).view(n, H).double().cpu()
+
+
 @pytest.mark.parametrize("n0,n,d,relu", [(0, 1, 128, 0), (100, 65, 128, 0), (64, 640, 128, 0), (1, 1000, 64, 0), (70, 300, 128, 1),
                                          (0, 129, 64, 1)])
 def test_causal_partials_carry_24_bits(n0, n, d, relu, cuda_device):
@@ -71,17 +83,47 @@ def test_causal_partials_carry_24_bits(n0, n, d, relu, cuda_device):
     ctx.append_kv(k.to(cuda_device), v.to(cuda_device))
     ctx.forward(q.to(cuda_device), None, None, q_pos0=n0, causal=True, flags=hsa.HSA_FWD_NO_SPARSE)
     assert ctx.device_status() == 0
-    # the partials come first in what the causal flag adds to the workspace
-    plain = hsa.hsa_config.from_buffer_copy(ctx.cfg)
-    plain.flags = 0
-    lo = hsa.hsa_query_sizes(plain).workspace
-    num = ctx.workspace[lo:lo + 4 * n * H * d].view(torch.float32).view(n, H, d).double().cpu()
-    lo += (4 * size * H * d + 255) // 256 * 256
-    den = ctx.workspace[lo:lo + 4 * n * H].view(torch.float32).view(n, H).double().cpu()
+    num, den = _causal_partials(ctx, n, size)
     phi = lambda x: x.clamp(min=0) if relu else torch.where(x > 0, x + 1, x.exp())
     A = torch.einsum("ihd,jhd->hij", phi(q.double()), phi(k.double())).tril()
     for got, ref in ((num, torch.einsum("hij,jhd->ihd", A, v.double())), (den, A.sum(2).T)):
         assert float((got - ref).norm()) <= 2.0 ** -21 * float(ref.norm())
+    ctx.destroy()
+
+@pytest.mark.parametrize("n0,n,d,relu", [(0, 100, 128, 0), (100, 300, 128, 0), (70, 300, 64, 0), (64, 300, 128, 1)])
+def test_causal_not_finite_values_stay_behind_their_position(n0, n, d, relu, cuda_device):
+    """Inf and NaN in K, V and queries of a causal chunk reach the rows at and behind them, and there what they
+    reach in a plain sum, and nothing before them."""
+    from paper_2609_34606_b200 import hsa
+    H, inf, nan = 4, float("inf"), float("nan")
+    g = torch.Generator().manual_seed(n0 + d)
+    k, v, q = _randn(g, n, H, d), _randn(g, n, H, d), _randn(g, n, H, d)
+    t = n - 30
+    v[t, 0, 5], v[t, 0, 6], v[3, 0, 7] = inf, -inf, nan
+    k[t, 1, 9], k[t + 9, 1, 2] = inf, -inf
+    q[20, 2, 33], q[t, 2, 0], q[t + 1, 2, 1] = inf, -inf, nan
+    size = max(n, n0)
+    ctx = hsa.HSAContext(H, d, max_pages=(n0 + n + 63) // 64, max_q_tokens=size, max_topk=1, causal=True, device=cuda_device,
+                         feature_map=relu)
+    if n0:
+        ctx.append_kv(_randn(g, n0, H, d).to(cuda_device), _randn(g, n0, H, d).to(cuda_device))
+    ctx.append_kv(k.to(cuda_device), v.to(cuda_device))
+    ctx.forward(q.to(cuda_device), None, None, q_pos0=n0, causal=True, flags=hsa.HSA_FWD_NO_SPARSE)
+    assert ctx.device_status() == 0
+    num, den = _causal_partials(ctx, n, size)
+
+    def phi(x):
+        x = x.double()  # (max(NaN, 0) is 0 on the GPU)
+        return torch.nan_to_num(x, nan=0.0, posinf=inf, neginf=-inf).clamp(min=0) if relu else torch.where(x > 0, x + 1, x.exp())
+
+    ref_num, ref_den = torch.zeros(n, H, d, dtype=torch.float64), torch.zeros(n, H, dtype=torch.float64)
+    for i in range(n):
+        w = (phi(q[i])[None] * phi(k[:i + 1])).sum(2)
+        ref_num[i], ref_den[i] = (w[:, :, None] * v[:i + 1].double()).sum(0), w.sum(0)
+    for got, ref in ((num, ref_num), (den, ref_den)):
+        odd = ~ref.isfinite()
+        assert torch.equal(torch.nan_to_num(got[odd], nan=1.0), torch.nan_to_num(ref[odd], nan=1.0))
+        assert float((got[~odd] - ref[~odd]).norm()) <= 2.0 ** -21 * float(ref[~odd].norm())
     ctx.destroy()
 
 @pytest.mark.parametrize("d", [64, 128])
