@@ -298,8 +298,9 @@ int hsa_state_layout(hsa_ctx* ctx, size_t* off_S, size_t* off_z, size_t* off_ksu
 
 /* Synchronises the device, reads and clears the status word: HSA_OK or a DEVICE_* code.
  * After HSA_ERR_DEVICE_TIMEOUT the selection written by the call that timed out has every count
- * set to zero (a forward call on it computes the linear branch alone), and this call also puts
- * the selection kernel's grid barrier back to its initial state, so the next call starts clean. */
+ * set to zero (a forward call on it computes the linear branch alone).  After any code this call also
+ * puts the selection kernel's grid barrier and the forward kernel's counters of split lists back to
+ * their initial state, so the next call starts clean. */
 int hsa_device_status(hsa_ctx* ctx, int32_t* status_out);
 
 /* Bound, in nanoseconds, of a wait at the grid barrier of the selection kernel (the one place

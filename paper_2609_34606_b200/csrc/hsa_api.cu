@@ -69,6 +69,10 @@ bool config_ok(const hsa_config* c) {
   return true;
 }
 
+size_t ticket_bytes(const hsa_config* c) {
+  return static_cast<size_t>((c->max_q_tokens + kTileM - 1) / kTileM) * c->num_heads * 4;
+}
+
 Layout make_layout(const hsa_config* c) {
   Layout L{};
   const size_t H = c->num_heads, D = c->head_dim, P = c->max_pages;
@@ -127,7 +131,7 @@ Layout make_layout(const hsa_config* c) {
     L.part_o = o;      o = align_up(o + slots * kTileM * D * 4, 256);
     L.part_l = o;      o = align_up(o + slots * kTileM * 4, 256);
     L.part_ref = o;    o = align_up(o + slots * kTileM * 4, 256);
-    L.part_ticket = o; o = align_up(o + tiles * H * 4, 256);
+    L.part_ticket = o; o = align_up(o + ticket_bytes(c), 256);
   }
   L.ws_total = o;
   return L;
@@ -286,8 +290,7 @@ int hsa_create(hsa_ctx** out, const hsa_config* cfg, const hsa_buffers* bufs,
   e = cudaMemcpy(ws + ctx->lay.page_table, pt.data(), pt.size() * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(ws + ctx->lay.status, 0, 16);
   if (e == cudaSuccess && ctx->lay.part_slots > 0)
-    e = cudaMemset(ws + ctx->lay.part_ticket, 0,
-                   static_cast<size_t>((cfg->max_q_tokens + kTileM - 1) / kTileM) * cfg->num_heads * 4);
+    e = cudaMemset(ws + ctx->lay.part_ticket, 0, ticket_bytes(cfg));
   if (e == cudaSuccess) e = cudaMemset(bufs->state, 0, ctx->lay.state_total);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e == cudaSuccess) e = forward_init();
@@ -860,8 +863,11 @@ int hsa_device_status(hsa_ctx* ctx, int32_t* status_out) {
   int32_t v = 0;
   e = cudaMemcpy(&v, ws + ctx->lay.status, 4, cudaMemcpyDeviceToHost);
   if (e == cudaSuccess && v != 0) e = cudaMemset(ws + ctx->lay.status, 0, 4);
-  // a grid barrier that ran out leaves its arrive count behind: both of its words start over
-  if (e == cudaSuccess && v == HSA_ERR_DEVICE_TIMEOUT) e = cudaMemset(ws + ctx->lay.status + 8, 0, 8);
+  // (the word keeps the first code only, so any may hide a wait that ran out)  A grid barrier that ran out leaves
+  // its arrive count behind: both of its words start over.  A part of a split list that gave up has drawn no
+  // ticket, which leaves its list's counter short: they start over too.
+  if (e == cudaSuccess && v != 0) e = cudaMemset(ws + ctx->lay.status + 8, 0, 8);
+  if (e == cudaSuccess && v != 0 && ctx->lay.part_slots > 0) e = cudaMemset(ws + ctx->lay.part_ticket, 0, ticket_bytes(&ctx->cfg));
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   *status_out = v;
   return HSA_OK;

@@ -407,3 +407,29 @@ def test_lists_of_few_items_split_over_ctas(d, H, n_q, budgets, gates, causal, c
     # the parts take their exponent references from other keys: weights round to bf16 differently
     assert float((a - b).norm() / b.norm()) <= BF16_REL
     ctx.destroy()
+
+
+@pytest.mark.parametrize("split_blocks,code", [(4, -5), (4, -6), (0, -5)])
+def test_counters_of_split_lists_start_over_with_the_status_word(split_blocks, code, cuda_device):
+    """A part of a split list that gives up draws no ticket; reading the status word puts the counters back (written
+    here by the host, as such a launch leaves them), so that the next launch merges all of its parts."""
+    from paper_2609_34606_b200 import hsa
+    H, d, n, n_q = 2, 128, 130 * 64, 200
+    g = torch.Generator().manual_seed(3)
+    ctx = hsa.HSAContext(H, d, max_pages=130, max_q_tokens=n, max_topk=128, device=cuda_device, split_blocks=split_blocks)
+    ctx.append_kv(_randn(g, n, H, d).to(cuda_device), _randn(g, n, H, d).to(cuda_device))
+    q = _randn(g, n_q, H, d).to(cuda_device)
+    idx, cnt = ctx.select_blocks(q, torch.full((H,), 128, dtype=torch.int32, device=cuda_device))
+    want = ctx.forward(q, idx, cnt)
+    assert ctx.device_status() == 0
+    tickets = (n + 127) // 128 * H  # the last words of the workspace, in whole 256 bytes
+    words = ctx.workspace.view(torch.int32)
+    end = hsa.hsa_query_sizes(ctx.cfg).workspace // 4 - (4 * tickets + 255) // 256 * 64
+    assert words[end:end + tickets].abs().sum().item() == 0
+    words[end:end + tickets] = 1
+    words[hsa.hsa_workspace_layout(ctx.ctx)[0] // 4] = code
+    assert ctx.device_status() == code
+    assert words[end:end + tickets].abs().sum().item() == 0
+    out = ctx.forward(q, idx, cnt)
+    assert ctx.device_status() == 0 and torch.equal(out, want)
+    ctx.destroy()
