@@ -1092,18 +1092,30 @@ __global__ void __launch_bounds__(256 * kSubBlocks, 1) select_cluster_kernel(Sel
 }
 
 namespace {
-// cooperative launch support and SM count of the current device (queried once per device)
+// What is looked up once per device of the process, by whichever thread gets there first.
+struct DeviceInfo {
+  bool known;
+  int coop, nsm;
+  bool cluster_known[2][2][2][2];  // per instance of the cluster form: D == 128, mixed, own, adaptive
+  int cluster[2][2][2][2];         // CTAs of its clusters, 0: cannot be launched
+};
+constexpr int kMaxDevices = 64;
+DeviceInfo g_device_info[kMaxDevices];
+std::mutex g_device_mutex;
+
+// cooperative launch support and SM count of the current device
 bool coop_info(int* nsm) {
-  static int cached_dev = -1, cached_coop = 0, cached_sm = 0;
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess) return false;
-  if (dev != cached_dev) {
-    cudaDeviceGetAttribute(&cached_coop, cudaDevAttrCooperativeLaunch, dev);
-    cudaDeviceGetAttribute(&cached_sm, cudaDevAttrMultiProcessorCount, dev);
-    cached_dev = dev;
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+  std::lock_guard<std::mutex> lock(g_device_mutex);
+  DeviceInfo& info = g_device_info[dev];
+  if (!info.known) {
+    cudaDeviceGetAttribute(&info.coop, cudaDevAttrCooperativeLaunch, dev);
+    cudaDeviceGetAttribute(&info.nsm, cudaDevAttrMultiProcessorCount, dev);
+    info.known = true;
   }
-  *nsm = cached_sm;
-  return cached_coop != 0 && cached_sm > 0;
+  *nsm = info.nsm;
+  return info.coop != 0 && info.nsm > 0;
 }
 }  // namespace
 
@@ -1203,16 +1215,24 @@ bool launch_cluster(const SelectArgs& a, const AdaptiveArgs* ad, bool mixed, cud
   const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
   const bool own = n_tiles <= kOwnQueryTiles;
   const void* fn = a.D == 128 ? cluster_kernel<128>(mixed, own, ad != nullptr) : cluster_kernel<64>(mixed, own, ad != nullptr);
-  // the cluster size is looked up once per instance, for the largest shared-memory size the form
-  // is used with (a cluster that fits with that fits with less)
+  // the cluster size is looked up, and the shared-memory limit set, once per instance and device, for the
+  // largest size the form is used with (a cluster that fits with that fits with less)
   constexpr size_t kMaxSmem = 120 * 1024;
   if (smem > kMaxSmem) return false;
-  static int cached_cs[2][2][2][2] = {{{{-1, -1}, {-1, -1}}, {{-1, -1}, {-1, -1}}}, {{{-1, -1}, {-1, -1}}, {{-1, -1}, {-1, -1}}}};
-  int& cs = cached_cs[a.D == 128][mixed][own][ad != nullptr];
-  if (cs < 0) {
-    const bool ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMaxSmem)) == cudaSuccess;
-    cs = ok ? cluster_size_for(fn, kMaxSmem, 256 * kSubBlocks) : 0;
-    if (cs == 0) cudaGetLastError();  // no cluster of that shape on this device: the other forms
+  int dev = -1;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
+  int cs;
+  {
+    std::lock_guard<std::mutex> lock(g_device_mutex);
+    bool& known = g_device_info[dev].cluster_known[a.D == 128][mixed][own][ad != nullptr];
+    int& size = g_device_info[dev].cluster[a.D == 128][mixed][own][ad != nullptr];
+    if (!known) {
+      const bool ok = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kMaxSmem)) == cudaSuccess;
+      size = ok ? cluster_size_for(fn, kMaxSmem, 256 * kSubBlocks) : 0;
+      if (size == 0) cudaGetLastError();  // no cluster of that shape on this device: the other forms
+      known = true;
+    }
+    cs = size;
   }
   if (cs == 0) return false;
   SelectArgs aa = a;
