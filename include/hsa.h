@@ -21,6 +21,10 @@
  *   - Every call only enqueues work on the given CUDA stream (a cudaStream_t
  *     passed as void*; NULL = default stream) and returns; nothing synchronises
  *     except hsa_device_status.  A context is not thread-safe.
+ *   - Calls of one context share its pool, state and workspace: work of two calls that is not ordered
+ *     on the GPU (two streams, two graphs) must not overlap.  The one exception: hsa_forward calls may
+ *     overlap one another while max_topk <= split_blocks, unless they are causal with the linear
+ *     branch on.
  *   - Return value: HSA_OK (0) or a negative hsa_status.  Device-side problems
  *     (a bounded wait that ran out, an out-of-range block index) never trap:
  *     the kernel records a code in a status word that hsa_device_status reads.
@@ -94,9 +98,8 @@ typedef struct {
   uint32_t flags;         /* HSA_CFG_* bits                                                    */
   int32_t lin_rank;       /* HSA_LIN_LINFORMER: projection rank r, a multiple of 64, 64..2048 (else 0) */
   int32_t lin_seg_tokens; /* HSA_LIN_LINFORMER: segment length L; every append must be exactly L      */
-  int32_t split_blocks;   /* a (query tile, head) with more selected blocks than this is split over
-                             several CTAs whose partial results the last one to finish merges
-                             (0 -> 256; only matters when max_topk exceeds it)                     */
+  int32_t split_blocks;   /* 0 -> 256.  When max_topk exceeds it, long lists are split over several CTAs
+                             whose partial results, in the workspace, the last one to finish merges   */
   int32_t feature_map;    /* HSA_LIN_STATE: HSA_PHI_ELU1 (0) or HSA_PHI_RELU                           */
 } hsa_config;
 
@@ -104,7 +107,8 @@ typedef struct {
   size_t k_pool;     /* bytes: [max_pages][H][64][d] bf16                                      */
   size_t v_pool;     /* same                                                                   */
   size_t state;      /* linear-branch state + per-block key sums                               */
-  size_t workspace;  /* page table copy, partial sums, status word                             */
+  size_t workspace;  /* page table copy, partial sums, status word; HSA_CFG_CAUSAL: phi(K) of a chunk,
+                        partial sums of the intra-chunk part                                   */
   size_t kc_pool;    /* HSA_LIN_LINFORMER: compressed keys, [segments * r / 64][H][64][d] bf16, else 0  */
   size_t vc_pool;    /* same for the compressed values                                         */
 } hsa_sizes;

@@ -120,6 +120,25 @@ __device__ __forceinline__ float ex2v(float x) {
   asm volatile("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// from the same place in the shared memory of the cluster's CTA `rank`
+__device__ __forceinline__ uint32_t cluster_addr(const float* p, int rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float ld_cluster(const float* p, int rank) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr(p, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster4(const float* p, int rank) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_addr(p, rank))
+               : "memory");
+  return v;
+}
 // either feature map without a branch: max(x, 0) + w * exp(min(x, 0)) with w = 1 (elu + 1) or 0 (relu)
 __device__ __forceinline__ float phi_q(float x, float w) {
   return fmaf(w, ex2(fminf(x, 0.f) * 1.4426950408889634f), fmaxf(x, 0.f));
@@ -156,11 +175,12 @@ __device__ __forceinline__ void init_barriers(Bars* bars) {
 
 }  // namespace
 
-// SPLIT: compiled with the split-tile path (grid z > 1); the plain kernel carries none of it
+// SPLIT: 1: compiled with the split-tile path (grid z > 1), parts in the workspace; 2: the parts of a list are the
+// CTAs of a cluster and meet in shared memory; the plain kernel (0) carries none of either
 // LINF: compiled with the compressed-pool segment in front of the selected pages (tm_kc, tm_vc)
 // GT: per-dim gate logits arrive as tiles by TMA (tm_gl, tm_gs); an instance of its own, so that the others
 // keep their registers
-template <int D, bool SPLIT, bool LINF, bool GT>
+template <int D, int SPLIT, bool LINF, bool GT>
 __global__ void __launch_bounds__(kThreads, 1)
 hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v,
@@ -175,7 +195,9 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   // two score buffers this shortens the chain that bounds the loop: Linformer pass 245.4 -> 236.5 us; long
   // split lists 418.8 -> 415.4.  With three buffers and short lists it does not pay: 64 blocks 152.5 against
   // 153.2, 128 blocks 272.6 against 270.2.
-  constexpr bool AHEAD = SPLIT || LINF;
+  constexpr bool AHEAD = SPLIT == 1 || LINF;
+  constexpr bool PARTS = SPLIT == 1;                     // partial results in the workspace
+  constexpr int kMaxParts = SPLIT == 1 ? kFwdSplitMax : SPLIT == 2 ? kClusterParts : 1;
   constexpr int NSB = LINF ? 2 : kSBufs;                 // score buffers in use
   constexpr uint32_t kColSb = LINF ? 256 : kColS;        // first score buffer
   constexpr uint32_t kColLn = LINF ? 128 : kColLin;      // linear-branch accumulator
@@ -204,19 +226,24 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   };
   // Launched with programmatic stream serialization: this grid may be scheduled while the kernel
   // before it (block selection) is still extracting its lists.  Nothing of that kernel's output is
-  // read before the wait; the plain kernel does its set-up first, under that kernel's tail (a split
-  // CTA may still leave without any set-up, so it sets up after it has seen its list).
-  if (!SPLIT) setup();
+  // read before the wait; the set-up is done first, under that kernel's tail (a CTA of the workspace form may
+  // still leave without any, so it sets up after it has seen its list).
+  if (!PARTS) setup();
   // wait_late: the kernel before this one supplies the causal partials only, which the epilogue reads;
   // it let this grid start after it had itself waited for everything before it (lists, pages, state),
   // so that the tiles' loops run on the SMs it has left already while its longest tiles finish
-  if (SPLIT || !p.wait_late) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (PARTS || !p.wait_late) asm volatile("griddepcontrol.wait;" ::: "memory");
   int tile = blockIdx.x, h = blockIdx.y, part = blockIdx.z;
+  if (SPLIT == 2) {
+    // (a cluster's CTAs follow one another in x, and there are 2, 4 or 8 of them)
+    part = tile & (p.cluster - 1);
+    tile >>= p.cluster >> 2 == 2 ? 3 : p.cluster >> 1;
+  }
   // Parts of a list of `st` two-page steps.  balance > 0: the steps one SM would run if the whole
   // launch were spread evenly; a list is cut into the fewest parts none of which is longer than that
-  // (no part shorter than min_part_steps).  balance == 0: parts of split_blocks blocks.
+  // (no part shorter than 16 steps).  balance == 0: parts of split_blocks blocks.
   auto parts_of = [&](int st, int balance) -> int {
-    const int want = balance > 0 ? min((st + balance - 1) / balance, max(1, st / p.min_part_steps))
+    const int want = balance > 0 ? min((st + balance - 1) / balance, max(1, st / 16))
                                  : (st + p.split_blocks / 2 - 1) / (p.split_blocks / 2);
     int ns = min(p.max_splits, max(1, want));
     const int per = (st + ns - 1) / ns;
@@ -225,7 +252,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   };
   int balance = 0;
   int slot_step = 1;  // from one part's partial-result slot to the next part's
-  if (SPLIT && p.remap) {
+  if (PARTS && p.remap) {
     // Longest lists first.  With one list per head every (tile, part) of a head costs the same, so the
     // heads are ranked by the steps one part of theirs takes and the grid walks through them in that
     // order (part-major inside a head: CTAs that run side by side gather the same pages); the heavy
@@ -238,7 +265,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     int total = st;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) total += __shfl_xor_sync(0xffffffffu, total, o);
-    balance = max(1, static_cast<int>((static_cast<int64_t>(total) * n_tiles + p.balance_sms - 1) / p.balance_sms));
+    balance = max(1, static_cast<int>((static_cast<int64_t>(total) * n_tiles + p.nsm - 1) / p.nsm));
     const int ns = parts_of(st, balance);
     const int per = (st + ns - 1) / ns;
     const int n_items = lane < p.H ? ns * n_tiles : 0;
@@ -270,7 +297,19 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   // A long list is split over the CTAs (tile, head, 0 .. nsplit - 1): each takes a run of whole
   // two-page steps; CTAs beyond nsplit leave before they set anything up.
   int nsplit = 1;
-  if (SPLIT && p.max_splits > 1) {
+  if (SPLIT == 2) {
+    // a power of two of parts, of about equal length
+    const int steps_total = (cnt + 1) / 2, lg = cluster_parts_log2(p.cluster, steps_total);
+    nsplit = 1 << lg;
+    if (part >= nsplit) {  // (the others do not wait for it)
+      if (warp == 0) tmem_dealloc(bars->tmem_base, kTmemCols);
+      return;
+    }
+    const int b_lo = 2 * ((part * steps_total) >> lg);
+    sel += b_lo;
+    cnt = min(cnt, 2 * (((part + 1) * steps_total) >> lg)) - b_lo;
+  }
+  if (SPLIT == 1 && p.max_splits > 1) {
     const int steps_total = (cnt + 1) / 2;
     nsplit = parts_of(steps_total, balance);
     const int steps_per = (steps_total + nsplit - 1) / nsplit;
@@ -283,7 +322,15 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     }
   }
   // this CTA's partial-result slot: the CTA's own number where the grid is one-dimensional
-  const int slot = (SPLIT && p.remap) ? static_cast<int>(blockIdx.x) : (tile * p.H + h) * p.max_splits + part;
+  const int slot = (PARTS && p.remap) ? static_cast<int>(blockIdx.x) : (tile * p.H + h) * p.max_splits + part;
+  // cluster form: the first part merges the others and alone has a linear branch, gates and output
+  const bool lead = SPLIT != 2 || part == 0;
+  const bool do_lin = p.do_linear && lead;
+  // The two phases of the cluster barrier: A, a softmax thread has left its part's results in shared memory (for the
+  // other warps of no meaning: they arrive at once); B, the first part has read them.
+  auto cluster_arrive = [] { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); };
+  auto cluster_wait = [] { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); };
+  bool a_arrived = false, a_waited = false;
   // steps of the compressed segment (LINF), then of the selected pages
   const int lf_pages = LINF ? p.lf_pages : 0;
   const int nA = (lf_pages + 1) / 2;
@@ -295,7 +342,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   // K steps that pass through ring stage s: a gate tile is the next one of its stage
   auto gate_uses = [&](int s) -> int { return nsteps > s ? (nsteps - 1 - s) / kStages + 1 : 0; };
 
-  if (SPLIT) setup();
+  if (PARTS) setup();
   const uint32_t tmem = bars->tmem_base;
 
   // attempt 0: fast pass (fixed exponent reference); attempt 1 only if a step overflowed: safe
@@ -322,6 +369,10 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     // a split that asks for more than is given back would block at setmaxnreg.inc for ever.
     static_assert(128 * (168 - 56) >= 256 * (kSoftmaxRegs - 168), "setmaxnreg.inc would never be satisfied");
     asm volatile("setmaxnreg.dec.sync.aligned.u32 56;");
+    if (SPLIT == 2 && nsplit > 1) {
+      cluster_arrive();  // A
+      a_arrived = true;
+    }
 #pragma unroll 1
     for (int attempt = 0; attempt < 2; ++attempt) {
     if (warp == 0) {
@@ -375,7 +426,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           ok = load_kv(j, false);
           if (ok && j + NSB < nsteps) ok = load_kv(j + NSB, true);
         }
-        if (ok && p.do_linear && !LINF) {
+        if (ok && do_lin && !LINF) {
           // hi and lo halves of the D x D state ride the V ring as two more "steps"
           for (int hl = 0; hl < 2 && ok; ++hl) {
             const int j = nsteps + hl;
@@ -392,7 +443,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             ++armed_v;
           }
         }
-        if (GT && ok) {
+        if (GT && ok && lead) {
           // per-dim gates: the tile's logits follow the last K pages into stages 1 and 2 of the K ring
           // (stage 0 holds the row statistics by then), ahead of the epilogue that applies them
           for (int i = 0; i < 2 && ok; ++i) {
@@ -425,7 +476,8 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       // The tiles of a (head, group) walk through the same list at about the same time.  Each of
       // them asks a slice of the list (entries tile-in-group, + tiles-per-group, ...) into L2 when
       // it starts, so that between them the whole list is on its way long before the rings reach it.
-      if (!SPLIT && p.k_pool != nullptr && elect_one_sync()) {  // (split tiles: measured slower with it)
+      // (split tiles: measured slower with it)
+      if (!PARTS && nsplit == 1 && p.k_pool != nullptr && elect_one_sync()) {
         const int n_tiles = p.n_tiles;
         const int tpg = p.group_tokens > 0 ? max(1, p.group_tokens / kTileM) : n_tiles;  // tiles per group
         for (int e = kStages * 2 + tile % tpg; e < cnt; e += tpg) {
@@ -507,7 +559,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           if (j + NSB < nsteps) ok = issue_qk(j + NSB, k_landed);
         }
         if (ok) tc_commit(&bars->o_done);
-        if (ok && p.do_linear && !LINF) {
+        if (ok && do_lin && !LINF) {
           ok = wait_bar(&bars->lin_a_full, 0, bars, p.status);
           for (int hl = 0; hl < 2 && ok; ++hl) {
             const int j = nsteps + hl;
@@ -565,7 +617,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       const int cbase = (grp & 1) * HC;
       float den_part = 0.f, den_part2 = 0.f;
       uint32_t fr[HC / 2];
-      if (ok && p.do_linear && epi && !LINF) {
+      if (ok && do_lin && epi && !LINF) {
         // phi(q) of this thread's row for its half of the dims (bf16 A operand of the linear
         // MMA) and the partial denominator phi(q) . z -- computed up front, while the first scores are on their way,
         // and kept in registers until the epilogue
@@ -815,9 +867,9 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           w[2 * i + 1] = gate_w(__uint_as_float(gw[i] & 0xffff0000u));
         }
       };
-      // (every attempt and every part of a split list waits for the tiles: they must have landed before the
+      // (every attempt and every part that asked for the tiles waits for them: they must have landed before the
       // barriers start over or the CTA leaves)
-      if (GT && ok) {
+      if (GT && ok && lead) {
         for (int i = 0; i < 2; ++i)
           if (p.gate_tiles & (1 << i)) ok = ok && wait_bar(&bars->k_full[1 + i], gate_uses(1 + i) & 1, bars, p.status);
         ok = __all_sync(0xffffffffu, ok);
@@ -830,7 +882,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         l_a = l;
         l = 0.f;
       }
-      if (ok && p.do_linear && epi && !LINF) {
+      if (ok && do_lin && epi && !LINF) {
         if constexpr (D == 128) {
           tmem_st32(tmem + lane_off + kColPhi + grp * 32, reinterpret_cast<uint32_t(&)[32]>(fr[0]));
         } else {
@@ -843,6 +895,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       // publish this group's partial row sum and denominator, then read the other group's
       stats[(grp * 128 + r) * 4 + 0] = l;
       stats[(grp * 128 + r) * 4 + 1] = LINF ? l_a : den_part;  // LINF: the denominator is the compressed segment's row sum
+      if (SPLIT == 2) stats[(grp * 128 + r) * 4 + 2] = t_ref;   // (in the safe pass only the first group has one)
       named_bar_sync(1, 128 * kGroups);
       float lsum = 0.f, den = 0.f;
 #pragma unroll
@@ -852,15 +905,90 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       }
       float inv_l = (nsteps > nA && lsum > 0.f) ? 1.f / lsum : 0.f;
       const bool has_o = nsteps > nA;                       // the selected pages wrote an accumulator
-      const bool has_lin = LINF ? nA > 0 : p.do_linear != 0;  // the linear branch wrote one
+      const bool has_lin = LINF ? nA > 0 : do_lin;  // the linear branch wrote one
       // Split tile: every part dumps its unnormalised accumulator with the row sums and the
       // exponent references, then takes a ticket; the part that draws the last ticket merges all of
       // them (its own included) in the epilogue below, the others write no output.  Only the attempt
       // that stands (no redo pending) takes part.
       const bool final_attempt = safe || bars->redo == 0;
       bool do_output = final_attempt;
-      float pf[SPLIT ? kFwdSplitMax : 1];  // merge factors 2^(ref_p - max ref) of the parts (split tiles only)
-      if (SPLIT && nsplit > 1 && final_attempt) {
+      float pf[kMaxParts];  // merge factors 2^(ref_p - max ref) of the parts (split tiles only)
+      if (SPLIT == 2 && nsplit > 1 && final_attempt) {
+        // The other parts leave accumulator, row sums and references in the V ring, which nothing uses any more:
+        // column groups of four outermost, then rows, so that a warp writes and reads whole lines.  The first part
+        // reads them from there, its own accumulator from TMEM.
+        float* mine = reinterpret_cast<float*>(smem + L::kV);
+        float* mine_l = mine + kTileM * D;  // row sums, then references
+        do_output = part == 0;
+        if (part > 0) {
+          if (ok) {
+#pragma unroll 1
+            for (int c0 = cbase; c0 < cbase + HC; c0 += 16) {
+              uint32_t oa[16];
+              tmem_ld16(o_tmem + c0, oa);
+              tc_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 16; i += 4)
+                *reinterpret_cast<float4*>(mine + (c0 + i) * kTileM + r * 4) =
+                    make_float4(__uint_as_float(oa[i]), __uint_as_float(oa[i + 1]), __uint_as_float(oa[i + 2]),
+                                __uint_as_float(oa[i + 3]));
+            }
+          }
+          if (grp == 0) {
+            mine_l[r] = ok ? lsum : 0.f;  // (a part that gave up counts for nothing; the status word says so)
+            mine_l[kTileM + r] = t_ref;
+          }
+        }
+        cluster_arrive();  // A
+        a_arrived = true;
+        if (part == 0) {
+          cluster_wait();
+          a_waited = true;
+          float lq[kMaxParts], rmax = -INFINITY;
+#pragma unroll
+          for (int q = 0; q < kMaxParts; ++q) {
+            lq[q] = q == 0 ? lsum : q < nsplit ? ld_cluster(mine_l + r, q) : 0.f;
+            pf[q] = q == 0 ? stats[r * 4 + 2] : q < nsplit ? ld_cluster(mine_l + kTileM + r, q) : 0.f;
+            rmax = lq[q] > 0.f ? fmaxf(rmax, pf[q]) : rmax;
+          }
+          float ltot = 0.f;
+#pragma unroll
+          for (int q = 0; q < kMaxParts; ++q) {
+            pf[q] = lq[q] > 0.f ? ex2(pf[q] - rmax) : 0.f;
+            ltot = fmaf(lq[q], pf[q], ltot);
+          }
+          inv_l = ltot > 0.f ? 1.f / ltot : 0.f;
+          if (ok) {
+            // the merged accumulator, sum of factor * partial, takes the place of the first part's: from here on the
+            // tile is one that was never split
+#pragma unroll 1
+            for (int c0 = cbase; c0 < cbase + HC; c0 += 8) {
+              uint32_t oa[8];
+              float4 v[kMaxParts][2];
+              tmem_ld8(o_tmem + c0, oa);
+#pragma unroll
+              for (int q = 1; q < kMaxParts; ++q)
+#pragma unroll
+                for (int i = 0; i < 2; ++i)
+                  v[q][i] = q < nsplit ? ld_cluster4(mine + (c0 + 4 * i) * kTileM + r * 4, q) : make_float4(0.f, 0.f, 0.f, 0.f);
+              tc_wait_ld();
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                float acc = pf[0] * __uint_as_float(oa[i]);
+#pragma unroll
+                for (int q = 1; q < kMaxParts; ++q) {
+                  const float4 x = v[q][i >> 2];
+                  if (pf[q] != 0.f) acc = fmaf(pf[q], (i & 3) == 0 ? x.x : (i & 3) == 1 ? x.y : (i & 3) == 2 ? x.z : x.w, acc);
+                }
+                oa[i] = __float_as_uint(acc);
+              }
+              tmem_st8(o_tmem + c0, oa);
+            }
+            tc_wait_st();
+          }
+        }
+      }
+      if (PARTS && nsplit > 1 && final_attempt) {
         if (ok) {
           // (column groups of four outermost, then rows: the lanes of a warp write and, at the merge, read
           // whole lines; row by row, every access of a warp touched 32 lines)
@@ -897,25 +1025,25 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           const size_t s0 = static_cast<size_t>(slot - part * slot_step) * kTileM + r;
           const size_t sq = static_cast<size_t>(slot_step) * kTileM;
           // (all of them asked for at once: one round trip, where a loop took two or three per part)
-          float lq[SPLIT ? kFwdSplitMax : 1];
+          float lq[kMaxParts];
 #pragma unroll
-          for (int q = 0; q < (SPLIT ? kFwdSplitMax : 1); ++q) {
+          for (int q = 0; q < kMaxParts; ++q) {
             lq[q] = q < nsplit ? __ldcg(&p.part_l[s0 + q * sq]) : 0.f;
             pf[q] = q < nsplit ? __ldcg(&p.part_ref[s0 + q * sq]) : 0.f;
           }
           float rmax = -INFINITY;
 #pragma unroll
-          for (int q = 0; q < (SPLIT ? kFwdSplitMax : 1); ++q) rmax = lq[q] > 0.f ? fmaxf(rmax, pf[q]) : rmax;
+          for (int q = 0; q < kMaxParts; ++q) rmax = lq[q] > 0.f ? fmaxf(rmax, pf[q]) : rmax;
           float ltot = 0.f;
 #pragma unroll
-          for (int q = 0; q < (SPLIT ? kFwdSplitMax : 1); ++q) {
+          for (int q = 0; q < kMaxParts; ++q) {
             pf[q] = lq[q] > 0.f ? ex2(pf[q] - rmax) : 0.f;
             ltot = fmaf(lq[q], pf[q], ltot);
           }
           inv_l = ltot > 0.f ? 1.f / ltot : 0.f;
         }
       }
-      if (ok && p.do_linear && epi && !LINF) {
+      if (ok && do_lin && epi && !LINF) {
         ok = __all_sync(0xffffffffu, wait_bar(&bars->lin_done, 0, bars, p.status));
         tc_fence_after();
       }
@@ -923,7 +1051,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       // branch has not looked at Q at all: its TMA load may still be in flight and must land first.
       if (ok && epi && nsteps == 0 && (!p.do_linear || LINF))
         ok = __all_sync(0xffffffffu, wait_bar(&bars->q_full, 0, bars, p.status));
-      if (!SPLIT && p.wait_late) asm volatile("griddepcontrol.wait;" ::: "memory");  // the causal partials
+      if (!PARTS && p.wait_late) asm volatile("griddepcontrol.wait;" ::: "memory");  // the causal partials
       if (ok && epi && do_output) {  // warp-uniform: the TMEM loads below are warp-collective
         const bool wr = row < p.n_q;  // rows past the end of the chunk compute but never store
         float lin_den = den;
@@ -953,7 +1081,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         // (decided from the launch parameters, not from this thread's pointers: the branch holds
         // warp-collective TMEM loads and must not diverge inside a warp)
         const bool plain = !p.g_lin && !p.g_sp && !(p.do_linear && p.lin_num != nullptr) && !p.ext_lin &&
-                           !(SPLIT && nsplit > 1);
+                           !(PARTS && nsplit > 1);
         if (plain) {
           // no gates, no causal partials, no external linear output, no merge: 32 columns per trip
           const float il = has_o ? inv_l : 0.f, id = has_lin ? inv_den : 0.f;
@@ -984,7 +1112,7 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         // CTA runs once is fetched cold: 176 us a pass against 164 with this loop, 12 heads of 128, 4680
         // tokens; value by value from global memory, which this replaces: 207.)
         const bool gated = GT && (!p.g_lin || (p.gate_tiles & 1)) && (!p.g_sp || (p.gate_tiles & 2)) &&
-                           !(p.do_linear && p.lin_num != nullptr) && !p.ext_lin && !(SPLIT && nsplit > 1);
+                           !(p.do_linear && p.lin_num != nullptr) && !p.ext_lin && !(PARTS && nsplit > 1);
         if (gated) {
           const float il = has_o ? inv_l : 0.f, id = has_lin ? inv_den : 0.f;
 #pragma unroll 1
@@ -1021,14 +1149,14 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
           uint32_t oa[16], ln[16];
 #pragma unroll
           for (int i = 0; i < 16; ++i) oa[i] = ln[i] = 0u;
-          if (SPLIT && nsplit > 1) {
+          if (PARTS && nsplit > 1) {
             // merged accumulator: sum over the parts of factor * partial, from the dumps
             float acc[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) acc[i] = 0.f;
             const float* po = p.part_o + (static_cast<size_t>(slot - part * slot_step) * (D / 4) + c0 / 4) * (kTileM * 4) + r * 4;
 #pragma unroll
-            for (int q = 0; q < (SPLIT ? kFwdSplitMax : 1); ++q) {
+            for (int q = 0; q < kMaxParts; ++q) {
               if (q < nsplit && pf[q] != 0.f) {
 #pragma unroll
                 for (int i = 0; i < 16; i += 4) {
@@ -1133,6 +1261,12 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
     }
   }
 
+  if (SPLIT == 2 && nsplit > 1) {
+    if (!a_arrived) cluster_arrive();  // (a wait that ran out: no attempt stood)
+    if (!a_waited) cluster_wait();
+    cluster_arrive();  // B
+    cluster_wait();
+  }
   if (warp == 0) {
     tc_fence_after();
     tmem_dealloc(tmem, kTmemCols);
@@ -1143,23 +1277,55 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 namespace {
 using FwdKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap,
                            CUtensorMap, FwdParams);
+// split: see the kernel
 template <int D>
-FwdKernel fwd_kernel(bool split, bool linf, bool gt) {
+FwdKernel fwd_kernel(int split, bool linf, bool gt) {
   if constexpr (D == 128) {
-    if (linf) return gt ? hsa_forward_kernel<128, false, true, true> : hsa_forward_kernel<128, false, true, false>;
+    if (linf) return gt ? hsa_forward_kernel<128, 0, true, true> : hsa_forward_kernel<128, 0, true, false>;
   }
-  if (split) return gt ? hsa_forward_kernel<D, true, false, true> : hsa_forward_kernel<D, true, false, false>;
-  return gt ? hsa_forward_kernel<D, false, false, true> : hsa_forward_kernel<D, false, false, false>;
+  if (split == 2) return gt ? hsa_forward_kernel<D, 2, false, true> : hsa_forward_kernel<D, 2, false, false>;
+  if (split == 1) return gt ? hsa_forward_kernel<D, 1, false, true> : hsa_forward_kernel<D, 1, false, false>;
+  return gt ? hsa_forward_kernel<D, 0, false, true> : hsa_forward_kernel<D, 0, false, false>;
 }
+
+// a launch of `ctas` CTAs in clusters of `cluster` (0: none), as a programmatic dependent of the kernel before it
+struct FwdLaunch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[2];
+  FwdLaunch(int D, dim3 grid, int cluster, cudaStream_t st) {
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = D == 128 ? Smem<128>::kTotal : Smem<64>::kTotal;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 0 ? 2 : 1;
+  }
+};
 }  // namespace
 
-cudaError_t forward_init() {
+cudaError_t forward_init(int D, int (&clusters)[3]) {
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < 8 && e == cudaSuccess; ++i) {
-    const bool split = i & 1, linf = (i & 2) && !split, gt = i & 4;
+    const int split = i % 4 == 3 ? 0 : i % 4;
+    const bool linf = i % 4 == 3, gt = i >= 4;
     e = cudaFuncSetAttribute(fwd_kernel<128>(split, linf, gt), cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<128>::kTotal);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(fwd_kernel<64>(split, false, gt), cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<64>::kTotal);
+  }
+  for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
+    FwdLaunch l(D, dim3(2 << k), 2 << k, nullptr);
+    const void* fn = D == 128 ? reinterpret_cast<const void*>(fwd_kernel<128>(2, false, true))
+                              : reinterpret_cast<const void*>(fwd_kernel<64>(2, false, true));
+    if (cudaOccupancyMaxActiveClusters(&clusters[k], fn, &l.cfg) != cudaSuccess) {
+      cudaGetLastError();
+      clusters[k] = 0;  // no clusters of this size on this device
+    }
   }
   return e;
 }
@@ -1171,24 +1337,15 @@ cudaError_t launch_forward(const FwdParams& p_in, int D, const CUtensorMap& tm_q
   const int n_tiles = (p_in.n_q + kTileM - 1) / kTileM;
   FwdParams p = p_in;
   p.n_tiles = n_tiles;
-  const bool split = p.max_splits > 1;
+  const int split = p.max_splits > 1 ? 1 : p.cluster > 1 ? 2 : 0;
   const bool linf = p.lf_table != nullptr;
-  if (linf && (split || D != 128 || !tm_kc || !tm_vc)) return cudaErrorInvalidValue;
+  if (linf && (split != 0 || D != 128 || !tm_kc || !tm_vc)) return cudaErrorInvalidValue;
   // One list per head and few heads: the split kernel ranks the heads itself and walks a
   // one-dimensional grid longest lists first; its balance rule makes at most nsm + H * n_tiles parts.
-  p.remap = split && p.n_groups == 1 && p.H <= 32;
-  dim3 grid(n_tiles, p.H, split ? p.max_splits : 1);
+  p.remap = split == 1 && p.n_groups == 1 && p.H <= 32;
+  dim3 grid(split == 2 ? n_tiles * p.cluster : n_tiles, p.H, split == 1 ? p.max_splits : 1);
   if (p.remap) grid = dim3(p.nsm + p.H * n_tiles);
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = grid;
-  cfg.blockDim = dim3(kThreads);
-  cfg.dynamicSmemBytes = D == 128 ? Smem<128>::kTotal : Smem<64>::kTotal;
-  cfg.stream = st;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  FwdLaunch l(D, grid, split == 2 ? p.cluster : 0, st);
   // (kernels without the compressed segment never look at the last two maps)
   const CUtensorMap& kc = linf ? *tm_kc : tm_k;
   const CUtensorMap& vc = linf ? *tm_vc : tm_v;
@@ -1197,7 +1354,7 @@ cudaError_t launch_forward(const FwdParams& p_in, int D, const CUtensorMap& tm_q
   const CUtensorMap& gl = tm_gl ? *tm_gl : tm_q;
   const CUtensorMap& gs = tm_gs ? *tm_gs : tm_q;
   const bool gt = p.gate_tiles != 0;
-  return cudaLaunchKernelEx(&cfg, D == 128 ? fwd_kernel<128>(split, linf, gt) : fwd_kernel<64>(split, false, gt), tm_q, tm_k, tm_v,
+  return cudaLaunchKernelEx(&l.cfg, D == 128 ? fwd_kernel<128>(split, linf, gt) : fwd_kernel<64>(split, false, gt), tm_q, tm_k, tm_v,
                             tm_state, tm_out, kc, vc, gl, gs, p);
 }
 

@@ -41,7 +41,6 @@ struct Layout {
   size_t status, page_table, qpart, keys, spart, lin_num, lin_den, phik, rpart, ctable, csel, ccnt, olin, ad_w, ad_idx, ad_gini, ad_wsum,
       part_o, part_l, part_ref, part_ticket, ws_total;
   int fwd_splits, split_blocks;
-  size_t part_slots;
   int phik_blocks;  // pages a chunk can touch (causal contexts with a linear state, else 0)
   // Linformer
   size_t n_cpages, cpool;
@@ -124,10 +123,8 @@ Layout make_layout(const hsa_config* c) {
   L.split_blocks += L.split_blocks & 1;  // whole two-page steps
   L.fwd_splits = (c->max_topk + L.split_blocks - 1) / L.split_blocks;
   if (L.fwd_splits > kFwdSplitMax) L.fwd_splits = kFwdSplitMax;
-  L.part_slots = L.fwd_splits > 1 ? tiles * H * L.fwd_splits
-                                  : (c->max_topk >= kFewItemsMinBlocks && c->lin_mode != HSA_LIN_LINFORMER ? kFewItemsSlots : 0);
-  if (L.part_slots > 0) {
-    const size_t slots = L.part_slots;
+  if (L.fwd_splits > 1) {
+    const size_t slots = tiles * H * static_cast<size_t>(L.fwd_splits);
     L.part_o = o;      o = align_up(o + slots * kTileM * D * 4, 256);
     L.part_l = o;      o = align_up(o + slots * kTileM * 4, 256);
     L.part_ref = o;    o = align_up(o + slots * kTileM * 4, 256);
@@ -152,6 +149,7 @@ struct hsa_ctx {
   int cur_slot;         // state slot that holds the running state of the current history
   int64_t tail_saved_for;  // history length whose tail-block key sum sits in the saved-tail buffer (-1: none)
   int nsm;
+  int clusters[3];      // clusters of 2, 4 and 8 CTAs of the forward kernel that run at once
   CUtensorMap tm_k, tm_v, tm_state, tm_kc, tm_vc, tm_olin, tm_ek, tm_ev, tm_phik;
   int32_t n_segs;  // Linformer: complete segments compressed so far
   std::vector<int32_t> page_table_host;  // history block -> physical page
@@ -289,11 +287,11 @@ int hsa_create(hsa_ctx** out, const hsa_config* cfg, const hsa_buffers* bufs,
   uint8_t* ws = static_cast<uint8_t*>(bufs->workspace);
   e = cudaMemcpy(ws + ctx->lay.page_table, pt.data(), pt.size() * 4, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemset(ws + ctx->lay.status, 0, 16);
-  if (e == cudaSuccess && ctx->lay.part_slots > 0)
+  if (e == cudaSuccess && ctx->lay.fwd_splits > 1)
     e = cudaMemset(ws + ctx->lay.part_ticket, 0, ticket_bytes(cfg));
   if (e == cudaSuccess) e = cudaMemset(bufs->state, 0, ctx->lay.state_total);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
-  if (e == cudaSuccess) e = forward_init();
+  if (e == cudaSuccess) e = forward_init(cfg->head_dim, ctx->clusters);
   if (e == cudaSuccess) e = append_init();
   if (e == cudaSuccess) e = linear_only_init();
   if (e == cudaSuccess) e = causal_linear_init();
@@ -610,31 +608,22 @@ int hsa_forward(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride, in
   p.nsm = ctx->nsm;
   p.k_pool = static_cast<const uint8_t*>(ctx->buf.k_pool);
   p.v_pool = static_cast<const uint8_t*>(ctx->buf.v_pool);
-  // Lists are split over CTAs when they may be long (the context's split_blocks), or when one list per
-  // head makes at most half as many (query tile, head) items as there are SMs: then into as many
-  // parts as fill the SMs once, if that is worth it.  A step takes 0.9 us of a part's time; dumping,
-  // merging and finding its work cost a split item 14 us and 1 us per part (head_dim 128).  Forward alone,
-  // heads x tokens x blocks: 4 x 600 x 100 48.6 -> 32.9 us, 2 x 256 x 128 57.0 -> 30.7,
-  // 4 x 2300 x 128 62.5 -> 50.9, 8 x 512 x 64 34.1 -> 30.1; not taken: 12 x 768 x 64 35.6 against 35.4,
-  // 12 x 600 x 32 21.4 against 27.2.
-  const int64_t items = static_cast<int64_t>((n_q + kTileM - 1) / kTileM) * H;
-  bool few_items = false;
-  if (ctx->lay.fwd_splits == 1 && p.n_groups == 1 && H <= 32 && 2 * items <= ctx->nsm &&
-      static_cast<size_t>(ctx->nsm + items) <= ctx->lay.part_slots) {
-    const int64_t steps = (min64(p.kcap, p.n_blocks) + 1) / 2;
-    const int64_t parts = min64(min64(kFwdSplitMax, steps / kFewItemsPart), ctx->nsm / items);
-    few_items = 9 * steps * (parts - 1) > 10 * parts * (14 + parts);
-  }
-  if (do_sparse && (ctx->lay.fwd_splits > 1 || few_items)) {
-    p.max_splits = few_items ? kFwdSplitMax : ctx->lay.fwd_splits;
+  // Lists are split over CTAs when they may be long (the context's split_blocks), through the workspace, or, without
+  // it, when there are so few (query tile, head) items that clusters of 2, 4 or 8 CTAs, one per item, all run at
+  // once and a list can be long enough for it (the lists themselves are not known here: where they are short
+  // for all that, the clusters cost 0.3 us, those of 2 0.8, in a call of 11).
+  if (do_sparse && ctx->lay.fwd_splits > 1) {
+    p.max_splits = ctx->lay.fwd_splits;
     p.split_blocks = ctx->lay.split_blocks;
-    p.min_part_steps = few_items ? kFewItemsPart : 16;
-    // (a list's parts are rounded up, by less than one per item: these SMs make one wave of it)
-    p.balance_sms = few_items ? ctx->nsm - static_cast<int>(items) : ctx->nsm;
     p.part_o = reinterpret_cast<float*>(ws + ctx->lay.part_o);
     p.part_l = reinterpret_cast<float*>(ws + ctx->lay.part_l);
     p.part_ref = reinterpret_cast<float*>(ws + ctx->lay.part_ref);
     p.part_ticket = reinterpret_cast<int32_t*>(ws + ctx->lay.part_ticket);
+  } else if (do_sparse && !do_linformer && p.n_groups == 1) {
+    const int64_t items = static_cast<int64_t>((n_q + kTileM - 1) / kTileM) * H;
+    const int steps = static_cast<int>((min64(p.kcap, p.n_blocks) + 1) / 2);
+    for (int lg = 3; lg >= 1 && p.cluster == 0; --lg)
+      if (items <= ctx->clusters[lg - 1] && cluster_parts_log2(1 << lg, steps) > 0) p.cluster = 1 << lg;
   }
   if (causal_lin) {
     CausalLinArgs c{};
@@ -867,7 +856,7 @@ int hsa_device_status(hsa_ctx* ctx, int32_t* status_out) {
   // its arrive count behind: both of its words start over.  A part of a split list that gave up has drawn no
   // ticket, which leaves its list's counter short: they start over too.
   if (e == cudaSuccess && v != 0) e = cudaMemset(ws + ctx->lay.status + 8, 0, 8);
-  if (e == cudaSuccess && v != 0 && ctx->lay.part_slots > 0) e = cudaMemset(ws + ctx->lay.part_ticket, 0, ticket_bytes(&ctx->cfg));
+  if (e == cudaSuccess && v != 0 && ctx->lay.fwd_splits > 1) e = cudaMemset(ws + ctx->lay.part_ticket, 0, ticket_bytes(&ctx->cfg));
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   *status_out = v;
   return HSA_OK;

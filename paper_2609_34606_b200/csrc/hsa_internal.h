@@ -15,13 +15,19 @@ constexpr int kStateSplitMax = 16;       // token-axis splits of the state updat
 // the bf16 rounding of z, row 1 the bf16 rounding of the remainder, rows 2..15 are zero, so that
 // phi(Q) times it gives the denominator phi(q).z as the sum of two accumulator columns
 constexpr int kZopBytes = 4096;
-// partial-result slots of a context whose lists are too short to be split for their length: enough for a
-// launch that has at most half as many (query tile, head) items as the GPU has SMs (see hsa_forward)
-constexpr int kFewItemsSlots = 240;
-constexpr int kFewItemsMinBlocks = 48;   // shorter lists are not split for that
-constexpr int kFewItemsPart = 8;         // shortest part of such a launch, in two-page steps
+constexpr int kClusterParts = 8;         // CTAs of a cluster that a list of a launch with few items is split over
 constexpr int kPhiTerms = 3;             // bf16 terms of phi(K) for the causal products: 24 bits
 constexpr int kFwdSplitMax = 16;         // CTAs a long (query tile, head) of the forward kernel is split over
+
+// Parts (their log2) that a list of `steps` two-page steps is cut into by a cluster of 2, 4 or 8 CTAs.  A step takes
+// 0.74 us; meeting, dumping and merging cost 6 us and 0.5 us per part (head_dim 128; less at 64).  Forward alone,
+// heads x tokens x blocks, whole -> parts: 2 x 256 x 128 55.5 -> 24.0 us (8 parts), 4 x 600 x 128 55.7 -> 27.4 (4),
+// 4 x 600 x 32 19.8 -> 18.0, 4 x 2300 x 128 56.7 -> 39.8 (2), 12 x 768 x 64 32.7 -> 27.5; not taken: 4 x 600 x
+// 20 15.3 against 18.1, 12 x 768 x 32 20.6 against 22.2.
+__host__ __device__ inline int cluster_parts_log2(int cluster, int steps) {
+  if (cluster == 2) return steps >= 20 ? 1 : 0;
+  return cluster < 4 || steps < 16 ? 0 : cluster >= 8 && steps >= 24 ? 3 : 2;
+}
 
 __host__ __device__ inline int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
 __host__ __device__ inline int64_t max64(int64_t a, int64_t b) { return a > b ? a : b; }
@@ -142,8 +148,7 @@ struct FwdParams {
   // (grid z = max_splits); each dumps its unnormalised O, row sums and exponent references, the last
   // one to take a ticket merges them and writes the output
   int max_splits, split_blocks;
-  int min_part_steps;    // shortest part of the balance rule, in two-page steps
-  int balance_sms;       // SMs the balance rule spreads the steps over
+  int cluster;           // > 1 (max_splits 1): each (query tile, head) is a cluster of that many CTAs
   int n_tiles, remap;    // set by the launcher: query tiles; 1 = one-dimensional grid, longest lists first
   int nsm;               // SMs of the device (the split rule balances the launch over them)
   float* part_o;         // [slots][D / 4][128][4]: slot (tile H + h) max_splits + part, or the CTA's number (remap)
@@ -223,7 +228,8 @@ cudaError_t causal_linear_init();
 cudaError_t launch_linear_only(const FwdParams& p, int nsm, const CUtensorMap& tm_q, const CUtensorMap& tm_state,
                                const CUtensorMap& tm_out, cudaStream_t st);
 cudaError_t linear_only_init();
-cudaError_t forward_init();
+// clusters: how many clusters of 2, 4 and 8 CTAs of the forward kernel the device runs at once
+cudaError_t forward_init(int D, int (&clusters)[3]);
 cudaError_t append_init();  // opt in to the shared-memory size the fused append kernel needs
 
 }  // namespace hsa

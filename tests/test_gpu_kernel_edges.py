@@ -409,14 +409,14 @@ def test_lists_of_few_items_split_over_ctas(d, H, n_q, budgets, gates, causal, c
     ctx.destroy()
 
 
-@pytest.mark.parametrize("split_blocks,code", [(4, -5), (4, -6), (0, -5)])
-def test_counters_of_split_lists_start_over_with_the_status_word(split_blocks, code, cuda_device):
+@pytest.mark.parametrize("code", [-5, -6])
+def test_counters_of_split_lists_start_over_with_the_status_word(code, cuda_device):
     """A part of a split list that gives up draws no ticket; reading the status word puts the counters back (written
     here by the host, as such a launch leaves them), so that the next launch merges all of its parts."""
     from paper_2609_34606_b200 import hsa
     H, d, n, n_q = 2, 128, 130 * 64, 200
     g = torch.Generator().manual_seed(3)
-    ctx = hsa.HSAContext(H, d, max_pages=130, max_q_tokens=n, max_topk=128, device=cuda_device, split_blocks=split_blocks)
+    ctx = hsa.HSAContext(H, d, max_pages=130, max_q_tokens=n, max_topk=128, device=cuda_device, split_blocks=4)
     ctx.append_kv(_randn(g, n, H, d).to(cuda_device), _randn(g, n, H, d).to(cuda_device))
     q = _randn(g, n_q, H, d).to(cuda_device)
     idx, cnt = ctx.select_blocks(q, torch.full((H,), 128, dtype=torch.int32, device=cuda_device))
@@ -432,4 +432,90 @@ def test_counters_of_split_lists_start_over_with_the_status_word(split_blocks, c
     assert words[end:end + tickets].abs().sum().item() == 0
     out = ctx.forward(q, idx, cnt)
     assert ctx.device_status() == 0 and torch.equal(out, want)
+    ctx.destroy()
+
+
+def test_forwards_of_short_lists_on_two_streams(cuda_device):
+    """Forwards of one context with few items that run at the same time on two streams do not disturb each other."""
+    from paper_2609_34606_b200 import hsa
+    H, d, n, n_q = 2, 128, 130 * 64, 256
+    g = torch.Generator().manual_seed(9)
+    ctx = hsa.HSAContext(H, d, max_pages=130, max_q_tokens=n, max_topk=128, device=cuda_device)
+    ctx.append_kv(_randn(g, n, H, d).to(cuda_device), _randn(g, n, H, d).to(cuda_device))
+    q = [_randn(g, n_q, H, d).to(cuda_device) for _ in range(2)]
+    idx, cnt = ctx.select_blocks(q[0], torch.full((H,), 128, dtype=torch.int32, device=cuda_device))
+    streams = [torch.cuda.Stream(cuda_device) for _ in range(2)]
+    torch.cuda.synchronize()
+
+    def run(i, out):
+        with torch.cuda.stream(streams[i]):
+            ctx.forward(q[i], idx, cnt, out=out)
+
+    want = [torch.empty_like(x) for x in q]
+    for i in range(2):  # one after the other
+        run(i, want[i])
+        torch.cuda.synchronize()
+    outs = [[torch.empty_like(x) for _ in range(20)] for x in q]
+    for k in range(20):
+        for i in range(2):
+            run(i, outs[i][k])
+    torch.cuda.synchronize()
+    assert ctx.device_status() == 0
+    assert all(torch.equal(o, want[i]) for i in range(2) for o in outs[i])
+    ctx.destroy()
+
+
+@pytest.mark.parametrize("d,H,n_q,cnt,gates", [(128, 2, 100, (128, 7), ""), (64, 1, 1, (128,), "head"), (128, 1, 128, (24,), "dim"),
+                                               (128, 4, 600, (9, 127, 16, 0), ""), (64, 16, 200, (64,) * 16, "dim")])
+def test_lists_of_few_items_against_64_bits(d, H, n_q, cnt, gates, cuda_device):
+    """Lists split over the CTAs of a cluster (2, 4 and 8 of them; lists too short for as many parts, or for any)
+    against the oracle on the same lists."""
+    from paper_2609_34606_b200 import hsa
+    n = 130 * 64 - 11
+    g = torch.Generator().manual_seed(n_q + d)
+    K, V, q = _randn(g, n, H, d), _randn(g, n, H, d), _randn(g, n_q, H, d)
+    ctx = hsa.HSAContext(H, d, max_pages=130, max_q_tokens=n, max_topk=128, device=cuda_device)
+    ctx.append_kv(K.to(cuda_device), V.to(cuda_device))
+    qd = q.to(cuda_device)
+    idx, num = ctx.select_blocks(qd, torch.tensor(cnt, dtype=torch.int32, device=cuda_device))
+    gl = gs = gl_n = gs_n = None
+    if gates:
+        shape = (n_q, H, d) if gates == "dim" else (n_q, H)
+        gl, gs = _randn(g, *shape), _randn(g, *shape)
+        gl_n, gs_n = Hn.f64(gl), Hn.f64(gs)
+        gl, gs = gl.to(cuda_device), gs.to(cuda_device)
+    out = ctx.forward(qd, idx, num, g_lin=gl, g_sp=gs)
+    assert ctx.device_status() == 0
+    rows = sorted({0, n_q // 2, n_q - 1})
+    ref = O.hsa_forward(Hn.f32(q), Hn.f32(K), Hn.f32(V), n, False, Hn.selection_lists(idx, num), 0, gl_n, gs_n, 0, rows=rows)["out"]
+    got = Hn.f64(out)[rows]
+    ref = ref[rows]
+    # bf16 weights (2^-9 each, of random sign) and phi(q), and one rounding of the result
+    assert np.linalg.norm(got - ref) <= 1.5 * BF16_REL * np.linalg.norm(ref)
+    ctx.destroy()
+
+
+@pytest.mark.parametrize("hot", [6, 60, 98])
+@pytest.mark.parametrize("d,causal", [(128, False), (64, False), (128, True)])
+def test_safe_pass_of_lists_split_over_a_cluster(d, causal, hot, cuda_device):
+    """Later blocks that outscore the first by far, in one part of a list only (the merging one, one in the middle, the
+    last): that part is done again with a running maximum, the others are not, and the parts merge."""
+    from paper_2609_34606_b200 import hsa
+    H, n_q, n = 2, 150, 100 * 64
+    g = torch.Generator().manual_seed(d)
+    K, V, q = _randn(g, n, H, d), _randn(g, n, H, d), _randn(g, n_q, H, d)
+    K[hot * 64:(hot + 2) * 64] *= 24   # scores up to some 24 * 4 * sqrt(d) / sqrt(d) above the others
+    q = q * 4
+    ctx = hsa.HSAContext(H, d, max_pages=100, max_q_tokens=n, max_topk=100, device=cuda_device, causal=causal)
+    n0 = n - n_q
+    ctx.append_kv(K[:n0].to(cuda_device), V[:n0].to(cuda_device))
+    ctx.append_kv(K[n0:].to(cuda_device), V[n0:].to(cuda_device))
+    qd, pos = q.to(cuda_device), n0 if causal else n
+    idx, cnt = ctx.select_blocks(qd, torch.full((H,), -1, dtype=torch.int32, device=cuda_device), q_pos0=pos, causal=causal)
+    out = ctx.forward(qd, idx, cnt, q_pos0=pos, causal=causal, flags=hsa.HSA_FWD_NO_LINEAR)
+    redone = ctx.safe_pass_tiles()
+    assert ctx.device_status() == 0 and 0 < redone <= 4 * 2
+    ref = O.dense_attention(Hn.f32(q), Hn.f32(K), Hn.f32(V), pos, causal)
+    # (peaked rows: a weight is one bf16 rounding, and so is the result)
+    assert np.linalg.norm(Hn.f64(out) - ref) <= 2 * BF16_REL * np.linalg.norm(ref)
     ctx.destroy()

@@ -92,3 +92,27 @@ def test_selection_on_every_device_of_a_process(lib, d, n_blocks, adaptive):
             assert (ctx.select_adaptive(n_q) if adaptive else ctx.select(n_q)) == 0
             names = [l[0] for l in launches(lib)]
             assert names and all(l[3] == dev for l in launches(lib)) and "select_cluster" in names[-1]
+
+
+def test_forwards_of_short_lists_share_no_scratch(lib):
+    """Two forwards of one context may run at the same time if their lists are short: they are not split through
+    the workspace, which holds nothing for that, and take the same route on every stream and under capture."""
+    workspace, cluster, plain = ("hsa_forward_kernelILi128ELi%dE" % i for i in (1, 2, 0))
+
+    def kernel(ctx, n_q, stream=0):
+        lib.fake_reset()
+        assert ctx.forward(n_q, stream) == 0
+        (name, grid, _, _), = launches(lib)
+        return next(k for k in (workspace, cluster, plain) if k in name), grid
+
+    ctx = Context(lib, 2, 128, 130, 128, n=130 * 64)
+    routes = [kernel(ctx, 256, s) for s in (0, 0x70, 0)]
+    lib.fake_set_capturing(0x70, 1)
+    routes.append(kernel(ctx, 256, 0x70))
+    assert set(routes) == {(cluster, (2 * 8, 2, 1))}
+    assert kernel(ctx, 4680) == (plain, (37, 2, 1))
+    assert kernel(Context(lib, 2, 128, 20, 20, n=20 * 64), 256)[0] == plain      # never long enough
+    assert kernel(Context(lib, 2, 128, 300, 300, n=300 * 64), 256)[0] == workspace
+    from paper_2609_34606_b200 import hsa
+    sizes = {hsa.hsa_query_sizes(hsa.hsa_config(2, 128, 64, 300, 4680, k, 1, 0, 0.0, 0)).workspace for k in (1, 47, 48, 256)}
+    assert len(sizes) == 1
