@@ -357,7 +357,7 @@ class HSAContext:
         v = self._slots.get(off)
         if v is None:
             v = self._slots[off] = self._view(off, shape)
-        return v
+        return v.detach()  # (a tensor of the caller's own: what is done to its shape or flags stays with it)
 
     @property
     def S(self) -> torch.Tensor:
@@ -374,7 +374,7 @@ class HSAContext:
 
     @property
     def ksum(self) -> torch.Tensor:
-        return self._ksum
+        return self._ksum.detach()
 
     @property
     def n_tokens(self) -> int:

@@ -519,3 +519,17 @@ def test_safe_pass_of_lists_split_over_a_cluster(d, causal, hot, cuda_device):
     # (peaked rows: a weight is one bf16 rounding, and so is the result)
     assert np.linalg.norm(Hn.f64(out) - ref) <= 2 * BF16_REL * np.linalg.norm(ref)
     ctx.destroy()
+
+
+def test_state_views_are_the_callers_own(cuda_device):
+    """What a caller does to the shape or the flags of a state view stays with that view; the memory is shared."""
+    from paper_2609_34606_b200 import hsa
+    ctx = hsa.HSAContext(2, 64, max_pages=4, max_q_tokens=128, max_topk=4, device=cuda_device)
+    x = torch.randn(100, 2, 64, device=cuda_device).to(torch.bfloat16)
+    ctx.append_kv(x, x)
+    for name, shape in (("S", (2, 64, 64)), ("z", (2, 64)), ("ksum", (2, 4, 64))):
+        view = getattr(ctx, name)
+        view.unsqueeze_(0).requires_grad_()
+        again = getattr(ctx, name)
+        assert tuple(again.shape) == shape and not again.requires_grad and again.data_ptr() == view.data_ptr()
+    ctx.destroy()
