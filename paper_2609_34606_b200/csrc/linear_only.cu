@@ -302,7 +302,7 @@ hsa_linear_only_kernel(FwdParams p, int n_items, const __grid_constant__ CUtenso
           const float inv_den = RELU ? 1.f / (den + 1e-6f) : (den > 0.f ? 1.f / den : 0.f);
           const __nv_bfloat16* gl =
               (wr && p.g_lin) ? p.g_lin + static_cast<size_t>(row) * p.g_ts + static_cast<size_t>(h) * p.g_hs : nullptr;
-          const int g_ds = static_cast<int>(p.g_ds);
+          const int64_t g_ds = p.g_ds;
 #pragma unroll
           for (int i = 0; i < 32; i += 2) {
             float w0 = inv_den, w1 = inv_den, l0 = 0.f, l1 = 0.f;

@@ -533,3 +533,25 @@ def test_state_views_are_the_callers_own(cuda_device):
         again = getattr(ctx, name)
         assert tuple(again.shape) == shape and not again.requires_grad and again.data_ptr() == view.data_ptr()
     ctx.destroy()
+
+
+@pytest.mark.parametrize("flags", [1, 2, 0])
+def test_gates_with_a_dim_stride_beyond_32_bits(flags, cuda_device):
+    """Per-dim gates whose dims lie 2^24 and more elements apart: offsets inside a row need 64 bits, in the kernel of
+    both branches and in the one of the linear branch alone."""
+    from paper_2609_34606_b200 import hsa
+    H, d, n = 2, 128, 130
+    step = (1 << 24) + (1 << 18)
+    g = torch.Generator().manual_seed(flags)
+    ctx = hsa.HSAContext(H, d, max_pages=3, max_q_tokens=n, max_topk=3, device=cuda_device)
+    x, q = _randn(g, n, H, d).to(cuda_device), _randn(g, n, H, d).to(cuda_device)
+    ctx.append_kv(x, x)
+    idx, cnt = ctx.select_blocks(q, torch.full((H,), -1, dtype=torch.int32, device=cuda_device))
+    near = _randn(g, n, H, d).to(cuda_device)
+    far = torch.empty((d - 1) * step + n * H, dtype=torch.bfloat16, device=cuda_device).as_strided((n, H, d), (H, 1, step))
+    far.copy_(near)
+    want = ctx.forward(q, idx, cnt, g_lin=near, g_sp=near, flags=flags)
+    out = ctx.forward(q, idx, cnt, g_lin=far, g_sp=far, flags=flags)
+    assert ctx.device_status() == 0
+    assert float((out.double() - want.double()).norm()) <= BF16_REL * float(want.double().norm())
+    ctx.destroy()
