@@ -555,3 +555,50 @@ def test_gates_with_a_dim_stride_beyond_32_bits(flags, cuda_device):
     assert ctx.device_status() == 0
     assert float((out.double() - want.double()).norm()) <= BF16_REL * float(want.double().norm())
     ctx.destroy()
+
+
+@pytest.mark.parametrize("hot", [False, True])
+@pytest.mark.parametrize("form", ["plain", "causal", "linformer", "workspace", "cluster", "causal cluster"])
+@pytest.mark.parametrize("d", [64, 128])
+def test_gate_tiles_in_every_instance(d, form, hot, cuda_device):
+    """Per-dim gates as tiles in each instance of the forward kernel, beside causal partials, in merged lists and in
+    tiles that are done again with a running maximum: against the merge of the branches as the same kernel gives
+    them without gates."""
+    from paper_2609_34606_b200 import hsa
+    if form == "linformer" and d == 64:
+        pytest.skip("the Linformer form has head_dim 128")
+    H, n, causal = 3, 60 * 64, "causal" in form
+    n_q = 150 if "cluster" in form else 300
+    g = torch.Generator().manual_seed(d + len(form))
+    rand = lambda *s: _randn(g, *s).to(cuda_device)
+    opt = {}
+    if form == "linformer":
+        opt = dict(lin_mode=hsa.HSA_LIN_LINFORMER, lin_rank=64, lin_seg_tokens=n, e_k=rand(H, n, 64) * 0.02, e_v=rand(H, n, 64) * 0.02)
+    budget = 10 if form in ("plain", "causal") else 50
+    ctx = hsa.HSAContext(H, d, max_pages=60, max_q_tokens=n, max_topk=budget, device=cuda_device, gate_act=1, causal=causal,
+                         split_blocks=16 if form == "workspace" else 0, **opt)
+    K, V, q = rand(n, H, d), rand(n, H, d), rand(n_q, H, d)
+    if hot:
+        K[20 * 64:22 * 64] *= 24
+        q *= 4
+    n0 = n - n_q if causal else 0
+    for lo, hi in ((0, n0), (n0, n)):
+        if hi > lo:
+            ctx.append_kv(K[lo:hi], V[lo:hi])
+    pos = n0 if causal else n
+    # lists that hold the outscoring blocks, behind ordinary ones
+    idx, cnt = ctx.alloc_selection(n_q)
+    idx[:, 0] = torch.arange(60 - budget, 60) if budget < 50 and not hot else torch.arange(budget) + (14 if budget < 50 else 0)
+    cnt.fill_(budget)
+    gl, gs = rand(n_q, H, d), rand(n_q, H, d)
+    run = lambda **kw: ctx.forward(q, idx, cnt, q_pos0=pos, causal=causal, **kw).double()
+    ctx.safe_pass_tiles()
+    out = run(g_lin=gl, g_sp=gs)
+    assert (ctx.safe_pass_tiles() > 0) == hot
+    lin, sp = run(flags=hsa.HSA_FWD_NO_SPARSE), run(flags=hsa.HSA_FWD_NO_LINEAR)
+    assert ctx.device_status() == 0
+    a, b = torch.sigmoid(gl.double()) * lin, torch.sigmoid(gs.double()) * sp
+    # each branch and the result are rounded once, and a branch alone may take its exponent references from other
+    # keys, so that its bf16 weights round differently (2^-9 each, of random sign, of a sum of many)
+    assert float((out - a - b).norm()) <= 1.5 * BF16_REL * float((a + b).norm())
+    ctx.destroy()
