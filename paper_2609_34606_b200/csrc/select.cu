@@ -27,10 +27,10 @@ __device__ __forceinline__ void blk_sync(const Blk& blk) {
 }
 
 // ---------------------------------------------------------------------------------------
-// Stage 1: column sums of q over one 128-token tile and one head -> qpart[tile][h][D].
+// Stage 1: column sums of q over one 128-token tile and one head -> store(dim, sum).
 // ---------------------------------------------------------------------------------------
-template <int D>
-__device__ __forceinline__ void qsum_item(const Blk& blk, const SelectArgs& a, int tile, int h, float (*red)[D]) {
+template <int D, class Store>
+__device__ __forceinline__ void qsum_item(const Blk& blk, const SelectArgs& a, int tile, int h, float (*red)[D], Store store) {
   constexpr int CH = D / 8;
   constexpr int RP = 256 / CH;
   const int c8 = blk.tid % CH, rg = blk.tid / CH;
@@ -66,8 +66,12 @@ __device__ __forceinline__ void qsum_item(const Blk& blk, const SelectArgs& a, i
     float s = 0.f;
 #pragma unroll
     for (int r = 0; r < RP; ++r) s += red[r][blk.tid];
-    a.qpart[(static_cast<size_t>(tile) * a.H + h) * D + blk.tid] = s;
+    store(blk.tid, s);
   }
+}
+template <int D>
+__device__ __forceinline__ void qsum_item(const Blk& blk, const SelectArgs& a, int tile, int h, float (*red)[D]) {
+  qsum_item<D>(blk, a, tile, h, red, [&](int e, float s) { a.qpart[(static_cast<size_t>(tile) * a.H + h) * D + e] = s; });
 }
 
 template <int D>
@@ -992,12 +996,22 @@ __device__ __forceinline__ void adaptive_list(const SelectArgs& a, const Adaptiv
   }
 }
 
+constexpr int kClusterCtas = 8;  // the portable maximum
+// The query tile sums are taken inside the clusters while every sub-block gets at most one tile (24 of
+// 128 tokens): one launch instead of two.  Longer chunks want every SM for them, 96 of 148 are in a
+// cluster at 12 heads.  Selection alone, two launches against one, heads x tokens: 2 x 256 7.5 against 7.7 us, 16 x
+// 128 10.6 against 11.0, 8 x 1024 8.0 against 8.5, 12 x 1560 8.5 against 8.3, 12 x 3000 9.1 against 8.4; and
+// the caller needs 6.0 against 3.6 us to issue it.
+constexpr int kOwnQueryTiles = kClusterCtas * kSubBlocks;
+
 template <int D>
 struct ClusterSmem {
   // per sub-block: partial column sums of a query tile (fp32 [256 / (D / 8)][D]); together: mean query [D]
   // and partial sums [768 / D][D], fp64
   static constexpr int kScratch = 8192;
-  static constexpr int kFixed = (kSubBlocks * kScratch + static_cast<int>(sizeof(TopkShared)) + 15) / 16 * 16;
+  static constexpr int kTileSums = (kSubBlocks * kScratch + static_cast<int>(sizeof(TopkShared)) + 15) / 16 * 16;
+  // OWN_Q: the head's query tile sums, fp32 [kOwnQueryTiles][D], in every CTA of the cluster
+  __host__ __device__ static constexpr int fixed(bool own_q) { return kTileSums + (own_q ? kOwnQueryTiles * D * 4 : 0); }
 };
 
 // OWN_Q: the query tile sums are taken here as well, a tile per sub-block, instead of by the kernel in front
@@ -1011,7 +1025,8 @@ __global__ void __launch_bounds__(256 * kSubBlocks, 1) select_cluster_kernel(Sel
   const int sub = static_cast<int>(threadIdx.x) / 256;
   const Blk blk{static_cast<int>(threadIdx.x) % 256, 1 + sub};
   TopkShared* sh_all = reinterpret_cast<TopkShared*>(cl_smem + kSubBlocks * kScratch);
-  uint32_t* cl_keys = reinterpret_cast<uint32_t*>(cl_smem + ClusterSmem<D>::kFixed);
+  uint32_t* cl_keys = reinterpret_cast<uint32_t*>(cl_smem + ClusterSmem<D>::fixed(OWN_Q));
+  float* tile_sums = reinterpret_cast<float*>(cl_smem + ClusterSmem<D>::kTileSums);
   const int h = static_cast<int>(blockIdx.x) / cluster_ctas;
   const int slot = (static_cast<int>(blockIdx.x) % cluster_ctas) * kSubBlocks + sub;
   const int n_slots = cluster_ctas * kSubBlocks;
@@ -1031,12 +1046,24 @@ __global__ void __launch_bounds__(256 * kSubBlocks, 1) select_cluster_kernel(Sel
   if (OWN_Q) {
     if (slot < n_chunks) scores_load<D, MIXED>(blk, a, slot, h, op);
     const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
+    // a tile's sums go to every CTA of the cluster (through global memory they arrived 0.4 to 1.5 us later)
+    const uint32_t sums_addr = static_cast<uint32_t>(__cvta_generic_to_shared(tile_sums));
+    bool running = false;
     for (int tile = slot; tile < n_tiles; tile += n_slots) {
-      qsum_item<D>(blk, a, tile, h, reinterpret_cast<float(*)[D]>(cl_smem + sub * kScratch));
+      qsum_item<D>(blk, a, tile, h, reinterpret_cast<float(*)[D]>(cl_smem + sub * kScratch), [&](int e, float s) {
+        if (!running) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");  // every CTA of the cluster is running
+        running = true;
+        for (int r = 0; r < cluster_ctas; ++r) {
+          uint32_t addr;
+          asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(sums_addr + static_cast<uint32_t>(tile * D + e) * 4u), "r"(r));
+          asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(s) : "memory");
+        }
+      });
       blk_sync(blk);
     }
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every CTA of the cluster is running
-    cluster_sync_all();  // and the head's tile sums are written
+    if (!running) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    __syncwarp();
+    cluster_sync_all();  // and the head's tile sums are complete
   }
   // The head's mean query, once per CTA: all 768 threads add up the tile sums (a column's partials
   // split over 768 / D ways, every load of a thread in flight at once, fp64, fixed order), then one
@@ -1052,7 +1079,9 @@ __global__ void __launch_bounds__(256 * kSubBlocks, 1) select_cluster_kernel(Sel
       float v[kInFlight];
 #pragma unroll
       for (int i = 0; i < kInFlight; ++i)
-        v[i] = (t0 + i * WAYS < n_tiles) ? __ldcg(&a.qpart[(static_cast<size_t>(t0 + i * WAYS) * a.H + h) * D + col]) : 0.f;
+        v[i] = (t0 + i * WAYS >= n_tiles) ? 0.f
+               : OWN_Q                      ? tile_sums[(t0 + i * WAYS) * D + col]
+                                            : __ldcg(&a.qpart[(static_cast<size_t>(t0 + i * WAYS) * a.H + h) * D + col]);
 #pragma unroll
       for (int i = 0; i < kInFlight; ++i) sum += static_cast<double>(v[i]);
     }
@@ -1084,7 +1113,7 @@ __global__ void __launch_bounds__(256 * kSubBlocks, 1) select_cluster_kernel(Sel
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if constexpr (ADAPT) {
     if (slot < kSubBlocks)  // the cluster's first CTA
-      adaptive_list(a, ad, h, cl_keys, reinterpret_cast<unsigned long long*>(cl_smem + ClusterSmem<D>::kFixed + adaptive_key_bytes(a)),
+      adaptive_list(a, ad, h, cl_keys, reinterpret_cast<unsigned long long*>(cl_smem + ClusterSmem<D>::fixed(OWN_Q) + adaptive_key_bytes(a)),
                     reinterpret_cast<AdaptiveShared*>(cl_smem));
   } else {
     if (slot == 0) topk_item<MIXED>(blk, a, 0, h, cl_keys, sh_all, budget, intra_budget, true);
@@ -1124,7 +1153,7 @@ namespace {
 // Cluster size (8 CTAs, the portable maximum) if the cluster form can be launched on this device for
 // the given instance and shared-memory size, else 0.
 int cluster_size_for(const void* fn, size_t smem, int threads) {
-  const int cs = 8;
+  const int cs = kClusterCtas;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(cs);
   cfg.blockDim = dim3(threads);
@@ -1179,14 +1208,7 @@ cudaError_t launch_qsum(const SelectArgs& a, cudaStream_t st) {
 }
 
 namespace {
-// Cluster form of the selection, if this call and this device allow it (-1 in *done_as: not launched).
 constexpr int kClusterMaxChunks = 192;
-// The query tile sums are taken inside the clusters while every sub-block gets at most one tile (24 of
-// 128 tokens): one launch instead of two.  Longer chunks want every SM for them, 96 of 148 are in a
-// cluster at 12 heads.  Measured: 12.6 against 12.7 us of kernels for 8 tiles x 16 heads of 64, 10.4 against
-// 10.0 for 13 tiles x 12 heads of 128, and 3.6 against 6.0 us of the caller's time to issue the call.
-constexpr int kOwnQueryTiles = 8 * kSubBlocks;
-
 template <int D>
 const void* cluster_kernel(bool mixed, bool own, bool adapt) {
   if (adapt)
@@ -1204,7 +1226,9 @@ bool launch_cluster(const SelectArgs& a, const AdaptiveArgs* ad, bool mixed, cud
   const int64_t nblk = (a.n_tokens + kBlock - 1) / kBlock;
   const int64_t n_chunks = (nblk + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta;
   if (a.n_groups != 1 || n_chunks > kClusterMaxChunks) return false;
-  size_t smem = a.D == 128 ? ClusterSmem<128>::kFixed : ClusterSmem<64>::kFixed;
+  const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
+  const bool own = n_tiles <= kOwnQueryTiles;
+  size_t smem = a.D == 128 ? ClusterSmem<128>::fixed(own) : ClusterSmem<64>::fixed(own);
   if (ad) {
     size_t np2 = 32;
     while (static_cast<int64_t>(np2) < nblk) np2 <<= 1;
@@ -1212,12 +1236,10 @@ bool launch_cluster(const SelectArgs& a, const AdaptiveArgs* ad, bool mixed, cud
   } else {
     smem += static_cast<size_t>(nblk > 0 ? nblk : 1) * sizeof(uint32_t);
   }
-  const int n_tiles = (a.n_q + kTileM - 1) / kTileM;
-  const bool own = n_tiles <= kOwnQueryTiles;
   const void* fn = a.D == 128 ? cluster_kernel<128>(mixed, own, ad != nullptr) : cluster_kernel<64>(mixed, own, ad != nullptr);
   // the cluster size is looked up, and the shared-memory limit set, once per instance and device, for the
   // largest size the form is used with (a cluster that fits with that fits with less)
-  constexpr size_t kMaxSmem = 120 * 1024;
+  constexpr size_t kMaxSmem = 132 * 1024;
   if (smem > kMaxSmem) return false;
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return false;
