@@ -463,7 +463,7 @@ def bench_ours(args, rank: int, world: int):
             # (the Linformer form has as many: page write + projection instead of the fused append and
             # its reduction, one forward launch that walks the compressed pool before the selected pages)
             "device_status": status,
-            "roofline": {"kernel": "hsa_forward_kernel<128, false>", "bound": "tensor", "achieved": fwd_tf,
+            "roofline": {"kernel": "hsa_forward_kernel<128, 0, false, false>", "bound": "tensor", "achieved": fwd_tf,
                          "peak": peaks["bf16_tflops"], "unit": "TFLOP/s", "frac": fwd_tf / peaks["bf16_tflops"],
                          "traffic": ncu_traffic(w.name), "algorithmic_bytes": by["forward"],
                          "peak_source": peaks["source"] + " (burst)",

@@ -173,6 +173,9 @@ __global__ void state_reduce_kernel(AppendArgs a) {
 // Error against 64 bits, the fp32 SIMT kernels this replaced -> now (2-norm, N(0, 1) inputs): 16 heads, 1000
 // tokens, S 1.6e-7 -> 7.8e-8, z 7.4e-8 -> 5.1e-8; 40 heads, 4680 tokens, S 5.8e-7 -> 2.9e-7, z 4.9e-7 ->
 // 3.4e-8; with one accumulator per two blocks S was 8.4e-8 and 6.3e-7.
+// Measured, the whole append replayed from a graph: 16 heads, 1000 tokens 13.6 -> 7.6 us (the 8.3 MB take 1.3 us at
+// the copy bandwidth: what is left is latency, of launch, first data and two kernels), 8 heads, 4680 tokens
+// 26.2 -> 11.5 us.
 // Every wait is bounded; on expiry the CTA records a timeout and leaves.
 // ---------------------------------------------------------------------------------------
 

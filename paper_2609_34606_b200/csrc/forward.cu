@@ -192,9 +192,9 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   // AHEAD: a step's bookkeeping before the wait for its scores (350 cycles that came after it), and the
   // issuing lane's barriers looked at while P V runs (a barrier costs some 100 cycles to ask even if it is
   // complete: shared memory is the busiest unit of this loop, 160 KB per step at 128 B per clock).  With
-  // two score buffers this shortens the chain that bounds the loop: Linformer pass 245.4 -> 236.5 us; long
-  // split lists 418.8 -> 415.4.  With three buffers and short lists it does not pay: 64 blocks 152.5 against
-  // 153.2, 128 blocks 272.6 against 270.2.
+  // two score buffers this shortens the chain that bounds the loop: Linformer pass 247 -> 239 us.  (Long split
+  // lists 419 -> 415, about what runs differ by.)  With three buffers and short lists it does not pay: 64 blocks
+  // 152.5 against 153.2, 128 blocks 272.6 against 270.2.
   constexpr bool AHEAD = SPLIT == 1 || LINF;
   constexpr bool PARTS = SPLIT == 1;                     // partial results in the workspace
   constexpr int kMaxParts = SPLIT == 1 ? kFwdSplitMax : SPLIT == 2 ? kClusterParts : 1;
