@@ -279,44 +279,61 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
     if (elect_one_sync()) {
       constexpr uint32_t kHiSw = desc_hi_sw128(1024);
       const uint32_t q_lo = desc_lo_sw128(smem_u32(smem + L::kQ), 16);
-      auto issue_qk = [&](int j) -> bool {
+      // What is waited for next is asked about while the products just issued still keep the pipe busy: a barrier
+      // costs some 100 cycles to ask even if it is complete, and few products queue up.
+      bool k_landed = false, ready = false;
+      auto issue_qk = [&](int j, int next) -> bool {
         const uint32_t d = tmem + kClColBuf + kClBuf * (j & 1);
         const int s = j % kClStages;
-        if (!cl_wait(&bars->k_full[s], (j / kClStages) & 1, bars, a.status)) return false;
+        if (!k_landed && !cl_wait(&bars->k_full[s], (j / kClStages) & 1, bars, a.status)) return false;
         tc_fence_after();
         const uint32_t k_lo = desc_lo_sw128(smem_u32(smem + L::kK + s * kClTerms * L::kPage), 16);
         // term t of phi(Q) with the first 3 - t of phi(K), onto the sums from the t-th on
+        auto product = [&](int t, int kk) {
+          tc_mma_ss_lo(d + kBlock * t, q_lo + ((t * L::kQTile + (kk / 4) * L::kQHalf + (kk % 4) * 32) >> 4),
+                       k_lo + (((kk / 4) * kClTerms * L::kSlab + (kk % 4) * 32) >> 4), kHiSw,
+                       idesc_bf16_f32(128, kBlock * (kClTerms - t), 0, 0), (t > 0 || kk > 0) ? 1u : 0u);
+        };
+        // (the largest products last: the most work in the queue while the lane turns to the next step)
+        product(0, 0);
 #pragma unroll
-        for (int t = 0; t < kClTerms; ++t)
+        for (int t = kClTerms - 1; t > 0; --t)
 #pragma unroll
-          for (int kk = 0; kk < D / 16; ++kk)
-            tc_mma_ss_lo(d + kBlock * t, q_lo + ((t * L::kQTile + (kk / 4) * L::kQHalf + (kk % 4) * 32) >> 4),
-                         k_lo + (((kk / 4) * kClTerms * L::kSlab + (kk % 4) * 32) >> 4), kHiSw,
-                         idesc_bf16_f32(128, kBlock * (kClTerms - t), 0, 0), (t > 0 || kk > 0) ? 1u : 0u);
+          for (int kk = 0; kk < D / 16; ++kk) product(t, kk);
+        ready = next < nsteps && mbar_test_wait(&bars->v_full[next % kClStages], (next / kClStages) & 1) &&
+                mbar_test_wait(&bars->p_ready, next & 1);
+#pragma unroll
+        for (int kk = 1; kk < D / 16; ++kk) product(0, kk);
         tc_commit(&bars->a_full[j & 1]);
         return true;
       };
       bool ok = cl_wait(&bars->q_read, 0, bars, a.status);  // phi(Q) is in shared memory
-      for (int j = 0; j < min(2, nsteps) && ok; ++j) ok = issue_qk(j);
+      for (int j = 0; j < min(2, nsteps) && ok; ++j) {
+        k_landed = false;
+        ok = issue_qk(j, nsteps);
+      }
 #pragma unroll 1
       for (int j = 0; j < nsteps && ok; ++j) {
         const int s = j % kClStages;
-        // (V first, which has long landed: it is asked for while the tensor pipe still works)
-        ok = cl_wait(&bars->v_full[s], (j / kClStages) & 1, bars, a.status) && cl_wait(&bars->p_ready, j & 1, bars, a.status);
+        if (!ready)
+          ok = cl_wait(&bars->v_full[s], (j / kClStages) & 1, bars, a.status) && cl_wait(&bars->p_ready, j & 1, bars, a.status);
         if (!ok) break;
         tc_fence_after();
         constexpr uint32_t idesc = idesc_bf16_f32(128, D, 0, 1);
         const uint32_t v_lo = desc_lo_sw128(smem_u32(smem + L::kV + s * L::kPage), L::kSlab);
         const uint32_t p_op = tmem + kClColBuf + kClBuf * (j & 1);
 #pragma unroll
-        for (int t = kClTerms - 1; t >= 0; --t)
+        for (int t = kClTerms - 1; t >= 0; --t) {
 #pragma unroll
           for (int kk = 0; kk < kBlock / 16; ++kk)
             tc_mma_ts_lo(tmem + kClColNum, p_op + (t == 2 ? kBlock + 16 * kk : 16 * kk + 8 * t), v_lo + kk * 128, kHiSw, idesc,
                          (t < kClTerms - 1 || kk > 0) ? 1u : 0u);
+          if (t == 1) k_landed = j + 2 < nsteps && mbar_test_wait(&bars->k_full[s], ((j + 2) / kClStages) & 1);
+        }
         tc_commit(&bars->num_full[s]);
         // the weights of step j + 2 overwrite the ones just consumed: the tensor pipe runs in order
-        if (j + 2 < nsteps) ok = issue_qk(j + 2);
+        ready = false;
+        if (j + 2 < nsteps) ok = issue_qk(j + 2, j + 1);
       }
     }
   } else {
