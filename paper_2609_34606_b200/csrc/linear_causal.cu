@@ -32,7 +32,7 @@
 // What bounds it: the tensor pipe along the longest tile, 25 steps at a chunk of 1560 tokens.  The terms of
 // phi(K) lie side by side, so that one product of phi(Q) hi with all three, one of mid with the first two and
 // one of lo with the first form all sums: 8 x (96 + 64 + 32) cycles per step at head_dim 128, and 768 for num.
-// Measured there (time stamps): 7400 cycles up to the first product (phi(Q)), then 2950 per step, 44 us for
+// Measured there (time stamps): 7500 cycles up to the first product (phi(Q)), then 2450 per step, 36 us for
 // the tile; all tiles of 12 heads together are 2184 steps, 18 us of the pipe on 148 SMs, and the forward
 // kernel runs on the SMs that are through.  One CTA per query and head in fp32 on the CUDA cores took 1678 us.
 // The steps of a tile grow with its position, so the longest tiles are launched first and the forward kernel
