@@ -38,7 +38,7 @@ struct Layout {
   // state
   size_t S, z, slot_S, slot_z, hilo, zop, ksum_saved, ksum, state_total;  // S, z: slot 0; slot_*: bytes per slot
   // workspace
-  size_t status, page_table, qpart, keys, spart, lin_num, lin_den, phik, rpart, ctable, csel, ccnt, olin, ad_w, ad_idx, ad_gini, ad_wsum,
+  size_t status, page_table, qpart, keys, spart, lin_num, lin_den, phik, sums, rpart, ctable, csel, ccnt, olin, ad_w, ad_idx, ad_gini, ad_wsum,
       part_o, part_l, part_ref, part_ticket, ws_total;
   int fwd_splits, split_blocks;
   int phik_blocks;  // pages a chunk can touch (causal contexts with a linear state, else 0)
@@ -101,6 +101,9 @@ Layout make_layout(const hsa_config* c) {
     if (c->lin_mode == HSA_LIN_STATE) {
       L.phik_blocks = (c->max_q_tokens + kBlock - 1) / kBlock + 1;
       L.phik = o;   o = align_up(o + H * kPhiTerms * static_cast<size_t>(L.phik_blocks) * kBlock * D * 2, 256);
+      if (D == 128) {
+        L.sums = o; o = align_up(o + causal_sums_bytes(c->num_heads, c->max_q_tokens), 256);
+      }
     }
   }
   if (c->flags & HSA_CFG_ADAPTIVE) {
@@ -632,6 +635,8 @@ int hsa_forward(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride, in
     c.v_pool = static_cast<const __nv_bfloat16*>(ctx->buf.v_pool);
     c.phik = reinterpret_cast<__nv_bfloat16*>(ws + ctx->lay.phik);
     c.phik_blocks = ctx->lay.phik_blocks;
+    if (D == 128) c.sums = reinterpret_cast<float*>(ws + ctx->lay.sums);
+    c.sum_groups = causal_sum_groups(ctx->cfg.max_q_tokens);
     c.page_table = p.page_table;
     c.q_pos0 = q_pos0;
     c.H = H;

@@ -170,6 +170,8 @@ struct CausalLinArgs {
   // being the chunk's first page (its rows before the chunk included)
   __nv_bfloat16* phik;
   int phik_blocks;
+  float* sums;     // workspace: sums over groups of pages, [H][sum_groups][...] (causal_sums_bytes; null: none)
+  int sum_groups;
   int64_t q_pos0;   // first query position == first token of the intra-chunk part
   int H, D;
   int relu;  // feature map: 0 elu(x) + 1, 1 max(x, 0)
@@ -224,6 +226,8 @@ cudaError_t launch_forward(const FwdParams& p, int D, const CUtensorMap& tm_q,
 cudaError_t launch_causal_linear(const CausalLinArgs& a, const CUtensorMap& tm_q, const CUtensorMap& tm_phik,
                                  const CUtensorMap& tm_v, cudaStream_t st);
 cudaError_t causal_linear_init();
+int causal_sum_groups(int tokens);
+size_t causal_sums_bytes(int heads, int tokens);  // head_dim 128
 // linear branch alone (head_dim 128): lean HBM-bound kernel, nsm = SMs of the device
 cudaError_t launch_linear_only(const FwdParams& p, int nsm, const CUtensorMap& tm_q, const CUtensorMap& tm_state,
                                const CUtensorMap& tm_out, cudaStream_t st);

@@ -90,6 +90,41 @@ def test_causal_partials_carry_24_bits(n0, n, d, relu, cuda_device):
         assert float((got - ref).norm()) <= 2.0 ** -21 * float(ref.norm())
     ctx.destroy()
 
+@pytest.mark.parametrize("n0,n,relu,odd", [(0, 641, 0, False), (63, 768, 0, False), (64, 769, 1, False), (1, 1281, 0, False),
+                                           (100, 1500, 0, True), (0, 700, 1, True)])
+def test_causal_sums_over_groups(n0, n, relu, odd, cuda_device):
+    """Chunks long enough for sums over groups of pages (the first and the last tile of a group, one row in a last
+    tile or group, a group that starts inside a page): partials against 64 bits as above, and, with Inf and NaN in K and
+    V inside a group, what a plain sum has."""
+    from paper_2609_34606_b200 import hsa
+    H, d, inf, nan = 2, 128, float("inf"), float("nan")
+    g = torch.Generator().manual_seed(n)
+    k, v, q = _randn(g, n, H, d), _randn(g, n, H, d), _randn(g, n, H, d)
+    if odd:
+        t = n - 300
+        v[t, 0, 5], v[t + 70, 0, 6], v[t + 3, 0, 7] = inf, -inf, nan
+        k[t, 1, 9] = inf
+    ctx = hsa.HSAContext(H, d, max_pages=(n0 + n + 63) // 64, max_q_tokens=n, max_topk=1, causal=True, device=cuda_device,
+                         feature_map=relu)
+    if n0:
+        ctx.append_kv(_randn(g, n0, H, d).to(cuda_device), _randn(g, n0, H, d).to(cuda_device))
+    ctx.append_kv(k.to(cuda_device), v.to(cuda_device))
+    ctx.forward(q.to(cuda_device), None, None, q_pos0=n0, causal=True, flags=hsa.HSA_FWD_NO_SPARSE)
+    assert ctx.device_status() == 0
+    num, den = _causal_partials(ctx, n, n)
+    phi = lambda x: x.double().clamp(min=0) if relu else torch.where(x > 0, x.double() + 1, x.double().exp())
+    ref_num, ref_den = torch.zeros(n, H, d, dtype=torch.float64), torch.zeros(n, H, dtype=torch.float64)
+    for i in range(n):
+        w = (phi(q[i])[None] * phi(k[:i + 1])).sum(2)
+        ref_num[i], ref_den[i] = (w[:, :, None] * v[:i + 1].double()).sum(0), w.sum(0)
+    for got, ref in ((num, ref_num), (den, ref_den)):
+        wrong = ~ref.isfinite()
+        assert bool(wrong.any()) == (odd and (got is num or bool((~ref_den.isfinite()).any())))
+        assert torch.equal(torch.nan_to_num(got[wrong], nan=1.0), torch.nan_to_num(ref[wrong], nan=1.0))
+        assert float((got[~wrong] - ref[~wrong]).norm()) <= 2.0 ** -21 * float(ref[~wrong].norm())
+    ctx.destroy()
+
+
 @pytest.mark.parametrize("n0,n,d,relu", [(0, 100, 128, 0), (100, 300, 128, 0), (70, 300, 64, 0), (64, 300, 128, 1)])
 def test_causal_not_finite_values_stay_behind_their_position(n0, n, d, relu, cuda_device):
     """Inf and NaN in K, V and queries of a causal chunk reach the rows at and behind them, and there what they
