@@ -178,9 +178,9 @@ __device__ __forceinline__ void init_barriers(Bars* bars) {
 // SPLIT: 1: compiled with the split-tile path (grid z > 1), parts in the workspace; 2: the parts of a list are the
 // CTAs of a cluster and meet in shared memory; the plain kernel (0) carries none of either
 // LINF: compiled with the compressed-pool segment in front of the selected pages (tm_kc, tm_vc)
-// GT: per-dim gate logits arrive as tiles by TMA (tm_gl, tm_gs); an instance of its own, so that the others
-// keep their registers
-template <int D, int SPLIT, bool LINF, bool GT>
+// TILES: what the epilogue reads arrives as tiles by TMA: 1: per-dim gate logits (tm_gl, tm_gs), 2: causal partials
+// (tm_gl); instances of their own, so that the others keep their registers
+template <int D, int SPLIT, bool LINF, int TILES>
 __global__ void __launch_bounds__(kThreads, 1)
 hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v,
@@ -203,6 +203,8 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
   constexpr uint32_t kColLn = LINF ? 128 : kColLin;      // linear-branch accumulator
   using L = Smem<D>;
   constexpr int DH = D / 64;  // 64-element (128-byte) slabs per row
+  constexpr bool GT = TILES == 1, NUMT = TILES == 2;
+  static_assert(!NUMT || (D == 128 && SPLIT != 1 && !LINF), "causal partials as tiles: head_dim 128, no parts in the workspace");
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
@@ -455,6 +457,20 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             for (int dh = 0; dh < DH; ++dh)
               tma_load_3d(smem + L::kK + s * L::kTile + dh * L::kHalf, i == 0 ? &tm_gl : &tm_gs, &bars->k_full[s], dh * 64, h, row0);
             gates_armed |= 1 << i;
+          }
+        }
+        if (NUMT && ok && lead) {
+          // causal partials: [128 rows x 128 dims] fp32 in slabs of 32 dims into the same two stages, once the kernel
+          // that makes them is complete
+          for (int s = 1; s < 3 && ok; ++s) ok = wait_bar(&bars->k_empty[s], (gate_uses(s) & 1) ^ 1, bars, p.status);
+          if (ok) {
+            if (p.wait_late) asm volatile("griddepcontrol.wait;" ::: "memory");
+            for (int i = 0; i < 4; ++i) {
+              const int s = 1 + i / 2;
+              if (i % 2 == 0) mbar_expect_tx(&bars->k_full[s], L::kTile);
+              tma_load_3d(smem + L::kK + s * L::kTile + i % 2 * L::kHalf, &tm_gl, &bars->k_full[s], i * 32, h, row0);
+            }
+            gates_armed = 3;
           }
         }
         if (!ok) {
@@ -1052,12 +1068,16 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
       if (ok && epi && nsteps == 0 && (!p.do_linear || LINF))
         ok = __all_sync(0xffffffffu, wait_bar(&bars->q_full, 0, bars, p.status));
       if (!PARTS && p.wait_late) asm volatile("griddepcontrol.wait;" ::: "memory");  // the causal partials
+      if (NUMT && ok && lead) {
+        for (int s = 1; s < 3; ++s) ok = ok && wait_bar(&bars->k_full[s], gate_uses(s) & 1, bars, p.status);
+        ok = __all_sync(0xffffffffu, ok);
+      }
       if (ok && epi && do_output) {  // warp-uniform: the TMEM loads below are warp-collective
         const bool wr = row < p.n_q;  // rows past the end of the chunk compute but never store
         float lin_den = den;
         const float* lnum = nullptr;
         if (wr && p.do_linear && p.lin_num != nullptr) {
-          lnum = p.lin_num + (static_cast<size_t>(row) * p.H + h) * D;
+          if (!NUMT) lnum = p.lin_num + (static_cast<size_t>(row) * p.H + h) * D;
           lin_den += p.lin_den[static_cast<size_t>(row) * p.H + h];
         }
         // (relu: a row may have no weight at all, hence 1e-6 in its denominator; 0 / 1e-6 = 0)
@@ -1080,10 +1100,10 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         const int64_t g_ds = p.g_ds;
         // (decided from the launch parameters, not from this thread's pointers: the branch holds
         // warp-collective TMEM loads and must not diverge inside a warp)
-        const bool plain = !p.g_lin && !p.g_sp && !(p.do_linear && p.lin_num != nullptr) && !p.ext_lin &&
+        const bool plain = !p.g_lin && !p.g_sp && (NUMT || !(p.do_linear && p.lin_num != nullptr)) && !p.ext_lin &&
                            !(PARTS && nsplit > 1);
         if (plain) {
-          // no gates, no causal partials, no external linear output, no merge: 32 columns per trip
+          // no gates, no causal partials but a tile's, no external linear output, no merge: 32 columns per trip
           const float il = has_o ? inv_l : 0.f, id = has_lin ? inv_den : 0.f;
 #pragma unroll 1
           for (int c0 = cbase; c0 < cbase + HC; c0 += 32) {
@@ -1093,6 +1113,17 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
             if (has_o) tmem_ld32(o_tmem + c0, oa);
             if (has_lin) tmem_ld32(tmem + lane_off + kColLn + c0, ln);
             tc_wait_ld();
+            if (NUMT) {
+              const uint8_t* slab = smem + L::kK + L::kTile + (c0 >> 5) * L::kHalf + r * 128;
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const float4 v = *reinterpret_cast<const float4*>(slab + ((i ^ (r & 7)) << 4));
+                ln[4 * i] = __float_as_uint(__uint_as_float(ln[4 * i]) + v.x);
+                ln[4 * i + 1] = __float_as_uint(__uint_as_float(ln[4 * i + 1]) + v.y);
+                ln[4 * i + 2] = __float_as_uint(__uint_as_float(ln[4 * i + 2]) + v.z);
+                ln[4 * i + 3] = __float_as_uint(__uint_as_float(ln[4 * i + 3]) + v.w);
+              }
+            }
             uint32_t pk[16];
 #pragma unroll
             for (int i = 0; i < 32; i += 2)
@@ -1196,7 +1227,17 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 #pragma unroll
             for (int i = 0; i < 16; ++i) ws[i] = gate_w(__bfloat162float(gs[(c0 + i) * g_ds]));
           }
-          if (lnum) {
+          if constexpr (NUMT) {
+            const uint8_t* slab = smem + L::kK + L::kTile + (c0 >> 5) * L::kHalf + r * 128;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+              const float4 v = *reinterpret_cast<const float4*>(slab + (((((c0 & 31) >> 2) + i) ^ (r & 7)) << 4));
+              ladd[4 * i] = v.x;
+              ladd[4 * i + 1] = v.y;
+              ladd[4 * i + 2] = v.z;
+              ladd[4 * i + 3] = v.w;
+            }
+          } else if (lnum) {
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
               const float4 v = *reinterpret_cast<const float4*>(lnum + c0 + 4 * i);
@@ -1277,15 +1318,16 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 namespace {
 using FwdKernel = void (*)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap,
                            CUtensorMap, FwdParams);
-// split: see the kernel
+// split, tiles: see the kernel
 template <int D>
-FwdKernel fwd_kernel(int split, bool linf, bool gt) {
+FwdKernel fwd_kernel(int split, bool linf, int tiles) {
   if constexpr (D == 128) {
-    if (linf) return gt ? hsa_forward_kernel<128, 0, true, true> : hsa_forward_kernel<128, 0, true, false>;
+    if (linf) return tiles ? hsa_forward_kernel<128, 0, true, 1> : hsa_forward_kernel<128, 0, true, 0>;
+    if (tiles == 2) return split == 2 ? hsa_forward_kernel<128, 2, false, 2> : hsa_forward_kernel<128, 0, false, 2>;
   }
-  if (split == 2) return gt ? hsa_forward_kernel<D, 2, false, true> : hsa_forward_kernel<D, 2, false, false>;
-  if (split == 1) return gt ? hsa_forward_kernel<D, 1, false, true> : hsa_forward_kernel<D, 1, false, false>;
-  return gt ? hsa_forward_kernel<D, 0, false, true> : hsa_forward_kernel<D, 0, false, false>;
+  if (split == 2) return tiles ? hsa_forward_kernel<D, 2, false, 1> : hsa_forward_kernel<D, 2, false, 0>;
+  if (split == 1) return tiles ? hsa_forward_kernel<D, 1, false, 1> : hsa_forward_kernel<D, 1, false, 0>;
+  return tiles ? hsa_forward_kernel<D, 0, false, 1> : hsa_forward_kernel<D, 0, false, 0>;
 }
 
 // a launch of `ctas` CTAs in clusters of `cluster` (0: none), as a programmatic dependent of the kernel before it
@@ -1313,15 +1355,18 @@ cudaError_t forward_init(int D, int (&clusters)[3]) {
   cudaError_t e = cudaSuccess;
   for (int i = 0; i < 8 && e == cudaSuccess; ++i) {
     const int split = i % 4 == 3 ? 0 : i % 4;
-    const bool linf = i % 4 == 3, gt = i >= 4;
+    const bool linf = i % 4 == 3;
+    const int gt = i >= 4;
     e = cudaFuncSetAttribute(fwd_kernel<128>(split, linf, gt), cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<128>::kTotal);
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(fwd_kernel<64>(split, false, gt), cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<64>::kTotal);
   }
+  for (int split = 0; split <= 2 && e == cudaSuccess; split += 2)
+    e = cudaFuncSetAttribute(fwd_kernel<128>(split, false, 2), cudaFuncAttributeMaxDynamicSharedMemorySize, Smem<128>::kTotal);
   for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
     FwdLaunch l(D, dim3(2 << k), 2 << k, nullptr);
-    const void* fn = D == 128 ? reinterpret_cast<const void*>(fwd_kernel<128>(2, false, true))
-                              : reinterpret_cast<const void*>(fwd_kernel<64>(2, false, true));
+    const void* fn = D == 128 ? reinterpret_cast<const void*>(fwd_kernel<128>(2, false, 1))
+                              : reinterpret_cast<const void*>(fwd_kernel<64>(2, false, 1));
     if (cudaOccupancyMaxActiveClusters(&clusters[k], fn, &l.cfg) != cudaSuccess) {
       cudaGetLastError();
       clusters[k] = 0;  // no clusters of this size on this device
@@ -1333,7 +1378,7 @@ cudaError_t forward_init(int D, int (&clusters)[3]) {
 cudaError_t launch_forward(const FwdParams& p_in, int D, const CUtensorMap& tm_q, const CUtensorMap& tm_k,
                            const CUtensorMap& tm_v, const CUtensorMap& tm_state, const CUtensorMap& tm_out,
                            cudaStream_t st, const CUtensorMap* tm_kc, const CUtensorMap* tm_vc, const CUtensorMap* tm_gl,
-                           const CUtensorMap* tm_gs) {
+                           const CUtensorMap* tm_gs, const CUtensorMap* tm_num) {
   const int n_tiles = (p_in.n_q + kTileM - 1) / kTileM;
   FwdParams p = p_in;
   p.n_tiles = n_tiles;
@@ -1351,10 +1396,11 @@ cudaError_t launch_forward(const FwdParams& p_in, int D, const CUtensorMap& tm_q
   const CUtensorMap& vc = linf ? *tm_vc : tm_v;
   // (nor, without gate tiles, at these)
   p.gate_tiles = (tm_gl ? 1 : 0) | (tm_gs ? 2 : 0);
-  const CUtensorMap& gl = tm_gl ? *tm_gl : tm_q;
+  const bool num = p.lin_num && tm_num && D == 128 && split != 1 && !linf && p.gate_tiles == 0;
+  const CUtensorMap& gl = tm_gl ? *tm_gl : num ? *tm_num : tm_q;
   const CUtensorMap& gs = tm_gs ? *tm_gs : tm_q;
-  const bool gt = p.gate_tiles != 0;
-  return cudaLaunchKernelEx(&l.cfg, D == 128 ? fwd_kernel<128>(split, linf, gt) : fwd_kernel<64>(split, false, gt), tm_q, tm_k, tm_v,
+  const int tiles = p.gate_tiles != 0 ? 1 : num ? 2 : 0;
+  return cudaLaunchKernelEx(&l.cfg, D == 128 ? fwd_kernel<128>(split, linf, tiles) : fwd_kernel<64>(split, false, tiles), tm_q, tm_k, tm_v,
                             tm_state, tm_out, kc, vc, gl, gs, p);
 }
 

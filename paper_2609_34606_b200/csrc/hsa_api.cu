@@ -153,7 +153,7 @@ struct hsa_ctx {
   int64_t tail_saved_for;  // history length whose tail-block key sum sits in the saved-tail buffer (-1: none)
   int nsm;
   int clusters[3];      // clusters of 2, 4 and 8 CTAs of the forward kernel that run at once
-  CUtensorMap tm_k, tm_v, tm_state, tm_kc, tm_vc, tm_olin, tm_ek, tm_ev, tm_phik;
+  CUtensorMap tm_k, tm_v, tm_state, tm_kc, tm_vc, tm_olin, tm_ek, tm_ev, tm_phik, tm_num;
   int32_t n_segs;  // Linformer: complete segments compressed so far
   std::vector<int32_t> page_table_host;  // history block -> physical page
   std::vector<uint8_t> resident;         // per history block: tiles present in the pool (tier migration)
@@ -192,6 +192,19 @@ int encode_q(CUtensorMap* tm, const void* q, int n_q, int H, int D, int64_t ts, 
   CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(q), dims, strides, box,
                    estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                    CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? HSA_OK : HSA_ERR_CUDA;
+}
+
+// causal partials: fp32 [tokens][H][128], boxes of 32 dims x 1 x 128 tokens
+int encode_num(CUtensorMap* tm, void* num, int tokens, int H) {
+  EncodeTiledFn enc = get_encode_fn();
+  if (!enc) return HSA_ERR_CUDA;
+  cuuint64_t dims[3] = {128, static_cast<cuuint64_t>(H), static_cast<cuuint64_t>(tokens)};
+  cuuint64_t strides[2] = {512, static_cast<cuuint64_t>(H) * 512};
+  cuuint32_t box[3] = {32, 1, kTileM};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = enc(tm, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, num, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                   CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? HSA_OK : HSA_ERR_CUDA;
 }
 
@@ -321,6 +334,8 @@ int hsa_create(hsa_ctx** out, const hsa_config* cfg, const hsa_buffers* bufs,
                        static_cast<uint64_t>(cfg->num_heads) * 4 * D, D);
   if (r == HSA_OK && ctx->lay.phik_blocks > 0)
     r = encode_2d_rows(&ctx->tm_phik, ws + ctx->lay.phik, static_cast<uint64_t>(cfg->num_heads) * kPhiTerms * ctx->lay.phik_blocks * kBlock, D);
+  if (r == HSA_OK && ctx->lay.phik_blocks > 0 && D == 128)
+    r = encode_num(&ctx->tm_num, ws + ctx->lay.lin_num, cfg->max_q_tokens, cfg->num_heads);
   if (r == HSA_OK && linformer) {
     const uint64_t crows = static_cast<uint64_t>(ctx->lay.n_cpages) * cfg->num_heads * kBlock;
     r = encode_2d_rows(&ctx->tm_kc, bufs->kc_pool, crows, D);
@@ -708,7 +723,8 @@ int hsa_forward(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride, in
   if (D == 128 && do_linear && !do_sparse && !p.ext_lin)
     e = launch_linear_only(p, ctx->nsm, tm_q, ctx->tm_state, tm_out, st);  // nothing but Q in, out out
   else
-    e = launch_forward(p, D, tm_q, ctx->tm_k, ctx->tm_v, ctx->tm_state, tm_out, st, nullptr, nullptr, tm_gate[0], tm_gate[1]);
+    e = launch_forward(p, D, tm_q, ctx->tm_k, ctx->tm_v, ctx->tm_state, tm_out, st, nullptr, nullptr, tm_gate[0], tm_gate[1],
+                       causal_lin && D == 128 ? &ctx->tm_num : nullptr);
   if (e != cudaSuccess) return cuda_fail(ctx, e);
   return HSA_OK;
 }

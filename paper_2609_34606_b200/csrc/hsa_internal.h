@@ -216,12 +216,15 @@ cudaError_t launch_qsum(const SelectArgs& a, cudaStream_t st);  // stage 1 alone
 cudaError_t launch_retrieve(const RetrieveArgs& a, int n_pages, cudaStream_t st);
 cudaError_t launch_select_adaptive(const SelectArgs& a, const AdaptiveArgs& ad, cudaStream_t st);
 // tm_kc / tm_vc: maps of the compressed pools, used when p.lf_table is set (else null); tm_gl / tm_gs: maps
-// of per-dim gate logits with the geometry of tm_q (null: no such gate, or its strides do not allow one)
+// of per-dim gate logits with the geometry of tm_q (null: no such gate, or its strides do not allow one); tm_num: map
+// of p.lin_num, box 32 dims x 1 x 128 tokens (head_dim 128, may be null).  (Read by the rows' threads, 64 bytes of lines
+// 6 KB apart at a time, the partials took 4 to 6 us of each tile, 12 heads of 128, 1560 tokens; as a tile 2.)
 cudaError_t launch_forward(const FwdParams& p, int D, const CUtensorMap& tm_q,
                            const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                            const CUtensorMap& tm_state, const CUtensorMap& tm_out, cudaStream_t st,
                            const CUtensorMap* tm_kc = nullptr, const CUtensorMap* tm_vc = nullptr,
-                           const CUtensorMap* tm_gl = nullptr, const CUtensorMap* tm_gs = nullptr);
+                           const CUtensorMap* tm_gl = nullptr, const CUtensorMap* tm_gs = nullptr,
+                           const CUtensorMap* tm_num = nullptr);
 // tm_q: box of 128 tokens of one head; tm_phik, tm_v: rows of phik and of the V pool, box 64 x 64
 cudaError_t launch_causal_linear(const CausalLinArgs& a, const CUtensorMap& tm_q, const CUtensorMap& tm_phik,
                                  const CUtensorMap& tm_v, cudaStream_t st);
