@@ -418,6 +418,104 @@ __global__ void __launch_bounds__(256) block_scores_kernel(SelectArgs a) {
   scores_item<D, MIXED>(Blk{static_cast<int>(threadIdx.x), 0}, a, blockIdx.x, blockIdx.y, blockIdx.z, qs, op);
 }
 
+// The same as a kernel of its own: one CTA per (32 candidates, run of batches of 16 groups, head), launched behind the tile
+// sums as a programmatic dependent.  What bounds it is latency, so its chain is short: key sums and token counts are
+// asked for ahead of the wait (the tile-sum kernel writes none of them and has itself waited for everything before it), the
+// tile sums of a batch under the products of the one before; two accumulators per product chain; the scale of a mean
+// query is applied to the score, one division per thread.
+template <int D, bool MIXED>
+__global__ void __launch_bounds__(256) group_scores_kernel(SelectArgs a, int batches) {
+  constexpr int GB = kGroupBatch, PITCH = D + 4, KS = D / 4, NV = GB * D / 256;
+  __shared__ __align__(16) double qs[2][GB * PITCH];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, h = blockIdx.z;
+  const CandGeom cg = cand_geom<MIXED>(a);
+  const int c0 = blockIdx.x * kScoreBlocksPerCta + 8 * (warp & 3);  // this warp's eight candidates
+  float kb[KS];
+  {
+    const int c = c0 + (lane >> 2);
+    const int fp = c < cg.nc ? cand_first_page<MIXED>(cg, c) : 0;
+    const int np = c < cg.nc ? cand_pages<MIXED>(cg, c) : 0;
+    const float* k0 = a.ksum + (static_cast<size_t>(h) * a.max_pages + fp) * D + (lane & 3);
+#pragma unroll
+    for (int kk = 0; kk < KS; ++kk) {
+      float v = np > 0 ? k0[4 * kk] : 0.f;
+      if (MIXED && np > 1) v += k0[D + 4 * kk];
+      kb[kk] = v;
+    }
+  }
+  double inv_cnt[2];
+  bool masked[2];
+#pragma unroll
+  for (int t = 0; t < 2; ++t) {
+    const int c = c0 + 2 * (lane & 3) + t;
+    const int fp = c < cg.nc ? cand_first_page<MIXED>(cg, c) : 0;
+    const int np = c < cg.nc ? cand_pages<MIXED>(cg, c) : 0;
+    const int64_t cnt = max64(1, min64(static_cast<int64_t>(np) * kBlock, a.n_tokens - static_cast<int64_t>(fp) * kBlock));
+    inv_cnt[t] = cnt == kBlock ? 1.0 / kBlock : 1.0 / static_cast<double>(cnt);
+    masked[t] = false;
+    if (MIXED && a.kv_pages != nullptr && c < cg.ni) {
+      const int pl = fp + np - 1;
+      bool in_f = false, in_l = false;
+      for (int k = 0; k < a.n_kv_pages; ++k) {
+        const int kp = a.kv_pages[k];
+        in_f |= (fp / a.kv_page_blocks == kp);
+        in_l |= (pl / a.kv_page_blocks == kp);
+      }
+      masked[t] = !(in_f && in_l);
+    }
+  }
+  const int gtok = a.group_tokens, tiles_per_group = gtok / kTileM, n_tiles = (a.n_q + kTileM - 1) / kTileM;
+  const double scale_full = static_cast<double>(a.scale) / static_cast<double>(gtok);
+  const double scale_last = static_cast<double>(a.scale) / static_cast<double>(a.n_q - (a.n_groups - 1) * gtok);
+  const int g_lo = blockIdx.y * batches * GB, g_hi = min(a.n_groups, g_lo + batches * GB);
+  // tile sums of 16 groups, added in ascending tile order in fp64: column tid % D, groups tid / D + (256 / D) v
+  const int col = threadIdx.x % D, gr = threadIdx.x / D;
+  auto load = [&](int g0, int tt, float (&part)[NV]) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+      const int g = g0 + gr + 256 / D * v, t = g * tiles_per_group + tt;
+      part[v] = (g < g_hi && t < n_tiles) ? __ldcg(&a.qpart[(static_cast<size_t>(t) * a.H + h) * D + col]) : 0.f;
+    }
+  };
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  float part[NV];
+  load(g_lo, 0, part);
+  int buf = 0;
+#pragma unroll 1
+  for (int g0 = g_lo; g0 < g_hi; g0 += GB, buf ^= 1) {
+    double sum[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) sum[v] = static_cast<double>(part[v]);
+#pragma unroll 1
+    for (int tt = 1; tt < tiles_per_group; ++tt) {
+      load(g0, tt, part);
+#pragma unroll
+      for (int v = 0; v < NV; ++v) sum[v] += static_cast<double>(part[v]);
+    }
+#pragma unroll
+    for (int v = 0; v < NV; ++v) qs[buf][(gr + 256 / D * v) * PITCH + col] = sum[v];
+    if (g0 + GB < g_hi) load(g0 + GB, 0, part);
+    __syncthreads();  // (the other buffer is written again only behind the next one: one barrier per batch)
+    const int row0 = 8 * (warp >> 2);  // this warp's eight rows of the batch
+    if (g0 + row0 < g_hi && c0 < cg.nc) {  // warp-uniform
+      const double* arow = qs[buf] + (row0 + (lane >> 2)) * PITCH + (lane & 3);
+      double d[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+      for (int kk = 0; kk < KS; ++kk) dmma_m8n8k4(d[kk & 1][0], d[kk & 1][1], arow[4 * kk], static_cast<double>(kb[kk]));
+      const int g = g0 + row0 + (lane >> 2);
+      if (g < g_hi) {
+        uint32_t* keys = a.keys + (static_cast<size_t>(h) * a.n_groups + g) * a.max_pages;
+        const int c = c0 + 2 * (lane & 3);
+        const double sc = g == a.n_groups - 1 ? scale_last : scale_full;
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+          if (c + t < cg.nc) keys[c + t] = masked[t] ? 0u : order_key(static_cast<float>((d[0][t] + d[1][t]) * sc * inv_cnt[t]));
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------------------
 // Stage 3: one CTA per (group, head): k-th largest key by a 4-pass 8-bit radix select, then an
 // index-ordered compaction.  Exact ties at the threshold go to the lower block index.
@@ -1271,16 +1369,27 @@ bool launch_cluster(const SelectArgs& a, const AdaptiveArgs* ad, bool mixed, cud
 }
 }  // namespace
 
-// Three forms, all programmatic dependents of the kernel before them:
+namespace {
+const void* group_scores(int D, bool mixed) {
+  if (D == 128)
+    return mixed ? reinterpret_cast<const void*>(group_scores_kernel<128, true>) : reinterpret_cast<const void*>(group_scores_kernel<128, false>);
+  return mixed ? reinterpret_cast<const void*>(group_scores_kernel<64, true>) : reinterpret_cast<const void*>(group_scores_kernel<64, false>);
+}
+}  // namespace
+
+// Four forms, all programmatic dependents of the kernel before them:
 //   cluster form        query tile sums as a kernel of their own (they read the whole chunk and want
 //                       every SM; short chunks: inside the clusters), then one cluster of 8 CTAs per head for scores and lists, with one
 //                       hardware cluster barrier between them -- the default for one list per head while
 //                       a head has at most kClusterMaxChunks score items (6144 blocks; measured against
 //                       the grid-barrier form: 17.1 against 20.0 us at 2194 blocks, 24.8 against 25.1 us
 //                       at 4388)
-//   grid-barrier form   one cooperative launch over all SMs with two device barriers -- histories
-//                       beyond that, one list per query tile (37 x H lists want more than 24 blocks
-//                       of threads per head), and on request
+//   per query tile      several lists per head: tile sums, scores (matrix products in fp64, group_scores_kernel) and
+//                       lists as three launches.  The grid-barrier form spent 8 us at its barriers and ran the batches of
+//                       groups of a score item one after another, cold.  Heads x tokens x blocks, grid-barrier form ->
+//                       now: 12 x 4680 x 732 30.6 -> 20.7 us, x 4388 80 -> 64; 4 x 1000 x 157 20.7 -> 10.8;
+//                       16 x 4680 x 1563, groups of 512 tokens, 39 -> 28.6
+//   grid-barrier form   one cooperative launch over all SMs with two device barriers -- longer histories, and on request
 //   three launches      for devices without cooperative launch and for callers without a barrier word
 cudaError_t launch_select(const SelectArgs& a, cudaStream_t st) {
   int nsm = 0;
@@ -1295,7 +1404,9 @@ cudaError_t launch_select(const SelectArgs& a, cudaStream_t st) {
   const int64_t n_chunks_max = (nblk_all + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta;
   cudaError_t ec = cudaSuccess;
   if (a.use_clusters && launch_cluster(a, nullptr, mixed, st, &ec)) return ec;
-  if (a.barrier && coop_info(&nsm)) {
+  const bool by_groups = a.use_clusters && a.n_groups > 1;
+  const bool coop = coop_info(&nsm);  // (nsm is known either way)
+  if (!by_groups && a.barrier && coop) {
     // one cooperative launch for all three stages
     const size_t smem_keys = static_cast<size_t>(nblk_all > 0 ? nblk_all : 1) * sizeof(uint32_t);
     const void* fn = a.D == 128 ? (mixed ? reinterpret_cast<const void*>(select_fused_kernel<128, true>)
@@ -1320,11 +1431,21 @@ cudaError_t launch_select(const SelectArgs& a, cudaStream_t st) {
   if (e != cudaSuccess) return e;
   if (nblk_all > 0) {
     dim3 g2(static_cast<unsigned>(n_chunks_max), a.n_groups, a.H);
-    const void* f2 = a.D == 128 ? (mixed ? reinterpret_cast<const void*>(block_scores_kernel<128, true>)
+    // (batches of groups side by side only as far as the SMs hold them, two CTAs each: the key sums are read once per CTA)
+    const int n_batches = (a.n_groups + kGroupBatch - 1) / kGroupBatch;
+    int batches = n_batches;
+    void* g_args[2] = {&aa, &batches};
+    if (by_groups) {
+      const int64_t room = max64(1, 2 * nsm / max64(1, n_chunks_max * a.H));
+      g2.y = static_cast<unsigned>(min64(room, n_batches));
+      batches = (n_batches + static_cast<int>(g2.y) - 1) / static_cast<int>(g2.y);
+      g2.y = static_cast<unsigned>((n_batches + batches - 1) / batches);
+    }
+    const void* f2 = by_groups ? group_scores(a.D, mixed) : a.D == 128 ? (mixed ? reinterpret_cast<const void*>(block_scores_kernel<128, true>)
                                          : reinterpret_cast<const void*>(block_scores_kernel<128, false>))
                                 : (mixed ? reinterpret_cast<const void*>(block_scores_kernel<64, true>)
                                          : reinterpret_cast<const void*>(block_scores_kernel<64, false>));
-    e = launch_pdl(f2, g2, dim3(256), 0, p_args, st);
+    e = launch_pdl(f2, g2, dim3(256), 0, by_groups ? g_args : p_args, st);
     if (e != cudaSuccess) return e;
   }
   const size_t smem = static_cast<size_t>(nblk_all > 0 ? nblk_all : 1) * sizeof(uint32_t);

@@ -389,6 +389,34 @@ def test_adaptive_lists(d, H, n, n_q, causal, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("d,H,n_q,n,group,ex", [
+    (128, 3, 129, 64, 128, 0), (128, 2, 2048, 2049, 128, 0), (128, 2, 2049, 2112, 128, 2), (64, 3, 4300, 4000, 128, 0),
+    (128, 1, 1100, 9000, 512, 2), (64, 2, 700, 2100, 256, 2), (128, 12, 300, 40000, 128, 0)])
+def test_lists_per_query_tile_by_three_launches(d, H, n_q, n, group, ex, cuda_device):
+    """Scores of 2, 16, 17 and 34 groups (batches of 16), one and several tiles per group with a short last one, one candidate,
+    32, 33 and more, single pages and runs of pages: the lists of the grid-barrier form."""
+    from paper_2609_34606_b200 import hsa
+    g = torch.Generator().manual_seed(n_q + n)
+    K, V, q = _randn(g, n, H, d), _randn(g, n, H, d), _randn(g, n_q, H, d).to(cuda_device)
+    blocks = (n + 63) // 64
+    budgets = torch.tensor([max(1, blocks // 3 - h) for h in range(H)], dtype=torch.int32, device=cuda_device)
+    lists = []
+    for grid_form in (False, True):
+        ctx = hsa.HSAContext(H, d, max_pages=blocks, max_q_tokens=max(n_q, n), max_topk=blocks, device=cuda_device,
+                             grid_barrier_select=grid_form)
+        ctx.append_kv(K.to(cuda_device), V.to(cuda_device))
+        if ex:
+            lists.append(ctx.select_blocks_ex(q, budgets, ex, blocks // 2, None, group_tokens=group))
+        else:
+            lists.append(ctx.select_blocks(q, budgets, group_tokens=group))
+        assert ctx.device_status() == 0
+        ctx.destroy()
+    (ia, ca), (ib, cb) = lists
+    assert torch.equal(ca, cb) and int(ca.sum()) > 0
+    keep = torch.arange(ia.shape[2], device=cuda_device) < ca[:, :, None]
+    assert torch.equal(ia[keep], ib[keep])
+
+
 @pytest.mark.parametrize("n_q", [3072, 3073])
 def test_query_sums_inside_the_clusters(n_q, cuda_device):
     """24 query tiles are the most whose sums the clusters take themselves: lists as in the grid-barrier form."""
