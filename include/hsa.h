@@ -226,7 +226,8 @@ int hsa_block_resident(hsa_ctx* ctx, int32_t block, int32_t* resident_out);
  *   tau_h = tau_min + G_h (tau_max - tau_min),
  * G_h being the Gini coefficient of the sorted block weights averaged over the head's groups
  * (the paper's best setting is tau_max = 1.00, tau_min = 0.35).  Same candidates, tie rule and
- * output layout as hsa_select_blocks.  gini_tau_out_dev: optional device fp32 [2][H] receiving G_h
+ * output layout as hsa_select_blocks; entries behind a list are written as zeros.  gini_tau_out_dev:
+ * optional device fp32 [2][H] receiving G_h
  * and tau_h.  Needs HSA_CFG_ADAPTIVE; HSA_ERR_UNSUPPORTED when the history has more than 8192
  * blocks. */
 int hsa_select_blocks_adaptive(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride,

@@ -938,6 +938,7 @@ __global__ void __launch_bounds__(256) adaptive_pick_kernel(SelectArgs a, Adapti
       ++pos;
     }
   }
+  for (int i = total + static_cast<int>(threadIdx.x); i < a.kcap; i += 256) out[i] = 0;  // (zeros behind the list)
   if (threadIdx.x == 0) {
     a.sel_cnt[static_cast<size_t>(h) * a.n_groups + g] = min(total, a.kcap);
     if (total > a.kcap) atomicCAS(a.status, 0, kDevBounds);
@@ -1088,6 +1089,7 @@ __device__ __forceinline__ void adaptive_list(const SelectArgs& a, const Adaptiv
       if (pos < a.kcap) out[pos] = b;
       ++pos;
     }
+  for (int i = kk + tid; i < a.kcap; i += kAdThreads) out[i] = 0;  // (zeros behind the list)
   if (tid == 0) {
     a.sel_cnt[h] = min(kk, a.kcap);
     if (kk > a.kcap) atomicCAS(a.status, 0, kDevBounds);

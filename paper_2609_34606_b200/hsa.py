@@ -443,9 +443,9 @@ class HSAContext:
         with gini_tau fp32 [2, H] = (Gini, threshold) per head."""
         q_pos0 = self.n_tokens if q_pos0 is None else q_pos0
         g, H = self.n_groups(q.shape[0], group_tokens), self.H
-        # lists, counts and (as fp32) Gini and threshold in one zeroed buffer: one fill instead of three
+        # lists, counts and (as fp32) Gini and threshold in one buffer, which the call writes as a whole
         n_idx, n_cnt = H * g * self.max_topk, H * g
-        buf = torch.zeros(n_idx + n_cnt + 2 * H, dtype=torch.int32, device=self.device)
+        buf = torch.empty(n_idx + n_cnt + 2 * H, dtype=torch.int32, device=self.device)
         idx, cnt, gt = buf.split((n_idx, n_cnt, 2 * H))
         sel_idx, sel_cnt, gt = idx.view(H, g, self.max_topk), cnt.view(H, g), gt.view(torch.float32).view(2, H)
         hsa_select_blocks_adaptive(self.ctx, q, q_pos0, causal, tau_min, tau_max, group_tokens, sel_idx, sel_cnt, gt)

@@ -665,3 +665,22 @@ def test_gate_tiles_in_every_instance(d, form, hot, cuda_device):
     # keys, so that its bf16 weights round differently (2^-9 each, of random sign, of a sum of many)
     assert float((out - a - b).norm()) <= 1.5 * BF16_REL * float((a + b).norm())
     ctx.destroy()
+
+
+@pytest.mark.parametrize("n,group", [(700, 0), (64 * 40, 0), (700, 128)])
+def test_adaptive_lists_end_in_zeros(n, group, cuda_device):
+    """What a list buffer held before the call is gone, behind the list as well."""
+    from paper_2609_34606_b200 import hsa
+    H, d, n_q = 3, 128, 200
+    g = torch.Generator().manual_seed(n)
+    blocks = (n + 63) // 64
+    ctx = hsa.HSAContext(H, d, max_pages=blocks, max_q_tokens=n, max_topk=blocks + 3, device=cuda_device, adaptive=True)
+    ctx.append_kv(_randn(g, n, H, d).to(cuda_device), _randn(g, n, H, d).to(cuda_device))
+    q = _randn(g, n_q, H, d).to(cuda_device)
+    idx, cnt, gt = ctx.select_blocks_adaptive(q, 0.2, 0.4, group_tokens=group)
+    dirty, counts = torch.full_like(idx, 77), torch.full_like(cnt, 77)
+    hsa.hsa_select_blocks_adaptive(ctx.ctx, q, n, False, 0.2, 0.4, group, dirty, counts, None)
+    assert torch.equal(dirty, idx) and torch.equal(counts, cnt)
+    behind = torch.arange(idx.shape[2], device=cuda_device) >= cnt[:, :, None]
+    assert int(idx[behind].abs().sum()) == 0 and bool(behind.any()) and int(cnt.min()) > 0
+    ctx.destroy()
