@@ -34,20 +34,32 @@ __global__ void __launch_bounds__(256) append_pool_ksum_kernel(AppendArgs a) {
 #pragma unroll
   for (int i = 0; i < 8; ++i) acc[i] = 0.f;
 
-  for (int64_t t = t_lo + rg; t < t_hi; t += RP) {
-    const size_t src = static_cast<size_t>(t - a.n0) * a.tok_stride +
-                       static_cast<size_t>(h) * a.head_stride + c8 * 8;
-    const uint4 kk = *reinterpret_cast<const uint4*>(a.k + src);
-    const uint4 vv = *reinterpret_cast<const uint4*>(a.v + src);
-    const size_t dst = (row_base + (t - b * kBlock)) * D + c8 * 8;
-    *reinterpret_cast<uint4*>(a.k_pool + dst) = kk;
-    *reinterpret_cast<uint4*>(a.v_pool + dst) = vv;
-    const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kk);
+  // all of a thread's rows are asked for before the first is consumed (one round trip to memory, not one per row)
+  constexpr int NR = kBlock / RP;
+  uint4 kk[NR], vv[NR];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 f = __bfloat1622float2(k2[i]);
-      acc[2 * i] += f.x;
-      acc[2 * i + 1] += f.y;
+  for (int i = 0; i < NR; ++i) {
+    const int64_t t = t_lo + rg + i * RP;
+    if (t < t_hi) {
+      const size_t src = static_cast<size_t>(t - a.n0) * a.tok_stride + static_cast<size_t>(h) * a.head_stride + c8 * 8;
+      kk[i] = *reinterpret_cast<const uint4*>(a.k + src);
+      vv[i] = *reinterpret_cast<const uint4*>(a.v + src);
+    }
+  }
+#pragma unroll
+  for (int i = 0; i < NR; ++i) {
+    const int64_t t = t_lo + rg + i * RP;
+    if (t < t_hi) {
+      const size_t dst = (row_base + (t - b * kBlock)) * D + c8 * 8;
+      *reinterpret_cast<uint4*>(a.k_pool + dst) = kk[i];
+      *reinterpret_cast<uint4*>(a.v_pool + dst) = vv[i];
+      const __nv_bfloat162* k2 = reinterpret_cast<const __nv_bfloat162*>(&kk[i]);
+#pragma unroll
+      for (int e = 0; e < 4; ++e) {
+        const float2 f = __bfloat1622float2(k2[e]);
+        acc[2 * e] += f.x;
+        acc[2 * e + 1] += f.y;
+      }
     }
   }
   // Rows of a partial tail page past the last token are zero-filled: the forward kernel masks

@@ -120,25 +120,6 @@ __device__ __forceinline__ float ex2v(float x) {
   asm volatile("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// from the same place in the shared memory of the cluster's CTA `rank`
-__device__ __forceinline__ uint32_t cluster_addr(const float* p, int rank) {
-  uint32_t a;
-  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
-  return a;
-}
-__device__ __forceinline__ float ld_cluster(const float* p, int rank) {
-  float v;
-  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr(p, rank)) : "memory");
-  return v;
-}
-__device__ __forceinline__ float4 ld_cluster4(const float* p, int rank) {
-  float4 v;
-  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-               : "r"(cluster_addr(p, rank))
-               : "memory");
-  return v;
-}
 // either feature map without a branch: max(x, 0) + w * exp(min(x, 0)) with w = 1 (elu + 1) or 0 (relu)
 __device__ __forceinline__ float phi_q(float x, float w) {
   return fmaf(w, ex2(fminf(x, 0.f) * 1.4426950408889634f), fmaxf(x, 0.f));

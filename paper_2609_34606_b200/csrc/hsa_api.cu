@@ -153,6 +153,7 @@ struct hsa_ctx {
   int64_t tail_saved_for;  // history length whose tail-block key sum sits in the saved-tail buffer (-1: none)
   int nsm;
   int clusters[3];      // clusters of 2, 4 and 8 CTAs of the forward kernel that run at once
+  int lc_clusters[3];   // the same of the Linformer compression kernel
   CUtensorMap tm_k, tm_v, tm_state, tm_kc, tm_vc, tm_olin, tm_ek, tm_ev, tm_phik, tm_num;
   int32_t n_segs;  // Linformer: complete segments compressed so far
   std::vector<int32_t> page_table_host;  // history block -> physical page
@@ -312,7 +313,7 @@ int hsa_create(hsa_ctx** out, const hsa_config* cfg, const hsa_buffers* bufs,
   if (e == cudaSuccess) e = linear_only_init();
   if (e == cudaSuccess) e = causal_linear_init();
   if (e == cudaSuccess && linformer) {
-    e = linformer_init();
+    e = linformer_init(ctx->lc_clusters);
     // identity page table and "every page" selection of the compressed pool
     std::vector<int32_t> iota(ctx->lay.n_cpages);
     for (size_t i = 0; i < iota.size(); ++i) iota[i] = static_cast<int32_t>(i);
@@ -424,7 +425,7 @@ int hsa_append_kv(hsa_ctx* ctx, const void* k, const void* v, int32_t n_tokens, 
     la.seg_tokens = ctx->cfg.lin_seg_tokens;
     la.seg_index = ctx->n_segs;
     la.status = a.status;
-    e = launch_linformer_compress(la, ctx->tm_ek, ctx->tm_ev, maps.kin, maps.vin, static_cast<cudaStream_t>(stream));
+    e = launch_linformer_compress(la, ctx->lc_clusters, ctx->tm_ek, ctx->tm_ev, maps.kin, maps.vin, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     // pages and key sums of the chunk: launched behind the compression kernel, runs beside it (the
     // two write nothing in common) and ends after it

@@ -199,9 +199,11 @@ struct AppendMaps {
   CUtensorMap kin, vin, kpool, vpool;
 };
 cudaError_t launch_append(const AppendArgs& a, const AppendMaps* maps, cudaStream_t st);
-cudaError_t launch_linformer_compress(const LinformerArgs& a, const CUtensorMap& tm_ek, const CUtensorMap& tm_ev,
-                                      const CUtensorMap& tm_kin, const CUtensorMap& tm_vin, cudaStream_t st);
-cudaError_t linformer_init();
+// clusters: how many clusters of 2, 4 and 8 CTAs of the compression kernel the device runs at once (linformer_init)
+cudaError_t launch_linformer_compress(const LinformerArgs& a, const int (&clusters)[3], const CUtensorMap& tm_ek,
+                                      const CUtensorMap& tm_ev, const CUtensorMap& tm_kin, const CUtensorMap& tm_vin,
+                                      cudaStream_t st);
+cudaError_t linformer_init(int (&clusters)[3]);
 struct AdaptiveArgs {
   double* sorted_w;      // [H][n_groups][max_pages] softmax numerators in sorted order
   int32_t* sorted_idx;   // [H][n_groups][max_pages] block ids in sorted order

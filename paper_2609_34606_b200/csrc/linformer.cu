@@ -5,10 +5,17 @@
 //
 // One CTA computes a [128 rows of r] x [128 dims] tile of K~ or V~ for one head:
 //   C (fp32 in TMEM) = sum over token blocks of  E[tokens, 128 r]^T  X[tokens, 128 d]
-// One lane brings the [64 tokens x 128] tiles of E and of X into a four-stage ring by TMA (both land
+// One lane brings the [64 tokens x 128] tiles of E and of X into a ring by TMA (both land
 // in the 128-byte-swizzled MN-major layout the tensor cores take as they are; rows past the end of
 // the segment arrive as zeros), one lane issues four tcgen05 MMAs per block (K = tokens) and hands the
 // stage back, and at the end all warps write the bf16 rows to the compressed pool.
+//
+// What bounds a tile is what one SM has in flight, a ring of a stream with 1.5 us of latency, so the token blocks of a tile
+// are split over the 2, 4 or 8 CTAs of a cluster where the device runs that many at once: each leaves its fp32 sums
+// in its dead ring, and behind a cluster barrier adds up its share of the rows over all of them, in order.  The append of
+// a segment (this kernel, launched as a programmatic dependent, and the page write beside it), heads x tokens at rank
+// 256, a tile per CTA and a ring of four stages -> now, six stages: 12 x 4680 38.6 -> 28.3 us (144 MB), 16 x 4680 43.3 ->
+// 35.7, 2 x 4680 19.9 -> 14.5, 8 x 2000 14.5 -> 12.6; clusters with four stages 29.5, 35.8, 14.8, 12.8.
 #include <cuda_bf16.h>
 
 #include "hsa_internal.h"
@@ -19,7 +26,7 @@ namespace hsa {
 namespace {
 
 constexpr int kLcThreads = 512;
-constexpr int kLcDepth = 4;
+constexpr int kLcDepth = 6;
 constexpr int kLcTile = 64 * 128 * 2;
 constexpr int kLcStage = 2 * kLcTile;  // E tile | X tile
 constexpr int kLcSmem = kLcDepth * kLcStage + 256 + 1024;
@@ -31,6 +38,9 @@ struct LcBars {
   uint32_t tmem_base;
   volatile int abort_flag;
 };
+constexpr int kLcPitch = 132;  // floats per row of the sums left for the cluster
+static_assert(128 * kLcPitch * 4 <= kLcDepth * kLcStage, "the sums fit the ring");
+constexpr int kLcPart = 4;     // token blocks of a part at least
 
 __device__ __forceinline__ bool lc_wait(uint64_t* bar, uint32_t parity, LcBars* bars, int32_t* status) {
   if (mbar_try_wait(bar, parity)) return true;
@@ -45,6 +55,7 @@ __device__ __forceinline__ bool lc_wait(uint64_t* bar, uint32_t parity, LcBars* 
 
 }  // namespace
 
+template <int C>  // CTAs of a cluster, which share a tile
 __global__ void __launch_bounds__(kLcThreads, 1)
 linformer_compress_kernel(LinformerArgs a, const __grid_constant__ CUtensorMap tm_ek, const __grid_constant__ CUtensorMap tm_ev,
                           const __grid_constant__ CUtensorMap tm_kin, const __grid_constant__ CUtensorMap tm_vin) {
@@ -55,16 +66,15 @@ linformer_compress_kernel(LinformerArgs a, const __grid_constant__ CUtensorMap t
   LcBars* bars = reinterpret_cast<LcBars*>(smem + kLcDepth * kLcStage);
   const int h = blockIdx.y;
   const int rtiles = (a.rank + 127) / 128;  // (the last tile may hold 64 rows only: E reads as zeros beyond the rank)
-  const int which = blockIdx.x / rtiles;  // 0: keys, 1: values
-  const int rt = blockIdx.x % rtiles;
+  const int part_c = blockIdx.x % C, tile = blockIdx.x / C;
+  const int which = tile / rtiles;  // 0: keys, 1: values
+  const int rt = tile % rtiles;
   const CUtensorMap* tm_e = which == 0 ? &tm_ek : &tm_ev;  // [H][seg_tokens][rank], box 64 r x 64 tokens
   const CUtensorMap* tm_x = which == 0 ? &tm_kin : &tm_vin;  // [tokens][H][d], box 64 d x 1 x 64 tokens
   __nv_bfloat16* pool = which == 0 ? a.kc_pool : a.vc_pool;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int nblk = (a.seg_tokens + kBlock - 1) / kBlock;
-  // the page-write kernel of the same append is launched behind this one as a programmatic
-  // dependent and may run beside it (it touches none of this kernel's outputs)
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int blocks = (a.seg_tokens + kBlock - 1) / kBlock;
+  const int b_lo = blocks * part_c / C, nblk = blocks * (part_c + 1) / C - b_lo;  // this CTA's token blocks
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < kLcDepth; ++s) {
@@ -74,12 +84,18 @@ linformer_compress_kernel(LinformerArgs a, const __grid_constant__ CUtensorMap t
     mbar_init(&bars->all_done, 1);
     bars->abort_flag = 0;
     fence_mbar_init();
+    // launched as a programmatic dependent: everything before this kernel is complete from here on, for this CTA's
+    // loads and, since the trigger comes after the wait, for the page-write kernel of the same append, which is
+    // launched behind this one, may run beside it (it touches none of this kernel's outputs) and does not wait itself
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     if (blockIdx.x == 0) a.ccnt[h] = (a.seg_index + 1) * (a.rank / kBlock);  // compressed pages now valid
   }
   if (warp == 0) {
     tmem_alloc(&bars->tmem_base, 128);
     tmem_relinquish();
   }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -88,17 +104,22 @@ linformer_compress_kernel(LinformerArgs a, const __grid_constant__ CUtensorMap t
   if (warp == 1) {
     // ------------------------------------------------------------------ producer (one lane)
     if (elect_one_sync()) {
+      int armed = 0;
       for (int bi = 0; bi < nblk; ++bi) {
         const int s = bi % kLcDepth;
         if (bi >= kLcDepth && !lc_wait(&bars->empty[s], ((bi / kLcDepth) - 1) & 1, bars, a.status)) break;
+        ++armed;
         uint8_t* st_e = smem + s * kLcStage;
         uint8_t* st_x = st_e + kLcTile;
         mbar_expect_tx(&bars->full[s], kLcStage);
         for (int half = 0; half < 2; ++half) {
-          tma_load_3d(st_e + half * (kLcTile / 2), tm_e, &bars->full[s], rt * 128 + half * 64, bi * kBlock, h);
-          tma_load_3d(st_x + half * (kLcTile / 2), tm_x, &bars->full[s], half * 64, h, bi * kBlock);
+          tma_load_3d(st_e + half * (kLcTile / 2), tm_e, &bars->full[s], rt * 128 + half * 64, (b_lo + bi) * kBlock, h);
+          tma_load_3d(st_x + half * (kLcTile / 2), tm_x, &bars->full[s], half * 64, h, (b_lo + bi) * kBlock);
         }
       }
+      if (armed < nblk)  // let every copy already issued land before the CTA's shared memory goes away
+        for (int s = 0; s < kLcDepth; ++s)
+          if (armed > s) mbar_wait(&bars->full[s], ((armed - 1 - s) / kLcDepth) & 1, 1u << 16);
     }
   } else if (warp == 0) {
     // ------------------------------------------------------------------ MMA issuer (one lane)
@@ -124,20 +145,57 @@ linformer_compress_kernel(LinformerArgs a, const __grid_constant__ CUtensorMap t
   __syncwarp();
   const bool ok = lc_wait(&bars->all_done, 0, bars, a.status);
   tc_fence_after();
-  const int rr = rt * 128 + (warp & 3) * 32 + lane;  // row of the compressed segment
-  if (ok && rr < a.rank) {                            // (warp-uniform: the rank is a multiple of 64)
-    const int quad = warp & 3, part = warp >> 2;
-    uint32_t v[32];
-    tmem_ld32(tmem + (static_cast<uint32_t>(quad * 32) << 16) + part * 32, v);
-    tc_wait_ld();
+  const int quad = warp & 3, part = warp >> 2;
+  auto out_row = [&](int rr) {  // row of the compressed segment
     const int page = a.seg_index * (a.rank / kBlock) + rr / kBlock;
-    __nv_bfloat16* dst = pool + ((static_cast<size_t>(page) * a.H + h) * kBlock + (rr % kBlock)) * D + part * 32;
-    uint32_t pk[16];
+    return pool + ((static_cast<size_t>(page) * a.H + h) * kBlock + (rr % kBlock)) * D;
+  };
+  uint32_t v[32];
+  if constexpr (C > 1) {
+    auto cluster_sync = [] {
+      asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+      asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    };
+    float* sums = reinterpret_cast<float*>(smem);
+    float* mine = sums + (quad * 32 + lane) * kLcPitch + part * 32;
+    if (ok) {
+      tmem_ld32(tmem + (static_cast<uint32_t>(quad * 32) << 16) + part * 32, v);
+      tc_wait_ld();
+    }
 #pragma unroll
-    for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+    for (int i = 0; i < 32; i += 4)  // (a part that gave up counts for nothing; the status word says so)
+      *reinterpret_cast<float4*>(mine + i) = ok ? make_float4(__uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]),
+                                                               __uint_as_float(v[i + 3]))
+                                                : make_float4(0.f, 0.f, 0.f, 0.f);
+    __syncwarp();
+    cluster_sync();
 #pragma unroll
-    for (int i = 0; i < 4; ++i)
-      reinterpret_cast<uint4*>(dst)[i] = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+    for (int i = 0; i < 128 / C * 32 / kLcThreads; ++i) {
+      const int f = threadIdx.x + kLcThreads * i;  // (row of this CTA's share, four columns)
+      const int row = part_c * (128 / C) + f / 32, col = f % 32 * 4;
+      float4 x[C];
+#pragma unroll
+      for (int c = 0; c < C; ++c) x[c] = ld_cluster4(sums + row * kLcPitch + col, c);
+      float4 t = x[0];
+#pragma unroll
+      for (int c = 1; c < C; ++c) t = make_float4(t.x + x[c].x, t.y + x[c].y, t.z + x[c].z, t.w + x[c].w);
+      const int rr = rt * 128 + row;
+      if (rr < a.rank) *reinterpret_cast<uint2*>(out_row(rr) + col) = make_uint2(pack_bf16(t.x, t.y), pack_bf16(t.z, t.w));
+    }
+    cluster_sync();  // (nobody leaves while its sums are being read)
+  } else {
+    const int rr = rt * 128 + quad * 32 + lane;
+    if (ok && rr < a.rank) {  // (warp-uniform: the rank is a multiple of 64)
+      tmem_ld32(tmem + (static_cast<uint32_t>(quad * 32) << 16) + part * 32, v);
+      tc_wait_ld();
+      uint32_t pk[16];
+#pragma unroll
+      for (int i = 0; i < 16; ++i) pk[i] = pack_bf16(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+      __nv_bfloat16* dst = out_row(rr) + part * 32;
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        reinterpret_cast<uint4*>(dst)[i] = make_uint4(pk[4 * i], pk[4 * i + 1], pk[4 * i + 2], pk[4 * i + 3]);
+    }
   }
   tc_fence_before();
   __syncthreads();
@@ -147,16 +205,53 @@ linformer_compress_kernel(LinformerArgs a, const __grid_constant__ CUtensorMap t
   }
 }
 
-cudaError_t linformer_init() {
-  return cudaFuncSetAttribute(linformer_compress_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kLcSmem);
+namespace {
+using LcKernel = void (*)(LinformerArgs, CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap);
+LcKernel lc_kernel(int lg) {
+  return lg == 3 ? linformer_compress_kernel<8> : lg == 2 ? linformer_compress_kernel<4> : lg == 1 ? linformer_compress_kernel<2>
+                                                                                                   : linformer_compress_kernel<1>;
+}
+struct LcLaunch {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr[2];
+  LcLaunch(dim3 grid, int cluster, cudaStream_t st) {
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kLcThreads);
+    cfg.dynamicSmemBytes = kLcSmem;
+    cfg.stream = st;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = cluster;
+    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = cluster > 1 ? 2 : 1;
+  }
+};
+}  // namespace
+
+cudaError_t linformer_init(int (&clusters)[3]) {
+  cudaError_t e = cudaSuccess;
+  for (int lg = 0; lg <= 3 && e == cudaSuccess; ++lg)
+    e = cudaFuncSetAttribute(lc_kernel(lg), cudaFuncAttributeMaxDynamicSharedMemorySize, kLcSmem);
+  for (int lg = 1; lg <= 3 && e == cudaSuccess; ++lg) {
+    LcLaunch l(dim3(1 << lg), 1 << lg, nullptr);
+    if (cudaOccupancyMaxActiveClusters(&clusters[lg - 1], reinterpret_cast<const void*>(lc_kernel(lg)), &l.cfg) != cudaSuccess) {
+      cudaGetLastError();
+      clusters[lg - 1] = 0;  // no clusters of this size on this device
+    }
+  }
+  return e;
 }
 
-cudaError_t launch_linformer_compress(const LinformerArgs& a, const CUtensorMap& tm_ek, const CUtensorMap& tm_ev,
-                                      const CUtensorMap& tm_kin, const CUtensorMap& tm_vin, cudaStream_t st) {
-  dim3 grid(2 * ((a.rank + 127) / 128), a.H);
-  linformer_compress_kernel<<<grid, kLcThreads, kLcSmem, st>>>(a, tm_ek, tm_ev, tm_kin, tm_vin);
-  return cudaGetLastError();
+cudaError_t launch_linformer_compress(const LinformerArgs& a, const int (&clusters)[3], const CUtensorMap& tm_ek,
+                                      const CUtensorMap& tm_ev, const CUtensorMap& tm_kin, const CUtensorMap& tm_vin,
+                                      cudaStream_t st) {
+  const int tiles = 2 * ((a.rank + 127) / 128), blocks = (a.seg_tokens + kBlock - 1) / kBlock;
+  int lg = 0;
+  while (lg < 3 && tiles * a.H <= clusters[lg] && blocks >> (lg + 1) >= kLcPart) ++lg;
+  LcLaunch l(dim3(tiles << lg, a.H), 1 << lg, st);
+  return cudaLaunchKernelEx(&l.cfg, lc_kernel(lg), a, tm_ek, tm_ev, tm_kin, tm_vin);
 }
 
 }  // namespace hsa

@@ -281,6 +281,27 @@ __device__ __forceinline__ void tmem_st16(uint32_t taddr, const uint32_t (&r)[16
       : "memory");
 }
 
+// ----------------------------------------------------------------------------- clusters
+// from the same place in the shared memory of the cluster's CTA `rank`
+__device__ __forceinline__ uint32_t cluster_addr(const float* p, int rank) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(smem_u32(p)), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ float ld_cluster(const float* p, int rank) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr(p, rank)) : "memory");
+  return v;
+}
+__device__ __forceinline__ float4 ld_cluster4(const float* p, int rank) {
+  float4 v;
+  asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(cluster_addr(p, rank))
+               : "memory");
+  return v;
+}
+
 // ----------------------------------------------------------------------------- descriptors
 // Shared-memory matrix descriptor, 128-byte swizzle, tiles whose rows are 128 bytes long and
 // whose 8-row groups are 1024 bytes apart (exactly what a TMA box with a 128-byte inner extent

@@ -667,6 +667,31 @@ def test_gate_tiles_in_every_instance(d, form, hot, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("H,tokens,rank", [(20, 600, 256), (12, 300, 128), (12, 513, 256), (3, 1088, 64), (2, 2049, 192), (1, 64, 64)])
+def test_compressed_segments_by_clusters(H, tokens, rank, cuda_device):
+    """A tile's token blocks in one CTA (many tiles, few blocks) and over clusters of 2, 4 and 8, parts of unequal length, a
+    last block of one token, a half-filled last tile: compressed rows against 64 bits, two segments."""
+    from paper_2609_34606_b200 import hsa
+    d = 128
+    g = torch.Generator().manual_seed(tokens)
+    scale = tokens ** -0.5
+    e_k, e_v = ((torch.randn(H, tokens, rank, generator=g) * scale).to(torch.bfloat16) for _ in range(2))
+    ctx = hsa.HSAContext(H, d, max_pages=(2 * tokens + 63) // 64, max_q_tokens=tokens, max_topk=1, device=cuda_device,
+                         lin_mode=hsa.HSA_LIN_LINFORMER, lin_rank=rank, lin_seg_tokens=tokens, e_k=e_k.to(cuda_device),
+                         e_v=e_v.to(cuda_device))
+    for seg in range(2):
+        k, v = _randn(g, tokens, H, d), _randn(g, tokens, H, d)
+        ctx.append_kv(k.to(cuda_device), v.to(cuda_device))
+        assert ctx.device_status() == 0
+        pages = rank // 64
+        for pool, e, x in ((ctx.kc_pool, e_k, k), (ctx.vc_pool, e_v, v)):
+            got = pool.view(torch.bfloat16).view(-1, H, 64, d)[seg * pages:(seg + 1) * pages].double().cpu()
+            got = got.permute(1, 0, 2, 3).reshape(H, rank, d)
+            ref = torch.einsum("htr,thd->hrd", e.double(), x.double())
+            assert float((got - ref).norm()) <= BF16_REL * float(ref.norm())
+    ctx.destroy()
+
+
 @pytest.mark.parametrize("n,group", [(700, 0), (64 * 40, 0), (700, 128)])
 def test_adaptive_lists_end_in_zeros(n, group, cuda_device):
     """What a list buffer held before the call is gone, behind the list as well."""
