@@ -75,8 +75,9 @@ typedef enum {
 #define HSA_CFG_ADAPTIVE 2u
 /* hsa_config.flags: run the selection kernel in its grid-barrier form (one cooperative launch whose
  * CTAs meet at two device-wide barriers in global memory) instead of the default form, in which the
- * CTAs of a head form a thread-block cluster and meet at hardware cluster barriers.  The library
- * falls back to the grid-barrier form by itself where clusters of 8 CTAs cannot be launched. */
+ * CTAs of a head form a thread-block cluster and meet at hardware cluster barriers (several lists per
+ * head: three kernels behind one another).  The library falls back to the grid-barrier form by itself
+ * where clusters of 8 CTAs cannot be launched. */
 #define HSA_CFG_GRID_BARRIER_SELECT 4u
 
 /* hsa_forward flags: the paper's "linear only" / "sparse only" ablation modes (Table 4) */
@@ -152,7 +153,7 @@ int hsa_append_kv(hsa_ctx* ctx, const void* k, const void* v, int32_t n_tokens,
  *   sel_cnt_dev      device int32[H][n_groups] (output).
  * Candidates: blocks with at least one token and, if causal, first token <= last query
  * position of the group.  Counts are clamped to max_topk (flagged in the status word).
- * The work is enqueued as one or two kernels (see HSA_CFG_GRID_BARRIER_SELECT); the lists are the
+ * The work is enqueued as one to three kernels (see HSA_CFG_GRID_BARRIER_SELECT); the lists are the
  * same bit for bit either way. */
 int hsa_select_blocks(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride,
                       int64_t head_stride, int64_t q_pos0, int32_t causal,
@@ -227,9 +228,8 @@ int hsa_block_resident(hsa_ctx* ctx, int32_t block, int32_t* resident_out);
  * G_h being the Gini coefficient of the sorted block weights averaged over the head's groups
  * (the paper's best setting is tau_max = 1.00, tau_min = 0.35).  Same candidates, tie rule and
  * output layout as hsa_select_blocks; entries behind a list are written as zeros.  gini_tau_out_dev:
- * optional device fp32 [2][H] receiving G_h
- * and tau_h.  Needs HSA_CFG_ADAPTIVE; HSA_ERR_UNSUPPORTED when the history has more than 8192
- * blocks. */
+ * optional device fp32 [2][H] receiving G_h and tau_h.  Needs HSA_CFG_ADAPTIVE; HSA_ERR_UNSUPPORTED
+ * when the history has more than 8192 blocks. */
 int hsa_select_blocks_adaptive(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride,
                                int64_t head_stride, int64_t q_pos0, int32_t causal, float tau_min,
                                float tau_max, int32_t q_group_tokens, int32_t* sel_idx_dev,

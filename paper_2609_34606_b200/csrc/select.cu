@@ -2,9 +2,9 @@
 //   s[h,g,b] = mean_q(g) . (Ksum[h,b] / cnt_b) * scale
 // and an exact per-(head, group) top-k by radix select, all on the device:
 // query partial sums -> scores (many CTAs) -> top-k (one block of 256 threads per head and group).
-// The stages run in one of three forms (see launch_select): a kernel for the query sums followed
-// by one thread-block cluster per head, one cooperative launch with two grid barriers, or three
-// launches.
+// The stages run in one of four forms (see launch_select): a kernel for the query sums followed
+// by one thread-block cluster per head, three launches with a score kernel for several lists per head, one
+// cooperative launch with two grid barriers, or three launches.
 #include <cuda_bf16.h>
 
 #include <cmath>
@@ -304,7 +304,7 @@ __device__ __forceinline__ void scores_item(const Blk& blk, const SelectArgs& a,
 // (mma.sync m8n8k4).  One item is a chunk of 32 candidates of one head for ALL groups, so that the
 // key sums are read once: warp w owns candidates 8 (w & 3) .. + 7 (their key sums sit in registers as
 // the B fragments of all k-steps) and rows 8 (w >> 2) .. + 7 of each batch of 16 groups, whose mean
-// queries are rebuilt in shared memory (qs: 16 rows of D + 4 doubles; the pad keeps the fragment
+// query sums are rebuilt in shared memory (qs: 16 rows of D + 4 doubles; the pad keeps the fragment
 // loads at the two wavefronts a 256-byte access needs anyway).
 constexpr int kGroupBatch = 16;
 
@@ -312,6 +312,17 @@ __device__ __forceinline__ void dmma_m8n8k4(double& d0, double& d1, double a, do
   asm volatile("mma.sync.aligned.m8n8k4.row.col.f64.f64.f64.f64 {%0, %1}, {%2}, {%3}, {%0, %1};"
                : "+d"(d0), "+d"(d1)
                : "d"(a), "d"(b));
+}
+
+// A warp's eight groups by eight candidates: arow is the lane's A fragment, kb its B fragments; s the sums at the lane's two
+// accumulator columns.  Two accumulator chains (both forms that call this round alike).
+template <int D>
+__device__ __forceinline__ void group_products(const double* arow, const float (&kb)[D / 4], double (&s)[2]) {
+  double d[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
+#pragma unroll
+  for (int kk = 0; kk < D / 4; ++kk) dmma_m8n8k4(d[kk & 1][0], d[kk & 1][1], arow[4 * kk], static_cast<double>(kb[kk]));
+  s[0] = d[0][0] + d[1][0];
+  s[1] = d[0][1] + d[1][1];
 }
 
 template <int D, bool MIXED>
@@ -361,7 +372,8 @@ __device__ __forceinline__ void scores_item_groups(const Blk& blk, const SelectA
     }
   }
   const int tiles_per_group = gtok / kTileM;
-  const double mean_scale_full = static_cast<double>(a.scale) / static_cast<double>(gtok);  // all groups but a short last one
+  const double scale_full = static_cast<double>(a.scale) / static_cast<double>(gtok);  // all groups but a short last one
+  const double scale_last = static_cast<double>(a.scale) / static_cast<double>(a.n_q - (a.n_groups - 1) * gtok);
   for (int g0 = 0; g0 < a.n_groups; g0 += GB) {
     // mean queries of groups g0 .. g0 + 15 (tile sums added in ascending tile order, fp64)
     constexpr int NV = GB * D / 256;  // values per thread
@@ -383,26 +395,24 @@ __device__ __forceinline__ void scores_item_groups(const Blk& blk, const SelectA
 #pragma unroll
     for (int v = 0; v < NV; ++v) {
       const int idx = blk.tid + 256 * v;
-      const int gi = idx / D, g = g0 + gi;
-      const int q_lo = g * gtok, q_hi = min(a.n_q, q_lo + gtok);
-      const double ms = (q_hi - q_lo == gtok) ? mean_scale_full : static_cast<double>(a.scale) / static_cast<double>(q_hi - q_lo);
-      qs[gi * PITCH + idx % D] = g < a.n_groups ? sum[v] * ms : 0.0;
+      qs[idx / D * PITCH + idx % D] = sum[v];
     }
     blk_sync(blk);
     const int row0 = 8 * (warp >> 2);  // this warp's eight rows of the batch
     if (g0 + row0 < a.n_groups && c0 < cg.nc) {  // warp-uniform
       // A fragment: element (m = lane / 4, k = lane % 4) of every k-step
       const double* arow = qs + (row0 + (lane >> 2)) * PITCH + (lane & 3);
-      double d0 = 0.0, d1 = 0.0;
-#pragma unroll
-      for (int kk = 0; kk < KS; ++kk) dmma_m8n8k4(d0, d1, arow[4 * kk], static_cast<double>(kb[kk]));
+      double d[2];
+      group_products<D>(arow, kb, d);
       // accumulator: row lane / 4 (group), columns 2 (lane % 4) and + 1 (candidates)
       const int g = g0 + row0 + (lane >> 2);
       if (g < a.n_groups) {
         uint32_t* keys = a.keys + (static_cast<size_t>(h) * a.n_groups + g) * a.max_pages;
         const int c = c0 + 2 * (lane & 3);
-        if (c < cg.nc) keys[c] = masked[0] ? 0u : order_key(static_cast<float>(d0 * inv_cnt[0]));
-        if (c + 1 < cg.nc) keys[c + 1] = masked[1] ? 0u : order_key(static_cast<float>(d1 * inv_cnt[1]));
+        const double sc = g == a.n_groups - 1 ? scale_last : scale_full;
+#pragma unroll
+        for (int t = 0; t < 2; ++t)
+          if (c + t < cg.nc) keys[c + t] = masked[t] ? 0u : order_key(static_cast<float>(d[t] * sc * inv_cnt[t]));
       }
     }
     blk_sync(blk);
@@ -500,9 +510,8 @@ __global__ void __launch_bounds__(256) group_scores_kernel(SelectArgs a, int bat
     const int row0 = 8 * (warp >> 2);  // this warp's eight rows of the batch
     if (g0 + row0 < g_hi && c0 < cg.nc) {  // warp-uniform
       const double* arow = qs[buf] + (row0 + (lane >> 2)) * PITCH + (lane & 3);
-      double d[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-#pragma unroll
-      for (int kk = 0; kk < KS; ++kk) dmma_m8n8k4(d[kk & 1][0], d[kk & 1][1], arow[4 * kk], static_cast<double>(kb[kk]));
+      double d[2];
+      group_products<D>(arow, kb, d);
       const int g = g0 + row0 + (lane >> 2);
       if (g < g_hi) {
         uint32_t* keys = a.keys + (static_cast<size_t>(h) * a.n_groups + g) * a.max_pages;
@@ -510,7 +519,7 @@ __global__ void __launch_bounds__(256) group_scores_kernel(SelectArgs a, int bat
         const double sc = g == a.n_groups - 1 ? scale_last : scale_full;
 #pragma unroll
         for (int t = 0; t < 2; ++t)
-          if (c + t < cg.nc) keys[c + t] = masked[t] ? 0u : order_key(static_cast<float>((d[0][t] + d[1][t]) * sc * inv_cnt[t]));
+          if (c + t < cg.nc) keys[c + t] = masked[t] ? 0u : order_key(static_cast<float>(d[t] * sc * inv_cnt[t]));
       }
     }
   }
@@ -1131,7 +1140,7 @@ __global__ void __launch_bounds__(256 * kSubBlocks, 1) select_cluster_kernel(Sel
   const int slot = (static_cast<int>(blockIdx.x) % cluster_ctas) * kSubBlocks + sub;
   const int n_slots = cluster_ctas * kSubBlocks;
   const int n_chunks = (cand_geom<MIXED>(a).nc + kScoreBlocksPerCta - 1) / kScoreBlocksPerCta;
-  // (one list per head: the launcher sends per-tile selections to the grid-barrier form)
+  // (one list per head: the launcher sends per-tile selections elsewhere)
   // The key sums of this block's first score item are requested first, ahead of the wait for the
   // kernel before this one: that kernel (the query tile sums) writes none of them, and it has itself
   // waited for everything before it, so they are final when any CTA of this grid runs.
