@@ -1381,6 +1381,14 @@ bool launch_cluster(const SelectArgs& a, const AdaptiveArgs* ad, bool mixed, cud
 }  // namespace
 
 namespace {
+// Dynamic shared memory for the keys of a head: launch_select takes no more (nblk * 4, see the entry points).  The limit is
+// the same whoever sets it, so that threads with histories of different lengths never lower it for one another
+// between setting it and launching.
+constexpr int kKeysSmemMax = 200 * 1024;
+cudaError_t allow_keys_smem(const void* fn) {
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kKeysSmemMax);
+}
+
 const void* group_scores(int D, bool mixed) {
   if (D == 128)
     return mixed ? reinterpret_cast<const void*>(group_scores_kernel<128, true>) : reinterpret_cast<const void*>(group_scores_kernel<128, false>);
@@ -1424,8 +1432,10 @@ cudaError_t launch_select(const SelectArgs& a, cudaStream_t st) {
                                          : reinterpret_cast<const void*>(select_fused_kernel<128, false>))
                                 : (mixed ? reinterpret_cast<const void*>(select_fused_kernel<64, true>)
                                          : reinterpret_cast<const void*>(select_fused_kernel<64, false>));
-    if (smem_keys > 24 * 1024)
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem_keys));
+    if (smem_keys > 24 * 1024) {
+      const cudaError_t e = allow_keys_smem(fn);
+      if (e != cudaSuccess) return e;
+    }
     // 256 threads, at most 80 registers and under 12 KB of shared memory per CTA plus the keys:
     // three CTAs per SM are co-resident while the keys stay below 48 KB
     int per_sm = 3;
@@ -1461,7 +1471,7 @@ cudaError_t launch_select(const SelectArgs& a, cudaStream_t st) {
   }
   const size_t smem = static_cast<size_t>(nblk_all > 0 ? nblk_all : 1) * sizeof(uint32_t);
   const void* f3 = mixed ? reinterpret_cast<const void*>(topk_kernel<true>) : reinterpret_cast<const void*>(topk_kernel<false>);
-  if (smem > 40 * 1024) cudaFuncSetAttribute(f3, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  if (smem > 40 * 1024 && (e = allow_keys_smem(f3)) != cudaSuccess) return e;
   return launch_pdl(f3, dim3(a.n_groups, a.H), dim3(256), smem, p_args, st);
 }
 

@@ -25,6 +25,7 @@ std::map<std::pair<int, const void*>, int> g_smem_limit;
 std::map<unsigned long long, int> g_capturing;
 std::vector<Launch> g_launches;
 int g_device = 0, g_set_attribute_calls = 0;
+void (*g_on_smem_limit)() = nullptr;
 cudaError_t g_last = cudaSuccess;
 dim3 g_push_grid, g_push_block;
 size_t g_push_smem;
@@ -49,6 +50,8 @@ void fake_reset() {
 }
 void fake_set_device(int d) { g_device = d; }
 void fake_set_capturing(unsigned long long stream, int on) { g_capturing[stream] = on; }
+// called once, behind the next shared-memory limit that is set: what another thread may do there
+void fake_on_smem_limit(void (*fn)()) { g_on_smem_limit = fn; }
 int fake_launches() { return static_cast<int>(g_launches.size()); }
 int fake_set_attribute_calls() { return g_set_attribute_calls; }
 int fake_launch(int i, char* name, int size, int* grid3, long long* smem) {
@@ -92,7 +95,13 @@ cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* fn, voi
 }
 cudaError_t cudaFuncSetAttribute(const void* fn, cudaFuncAttribute attr, int value) {
   ++g_set_attribute_calls;
-  if (attr == cudaFuncAttributeMaxDynamicSharedMemorySize) g_smem_limit[{g_device, fn}] = value;
+  if (attr == cudaFuncAttributeMaxDynamicSharedMemorySize) {
+    g_smem_limit[{g_device, fn}] = value;
+    if (void (*other)() = g_on_smem_limit) {
+      g_on_smem_limit = nullptr;
+      other();
+    }
+  }
   return cudaSuccess;
 }
 cudaError_t cudaGetDevice(int* d) {

@@ -57,8 +57,8 @@ class Context:
     def q_args(self, n_q):
         return self.ctx, C.c_void_p(0x1000), n_q, C.c_int64(self.H * self.d), C.c_int64(self.d), C.c_int64(1 << 40), 0
 
-    def select(self, n_q=256):
-        return self.lib.hsa_select_blocks(*self.q_args(n_q), C.c_void_p(0x3000), 0, C.c_void_p(0x4000), C.c_void_p(0x5000), None)
+    def select(self, n_q=256, group=0):
+        return self.lib.hsa_select_blocks(*self.q_args(n_q), C.c_void_p(0x3000), group, C.c_void_p(0x4000), C.c_void_p(0x5000), None)
 
     def select_adaptive(self, n_q=256):
         return self.lib.hsa_select_blocks_adaptive(*self.q_args(n_q), C.c_float(0.35), C.c_float(1.0), 0, C.c_void_p(0x4000),
@@ -92,6 +92,20 @@ def test_selection_on_every_device_of_a_process(lib, d, n_blocks, adaptive):
             assert (ctx.select_adaptive(n_q) if adaptive else ctx.select(n_q)) == 0
             names = [l[0] for l in launches(lib)]
             assert names and all(l[3] == dev for l in launches(lib)) and "select_cluster" in names[-1]
+
+
+@pytest.mark.parametrize("kernel,group,flags", [("topk_kernel", 128, 0), ("select_fused", 0, 4), ("select_fused", 128, 4)])
+def test_selections_of_two_threads_keep_each_others_shared_memory(lib, kernel, group, flags):
+    """A selection over a shorter history that another thread issues between the shared-memory limit and the launch
+    of one over a longer history does not lower the limit under it."""
+    long, short = (Context(lib, 2, 128, n, 64, n=n * 64, flags=flags) for n in (50000, 11000))
+    results = []
+    other = C.CFUNCTYPE(None)(lambda: results.append(short.select(256, group)))
+    lib.fake_reset()
+    lib.fake_on_smem_limit(other)
+    assert long.select(256, group) == 0 and results == [0]
+    used = [l[2] for l in launches(lib) if kernel in l[0]]
+    assert used == [11000 * 4, 50000 * 4]
 
 
 def test_forwards_of_short_lists_share_no_scratch(lib):
