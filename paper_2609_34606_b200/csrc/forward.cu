@@ -1081,12 +1081,14 @@ hsa_forward_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
         const int64_t g_ds = p.g_ds;
         // (decided from the launch parameters, not from this thread's pointers: the branch holds
         // warp-collective TMEM loads and must not diverge inside a warp)
-        const bool plain = (p.g_ds == 0 || (!p.g_lin && !p.g_sp)) && (NUMT || !(p.do_linear && p.lin_num != nullptr)) && !p.ext_lin &&
+        const bool plain = ((p.g_ds == 0 && p.gate_act == 1) || (!p.g_lin && !p.g_sp)) && (NUMT || !(p.do_linear && p.lin_num != nullptr)) && !p.ext_lin &&
                            !(PARTS && nsplit > 1);
         if (plain) {
-          // no gates but one per token and head, which go into the row's two factors, no causal partials but a tile's, no
-          // external linear output, no merge: 32 columns per trip.  (Gates per token and head in the 16-column trips of
-          // the general loop: 42.2 us a pass, 16 heads of 64, 1000 tokens, against 41.4.)
+          // no gates but the sigmoid of one per token and head, which goes into the row's two factors, no causal partials but
+          // a tile's, no external linear output, no merge: 32 columns per trip.  (Such gates in the 16-column trips of
+          // the general loop: 42.2 us a pass, 16 heads of 64, 1000 tokens, against 41.4.  Gates that are used as given
+          // take that loop, where they meet a branch that is normalised already: gate over denominator alone
+          // can leave the range of fp32 where the result does not.)
           const float il = has_o ? inv_l * ws0 : 0.f, id = has_lin ? inv_den * wl0 : 0.f;
 #pragma unroll 1
           for (int c0 = cbase; c0 < cbase + HC; c0 += 32) {

@@ -620,6 +620,34 @@ def test_gates_with_a_dim_stride_beyond_32_bits(flags, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("d,causal", [(64, False), (128, False), (128, True)])
+def test_large_gates_over_a_small_denominator(d, causal, cuda_device):
+    """Gates that are used as given, 1e7 and more, on rows whose phi(q) . z is below 1e-32: the gate over the denominator
+    alone would be beyond fp32, the result is not; per token and head as per dim."""
+    from paper_2609_34606_b200 import hsa
+    H, n = 2, 200
+    g = torch.Generator().manual_seed(d)
+    V = _randn(g, n, H, d)
+    K, q = torch.zeros_like(V), torch.full_like(V, -84.0)
+    ctx = hsa.HSAContext(H, d, max_pages=4, max_q_tokens=n, max_topk=4, causal=causal, device=cuda_device)
+    ctx.append_kv(K.to(cuda_device), V.to(cuda_device))
+    qd, pos = q.to(cuda_device), 0 if causal else n
+    idx, cnt = ctx.select_blocks(qd, torch.full((H,), -1, dtype=torch.int32, device=cuda_device), q_pos0=pos, causal=causal)
+    gl = (torch.rand(n, H, generator=g) * 9e7 + 1e7).to(torch.bfloat16)
+    assert float(gl.min()) / (n * d * np.exp(-84.0)) > torch.finfo(torch.float32).max  # (phi(0) = 1)
+    gs = torch.zeros(n, H, dtype=torch.bfloat16)
+    gates = lambda wide: {k: (x[:, :, None].expand(n, H, d).contiguous() if wide else x).to(cuda_device) for k, x in (("g_lin", gl), ("g_sp", gs))}
+    per_head, per_dim = (ctx.forward(qd, idx, cnt, q_pos0=pos, causal=causal, **gates(wide)).double().cpu() for wide in (False, True))
+    assert ctx.device_status() == 0
+    # every key weighs the same: the branch is the mean of the visible values
+    vd = V.double()
+    mean = vd.cumsum(0) / torch.arange(1, n + 1).view(n, 1, 1) if causal else vd.mean(0, keepdim=True).expand(n, H, d)
+    ref = gl.double()[:, :, None] * mean
+    for out in (per_head, per_dim):
+        assert float((out - ref).norm()) <= BF16_REL * float(ref.norm())
+    ctx.destroy()
+
+
 @pytest.mark.parametrize("hot", [False, True])
 @pytest.mark.parametrize("form", ["plain", "causal", "linformer", "workspace", "cluster", "causal cluster"])
 @pytest.mark.parametrize("d", [64, 128])
