@@ -348,7 +348,9 @@ chunk_sums_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_k, con
   }
 }
 
-template <int D>
+// SUMS: compiled with the sums over earlier groups; an instance of its own, since a step without them takes 4 % longer in one
+// that carries them (linear branch alone, 4 heads, 5 tiles: 43.9 us a call against 42.9)
+template <int D, bool SUMS>
 __global__ void __launch_bounds__(kClThreads, 1)
 causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_v) {  // tm_k: the phi(K) tiles
@@ -396,8 +398,8 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
   // group on (the pages of a group start where its two tiles do, less the first page's older rows).
   const int b_first = static_cast<int>(a.q_pos0 / kBlock);
   const int64_t last = a.q_pos0 + min(row0 + kTileM, a.n_q) - 1;
-  const int groups = D == 128 && a.sums ? row0 / kTileM * 2 / kClGroup : 0;  // groups before the tile's own
-  const int p0 = groups * kClGroup;                                          // first page of the steps
+  const int groups = SUMS ? row0 / kTileM * 2 / kClGroup : 0;  // groups before the tile's own
+  const int p0 = groups * kClGroup;                            // first page of the steps
   const int nsteps = static_cast<int>(last / kBlock) - b_first + 1 - p0;
 
   if (warp == 0) {
@@ -429,8 +431,8 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
       };
       // phi(K) one step further than V: its stage is free as soon as the sums of step j - 2 are formed, before
       // the weights of that step have met the V whose stage the next V takes (in one order 3500 cycles per step)
-      bool ok = groups == 0 || cl_wait(&bars->pre_low, 0, bars, a.status);
-      ok = ok && load_k(0) && (groups == 0 || cl_wait(&bars->pre_full, 0, bars, a.status));
+      bool ok = !SUMS || groups == 0 || cl_wait(&bars->pre_low, 0, bars, a.status);
+      ok = ok && load_k(0) && (!SUMS || groups == 0 || cl_wait(&bars->pre_full, 0, bars, a.status));
       for (int j = 0; j < nsteps && ok; ++j) ok = (j + 1 >= nsteps || load_k(j + 1)) && load_v(j);
       if (!ok) {  // let every copy already issued land before the CTA's shared memory goes away
         mbar_wait(&bars->q_full, 0, 1u << 16);
@@ -474,7 +476,7 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
         return true;
       };
       bool ok = cl_wait(&bars->q_read, 0, bars, a.status);  // phi(Q) is in shared memory
-      if (D == 128 && groups > 0 && ok) {
+      if (SUMS && groups > 0 && ok) {
         // the sums over earlier groups: hi hi into the place of num, the smaller products into the second buffer's
         ok = cl_wait(&bars->s_ready, 0, bars, a.status);
         if (ok) {
@@ -541,7 +543,7 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
     for (int i = 0; i < NC; ++i) num[i] = 0.f;
     const float* sums = a.sums + static_cast<size_t>(h) * a.sum_groups * kClSums;
     float* zs = reinterpret_cast<float*>(bars + 1);  // z over the groups before the tile's own
-    if (D == 128 && groups > 0) {
+    if (SUMS && groups > 0) {
       if (set == 0) {
         float z = 0.f;
         for (int u = 0; u < groups; ++u) z += __ldcg(sums + static_cast<size_t>(u) * kClSums + D * D + r);
@@ -603,7 +605,7 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
             largest = fmaxf(largest, f[c * 8 + e]);
           }
         }
-        if (D == 128 && groups > 0) {
+        if (SUMS && groups > 0) {
           float d8[8];
 #pragma unroll
           for (int i = 0; i < 32; i += 4) {
@@ -625,7 +627,7 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
       }
       __syncwarp();
       if (lane == 0) mbar_arrive(&bars->q_read);
-      if (D == 128 && groups > 0) {
+      if (SUMS && groups > 0) {
         ok = __all_sync(0xffffffffu, cl_wait(&bars->pre_full, 0, bars, a.status));
         if (ok) {
           tc_fence_after();
@@ -734,11 +736,18 @@ causal_linear_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_q, 
   }
 }
 
+namespace {
+using ClKernel = void (*)(CausalLinArgs, CUtensorMap, CUtensorMap, CUtensorMap);
+ClKernel cl_kernel(int D, bool sums) {
+  return D == 64 ? causal_linear_kernel<64, false> : sums ? causal_linear_kernel<128, true> : causal_linear_kernel<128, false>;
+}
+int cl_smem(int D) { return D == 128 ? ClSmem<128>::kTotal : ClSmem<64>::kTotal; }
+}  // namespace
+
 cudaError_t causal_linear_init() {
-  cudaError_t e = cudaFuncSetAttribute(causal_linear_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, ClSmem<128>::kTotal);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(causal_linear_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, ClSmem<64>::kTotal);
-  if (e == cudaSuccess) e = cudaFuncSetAttribute(chunk_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCsSmem);
+  cudaError_t e = cudaFuncSetAttribute(chunk_sums_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCsSmem);
+  for (int i = 0; i < 3 && e == cudaSuccess; ++i)
+    e = cudaFuncSetAttribute(cl_kernel(i == 2 ? 64 : 128, i == 1), cudaFuncAttributeMaxDynamicSharedMemorySize, cl_smem(i == 2 ? 64 : 128));
   return e;
 }
 
@@ -771,9 +780,8 @@ cudaError_t launch_causal_linear(const CausalLinArgs& a_in, const CUtensorMap& t
   }
   cfg.gridDim = dim3(static_cast<unsigned>(n_tiles) * a.H);
   cfg.blockDim = dim3(kClThreads);
-  cfg.dynamicSmemBytes = a.D == 128 ? ClSmem<128>::kTotal : ClSmem<64>::kTotal;
-  if (a.D == 128) return cudaLaunchKernelEx(&cfg, causal_linear_kernel<128>, a, tm_q, tm_k, tm_v);
-  return cudaLaunchKernelEx(&cfg, causal_linear_kernel<64>, a, tm_q, tm_k, tm_v);
+  cfg.dynamicSmemBytes = cl_smem(a.D);
+  return cudaLaunchKernelEx(&cfg, cl_kernel(a.D, a.sums != nullptr), a, tm_q, tm_k, tm_v);
 }
 
 }  // namespace hsa
