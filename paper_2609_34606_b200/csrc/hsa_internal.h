@@ -175,6 +175,8 @@ struct CausalLinArgs {
   int64_t q_pos0;   // first query position == first token of the intra-chunk part
   int H, D;
   int relu;  // feature map: 0 elu(x) + 1, 1 max(x, 0)
+  int nsm;    // SMs of the device
+  int alone;  // 1: the forward behind it is the linear branch alone
   float* lin_num;
   float* lin_den;
   int32_t* status;  // device status word

@@ -8,7 +8,7 @@
 // of the products it would be made again for every query tile behind a key; left there by the append, every
 // append would pay for it): 5 us for a chunk of 1560 tokens, 12 heads of 128.
 //
-// From kClMinTiles query tiles on (head_dim 128) a tile does not walk through all of the chunk's pages in front of it:
+// In chunks of enough query tiles (sums_pay; head_dim 128) a tile does not walk through all of the chunk's pages in front of it:
 // chunk_sums_kernel leaves T = sum_j phi(k_j) v_j^T and z = sum_j phi(k_j) over every group of four pages (two tiles)
 // in the workspace, and a tile takes phi(Q) times the sum of T over the groups before its own, then the pages from
 // its group's first on, at most five.
@@ -62,11 +62,22 @@ constexpr int kClThreads = 64 + kClWorkers;
 constexpr int kClTerms = kPhiTerms;
 constexpr int kClStages = 2;
 constexpr int kClGroup = 4;       // pages of a group: two query tiles
-// Fewest query tiles for which the sums over groups are made: their kernel is 7 us in front of the tiles, the steps that
-// they save are 1.3 us each along the longest tile.  A whole causal pass, all pages step by step -> with sums, heads x
-// tokens: 12 x 384 49.0 -> 54.3 us, 4 x 640 52.8 -> 56.1, 12 x 768 60.1 -> 59.4, 8 x 900 63.2 -> 60.4, 2 x 3000 104 ->
-// 63, 12 x 3120 211 -> 165.
-constexpr int kClMinTiles = 6;
+// Whether the sums over groups are made.  Their kernel is 5 us in front of the tiles, and the steps that they save, 1.3 us each,
+// count along the longest tile: six query tiles at least.  Step by step the tiles also end one after another, and the
+// forward's tiles start on the SMs that are left; with sums they all end together.  So on more than half of the
+// SMs, and again where the tiles take a second wave, the work has to be larger: tiles * (heads + 15), the overheads of
+// both ways being about 15 heads' worth.  A causal forward, lists of 32 blocks, all pages step by step -> with sums, heads x
+// tiles (the rule's choice last): 2 x 6 38.9 -> 37.8 us (sums), 12 x 7 45.3 -> 51.6 (steps), 12 x 8 51.4 -> 54.8 (steps), 12 x 9
+// 56.3 -> 54.5 (sums), 16 x 6 48.0 -> 53.1 (steps), 16 x 8 59.4 -> 56.9 (sums), 20 x 8 72.4 -> 80.2 (steps), 20 x 10 87.8 -> 86.1
+// (sums), 24 x 7 74.4 -> 81.1 (steps), 24 x 9 89.3 -> 85.5 (sums), 40 x 16 314 -> 243 (sums).  It errs at 4 x 7 (40.7 -> 44.7) and,
+// with lists of 8 blocks, at 12 x 8 (46.5 -> 44.4).
+constexpr int kClMinTiles = 6, kClHalfWork = 220, kClWaveWork = 340;
+bool sums_pay(int tiles, int heads, int nsm, bool alone) {
+  const int64_t items = static_cast<int64_t>(tiles) * heads, work = items + 15 * static_cast<int64_t>(tiles);
+  if (tiles < kClMinTiles) return false;
+  if (items <= (alone ? nsm : nsm / 2)) return true;
+  return work >= (items <= nsm ? kClHalfWork : kClWaveWork);
+}
 constexpr int kClSums = 128 * 128 + 128;  // floats of a group's sums
 constexpr int kCsStages = 3, kCsThreads = 192;
 constexpr int kCsSmem = kCsStages * (kClTerms + 1) * kBlock * 128 * 2 + 2048 + 256 + 1024;
@@ -770,7 +781,7 @@ cudaError_t launch_causal_linear(const CausalLinArgs& a_in, const CUtensorMap& t
   cfg.numAttrs = 1;
   const cudaError_t e = cudaLaunchKernelEx(&cfg, a.D == 128 ? phi_terms_kernel<128> : phi_terms_kernel<64>, a);
   if (e != cudaSuccess) return e;
-  if (a.D != 128 || n_tiles < kClMinTiles) a.sums = nullptr;
+  if (a.D != 128 || !sums_pay(n_tiles, a.H, a.nsm, a.alone)) a.sums = nullptr;
   if (a.sums) {
     cfg.gridDim = dim3(static_cast<unsigned>((n_tiles - 1) * 2 / kClGroup), a.H);  // (nothing reads the last tiles' own group)
     cfg.blockDim = dim3(kCsThreads);

@@ -108,6 +108,24 @@ def test_selections_of_two_threads_keep_each_others_shared_memory(lib, kernel, g
     assert used == [11000 * 4, 50000 * 4]
 
 
+@pytest.mark.parametrize("H,tiles,alone,sums", [
+    (2, 5, 0, False), (2, 6, 0, True), (12, 6, 0, True), (12, 7, 0, False), (12, 7, 1, True), (12, 8, 0, False), (12, 9, 0, True),
+    (16, 6, 0, False), (16, 8, 0, True), (20, 8, 0, False), (20, 8, 1, False), (20, 10, 0, True), (24, 9, 1, True), (40, 5, 1, False)])
+def test_causal_sums_where_they_pay(lib, H, tiles, alone, sums):
+    """Which causal chunks make sums over page groups: by query tiles, heads and whether a sparse branch follows; the products run
+    in the instance that goes with it."""
+    n = tiles * 128 - 5
+    ctx = Context(lib, H, 128, 80, 32, max_q=n, n=n, flags=1, lin_mode=1)
+    none, ts = C.c_void_p(None), C.c_int64(H * 128)
+    lib.fake_reset()
+    assert lib.hsa_forward(ctx.ctx, C.c_void_p(0x1000), n, ts, C.c_int64(128), C.c_int64(0), 1, C.c_void_p(0x4000), C.c_void_p(0x5000), 0,
+                           none, none, C.c_int64(0), C.c_int64(0), C.c_int64(0), C.c_void_p(0x6000), ts, C.c_int64(128),
+                           2 if alone else 0, none) == 0
+    names = [l[0] for l in launches(lib)]
+    assert sum("chunk_sums_kernel" in x for x in names) == sums
+    assert sum("causal_linear_kernelILi128ELb%d" % sums in x for x in names) == 1
+
+
 def test_forwards_of_short_lists_share_no_scratch(lib):
     """Two forwards of one context may run at the same time if their lists are short: they are not split through
     the workspace, which holds nothing for that, and take the same route on every stream and under capture."""
