@@ -393,6 +393,7 @@ int hsa_append_kv(hsa_ctx* ctx, const void* k, const void* v, int32_t n_tokens, 
   a.lin_state = ctx->cfg.lin_mode == HSA_LIN_STATE;
   a.relu = ctx->cfg.feature_map == HSA_PHI_RELU;
   a.status = reinterpret_cast<int32_t*>(ws + ctx->lay.status);
+  a.nsm = ctx->nsm;
   const bool linformer = ctx->cfg.lin_mode == HSA_LIN_LINFORMER;
   if (linformer && (n_tokens != ctx->cfg.lin_seg_tokens || ctx->n_tokens != static_cast<int64_t>(ctx->n_segs) * n_tokens))
     return HSA_ERR_UNSUPPORTED;  // this mode appends whole segments only
@@ -424,8 +425,9 @@ int hsa_append_kv(hsa_ctx* ctx, const void* k, const void* v, int32_t n_tokens, 
     la.rank = ctx->cfg.lin_rank;
     la.seg_tokens = ctx->cfg.lin_seg_tokens;
     la.seg_index = ctx->n_segs;
+    la.nsm = ctx->nsm;
     la.status = a.status;
-    e = launch_linformer_compress(la, ctx->lc_clusters, ctx->tm_ek, ctx->tm_ev, maps.kin, maps.vin, static_cast<cudaStream_t>(stream));
+    e = launch_linformer_compress(la, ctx->lc_clusters, &a.one_row, ctx->tm_ek, ctx->tm_ev, maps.kin, maps.vin, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(ctx, e);
     // pages and key sums of the chunk: launched behind the compression kernel, runs beside it (the
     // two write nothing in common) and ends after it

@@ -63,6 +63,8 @@ struct AppendArgs {
   int nsplit;
   int lin_state;  // update the linear state?
   int beside_prior;  // SIMT page write: may run beside the kernel launched just before it (see launch_append)
+  int one_row;       // with beside_prior: a row of a thread at a time (see launch_linformer_compress)
+  int nsm;           // SMs of the device
   int relu;       // feature map of the state: 0 elu(x) + 1, 1 max(x, 0)
   int32_t* status;  // device status word
 };
@@ -182,6 +184,8 @@ struct CausalLinArgs {
   int32_t* status;  // device status word
 };
 
+constexpr int kPageCtasPerSm = 6;  // CTAs of the page write, a row of a thread at a time, on an SM (see launch_append)
+
 struct LinformerArgs {
   const __nv_bfloat16* k;
   const __nv_bfloat16* v;
@@ -192,6 +196,7 @@ struct LinformerArgs {
   __nv_bfloat16* vc_pool;
   int32_t* ccnt;             // [H] number of valid compressed pages
   int H, rank, seg_tokens, seg_index;
+  int nsm;                   // SMs of the device
   int32_t* status;
 };
 
@@ -201,8 +206,9 @@ struct AppendMaps {
   CUtensorMap kin, vin, kpool, vpool;
 };
 cudaError_t launch_append(const AppendArgs& a, const AppendMaps* maps, cudaStream_t st);
-// clusters: how many clusters of 2, 4 and 8 CTAs of the compression kernel the device runs at once (linformer_init)
-cudaError_t launch_linformer_compress(const LinformerArgs& a, const int (&clusters)[3], const CUtensorMap& tm_ek,
+// clusters: how many clusters of 2, 4 and 8 CTAs of the compression kernel the device runs at once (linformer_init);
+// one_row (output): which form of the page write runs best beside this launch
+cudaError_t launch_linformer_compress(const LinformerArgs& a, const int (&clusters)[3], int* one_row, const CUtensorMap& tm_ek,
                                       const CUtensorMap& tm_ev, const CUtensorMap& tm_kin, const CUtensorMap& tm_vin,
                                       cudaStream_t st);
 cudaError_t linformer_init(int (&clusters)[3]);

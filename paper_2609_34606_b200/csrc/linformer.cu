@@ -213,19 +213,27 @@ LcKernel lc_kernel(int lg) {
 }
 struct LcLaunch {
   cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute attr[2];
-  LcLaunch(dim3 grid, int cluster, cudaStream_t st) {
+  cudaLaunchAttribute attr[3];
+  LcLaunch(dim3 grid, int cluster, cudaStream_t st, bool room = false) {
     cfg.gridDim = grid;
     cfg.blockDim = dim3(kLcThreads);
     cfg.dynamicSmemBytes = kLcSmem;
     cfg.stream = st;
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
-    attr[1].id = cudaLaunchAttributeClusterDimension;
-    attr[1].val.clusterDim.x = cluster;
-    attr[1].val.clusterDim.y = attr[1].val.clusterDim.z = 1;
+    int n = 1;
+    if (cluster > 1) {
+      attr[n].id = cudaLaunchAttributeClusterDimension;
+      attr[n].val.clusterDim.x = cluster;
+      attr[n].val.clusterDim.y = attr[n].val.clusterDim.z = 1;
+      ++n;
+    }
+    if (room) {
+      attr[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+      attr[n++].val.sharedMemCarveout = cudaSharedmemCarveoutMaxShared;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = cluster > 1 ? 2 : 1;
+    cfg.numAttrs = n;
   }
 };
 }  // namespace
@@ -244,13 +252,20 @@ cudaError_t linformer_init(int (&clusters)[3]) {
   return e;
 }
 
-cudaError_t launch_linformer_compress(const LinformerArgs& a, const int (&clusters)[3], const CUtensorMap& tm_ek,
+cudaError_t launch_linformer_compress(const LinformerArgs& a, const int (&clusters)[3], int* one_row, const CUtensorMap& tm_ek,
                                       const CUtensorMap& tm_ev, const CUtensorMap& tm_kin, const CUtensorMap& tm_vin,
                                       cudaStream_t st) {
-  const int tiles = 2 * ((a.rank + 127) / 128), blocks = (a.seg_tokens + kBlock - 1) / kBlock;
+  const int tiles = 2 * ((a.rank + 127) / 128), blocks = (a.seg_tokens + kBlock - 1) / kBlock, items = tiles * a.H;
   int lg = 0;
-  while (lg < 3 && tiles * a.H <= clusters[lg] && blocks >> (lg + 1) >= kLcPart) ++lg;
-  LcLaunch l(dim3(tiles << lg, a.H), 1 << lg, st);
+  while (lg < 3 && items <= clusters[lg] && blocks >> (lg + 1) >= kLcPart) ++lg;
+  // The page write beside this kernel, a CTA per block and head, a row of a thread at a time: six CTAs fit an SM that this kernel
+  // leaves free, three beside one of its CTAs, but these only if the SM's memory is split for it (the ring alone asks
+  // for the next smaller split, all of which it takes).  Where not even that runs all of them at once, they ask for
+  // all rows of a thread, four to a free SM, and come in waves.
+  const int pages = blocks * a.H, ctas = items << lg, free_ctas = kPageCtasPerSm * (a.nsm - ctas);
+  const bool room = pages > free_ctas && pages <= free_ctas + 3 * ctas;
+  *one_row = pages <= free_ctas || room;
+  LcLaunch l(dim3(tiles << lg, a.H), 1 << lg, st, room);
   return cudaLaunchKernelEx(&l.cfg, lc_kernel(lg), a, tm_ek, tm_ev, tm_kin, tm_vin);
 }
 

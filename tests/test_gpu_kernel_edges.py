@@ -720,6 +720,25 @@ def test_compressed_segments_by_clusters(H, tokens, rank, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("H,n", [(1, 1), (12, 3136), (12, 4680), (16, 4680)])
+def test_page_write_takes_rows_one_by_one_or_at_once(H, n, cuda_device):
+    """Contexts without a linear state: few CTAs, more than fit at once with all rows asked for, as many as fit one row at a
+    time, and more.  Pages bit for bit, key sums."""
+    from paper_2609_34606_b200 import hsa
+    d, blocks = 128, (n + 63) // 64
+    g = torch.Generator(device=cuda_device).manual_seed(n)
+    k, v = (torch.randn(n, H, d, generator=g, device=cuda_device).to(torch.bfloat16) for _ in range(2))
+    ctx = hsa.HSAContext(H, d, max_pages=blocks, max_q_tokens=n, max_topk=1, lin_mode=hsa.HSA_LIN_NONE, device=cuda_device)
+    ctx.append_kv(k, v)
+    assert ctx.device_status() == 0
+    pad = torch.zeros(blocks * 64 - n, H, d, dtype=torch.bfloat16, device=cuda_device)
+    for pool, x in ((ctx.k_pool, k), (ctx.v_pool, v)):
+        assert torch.equal(pool.view(torch.bfloat16).view(-1, H, 64, d), torch.cat([x, pad]).view(blocks, 64, H, d).permute(0, 2, 1, 3))
+    ref = torch.cat([k, pad]).double().view(blocks, 64, H, d).sum(1).permute(1, 0, 2)
+    assert float((ctx.ksum.double() - ref).norm()) <= 2.0 ** -24 * 12 * float(ref.norm())  # (as above)
+    ctx.destroy()
+
+
 @pytest.mark.parametrize("n,group", [(700, 0), (64 * 40, 0), (700, 128)])
 def test_adaptive_lists_end_in_zeros(n, group, cuda_device):
     """What a list buffer held before the call is gone, behind the list as well."""
