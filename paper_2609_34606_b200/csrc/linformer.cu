@@ -40,7 +40,13 @@ struct LcBars {
 };
 constexpr int kLcPitch = 132;  // floats per row of the sums left for the cluster
 static_assert(128 * kLcPitch * 4 <= kLcDepth * kLcStage, "the sums fit the ring");
-constexpr int kLcPart = 4;     // token blocks of a part at least
+// Which segments are split: the merge of a cluster is 2 us, a token block of a tile 0.15 us while few CTAs stream.  On more than
+// half of the SMs the page write beside this kernel is in the way, so only long segments go there.  An append, heads x
+// tokens at rank 256, without clusters -> with (2 CTAs unless noted): 4 x 600 6.2 -> 7.0 us, 4 x 1280 7.8 -> 7.8, 4 x 2000 9.5 -> 8.4
+// (4 CTAs), 16 x 1024 8.0 -> 9.2, 12 x 2400 12.6 -> 12.8, 12 x 3120 16.8 -> 16.3, 12 x 4680 31.7 -> 28.0.
+constexpr int kLcPart = 4;       // token blocks of a part at least
+constexpr int kLcShortest = 20;  // token blocks of a segment at least
+constexpr int kLcLong = 49;      // the same for clusters on more than half of the SMs
 
 __device__ __forceinline__ bool lc_wait(uint64_t* bar, uint32_t parity, LcBars* bars, int32_t* status) {
   if (mbar_try_wait(bar, parity)) return true;
@@ -257,7 +263,11 @@ cudaError_t launch_linformer_compress(const LinformerArgs& a, const int (&cluste
                                       cudaStream_t st) {
   const int tiles = 2 * ((a.rank + 127) / 128), blocks = (a.seg_tokens + kBlock - 1) / kBlock, items = tiles * a.H;
   int lg = 0;
-  while (lg < 3 && items <= clusters[lg] && blocks >> (lg + 1) >= kLcPart) ++lg;
+  while (lg < 3 && items <= clusters[lg] && blocks >= kLcShortest && blocks >> (lg + 1) >= kLcPart) {
+    const int ctas = items << (lg + 1);
+    if (ctas > a.nsm / 2 && (blocks < kLcLong || (lg > 0 && 3 * ctas > 2 * a.nsm))) break;
+    ++lg;
+  }
   // The page write beside this kernel, a CTA per block and head, a row of a thread at a time: six CTAs fit an SM that this kernel
   // leaves free, three beside one of its CTAs, but these only if the SM's memory is split for it (the ring alone asks
   // for the next smaller split, all of which it takes).  Where not even that runs all of them at once, they ask for

@@ -720,6 +720,38 @@ def test_compressed_segments_by_clusters(H, tokens, rank, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("H,tokens,rank", [(4, 1216, 256), (4, 1217, 256), (2, 2049, 256), (12, 3072, 256), (12, 3073, 256), (12, 3900, 256),
+                                           (16, 2000, 256), (16, 2900, 256)])
+def test_segments_at_the_edges_of_the_launch_rules(H, tokens, rank, cuda_device):
+    """Segments on both sides of the lengths that are split over clusters (of 2, 4 and 8 CTAs), with the page write in either of
+    its forms beside them and with and without room on their SMs: compressed rows against 64 bits, pages bit for
+    bit, key sums."""
+    from paper_2609_34606_b200 import hsa
+    d = 128
+    g = torch.Generator(device=cuda_device).manual_seed(tokens)
+    rand = lambda *s: torch.randn(*s, generator=g, device=cuda_device)
+    e_k, e_v = ((rand(H, tokens, rank) * tokens ** -0.5).to(torch.bfloat16) for _ in range(2))
+    blocks = (tokens + 63) // 64
+    ctx = hsa.HSAContext(H, d, max_pages=blocks, max_q_tokens=tokens, max_topk=1, device=cuda_device,
+                         lin_mode=hsa.HSA_LIN_LINFORMER, lin_rank=rank, lin_seg_tokens=tokens, e_k=e_k, e_v=e_v)
+    ctx.k_pool.fill_(0xFF)
+    ctx.v_pool.fill_(0xFF)
+    k, v = rand(tokens, H, d).to(torch.bfloat16), rand(tokens, H, d).to(torch.bfloat16)
+    ctx.append_kv(k, v)
+    assert ctx.device_status() == 0
+    pad = torch.zeros(blocks * 64 - tokens, H, d, dtype=torch.bfloat16, device=cuda_device)
+    for pool, cpool, e, x in ((ctx.k_pool, ctx.kc_pool, e_k, k), (ctx.v_pool, ctx.vc_pool, e_v, v)):
+        got = cpool.view(torch.bfloat16).view(-1, H, 64, d)[:rank // 64].double().permute(1, 0, 2, 3).reshape(H, rank, d)
+        ref = torch.einsum("htr,thd->hrd", e.double(), x.double())
+        assert float((got - ref).norm()) <= BF16_REL * float(ref.norm())
+        want = torch.cat([x, pad]).view(blocks, 64, H, d).permute(0, 2, 1, 3)
+        assert torch.equal(pool.view(torch.bfloat16).view(-1, H, 64, d)[:blocks], want)
+    ref = torch.cat([k, pad]).double().view(blocks, 64, H, d).sum(1).permute(1, 0, 2)
+    # fp32 sums of 64 values: every addition rounds by 2^-24 of a partial sum of the order of the result
+    assert float((ctx.ksum.double() - ref).norm()) <= 2.0 ** -24 * 12 * float(ref.norm())
+    ctx.destroy()
+
+
 @pytest.mark.parametrize("H,n", [(1, 1), (12, 3136), (12, 4680), (16, 4680)])
 def test_page_write_takes_rows_one_by_one_or_at_once(H, n, cuda_device):
     """Contexts without a linear state: few CTAs, more than fit at once with all rows asked for, as many as fit one row at a
