@@ -142,7 +142,7 @@ bool aligned(const void* p, size_t a) { return (reinterpret_cast<uintptr_t>(p) %
 }  // namespace
 
 struct hsa_ctx {
-  unsigned long long wait_ns;  // bound of the selection kernel's grid-barrier waits
+  unsigned long long wait_ns;  // bound of waits (hsa_set_wait_limit_ns)
   hsa_config cfg;
   hsa_buffers buf;
   Layout lay;
@@ -426,6 +426,7 @@ int hsa_append_kv(hsa_ctx* ctx, const void* k, const void* v, int32_t n_tokens, 
     la.seg_tokens = ctx->cfg.lin_seg_tokens;
     la.seg_index = ctx->n_segs;
     la.nsm = ctx->nsm;
+    la.give_up = ctx->wait_ns < kNoWaitNs;
     la.status = a.status;
     e = launch_linformer_compress(la, ctx->lc_clusters, &a.one_row, ctx->tm_ek, ctx->tm_ev, maps.kin, maps.vin, static_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return cuda_fail(ctx, e);

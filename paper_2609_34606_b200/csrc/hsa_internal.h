@@ -184,6 +184,7 @@ struct CausalLinArgs {
   int32_t* status;  // device status word
 };
 
+constexpr unsigned long long kNoWaitNs = 128;  // wait limits below this: kernels give up at their first wait
 constexpr int kPageCtasPerSm = 6;  // CTAs of the page write, a row of a thread at a time, on an SM (see launch_append)
 
 struct LinformerArgs {
@@ -197,6 +198,7 @@ struct LinformerArgs {
   int32_t* ccnt;             // [H] number of valid compressed pages
   int H, rank, seg_tokens, seg_index;
   int nsm;                   // SMs of the device
+  int give_up;               // 1: the products are given up before the first (a wait limit of next to nothing)
   int32_t* status;
 };
 

@@ -107,10 +107,10 @@ linformer_compress_kernel(LinformerArgs a, const __grid_constant__ CUtensorMap t
   tc_fence_after();
   const uint32_t tmem = bars->tmem_base;
 
+  int armed = 0;  // blocks asked for (producer's lane)
   if (warp == 1) {
     // ------------------------------------------------------------------ producer (one lane)
     if (elect_one_sync()) {
-      int armed = 0;
       for (int bi = 0; bi < nblk; ++bi) {
         const int s = bi % kLcDepth;
         if (bi >= kLcDepth && !lc_wait(&bars->empty[s], ((bi / kLcDepth) - 1) & 1, bars, a.status)) break;
@@ -123,16 +123,17 @@ linformer_compress_kernel(LinformerArgs a, const __grid_constant__ CUtensorMap t
           tma_load_3d(st_x + half * (kLcTile / 2), tm_x, &bars->full[s], half * 64, h, (b_lo + bi) * kBlock);
         }
       }
-      if (armed < nblk)  // let every copy already issued land before the CTA's shared memory goes away
-        for (int s = 0; s < kLcDepth; ++s)
-          if (armed > s) mbar_wait(&bars->full[s], ((armed - 1 - s) / kLcDepth) & 1, 1u << 16);
     }
   } else if (warp == 0) {
     // ------------------------------------------------------------------ MMA issuer (one lane)
     if (elect_one_sync()) {
       constexpr uint32_t idesc = idesc_bf16_f32(128, 128, 1, 1);
       constexpr uint32_t hi = desc_hi_sw128(1024);
-      bool ok = true;
+      bool ok = a.give_up == 0;
+      if (!ok) {
+        bars->abort_flag = 1;
+        atomicCAS(a.status, 0, kDevTimeout);
+      }
       for (int bi = 0; bi < nblk && ok; ++bi) {
         const int s = bi % kLcDepth;
         ok = lc_wait(&bars->full[s], (bi / kLcDepth) & 1, bars, a.status);
@@ -149,7 +150,17 @@ linformer_compress_kernel(LinformerArgs a, const __grid_constant__ CUtensorMap t
     }
   }
   __syncwarp();
-  const bool ok = lc_wait(&bars->all_done, 0, bars, a.status);
+  lc_wait(&bars->all_done, 0, bars, a.status);
+  __syncthreads();
+  const bool ok = bars->abort_flag == 0;  // (one answer for the CTA: all_done alone does not say that every block is in)
+  if (!ok) {
+    // whoever has given up: the copies issued land before the ring is used for the sums or goes away, and the products end
+    // before TMEM goes
+    for (int s = 0; s < kLcDepth; ++s)
+      if (armed > s) mbar_wait(&bars->full[s], ((armed - 1 - s) / kLcDepth) & 1, 1u << 16);
+    if (warp == 0) mbar_wait(&bars->all_done, 0, 1u << 16);
+    __syncthreads();
+  }
   tc_fence_after();
   const int quad = warp & 3, part = warp >> 2;
   auto out_row = [&](int rr) {  // row of the compressed segment

@@ -752,6 +752,36 @@ def test_segments_at_the_edges_of_the_launch_rules(H, tokens, rank, cuda_device)
     ctx.destroy()
 
 
+@pytest.mark.parametrize("H,tokens", [(3, 300), (3, 1000), (4, 1300), (12, 3200), (1, 2100)])
+def test_compression_that_gives_up_leaves_the_context_usable(H, tokens, cuda_device):
+    """The products of the compression kernel are given up with copies in flight (a wait limit of one nanosecond; one CTA per tile
+    with fewer and more blocks than ring stages, clusters of 2, 4 and 8): it ends by itself and says so, and the segment
+    appended again is what it was."""
+    from paper_2609_34606_b200 import hsa
+    d, rank = 128, 256
+    g = torch.Generator(device=cuda_device).manual_seed(tokens)
+    rand = lambda *s: torch.randn(*s, generator=g, device=cuda_device).to(torch.bfloat16)
+    ctx = hsa.HSAContext(H, d, max_pages=(tokens + 63) // 64, max_q_tokens=tokens, max_topk=1, device=cuda_device,
+                         lin_mode=hsa.HSA_LIN_LINFORMER, lin_rank=rank, lin_seg_tokens=tokens, e_k=rand(H, tokens, rank),
+                         e_v=rand(H, tokens, rank))
+    k, v = rand(tokens, H, d), rand(tokens, H, d)
+    ctx.append_kv(k, v)
+    assert ctx.device_status() == 0
+    want = ctx.kc_pool.clone(), ctx.vc_pool.clone(), ctx.ksum.clone(), ctx.k_pool.clone()
+    ctx.set_wait_limit_ns(1)
+    for _ in range(3):
+        ctx.rewind(0)
+        ctx.append_kv(k, v)
+        assert ctx.device_status() == hsa.HSA_ERR_DEVICE_TIMEOUT
+    ctx.set_wait_limit_ns(2_000_000_000)
+    ctx.rewind(0)
+    ctx.append_kv(k, v)
+    assert ctx.device_status() == 0
+    for a, b in zip((ctx.kc_pool, ctx.vc_pool, ctx.ksum, ctx.k_pool), want):
+        assert torch.equal(a, b)
+    ctx.destroy()
+
+
 @pytest.mark.parametrize("H,n", [(1, 1), (12, 3136), (12, 4680), (16, 4680)])
 def test_page_write_takes_rows_one_by_one_or_at_once(H, n, cuda_device):
     """Contexts without a linear state: few CTAs, more than fit at once with all rows asked for, as many as fit one row at a
