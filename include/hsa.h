@@ -311,8 +311,9 @@ int hsa_device_status(hsa_ctx* ctx, int32_t* status_out);
 /* Bound, in nanoseconds, of a wait at the grid barrier of the selection kernel (the one place
  * where CTAs wait for each other; default 2e9).  When it runs out the kernel ends, the status word
  * holds HSA_ERR_DEVICE_TIMEOUT and the call's selection is empty.   Below
- * 128 ns the Linformer compression kernel, too, gives up (its waits are else bounded by a count of polls,
- * some seconds), which leaves the segment's rows undefined.  wait_ns > 0. */
+ * 128 ns two more kernels give up (their waits are else bounded by a count of polls, some seconds): the Linformer
+ * compression, which leaves the segment's rows undefined, and the sums over page groups of a causal forward, which leaves
+ * its linear branch undefined.  wait_ns > 0. */
 int hsa_set_wait_limit_ns(hsa_ctx* ctx, uint64_t wait_ns);
 
 /* Byte offsets inside the workspace, for tests and monitoring: the int32 status word, and the

@@ -663,6 +663,7 @@ int hsa_forward(hsa_ctx* ctx, const void* q, int32_t n_q, int64_t tok_stride, in
     c.relu = p.relu;
     c.nsm = ctx->nsm;
     c.alone = !do_sparse;
+    c.give_up = ctx->wait_ns < kNoWaitNs;
     c.lin_num = reinterpret_cast<float*>(ws + ctx->lay.lin_num);
     c.lin_den = reinterpret_cast<float*>(ws + ctx->lay.lin_den);
     c.status = p.status;

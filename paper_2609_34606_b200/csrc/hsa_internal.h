@@ -163,6 +163,8 @@ struct FwdParams {
   const uint8_t* v_pool;
 };
 
+constexpr unsigned long long kNoWaitNs = 128;  // wait limits below this: kernels give up at their first wait
+
 struct CausalLinArgs {
   int n_q;
   const int32_t* page_table;
@@ -179,12 +181,12 @@ struct CausalLinArgs {
   int relu;  // feature map: 0 elu(x) + 1, 1 max(x, 0)
   int nsm;    // SMs of the device
   int alone;  // 1: the forward behind it is the linear branch alone
+  int give_up;  // 1: the sums over groups are given up before the first product (a wait limit of next to nothing)
   float* lin_num;
   float* lin_den;
   int32_t* status;  // device status word
 };
 
-constexpr unsigned long long kNoWaitNs = 128;  // wait limits below this: kernels give up at their first wait
 constexpr int kPageCtasPerSm = 6;  // CTAs of the page write, a row of a thread at a time, on an SM (see launch_append)
 
 struct LinformerArgs {

@@ -277,11 +277,11 @@ chunk_sums_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_k, con
     return false;
   };
   constexpr uint32_t kColHi = 128, kColZ = 384;
+  int armed = 0;  // pages asked for (producer's lane)
   if (warp == 0) {
     if (elect_one_sync()) {
       const int64_t b0 = a.q_pos0 / kBlock + u * kClGroup;
       bool ok = true;
-      int armed = 0;
       for (int i = 0; i < kClGroup && ok; ++i) {
         const int s = i % kCsStages;
         uint8_t* st = smem + s * kStage;
@@ -296,15 +296,16 @@ chunk_sums_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_k, con
                         ((h * kClTerms + t) * a.phik_blocks + u * kClGroup + i) * kBlock);
         ++armed;
       }
-      if (!ok)  // let every copy already issued land before the CTA's shared memory goes away
-        for (int s = 0; s < kCsStages; ++s)
-          if (armed > s) mbar_wait(&bars->full[s], ((armed - 1 - s) / kCsStages) & 1, 1u << 16);
     }
   } else if (warp == 1) {
     if (elect_one_sync()) {
       constexpr uint32_t kHiSw = desc_hi_sw128(1024), idesc = idesc_bf16_f32(128, D, 1, 1), idesc_1 = idesc_bf16_f32(128, 16, 1, 0);
       const uint32_t b_ones = desc_lo_sw128(smem_u32(ones), 16);
-      bool ok = true;
+      bool ok = a.give_up == 0;
+      if (!ok) {
+        bars->abort_flag = 1;
+        atomicCAS(a.status, 0, kDevTimeout);
+      }
       for (int i = 0; i < kClGroup && ok; ++i) {
         const int s = i % kCsStages;
         ok = wait(&bars->full[s], (i / kCsStages) & 1);
@@ -324,12 +325,13 @@ chunk_sums_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_k, con
         }
         tc_commit(&bars->empty[s]);
       }
-      if (ok) tc_commit(&bars->done);
+      tc_commit(&bars->done);
     }
   } else {
     const int quad = warp & 3, r = quad * 32 + lane;
     const uint32_t row = tmem + (static_cast<uint32_t>(quad * 32) << 16);
-    if (__all_sync(0xffffffffu, wait(&bars->done, 0))) {
+    // (done alone does not say that every page is in)
+    if (__all_sync(0xffffffffu, wait(&bars->done, 0) && bars->abort_flag == 0)) {
       tc_fence_after();
       float* dst = a.sums + (static_cast<size_t>(h) * a.sum_groups + u) * kClSums;
 #pragma unroll 1
@@ -353,6 +355,14 @@ chunk_sums_kernel(CausalLinArgs a, const __grid_constant__ CUtensorMap tm_k, con
   }
   tc_fence_before();
   __syncthreads();
+  if (bars->abort_flag) {
+    // whoever has given up: the copies issued land before the CTA's shared memory goes away, and the products end before TMEM
+    // goes
+    for (int s = 0; s < kCsStages; ++s)
+      if (armed > s) mbar_wait(&bars->full[s], ((armed - 1 - s) / kCsStages) & 1, 1u << 16);
+    if (warp == 1) mbar_wait(&bars->done, 0, 1u << 16);
+  }
+  __syncwarp();
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem, 512);

@@ -125,6 +125,31 @@ def test_causal_sums_over_groups(n0, n, relu, odd, cuda_device):
     ctx.destroy()
 
 
+@pytest.mark.parametrize("H,n", [(1, 769), (12, 1560)])
+def test_causal_sums_that_give_up_leave_the_context_usable(H, n, cuda_device):
+    """The sums over page groups are given up with copies in flight (a wait limit of one nanosecond): their kernel ends by itself
+    and says so, and the next forward is what it was."""
+    from paper_2609_34606_b200 import hsa
+    d, n0 = 128, 100
+    g = torch.Generator(device=cuda_device).manual_seed(n)
+    rand = lambda *s: torch.randn(*s, generator=g, device=cuda_device).to(torch.bfloat16)
+    ctx = hsa.HSAContext(H, d, max_pages=(n0 + n + 63) // 64, max_q_tokens=n, max_topk=8, causal=True, device=cuda_device)
+    ctx.append_kv(rand(n0, H, d), rand(n0, H, d))
+    ctx.append_kv(rand(n, H, d), rand(n, H, d))
+    q = rand(n, H, d)
+    idx, cnt = ctx.select_blocks(q, torch.full((H,), 8, dtype=torch.int32, device=cuda_device), q_pos0=n0, causal=True)
+    want = ctx.forward(q, idx, cnt, q_pos0=n0, causal=True)
+    assert ctx.device_status() == 0
+    ctx.set_wait_limit_ns(1)
+    for _ in range(3):
+        ctx.forward(q, idx, cnt, q_pos0=n0, causal=True)
+        assert ctx.device_status() == hsa.HSA_ERR_DEVICE_TIMEOUT
+    ctx.set_wait_limit_ns(2_000_000_000)
+    out = ctx.forward(q, idx, cnt, q_pos0=n0, causal=True)
+    assert ctx.device_status() == 0 and torch.equal(out, want)
+    ctx.destroy()
+
+
 @pytest.mark.parametrize("n0,n,d,relu", [(0, 100, 128, 0), (100, 300, 128, 0), (70, 300, 64, 0), (64, 300, 128, 1)])
 def test_causal_not_finite_values_stay_behind_their_position(n0, n, d, relu, cuda_device):
     """Inf and NaN in K, V and queries of a causal chunk reach the rows at and behind them, and there what they
