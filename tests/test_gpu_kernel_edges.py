@@ -768,7 +768,10 @@ def test_segments_at_the_edges_of_the_launch_rules(H, tokens, rank, cuda_device)
     for pool, cpool, e, x in ((ctx.k_pool, ctx.kc_pool, e_k, k), (ctx.v_pool, ctx.vc_pool, e_v, v)):
         got = cpool.view(torch.bfloat16).view(-1, H, 64, d)[:rank // 64].double().permute(1, 0, 2, 3).reshape(H, rank, d)
         ref = torch.einsum("htr,thd->hrd", e.double(), x.double())
-        assert float((got - ref).norm()) <= BF16_REL * float(ref.norm())
+        # sums in 32 bits are off by no more than 2^-18 of the result here, rounding to bf16 by 2^-9.3 (2-norms): together
+        # hardly more than the rounding alone
+        alone = float((ref.to(torch.bfloat16).double() - ref).norm())
+        assert float((got - ref).norm()) <= (1 + 2.0 ** -8) * alone <= BF16_REL * float(ref.norm())
         want = torch.cat([x, pad]).view(blocks, 64, H, d).permute(0, 2, 1, 3)
         assert torch.equal(pool.view(torch.bfloat16).view(-1, H, 64, d)[:blocks], want)
     ref = torch.cat([k, pad]).double().view(blocks, 64, H, d).sum(1).permute(1, 0, 2)
@@ -842,4 +845,94 @@ def test_adaptive_lists_end_in_zeros(n, group, cuda_device):
     assert torch.equal(dirty, idx) and torch.equal(counts, cnt)
     behind = torch.arange(idx.shape[2], device=cuda_device) >= cnt[:, :, None]
     assert int(idx[behind].abs().sum()) == 0 and bool(behind.any()) and int(cnt.min()) > 0
+    ctx.destroy()
+
+
+def _causal_branches(q, K, V, n0, idx, cnt, group, relu):
+    """Both branches of a causal forward in 64 bits on the device, [n, H, d] each: q and the chunk start at position n0."""
+    n, H, d = q.shape
+    lin, sp = torch.empty(n, H, d, dtype=torch.float64, device=q.device), torch.empty(n, H, d, dtype=torch.float64, device=q.device)
+    phi = lambda x: x.clamp(min=0) if relu else torch.where(x > 0, x + 1, x.exp())
+    seen = torch.arange(K.shape[0], device=q.device)[None] <= n0 + torch.arange(n, device=q.device)[:, None]
+    for h in range(H):
+        qh, kh, vh = q[:, h].double(), K[:, h].double(), V[:, h].double()
+        A = (phi(qh) @ phi(kh).T) * seen
+        lin[:, h] = A @ vh / (A.sum(1, keepdim=True) + (1e-6 if relu else 0.0))
+        chosen = torch.zeros_like(seen)
+        for g in range(cnt.shape[1]):
+            rows = slice(g * group, (g + 1) * group) if group else slice(0, n)
+            for b in idx[h, g, :int(cnt[h, g])].tolist():
+                chosen[rows, 64 * b:64 * b + 64] = True
+        s = (qh @ kh.T * d ** -0.5).masked_fill(~(seen & chosen), -torch.inf)
+        sp[:, h] = torch.softmax(s, 1) @ vh
+    return lin, sp
+
+
+@pytest.mark.parametrize("H,n0,n,topk,group,relu", [
+    (2, 70, 769, -1, 0, 0), (12, 33, 1560, 6, 0, 0), (12, 100, 1500, 9, 128, 0), (16, 64, 1153, 4, 0, 1), (12, 640, 896, 8, 0, 0)])
+def test_causal_chunks_of_many_tiles_with_both_branches(H, n0, n, topk, group, relu, cuda_device):
+    """Terms, sums over page groups or steps through all pages, products, and the forward that takes the partials as tiles, more
+    than one wave of them: few items (clusters), 156 and 160 items, lists per query tile, against 64 bits."""
+    from paper_2609_34606_b200 import hsa
+    d = 128
+    g = torch.Generator(device=cuda_device).manual_seed(n)
+    K, V, q = (torch.randn(m, H, d, generator=g, device=cuda_device).to(torch.bfloat16) for m in (n0 + n, n0 + n, n))
+    blocks = (n0 + n + 63) // 64
+    ctx = hsa.HSAContext(H, d, max_pages=blocks, max_q_tokens=n, max_topk=blocks, causal=True, device=cuda_device, feature_map=relu,
+                         page_order=torch.arange(blocks - 1, -1, -1, dtype=torch.int32))
+    ctx.k_pool.fill_(0xFF)
+    ctx.v_pool.fill_(0xFF)
+    ctx.append_kv(K[:n0], V[:n0])
+    ctx.append_kv(K[n0:], V[n0:])
+    idx, cnt = ctx.select_blocks(q, torch.full((H,), topk, dtype=torch.int32, device=cuda_device), q_pos0=n0, causal=True, group_tokens=group)
+    idx[:, :, 0] = 0  # (the first block is one every query sees, so that no row is without a key)
+    cnt.clamp_(min=1)
+    out = ctx.forward(q, idx, cnt, q_pos0=n0, causal=True, group_tokens=group).double()
+    assert ctx.device_status() == 0
+    lin, sp = _causal_branches(q, K, V, n0, idx, cnt, group, relu)
+    # (the sparse branch's weights are bf16 as well as the result: two roundings, one of them of a sum's terms)
+    assert float((out - lin - sp).norm()) <= 1.5 * BF16_REL * float((lin + sp).norm())
+    ctx.destroy()
+
+
+@pytest.mark.parametrize("hot", [False, True])
+@pytest.mark.parametrize("gates", ["none", "sigmoid per head", "raw per head", "sigmoid strided per dim"])
+@pytest.mark.parametrize("group", [0, 128])
+def test_causal_partials_as_tiles(group, gates, hot, cuda_device):
+    """The causal partials as tiles beside every form of gate that is none itself, in lists split over a cluster and in whole ones
+    (per query tile), and where a tile is done again with a running maximum and asks for its partials a second time."""
+    from paper_2609_34606_b200 import hsa
+    H, d, n0, n = 2, 128, 58 * 64, 150
+    g = torch.Generator(device=cuda_device).manual_seed(len(gates))
+    rand = lambda *s: torch.randn(*s, generator=g, device=cuda_device).to(torch.bfloat16)
+    K, V, q = rand(n0 + n, H, d), rand(n0 + n, H, d), rand(n, H, d)
+    if hot:
+        K[30 * 64:32 * 64] *= 24  # scores far above those of the blocks in front
+        q *= 4
+    ctx = hsa.HSAContext(H, d, max_pages=61, max_q_tokens=n0, max_topk=50, causal=True, device=cuda_device,
+                         gate_act=0 if gates == "raw per head" else 1)
+    ctx.append_kv(K[:n0], V[:n0])
+    ctx.append_kv(K[n0:], V[n0:])
+    idx, cnt = ctx.alloc_selection(n, group)
+    idx[:, :] = torch.arange(50) + 8
+    cnt.fill_(50)
+    gl = gs = None
+    if gates == "sigmoid strided per dim":
+        gl, gs = rand(n, H, 2 * d)[:, :, ::2], rand(n, H, 2 * d)[:, :, ::2]
+    elif gates != "none":
+        gl, gs = rand(n, H), rand(n, H)
+    ctx.safe_pass_tiles()
+    out = ctx.forward(q, idx, cnt, q_pos0=n0, causal=True, group_tokens=group, g_lin=gl, g_sp=gs).double()
+    assert (ctx.safe_pass_tiles() > 0) == hot and ctx.device_status() == 0
+    lin, sp = _causal_branches(q, K, V, n0, idx, cnt, group, 0)
+
+    def weight(x):
+        if x is None:
+            return 1.0
+        x = x.double() if x.dim() == 3 else x.double()[:, :, None]
+        return x if gates == "raw per head" else torch.sigmoid(x)
+
+    a, b = weight(gl) * lin, weight(gs) * sp
+    # (hot rows are peaked: a weight is one bf16 rounding, and so is the result)
+    assert float((out - a - b).norm()) <= 2 * BF16_REL * float((a.square() + b.square()).sum().sqrt())
     ctx.destroy()
