@@ -456,14 +456,15 @@ def bench_ours(args, rank: int, world: int):
             "clocks": clocks,
             "e2e": {"value": agg_e2e / 1e12, "unit": UNIT, "ms_per_step": ms_e2e,
                     "h2d_bytes_per_step": 3 * w.Lq * w.H * w.d * 2, "d2h_bytes_per_step": w.Lq * w.H * w.d * 2},
-            # per step: append_fused, state_reduce, hsa_forward and the selection -- two kernels (query
-            # sums, then one cluster per head) for one list per head while a head has at most 192
-            # score items of 32 blocks, one cooperative kernel otherwise
-            "gpu_launches": (5 if (args.group_tokens == 0 and w.n_blocks <= 192 * 32) else 4) * K,
+            # per step: append_fused, state_reduce, hsa_forward and the selection -- for one list per head two
+            # kernels (query sums, then one cluster per head) while a head has at most 192 score items of 32
+            # blocks, one cooperative kernel beyond that; three kernels (query sums, scores, lists) for several
+            # lists per head
+            "gpu_launches": (6 if 0 < args.group_tokens < w.Lq else 5 if w.n_blocks <= 192 * 32 else 4) * K,
             # (the Linformer form has as many: page write + projection instead of the fused append and
             # its reduction, one forward launch that walks the compressed pool before the selected pages)
             "device_status": status,
-            "roofline": {"kernel": "hsa_forward_kernel<128, 0, false, false>", "bound": "tensor", "achieved": fwd_tf,
+            "roofline": {"kernel": "hsa_forward_kernel<128, 0, false, 0>", "bound": "tensor", "achieved": fwd_tf,
                          "peak": peaks["bf16_tflops"], "unit": "TFLOP/s", "frac": fwd_tf / peaks["bf16_tflops"],
                          "traffic": ncu_traffic(w.name), "algorithmic_bytes": by["forward"],
                          "peak_source": peaks["source"] + " (burst)",

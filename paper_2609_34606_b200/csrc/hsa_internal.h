@@ -232,7 +232,8 @@ cudaError_t launch_select_adaptive(const SelectArgs& a, const AdaptiveArgs& ad, 
 // tm_kc / tm_vc: maps of the compressed pools, used when p.lf_table is set (else null); tm_gl / tm_gs: maps
 // of per-dim gate logits with the geometry of tm_q (null: no such gate, or its strides do not allow one); tm_num: map
 // of p.lin_num, box 32 dims x 1 x 128 tokens (head_dim 128, may be null).  (Read by the rows' threads, 64 bytes of lines
-// 6 KB apart at a time, the partials took 4 to 6 us of each tile, 12 heads of 128, 1560 tokens; as a tile 2.)
+// 6 KB apart at a time, the partials took 4 to 6 us of each tile, 12 heads of 128, 1560 tokens; as a tile 2.  Beside per-dim
+// gate tiles, in lists split through the workspace and at head_dim 64 they still are.)
 cudaError_t launch_forward(const FwdParams& p, int D, const CUtensorMap& tm_q,
                            const CUtensorMap& tm_k, const CUtensorMap& tm_v,
                            const CUtensorMap& tm_state, const CUtensorMap& tm_out, cudaStream_t st,

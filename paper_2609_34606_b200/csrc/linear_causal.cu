@@ -11,7 +11,7 @@
 // In chunks of enough query tiles (sums_pay; head_dim 128) a tile does not walk through all of the chunk's pages in front of it:
 // chunk_sums_kernel leaves T = sum_j phi(k_j) v_j^T and z = sum_j phi(k_j) over every group of four pages (two tiles)
 // in the workspace, and a tile takes phi(Q) times the sum of T over the groups before its own, then the pages from
-// its group's first on, at most five.
+// its group's first on, at most five.  At head_dim 64 a tile always walks through all of them.
 //
 // One CTA per (128-row query tile, head), 576 threads:
 //   warp 0       TMA producer: Q tile, then, page by page up to the tile's diagonal, phi(K) and V (64 keys per
